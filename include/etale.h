@@ -228,10 +228,11 @@ etale_status etale_search_eval_count(etale_index *idx, const float *queries, uin
 /* Exact k nearest live nodes by brute force (measurement support for
  * Recall@10, Sec. 5.2): canonical fp32 distances, ties by smaller id.  k must
  * be 1..32.  Unless cfg.gt = 1, a tensor-core pass (bf16 inputs, fp32
- * accumulation; a hi/lo split when the data are not exact in bf16) keeps 32
- * candidates per query, which are reranked with the canonical distance; a
- * query whose result an a-priori error bound cannot certify is recomputed
- * on CUDA cores, so the output never depends on the path taken.            */
+ * accumulation; a hi/lo split when the data are not exact in bf16) gives
+ * approximate distances, and every row that an a-priori error bound on them
+ * cannot exclude is scored with the canonical distance; a query for which
+ * the bound excludes too little is recomputed on CUDA cores, so the output
+ * never depends on the path taken.                                         */
 etale_status etale_ground_truth(etale_index *idx, const float *queries, uint64_t nq,
                                 uint32_t k, uint32_t *out_ids, float *out_dists, void *stream);
 

@@ -1065,7 +1065,7 @@ static etale_status ground_truth_run(etale_index *idx, const Dev &d, const float
         }
         {
             PhaseScope ps(idx, ETALE_PH_GT_MERGE, st);
-            CK(launch_gt_rerank(d, qpad, q0, g, k, p, b, idx->next_id, oid, od, st), "ground truth (rerank)");
+            CK(launch_gt_rerank(d, qpad, q0, g, k, p, b, idx->next_id, oid, od, idx->num_sms, st), "ground truth (rerank)");
         }
         g_kernel_launches += 2;
     }

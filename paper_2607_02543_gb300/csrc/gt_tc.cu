@@ -19,16 +19,16 @@
 //      accumulator; eight epilogue warps read it with tcgen05.ld and write,
 //      per query and per block of 32 rows, the smallest approximate key
 //      key = |x|^2 - 2 q.x (L2) or -q.x (IP); dead rows have key +inf.
-//   3. gt_rerank_kernel (a warp per query): tau = the 32nd smallest block
-//      minimum (or the 2k-th for k > 16); every row of every block whose
-//      minimum is <= tau is reranked with the canonical fp32 distance (the
-//      same definition the rest of the index uses) into the top k.  Rows
-//      left out have approximate keys > tau; an a-priori bound E on
-//      |approximate - canonical| certifies that none of them can beat the
-//      k-th reranked distance.  Queries that fail the certificate (or have
-//      more than 256 candidate blocks) are recomputed by the CUDA-core exact
-//      kernel, so the result is always the exact top-k with canonical
-//      distances, ties by smaller id.
+//   3. gt_rerank_kernel: every row of the k blocks with the smallest minima
+//      is scored with the canonical fp32 distance (the same definition the
+//      rest of the index uses).  The k-th of these distances bounds the
+//      answer: an a-priori bound E on |approximate - canonical| turns it into
+//      a threshold T on approximate keys that no row of the top k can exceed,
+//      and the rows of the remaining blocks with a minimum <= T are scored
+//      too.  So the result is always the exact top-k with canonical
+//      distances, ties by smaller id.  Queries without a finite threshold
+//      (infinities or NaN in the data), or whose T admits more than half of
+//      all blocks, go to the CUDA-core exact kernel.
 #include <cuda.h>
 #include <cudaTypedefs.h>
 #include <cuda_bf16.h>
@@ -494,12 +494,13 @@ __global__ void gt_prep_queries(const float *q, u32 mp, u32 dim, u32 nq, u32 kp1
     }
 }
 
-// ---- the certificate ----------------------------------------------------------
-// Lower bound on the canonical fp32 distance of every row whose approximate
-// key exceeds LB.  qs: |q|^2, |q|, |lo_q|, |e_q| of the query; gs: max |x|^2,
-// max |lo_x|, max |e_x| over the rows (fp32 bits).  K = contracted length.
-__device__ double key_lower_bound(int metric, double m, double K, bool split, const float *qs, const u32 *gs,
-                                  double LB) {
+// ---- the error bound ----------------------------------------------------------
+// E, the most by which an approximate key can differ from |canonical distance
+// - |q|^2| (L2) or from canonical distance - 1 (IP), doubled for safety, up to
+// the factor 1 - 2 (m + 4) u of the L2 form below.  qs: |q|^2, |q|, |lo_q|,
+// |e_q| of the query; gs: max |x|^2, max |lo_x|, max |e_x| over the rows (fp32
+// bits).  K = contracted length.
+__device__ double key_error(int metric, double m, double K, bool split, const float *qs, const u32 *gs) {
     const double u = 1.0 / 16777216.0;
     const double qn = qs[0], qa = (double)qs[1] * 1.01, loq = (double)qs[2] * 1.01, eq = (double)qs[3] * 1.01;
     const double X2 = __uint_as_float(gs[0]), X1 = sqrt(X2) * 1.01;
@@ -507,24 +508,35 @@ __device__ double key_lower_bound(int metric, double m, double K, bool split, co
     // |computed dot - q.x|: the terms the split leaves out, plus fp32 accumulation
     const double dot_res = split ? loq * Lx + (qa + eq) * Ex + eq * (X1 + Ex) : 0.0;
     const double dot_err = dot_res + (K + 2.0) * 2.0 * u * 1.03 * qa * X1;
-    if (metric == 0) {
-        // norms (fp32 sums of squares), 2 x dot error, rounding of the key
-        const double E = 2.0 * ((m + 2.0) * u * qn * 1.01 + (m + 2.0) * u * X2 + 2.0 * dot_err +
-                                2.0 * u * (X2 + 2.1 * qa * X1));
-        const double y = qn + LB - E;
-        // the canonical fp32 distance is within (m + 4) u of the exact one
-        return y > 0.0 ? y * (1.0 - 2.0 * (m + 4.0) * u) : -1.0;
-    }
-    const double E = 2.0 * (dot_err + (m + 2.0) * u * qa * X1 + u * (1.0 + qa * X1));
-    return 1.0 + LB - E;
+    if (metric == 0)   // norms (fp32 sums of squares), 2 x dot error, rounding of the key
+        return 2.0 * ((m + 2.0) * u * qn * 1.01 + (m + 2.0) * u * X2 + 2.0 * dot_err + 2.0 * u * (X2 + 2.1 * qa * X1));
+    return 2.0 * (dot_err + (m + 2.0) * u * qa * X1 + u * (1.0 + qa * X1));
+}
+// Lower bound on the canonical fp32 distance of every row whose approximate
+// key exceeds LB.
+__device__ double key_lower_bound(int metric, double m, double K, bool split, const float *qs, const u32 *gs,
+                                  double LB) {
+    const double E = key_error(metric, m, K, split, qs, gs);
+    if (metric != 0) return 1.0 + LB - E;
+    const double y = (double)qs[0] + LB - E;
+    // the canonical fp32 distance is within (m + 4) u of the exact one
+    return y > 0.0 ? y * (1.0 - 2.0 * (m + 4.0) / 16777216.0) : -1.0;
+}
+// The inverse: no row with a canonical distance <= dk has an approximate key
+// above the returned value.
+__device__ double key_upper_bound(int metric, double m, double K, bool split, const float *qs, const u32 *gs,
+                                  double dk) {
+    const double E = key_error(metric, m, K, split, qs, gs);
+    if (metric != 0) return dk - 1.0 + E;
+    return dk / (1.0 - 2.0 * (m + 4.0) / 16777216.0) - (double)qs[0] + E;
 }
 
-// ---- threshold, exact rerank, certificate -------------------------------
-constexpr int RR_MAXB = 256;      // candidate blocks a query may keep
+// ---- threshold and exact rerank -----------------------------------------------
 constexpr int RR_WARPS = 8;
+constexpr int RR_LIST = 256;      // candidate blocks a warp collects before it scores them
 
 struct RerankArgs {
-    u32 nq, q0, k, nblk, rt, m, kprime, split;
+    u32 nq, q0, k, nblk, m, kprime, split;
     u64 n_rows;
     const float *q;       // all queries, nq_total x mp fp32
     const float *bmin;    // this group: nq x nblk
@@ -537,101 +549,251 @@ struct RerankArgs {
     const u32 *err;       // candidate pass error word: nonzero = minima incomplete
 };
 
+// canon_dist<8> of two rows against one query row (global memory), the column
+// blocks outermost: eight row loads in flight, the query's read once for both.
+// The same operations in the same order as canon_dist<8>.
+__device__ __forceinline__ void canon_dist_wide2(const float *__restrict__ q, const float *__restrict__ r0,
+                                                 const float *__restrict__ r1, int mp, int metric, int g, float &d0,
+                                                 float &d1) {
+    float p0[4], p1[4];
+#pragma unroll
+    for (int t = 0; t < 4; t++) p0[t] = p1[t] = 0.0f;
+    auto fold = [&](float acc, const float4 &u, const float4 &v) {
+        if (metric == 0) {
+            const float e0 = __fsub_rn(u.x, v.x), e1 = __fsub_rn(u.y, v.y);
+            const float e2 = __fsub_rn(u.z, v.z), e3 = __fsub_rn(u.w, v.w);
+            return __fmaf_rn(e3, e3, __fmaf_rn(e2, e2, __fmaf_rn(e1, e1, __fmaf_rn(e0, e0, acc))));
+        }
+        return __fmaf_rn(u.w, v.w, __fmaf_rn(u.z, v.z, __fmaf_rn(u.y, v.y, __fmaf_rn(u.x, v.x, acc))));
+    };
+    for (int base = 0; base < mp; base += 128) {
+        float4 u[4], v[4], w[4];
+#pragma unroll
+        for (int t = 0; t < 4; t++) {
+            const int i = base + 4 * (g + 8 * t);
+            if (i < mp) {
+                v[t] = *reinterpret_cast<const float4 *>(r0 + i);
+                w[t] = *reinterpret_cast<const float4 *>(r1 + i);
+                u[t] = *reinterpret_cast<const float4 *>(q + i);
+            }
+        }
+#pragma unroll
+        for (int t = 0; t < 4; t++)
+            if (base + 4 * (g + 8 * t) < mp) {
+                p0[t] = fold(p0[t], u[t], v[t]);
+                p1[t] = fold(p1[t], u[t], w[t]);
+            }
+    }
+    float s0 = __fadd_rn(__fadd_rn(p0[0], p0[2]), __fadd_rn(p0[1], p0[3]));
+    float s1 = __fadd_rn(__fadd_rn(p1[0], p1[2]), __fadd_rn(p1[1], p1[3]));
+#pragma unroll
+    for (int h = 4; h >= 1; h >>= 1) {
+        s0 = __fadd_rn(s0, __shfl_xor_sync(FULL, s0, h));
+        s1 = __fadd_rn(s1, __shfl_xor_sync(FULL, s1, h));
+    }
+    d0 = metric == 0 ? s0 : __fsub_rn(1.0f, s0);
+    d1 = metric == 0 ? s1 : __fsub_rn(1.0f, s1);
+}
+
+// Bound by the row reads (L2) and their latency.  Scoring what the k-th
+// distance leaves open, instead of a fixed 32 blocks with a certificate and a
+// full scan by gt_kernel where it fails: 10k queries x 300k x 128 integer rows
+// 0.97 -> 0.73 ms; 2,003 queries x 40k x 960 real-valued rows, all of which
+// failed the certificate, 53.5 -> 21.5 ms.
+// W warps per query (1 or 8): a block per query below 16 queries an SM, where
+// a warp per query would leave the SMs' slots empty.  Each lane keeps the four smallest minima of the
+// blocks it reads, with their numbers, so that a threshold met by at most four
+// blocks of any lane needs no second pass over the minima.
+template <int W>
 __global__ void __launch_bounds__(RR_WARPS * 32) gt_rerank_kernel(Dev d, RerankArgs a) {
-    __shared__ u32 cblk[RR_WARPS][RR_MAXB];
+    __shared__ u32 clist[RR_WARPS][RR_LIST];
+    __shared__ u64 ckey[RR_WARPS][32];
+    __shared__ u64 xbest[RR_WARPS][32];
+    __shared__ u32 xsum[2][RR_WARPS];
     const int warp = threadIdx.x >> 5, lane = lane_id();
-    const u32 li = blockIdx.x * RR_WARPS + warp;
-    if (li >= a.nq || *a.err) return;
+    const int tw = warp % W;                         // this warp's place among the query's warps
+    const u32 li = blockIdx.x * (RR_WARPS / W) + warp / W;
+    if (li >= a.nq || *a.err) return;                // the same for every warp of a query
     const u32 qi = a.q0 + li;
-    const float *row = a.bmin + (size_t)li * a.nblk;
-    // 1. each lane keeps the four smallest block minima of blocks lane, lane + 32, ...
-    u32 t0 = ~0u, t1 = ~0u, t2 = ~0u, t3 = ~0u;
-    for (u32 b = lane; b < a.nblk; b += 32) {
-        const u32 v = f2ord(__ldg(row + b));
+    const float *row = a.bmin + (size_t)li * a.nblk; // nblk is a multiple of 8
+    u32 parity = 0;
+    auto team_sum = [&](u32 v) -> u32 {
+        v = __reduce_add_sync(FULL, v);
+        if (W == 1) return v;
+        if (lane == 0) xsum[parity][warp] = v;
+        __syncthreads();
+        u32 s = 0;
+#pragma unroll
+        for (int w = 0; w < RR_WARPS; w++) s += xsum[parity][w];
+        parity ^= 1;
+        return s;
+    };
+    // 1. the four smallest minima of this lane's blocks
+    u32 t0 = ~0u, t1 = ~0u, t2 = ~0u, t3 = ~0u, b0 = 0, b1 = 0, b2 = 0, b3 = 0;
+    auto keep = [&](float f, u32 b) {
+        const u32 v = f2ord(f);
         if (v < t3) {
             if (v < t2) {
-                t3 = t2;
+                t3 = t2; b3 = b2;
                 if (v < t1) {
-                    t2 = t1;
-                    if (v < t0) { t1 = t0; t0 = v; } else t1 = v;
-                } else t2 = v;
-            } else t3 = v;
+                    t2 = t1; b2 = b1;
+                    if (v < t0) { t1 = t0; b1 = b0; t0 = v; b0 = b; } else { t1 = v; b1 = b; }
+                } else { t2 = v; b2 = b; }
+            } else { t3 = v; b3 = b; }
+        }
+    };
+    const u32 step = W * 128;
+    const float4 none = make_float4(__int_as_float(0x7fffffff), __int_as_float(0x7fffffff), __int_as_float(0x7fffffff),
+                                    __int_as_float(0x7fffffff));
+    for (u32 b = (u32)(tw * 32 + lane) * 4; b < a.nblk; b += 4 * step) {
+        float4 v[4];
+#pragma unroll
+        for (int u = 0; u < 4; u++)
+            v[u] = b + u * step < a.nblk ? __ldg(reinterpret_cast<const float4 *>(row + b + u * step)) : none;
+#pragma unroll
+        for (int u = 0; u < 4; u++) {
+            const u32 bb = b + u * step;
+            keep(v[u].x, bb);
+            keep(v[u].y, bb + 1);
+            keep(v[u].z, bb + 2);
+            keep(v[u].w, bb + 3);
         }
     }
-    // 2. tau = the rt-th smallest of the 128 kept values (bitwise search on
-    //    the order-preserving integer image); at least rt blocks have a
-    //    minimum <= tau
+    // 2. tau = the k-th smallest kept minimum (bitwise search on the
+    //    order-preserving integer image): at least k blocks are <= tau, and
+    //    each holds a live row
     u32 tau = 0;
     for (int bit = 31; bit >= 0; bit--) {
         const u32 tr = tau | (1u << bit);
-        const u32 c = (u32)(t0 < tr) + (u32)(t1 < tr) + (u32)(t2 < tr) + (u32)(t3 < tr);
-        if (__reduce_add_sync(FULL, c) < a.rt) tau = tr;
+        if (team_sum((u32)(t0 < tr) + (u32)(t1 < tr) + (u32)(t2 < tr) + (u32)(t3 < tr)) < a.k) tau = tr;
     }
-    // 3. candidate blocks: minimum <= tau (dead-only blocks have +inf)
-    u32 cnt = 0;
-    for (u32 b0 = 0; b0 < a.nblk; b0 += 32) {
-        const u32 b = b0 + lane;
-        const u32 v = b < a.nblk ? f2ord(__ldg(row + b)) : ~0u;
-        const bool c = v <= tau && v < ORD_INF;
-        const u32 m = __ballot_sync(FULL, c);
-        const u32 pos = cnt + __popc(m & lanemask_lt());
-        if (c && pos < RR_MAXB) cblk[warp][pos] = b;
-        cnt += __popc(m);
-    }
-    __syncwarp();
-    const bool over = cnt > RR_MAXB;
-    // 4. exact rerank of every live row of the candidate blocks
-    u64 best = KEY_INF;   // sorted across lanes
     const float *qv = a.q + (size_t)qi * d.mp;
     const int grp = lane >> 3, g = lane & 7;
-    for (u32 i = 0; i < (over ? 0u : cnt); i++) {
-        const u32 b = cblk[warp][i];
-        if (lane == 0 && i + 1 < cnt) {
-            // the next candidate block's rows on their way to L2
-            const u64 r0 = (u64)cblk[warp][i + 1] * 32u;
-            const u64 nr = min((u64)32, a.n_rows - r0);
-            bulk_prefetch_l2(d.x + r0 * d.mp, (u32)(nr * d.mp * 4u));
-        }
-        u64 cand = KEY_INF;
-        for (int r0 = 0; r0 < 32; r0 += 4) {
-            const u32 id = b * 32 + r0 + grp;
-            const bool inr = id < a.n_rows;
-            bool live = false;
-            if (inr) {
-                const u64 rf = d.ref[id];
-                live = !ref_del(rf) && ref_slab(rf) != NIL;
+    float4 qr[4];
+    if (d.mp <= 128) canon_row_q8(qv, (int)d.mp, g, qr);
+    u64 top = KEY_INF;    // the query's 32 smallest keys, sorted across lanes
+    u64 bound = KEY_INF;  // keys above it cannot be in the top k
+    bool cert = true;     // the rows not scored cannot be either
+    // 3. phase 0: the blocks with a minimum <= tau (dead-only blocks have
+    //    +inf); phase 1: those that the k-th distance found does not exclude
+    u32 lo = 0, hi = min(tau, ORD_INF - 1);
+    for (int phase = 0; phase < 2; phase++) {
+        auto in = [&](u32 v) { return v > lo && v <= hi; };
+        const bool kept = !__any_sync(FULL, t3 <= hi);   // every block in (lo, hi] is among the kept ones
+        if (phase == 1) {
+            u32 cnt = 0;
+            if (kept) {
+                cnt = (u32)in(t0) + (u32)in(t1) + (u32)in(t2) + (u32)in(t3);
+            } else {
+                for (u32 b = (u32)(tw * 32 + lane) * 4; b < a.nblk; b += step) {
+                    const float4 v = __ldg(reinterpret_cast<const float4 *>(row + b));
+                    cnt += (u32)in(f2ord(v.x)) + (u32)in(f2ord(v.y)) + (u32)in(f2ord(v.z)) + (u32)in(f2ord(v.w));
+                }
             }
-            // every lane computes (the distance shuffles over the full warp)
-            const float dd = canon_dist_wide<8>(qv, d.x + (size_t)(inr ? id : 0u) * d.mp, (int)d.mp, (int)d.metric, g);
-            const u64 kk = live ? mkkey(dd, id) : KEY_INF;
-#pragma unroll
-            for (int t = 0; t < 4; t++) {
-                const u64 v = __shfl_sync(FULL, kk, t * 8);
-                if (lane == r0 + t) cand = v;
-            }
+            const u32 all = team_sum(cnt);
+            if (all == 0) break;
+            cert = all <= max(64u, a.nblk / 2);
+            if (!cert) break;
         }
-        cand = warp_sort32(cand);
-        const u64 rev = __shfl_sync(FULL, cand, 31 - lane);
-        best = warp_sort32(best < rev ? best : rev);
+        u64 best = KEY_INF;   // this warp's 32 smallest keys of the phase
+        u32 cur = (u32)tw * 128;
+        for (bool more = true; more;) {
+            u32 pend = 0;
+            auto collect = [&](u32 v, u32 b) {
+                const bool c = in(v);
+                const u32 m = __ballot_sync(FULL, c);
+                if (c) clist[warp][pend + __popc(m & lanemask_lt())] = b;
+                pend += __popc(m);
+            };
+            if (kept) {
+                collect(t0, b0);
+                collect(t1, b1);
+                collect(t2, b2);
+                collect(t3, b3);
+                more = false;
+            } else {
+                for (; cur < a.nblk && pend <= RR_LIST - 128; cur += step) {
+                    const u32 b = cur + 4 * lane;
+                    const float4 v = b < a.nblk ? __ldg(reinterpret_cast<const float4 *>(row + b)) : none;
+                    collect(f2ord(v.x), b);
+                    collect(f2ord(v.y), b + 1);
+                    collect(f2ord(v.z), b + 2);
+                    collect(f2ord(v.w), b + 3);
+                }
+                more = cur < a.nblk;
+            }
+            __syncwarp();
+            for (u32 i = 0; i < pend; i++) {
+                const u32 id0 = clist[warp][i] * 32u;
+                if (lane == 0 && i + 1 < pend) {
+                    // the next candidate block's rows on their way to L2
+                    const u64 r0 = (u64)clist[warp][i + 1] * 32u;
+                    bulk_prefetch_l2(d.x + r0 * d.mp, (u32)(min((u64)32, a.n_rows - r0) * d.mp * 4u));
+                }
+                const int nr = (int)min((u64)32, a.n_rows - id0);
+                bool live = false;
+                if (lane < nr) {
+                    const u64 rf = d.ref[id0 + lane];
+                    live = !ref_del(rf) && ref_slab(rf) != NIL;
+                }
+                for (int r0 = 0; r0 < nr; r0 += 8) {
+                    // every lane computes (the distance shuffles over the full warp)
+                    const int ra = min(r0 + grp, nr - 1), rb = min(r0 + 4 + grp, nr - 1);
+                    const float *xa = d.x + (size_t)(id0 + ra) * d.mp, *xb = d.x + (size_t)(id0 + rb) * d.mp;
+                    float da, db;
+                    if (d.mp <= 128) {
+                        float4 va[4], vb[4];
+                        canon_row_q8(xa, (int)d.mp, g, va);
+                        canon_row_q8(xb, (int)d.mp, g, vb);
+                        da = canon_dist_q8v(qr, va, (int)d.mp, (int)d.metric, g);
+                        db = canon_dist_q8v(qr, vb, (int)d.mp, (int)d.metric, g);
+                    } else {
+                        canon_dist_wide2(qv, xa, xb, (int)d.mp, (int)d.metric, g, da, db);
+                    }
+                    if (g == 0) {
+                        ckey[warp][r0 + grp] = mkkey(da, id0 + ra);
+                        ckey[warp][r0 + 4 + grp] = mkkey(db, id0 + rb);
+                    }
+                }
+                __syncwarp();
+                u64 cand = live ? ckey[warp][lane] : KEY_INF;
+                __syncwarp();
+                // merge only when a key can still enter the top k
+                const u64 kth = __shfl_sync(FULL, best, (int)a.k - 1);
+                if (!__any_sync(FULL, cand < kth && cand < bound)) continue;
+                cand = warp_sort32(cand);
+                const u64 rev = __shfl_sync(FULL, cand, 31 - lane);
+                best = warp_sort32(best < rev ? best : rev);
+            }
+            __syncwarp();
+        }
+        // join the warps' lists
+        if (W > 1) {
+            xbest[warp][lane] = best;
+            __syncthreads();
+        }
+        for (int w = 0; w < W; w++) {
+            const u64 o = W > 1 ? xbest[w][31 - lane] : __shfl_sync(FULL, best, 31 - lane);
+            top = warp_sort32(top < o ? top : o);
+        }
+        if (W > 1) __syncthreads();
+        if (phase == 1 || tau >= ORD_INF) break;     // tau: every live row was scored
+        bound = __shfl_sync(FULL, top, (int)a.k - 1);
+        double T = __longlong_as_double(0x7ff0000000000000ll);
+        if (bound != KEY_INF)
+            T = key_upper_bound((int)d.metric, a.m, a.kprime, a.split != 0, a.qstat + 4 * (size_t)qi, a.gstat,
+                                (double)key_rho(bound));
+        const float Tf = __fadd_rn(__double2float_ru(T), 0.0f);   // +0 for -0: a minimum of +0 is not above it
+        cert = isfinite(Tf);
+        lo = hi;
+        hi = cert ? f2ord(Tf) : 0u;
+        if (!cert || hi <= lo) break;
     }
-    // 5. certificate: every row left out has an approximate key > tau
-    const u64 kth = __shfl_sync(FULL, best, a.k - 1);
-    bool cert;
-    if (over) {
-        cert = false;
-    } else if (tau >= ORD_INF) {
-        cert = true;                                  // every live row was reranked
-    } else if (kth == KEY_INF) {
-        cert = false;
-    } else {
-        const double lb = key_lower_bound((int)d.metric, a.m, a.kprime, a.split != 0, a.qstat + 4 * (size_t)qi,
-                                          a.gstat, (double)ord2f(tau));
-        cert = (double)key_rho(kth) < lb;
-    }
+    if (W > 1 && tw != 0) return;
     if (cert) {
         if (lane < (int)a.k) {
-            a.out_ids[(size_t)qi * a.k + lane] = best == KEY_INF ? NIL : key_id(best);
-            a.out_dist[(size_t)qi * a.k + lane] = best == KEY_INF ? __int_as_float(0x7f800000) : key_rho(best);
+            a.out_ids[(size_t)qi * a.k + lane] = top == KEY_INF ? NIL : key_id(top);
+            a.out_dist[(size_t)qi * a.k + lane] = top == KEY_INF ? __int_as_float(0x7f800000) : key_rho(top);
         }
     } else if (lane == 0) {
         a.fb[atomicAdd(a.fb_count, 1u)] = qi;
@@ -902,13 +1064,12 @@ cudaError_t launch_gt_tc(const Dev &d, u32 q0, u32 nq, const GtTcPlan &p, const 
 }
 
 cudaError_t launch_gt_rerank(const Dev &d, const float *q, u32 q0, u32 nq, u32 k, const GtTcPlan &p,
-                             const GtTcBufs &b, u64 next_id, u32 *out_ids, float *out_dist, cudaStream_t st) {
+                             const GtTcBufs &b, u64 next_id, u32 *out_ids, float *out_dist, int num_sms, cudaStream_t st) {
     RerankArgs r{};
     r.nq = nq;
     r.q0 = q0;
     r.k = k;
     r.nblk = p.nblk;
-    r.rt = k <= 16 ? 32 : 2 * k;
     r.m = d.dim;
     r.kprime = p.kprime;
     r.split = p.split;
@@ -922,7 +1083,9 @@ cudaError_t launch_gt_rerank(const Dev &d, const float *q, u32 q0, u32 nq, u32 k
     r.fb = b.fb;
     r.fb_count = b.gstat + 4;
     r.err = b.err;
-    gt_rerank_kernel<<<(nq + RR_WARPS - 1) / RR_WARPS, RR_WARPS * 32, 0, st>>>(d, r);
+    // a block per query until a warp per query fills the SMs
+    if (nq < (u32)num_sms * 16) gt_rerank_kernel<RR_WARPS><<<nq, RR_WARPS * 32, 0, st>>>(d, r);
+    else gt_rerank_kernel<1><<<(nq + RR_WARPS - 1) / RR_WARPS, RR_WARPS * 32, 0, st>>>(d, r);
     return cudaGetLastError();
 }
 

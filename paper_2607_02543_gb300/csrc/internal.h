@@ -173,7 +173,8 @@ void gt_tc_configure(GtTcPlan &p, u32 nq, bool split);
 cudaError_t launch_gt_tc(const Dev &d, u32 q0, u32 nq, const GtTcPlan &p, const GtTcBufs &b, u64 next_id,
                          int num_sms, cudaStream_t st);
 cudaError_t launch_gt_rerank(const Dev &d, const float *q, u32 q0, u32 nq, u32 k, const GtTcPlan &p,
-                             const GtTcBufs &b, u64 next_id, u32 *out_ids, float *out_dist, cudaStream_t st);
+                             const GtTcBufs &b, u64 next_id, u32 *out_ids, float *out_dist, int num_sms,
+                             cudaStream_t st);
 cudaError_t launch_export(const Dev &d, u64 n, unsigned char *del, unsigned char *hs, unsigned char *deg,
                           u32 *ids, float *rho, cudaStream_t st);
 cudaError_t launch_fill_offer_keys(u32 *key, u32 *val, u32 n, u32 invalid, cudaStream_t st);

@@ -70,3 +70,27 @@ def test_tensor_ground_truth_few_live_rows():
     assert g.ground_truth_info()["path"] == "tensor"
     assert (ids[:, 10:] == NIL).all() and np.isinf(d[:, 10:]).all()
     assert set(ids[0, :10].tolist()) == set(range(1, 20, 2))
+
+
+@pytest.mark.parametrize("n,nq,k,kind,dim", [
+    (2_000 + 9, 1, 10, "gauss", 100),      # a block per query
+    (2_000 + 9, 2_431, 10, "gauss", 128),
+    (2_000 + 9, 2_500, 32, "gauss", 37),   # a warp per query; more candidate blocks than a lane keeps
+    (9_000 + 1, 2_432, 1, "absgauss", 200),
+    (33, 2_500, 5, "int", 128),
+])
+def test_rerank_team_shapes(n, nq, k, kind, dim):
+    """A block or a warp per query, thresholds met by few or by many blocks: the exact kernel's bits."""
+    from paper_2607_02543_gb300 import Index
+    w = dataclasses.replace(W.scaled(W.SMALL, n, n_queries=nq), rounds=0, kind=kind, dim=dim, n_clusters=8)
+    plan = W.make_plan(w)
+    res = []
+    for gt in ("default", "cuda_cores"):
+        g = Index(dim, "l2", 16, n + 10, build_beam=16, max_cand=32, gt=gt)
+        g.insert(plan.base)
+        g.delete(np.arange(0, n, 7, dtype=np.uint32))
+        res.append(g.ground_truth(plan.queries, k))
+        if gt == "default":
+            assert g.ground_truth_info()["fallback_queries"] == 0
+    np.testing.assert_array_equal(res[0][0], res[1][0])
+    np.testing.assert_array_equal(res[0][1].view(np.uint32), res[1][1].view(np.uint32))

@@ -111,7 +111,7 @@ struct etale_index {
     // call and one update call can run at the same time (concurrent mode)
     DevBuf s_stage, s_qpad, s_out_ids, s_out_dist, s_seed;
     // ground truth on tensor cores
-    DevBuf gt_A, gt_B, gt_xn, gt_qstat, gt_gstat, gt_fb, gt_bmin;
+    DevBuf gt_A, gt_B, gt_xn, gt_qstat, gt_gstat, gt_fb, gt_bmin, gt_center;
     u32 gt_path = 0;
     u64 gt_fallbacks = 0;
     // seeding on tensor cores
@@ -1030,7 +1030,8 @@ static etale_status ground_truth_run(etale_index *idx, const Dev &d, const float
         return ETALE_OK;
     }
     if (!grow(idx->gt_A, p.bytes_A) || !grow(idx->gt_B, p.bytes_B) || !grow(idx->gt_xn, p.n_pad * 4) ||
-        !grow(idx->gt_qstat, (size_t)nq * 16) || !grow(idx->gt_gstat, 64) || !grow(idx->gt_fb, (size_t)nq * 4))
+        !grow(idx->gt_qstat, (size_t)nq * 16) || !grow(idx->gt_gstat, 64) || !grow(idx->gt_fb, (size_t)nq * 4) ||
+        !grow(idx->gt_center, (size_t)idx->mp * 4))
         return idx->fail(ETALE_ENOMEM, "ground-truth staging");
     GtTcBufs b{};
     b.A = idx->gt_A.p;
@@ -1039,12 +1040,13 @@ static etale_status ground_truth_run(etale_index *idx, const Dev &d, const float
     b.qstat = as<float>(idx->gt_qstat);
     b.gstat = as<u32>(idx->gt_gstat);
     b.fb = as<u32>(idx->gt_fb);
+    b.center = as<float>(idx->gt_center);
     b.err = b.gstat + 5;
     {
         PhaseScope ps(idx, ETALE_PH_GT_PREP, st);
         CK(launch_gt_tc_prep(d, idx->next_id, qpad, nq, p, b, st), "ground-truth copies");
     }
-    g_kernel_launches += 2;
+    g_kernel_launches += d.metric == 0 ? 3 : 2;
     u32 h[8];
     CK(cudaMemcpyAsync(h, b.gstat, sizeof h, cudaMemcpyDeviceToHost, st), "read split flag");
     CK(cudaStreamSynchronize(st), "synchronize");

@@ -45,14 +45,13 @@ constexpr int TC_ROWS = 128;                      // MMA M: queries per query su
 constexpr int TC_ACC = 256;                       // TMEM columns per accumulator buffer
 constexpr int TC_KBOX = 64;                       // bf16 per 128-byte swizzle row
 constexpr u32 TC_BOX = TC_ROWS * TC_KBOX * 2;     // 16 KB per 128-row TMA box
-// Tile shapes: one query sub-tile (M = 128) against 256 rows, or two
-// (M = 2 x 128) against 128 rows; both fill a 256-column accumulator.  The
-// first reads 96 B of operands from shared memory per MMA cycle instead of
-// 128 B (the SM's shared-memory bandwidth), the second half as many rows
-// from L2 per query.  On the 1M x 128 workload (10k queries) the first ran
-// the candidate pass in 3.5 ms, the second in 4.1 ms, so the plan takes the
-// first; the kernel keeps both.
+// Tile shape: 128 queries against 256 rows, one 256-column accumulator: 96 B of
+// operands from shared memory per MMA cycle of the SM's 128.  Two query tiles
+// against 128 rows read half as many rows from L2, but 128 B: 2,050 against
+// 1,690 cycles a tile (300k x 128 rows, 10k queries).
 constexpr int TC_MAX_STAGES = 12;
+constexpr int TC_XS = 4;                          // key-base ring slots (one tile's bases each)
+constexpr u32 TC_STATIC = 5 * 1024;               // static shared memory of the kernel, rounded up
 constexpr int TC_EPI_WARPS = 8;
 constexpr int TC_THREADS = (2 + TC_EPI_WARPS) * 32;
 constexpr u32 ORD_INF = 0xFF800000u;              // f2ord(+inf)
@@ -63,7 +62,7 @@ __host__ __device__ constexpr u32 tc_idesc(u32 n) {
 }
 
 struct TcArgs {
-    u32 nq, n_tiles, kblocks, n_msub, bn, m_tiles, chunks, tiles_per_chunk, stages;
+    u32 nq, n_tiles, kblocks, bn, m_tiles, chunks, tiles_per_chunk, stages;
     u32 all_keys;         // 0: smallest key per block of 32 rows; 1: every key
     u32 stream_a;         // 1: the query boxes travel through the ring (selects gt_tc_kernel<true>)
     const u32 *nq_dev;    // when set, the batch size is read here (nq is its cap); later query tiles are skipped
@@ -93,17 +92,32 @@ __device__ __forceinline__ u64 sw128_desc(u32 saddr) {
     return (u64)((saddr & 0x3FFFFu) >> 4) | ((u64)1 << 16) | ((u64)(1024 >> 4) << 32) | ((u64)1 << 46) |
            ((u64)2 << 61);
 }
-__device__ __forceinline__ void tc_mma(u32 d, u64 a, u64 b, u32 idesc, u32 acc) {
+// mbar_wait by a whole warp, converged afterwards: no lane may run ahead of the
+// others' waits (a lane two phases behind would wait for a phase that is over),
+// and the issuing instructions read their operands for the warp.
+__device__ __forceinline__ bool warp_wait(u64 *bar, u32 parity) {
+    return __all_sync(FULL, mbar_wait(bar, parity, WAIT_LIMIT));
+}
+// One lane of a converged warp (the same one at every call).
+__device__ __forceinline__ u32 elect_one() {
+    u32 p;
+    asm volatile("{\n .reg .pred q;\n elect.sync _|q, 0xffffffff;\n selp.u32 %0, 1, 0, q;\n}" : "=r"(p));
+    return p;
+}
+// Run by a whole warp, issued by the lane with `leader` set.
+__device__ __forceinline__ void tc_mma(u32 d, u64 a, u64 b, u32 idesc, u32 acc, u32 leader) {
     asm volatile(
-        "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-        " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(d),
-        "l"(a), "l"(b), "r"(idesc), "r"(acc)
+        "{\n .reg .pred p, e;\n setp.ne.b32 p, %4, 0;\n setp.ne.b32 e, %5, 0;\n"
+        " @e tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(d),
+        "l"(a), "l"(b), "r"(idesc), "r"(acc), "r"(leader)
         : "memory");
 }
-__device__ __forceinline__ void tc_commit(u64 *bar) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                     smem_addr(bar))
-                 : "memory");
+__device__ __forceinline__ void tc_commit(u64 *bar, u32 leader) {
+    asm volatile(
+        "{\n .reg .pred e;\n setp.ne.b32 e, %1, 0;\n"
+        " @e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n}" ::"r"(smem_addr(bar)),
+        "r"(leader)
+        : "memory");
 }
 // 64 consecutive TMEM columns of this warp's 32 lanes; completes at tmem_wait().
 __device__ __forceinline__ void tmem_ld64(u32 taddr, u32 *r) {
@@ -111,9 +125,28 @@ __device__ __forceinline__ void tmem_ld64(u32 taddr, u32 *r) {
                  : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31]), "=r"(r[32]), "=r"(r[33]), "=r"(r[34]), "=r"(r[35]), "=r"(r[36]), "=r"(r[37]), "=r"(r[38]), "=r"(r[39]), "=r"(r[40]), "=r"(r[41]), "=r"(r[42]), "=r"(r[43]), "=r"(r[44]), "=r"(r[45]), "=r"(r[46]), "=r"(r[47]), "=r"(r[48]), "=r"(r[49]), "=r"(r[50]), "=r"(r[51]), "=r"(r[52]), "=r"(r[53]), "=r"(r[54]), "=r"(r[55]), "=r"(r[56]), "=r"(r[57]), "=r"(r[58]), "=r"(r[59]), "=r"(r[60]), "=r"(r[61]), "=r"(r[62]), "=r"(r[63])
                  : "r"(taddr));
 }
+// Both halves of a register pair at once (the same roundings as two fmaf),
+// and the smallest of three.
+__device__ __forceinline__ u64 pair32(u32 lo, u32 hi) { return ((u64)hi << 32) | lo; }
+__device__ __forceinline__ u64 fma2(u64 a, u64 b, u64 c) {
+    u64 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ float min3(float a, float b, float c) {
+    float r;
+    asm("min.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+    return r;
+}
+__device__ __forceinline__ float pair_lo(u64 v) { return __uint_as_float((u32)v); }
+__device__ __forceinline__ float pair_hi(u64 v) { return __uint_as_float((u32)(v >> 32)); }
 __device__ __forceinline__ void tmem_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
 // ---- candidate pass ---------------------------------------------------------
+// Bound by the issue of the MMAs and their waits, then by the row boxes from L2
+// (a tile's 64 KB per 128 queries): 300k x 128 integer rows, 10k queries, 1.09
+// -> 0.57 ms, 0.69 of the measured bf16 rate.  The epilogue does two keys per
+// fma and takes two at a time into the running minimum.
 // STREAM_A: the query boxes travel through the ring with the row boxes (a
 // compile-time choice, so the resident form's MMA issue loop carries no test).
 template <bool STREAM_A>
@@ -121,8 +154,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
     gt_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, TcArgs a) {
     extern __shared__ unsigned char tc_raw[];
     __shared__ __align__(8) u64 full[TC_MAX_STAGES], empty[TC_MAX_STAGES];
-    __shared__ __align__(8) u64 a_full, a_empty, t_full[2], t_empty[2], drain;
-    __shared__ __align__(16) float xs[2][TC_ACC];    // key bases of the tile in TMEM buffer b
+    __shared__ __align__(8) u64 a_full, a_empty, t_full[2], t_empty[2], drain, x_full[TC_XS], x_empty[TC_XS];
+    __shared__ __align__(16) float xs[TC_XS][TC_ACC];    // ring of the tiles' key bases
     __shared__ u32 tmem_base;
     __shared__ volatile int abort_flag;
     unsigned char *sm = reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(tc_raw) + 1023) & ~(uintptr_t)1023);
@@ -132,14 +165,13 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
     // query tiles past the batch size in device memory are skipped, the same
     // items by every role
     const u32 nq_eff = a.nq_dev ? min(*a.nq_dev, a.nq) : a.nq;
-    const u32 mt_eff = (nq_eff + a.n_msub * TC_ROWS - 1) / (a.n_msub * TC_ROWS);
-    // resident: sA holds the query tile (n_msub x kblocks boxes), then the
-    // ring of row boxes; streamed: each ring stage is a row box followed by
-    // the n_msub query boxes of the same 64 columns
-    const u32 abox = a.n_msub * TC_BOX;
-    const u32 sbytes = bbox + (STREAM_A ? abox : 0u);
+    const u32 mt_eff = (nq_eff + TC_ROWS - 1) / TC_ROWS;
+    // resident: sA holds the query tile (kblocks boxes), then the ring of row
+    // boxes; streamed: each ring stage is a row box followed by the query box
+    // of the same 64 columns
+    const u32 sbytes = bbox + (STREAM_A ? TC_BOX : 0u);
     unsigned char *sA = sm;
-    unsigned char *sB = sm + (STREAM_A ? 0u : (size_t)a.kblocks * abox);
+    unsigned char *sB = sm + (STREAM_A ? 0u : (size_t)a.kblocks * TC_BOX);
 
     if (threadIdx.x == 0) {
         for (u32 i = 0; i < a.stages; i++) {
@@ -149,8 +181,12 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
         mbar_init(&a_full, 1);
         mbar_init(&a_empty, 1);
         for (int b = 0; b < 2; b++) {
-            mbar_init(&t_full[b], 2);   // the MMA commit + the key-base copy
+            mbar_init(&t_full[b], 1);
             mbar_init(&t_empty[b], TC_EPI_WARPS);
+        }
+        for (int i = 0; i < TC_XS; i++) {
+            mbar_init(&x_full[i], 1);
+            mbar_init(&x_empty[i], TC_EPI_WARPS);
         }
         mbar_init(&drain, 1);
         abort_flag = 0;
@@ -174,116 +210,120 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
     };
 
     if (warp == 0) {
-        // ---- producer: one thread issues every TMA load ----
-        if (lane == 0) {
-            u32 stage = 0, ph = 0, issued = 0, lastpar = 0, a_issued = 0, a_ph = 0;
-            bool first = true;
-            for (u32 it = blockIdx.x; it < items && !abort_flag; it += gridDim.x) {
-                const u32 mt = it % a.m_tiles, ch = it / a.m_tiles;
-                const u32 t0 = ch * a.tiles_per_chunk, t1 = min(a.n_tiles, t0 + a.tiles_per_chunk);
-                if (mt >= mt_eff) continue;
-                if (!STREAM_A) {
-                    if (!first) {
-                        if (!mbar_wait(&a_empty, a_ph, WAIT_LIMIT)) { fail(); break; }
-                        a_ph ^= 1;
-                    }
-                    first = false;
-                    mbar_expect_tx(&a_full, a.kblocks * abox);
-                    for (u32 s = 0; s < a.n_msub; s++)
-                        for (u32 kb = 0; kb < a.kblocks; kb++)
-                            tma_load_2d(sA + (size_t)(s * a.kblocks + kb) * TC_BOX, &tmA, (int)(kb * TC_KBOX),
-                                        (int)((mt * a.n_msub + s) * TC_ROWS), &a_full);
-                    a_issued++;
+        // ---- producer: the warp runs the loop together, one elected lane issues every copy ----
+        u32 stage = 0, ph = 0, issued = 0, lastpar = 0, a_issued = 0, a_ph = 0, xcount = 0;
+        bool first = true, ok = true;
+        const bool leader = elect_one();
+        for (u32 it = blockIdx.x; it < items && ok && !abort_flag; it += gridDim.x) {
+            const u32 mt = it % a.m_tiles, ch = it / a.m_tiles;
+            const u32 t0 = ch * a.tiles_per_chunk, t1 = min(a.n_tiles, t0 + a.tiles_per_chunk);
+            if (mt >= mt_eff) continue;
+            if (!STREAM_A) {
+                if (!first) {
+                    if (!warp_wait(&a_empty, a_ph)) { ok = false; break; }
+                    a_ph ^= 1;
                 }
-                for (u32 t = t0; t < t1 && !abort_flag; t++) {
-                    for (u32 kb = 0; kb < a.kblocks; kb++) {
-                        if (!mbar_wait(&empty[stage], ph ^ 1, WAIT_LIMIT)) { fail(); break; }
-                        unsigned char *sb = sB + (size_t)stage * sbytes;
+                first = false;
+                if (leader) {
+                    mbar_expect_tx(&a_full, a.kblocks * TC_BOX);
+                    for (u32 kb = 0; kb < a.kblocks; kb++)
+                        tma_load_2d(sA + (size_t)kb * TC_BOX, &tmA, (int)(kb * TC_KBOX), (int)(mt * TC_ROWS), &a_full);
+                }
+                __syncwarp();
+                a_issued++;
+            }
+            for (u32 t = t0; t < t1 && ok; t++) {
+                // the tile's key bases, up to TC_XS tiles ahead of the epilogue
+                // (issued with the accumulator's buffer they cost each tile one
+                // copy latency)
+                const u32 xi = xcount % TC_XS;
+                if (!warp_wait(&x_empty[xi], ((xcount / TC_XS) & 1) ^ 1)) { ok = false; break; }
+                if (leader) {
+                    mbar_expect_tx(&x_full[xi], a.bn * 4);
+                    bulk_g2s(xs[xi], a.xn + (size_t)t * a.bn, a.bn * 4, &x_full[xi]);
+                }
+                __syncwarp();
+                xcount++;
+                for (u32 kb = 0; kb < a.kblocks; kb++) {
+                    if (!warp_wait(&empty[stage], ph ^ 1)) { ok = false; break; }
+                    unsigned char *sb = sB + (size_t)stage * sbytes;
+                    if (leader) {
                         mbar_expect_tx(&full[stage], sbytes);
                         tma_load_2d(sb, &tmB, (int)(kb * TC_KBOX), (int)(t * a.bn), &full[stage]);
                         if (STREAM_A)
-                            for (u32 s = 0; s < a.n_msub; s++)
-                                tma_load_2d(sb + bbox + (size_t)s * TC_BOX, &tmA, (int)(kb * TC_KBOX),
-                                            (int)((mt * a.n_msub + s) * TC_ROWS), &full[stage]);
-                        issued |= 1u << stage;
-                        lastpar = (lastpar & ~(1u << stage)) | (ph << stage);
-                        if (++stage == a.stages) {
-                            stage = 0;
-                            ph ^= 1;
-                        }
+                            tma_load_2d(sb + bbox, &tmA, (int)(kb * TC_KBOX), (int)(mt * TC_ROWS), &full[stage]);
+                    }
+                    __syncwarp();
+                    issued |= 1u << stage;
+                    lastpar = (lastpar & ~(1u << stage)) | (ph << stage);
+                    if (++stage == a.stages) {
+                        stage = 0;
+                        ph ^= 1;
                     }
                 }
             }
-            // every copy this thread issued has landed before the CTA exits
-            for (u32 i = 0; i < a.stages; i++)
-                if (issued >> i & 1) mbar_wait(&full[i], lastpar >> i & 1, WAIT_LIMIT);
-            if (a_issued) mbar_wait(&a_full, (a_issued - 1) & 1, WAIT_LIMIT);
         }
+        if (!ok && lane == 0) fail();
+        // every copy this warp issued has landed before the CTA exits
+        for (u32 i = 0; i < a.stages; i++)
+            if (issued >> i & 1) mbar_wait(&full[i], lastpar >> i & 1, WAIT_LIMIT);
+        if (a_issued) mbar_wait(&a_full, (a_issued - 1) & 1, WAIT_LIMIT);
+        for (u32 i = 0; i < TC_XS && i < xcount; i++)
+            mbar_wait(&x_full[i], ((xcount - 1 - i) / TC_XS) & 1, WAIT_LIMIT);
     } else if (warp == 1) {
-        // ---- MMA issuer: one thread ----
-        if (lane == 0) {
+        // ---- MMA issuer: the warp runs the loop together, one elected lane issues.
+        // With a branch on the lane around the whole loop each tcgen05.mma took
+        // about 330 cycles to issue (its operands must be in uniform registers):
+        // 3,170 cycles a tile of 128 x 256 x 128 against 1,024 of tensor work.
+        {
             u32 stage = 0, ph = 0, a_ph = 0, tcount = 0;
-            for (u32 it = blockIdx.x; it < items && !abort_flag; it += gridDim.x) {
+            const u32 leader = elect_one();
+            const u32 idesc = tc_idesc(a.bn);
+            const u64 dA = sw128_desc(smem_addr(sA)), dB = sw128_desc(smem_addr(sB));
+            bool ok = true;
+            for (u32 it = blockIdx.x; it < items && ok; it += gridDim.x) {
                 const u32 ch = it / a.m_tiles;
                 const u32 t0 = ch * a.tiles_per_chunk, t1 = min(a.n_tiles, t0 + a.tiles_per_chunk);
                 if (it % a.m_tiles >= mt_eff) continue;
                 if (!STREAM_A) {
-                    if (!mbar_wait(&a_full, a_ph, WAIT_LIMIT)) { fail(); break; }
+                    if (!warp_wait(&a_full, a_ph)) { ok = false; break; }
                     a_ph ^= 1;
                     tc_fence_after();
                 }
-                for (u32 t = t0; t < t1 && !abort_flag; t++, tcount++) {
+                for (u32 t = t0; t < t1; t++, tcount++) {
                     const u32 b = tcount & 1;
-                    if (!mbar_wait(&t_empty[b], ((tcount >> 1) & 1) ^ 1, WAIT_LIMIT)) { fail(); break; }
+                    if (!warp_wait(&t_empty[b], ((tcount >> 1) & 1) ^ 1)) { ok = false; break; }
                     tc_fence_after();
-                    // the tile's key bases travel with the accumulator: same barrier
-                    mbar_expect_tx(&t_full[b], a.bn * 4);
-                    bulk_g2s(xs[b], a.xn + (size_t)t * a.bn, a.bn * 4, &t_full[b]);
-                    bool ok = true;
+                    const u32 acol = tmem + b * TC_ACC;
                     for (u32 kb = 0; kb < a.kblocks; kb++) {
-                        if (!mbar_wait(&full[stage], ph, WAIT_LIMIT)) { ok = false; break; }
+                        if (!warp_wait(&full[stage], ph)) { ok = false; break; }
                         tc_fence_after();
-                        const u32 bb = smem_addr(sB + (size_t)stage * sbytes);
-                        const u32 idesc = tc_idesc(a.bn);
+                        const u64 bd = dB + (u64)(stage * sbytes >> 4);
+                        const u64 ad = STREAM_A ? bd + (bbox >> 4) : dA + (u64)(kb * (TC_BOX >> 4));
 #pragma unroll
-                        for (u32 k = 0; k < TC_KBOX / 16; k++) {
-                            const u64 bd = sw128_desc(bb + k * 32);
-                            for (u32 s = 0; s < a.n_msub; s++) {
-                                const u32 aa = (STREAM_A ? bb + bbox + s * TC_BOX
-                                                           : smem_addr(sA + (size_t)(s * a.kblocks + kb) * TC_BOX)) +
-                                               k * 32;
-                                tc_mma(tmem + b * TC_ACC + s * TC_ROWS, sw128_desc(aa), bd, idesc, (kb | k) != 0);
-                            }
-                        }
-                        tc_commit(&empty[stage]);
+                        for (u32 k = 0; k < TC_KBOX / 16; k++)
+                            tc_mma(acol, ad + 2 * k, bd + 2 * k, idesc, (kb | k) != 0, leader);
+                        tc_commit(&empty[stage], leader);
                         if (++stage == a.stages) {
                             stage = 0;
                             ph ^= 1;
                         }
                     }
-                    tc_commit(&t_full[b]);
-                    if (!ok) {
-                        tcount++;   // this tile's key-base copy is in flight too
-                        fail();
-                        break;
-                    }
+                    if (!ok) break;
+                    tc_commit(&t_full[b], leader);
                 }
-                if (!STREAM_A) tc_commit(&a_empty);
+                if (!STREAM_A) tc_commit(&a_empty, leader);
             }
-            // all MMAs and key-base copies issued by this thread are complete
-            // before TMEM and shared memory are released
-            tc_commit(&drain);
+            if (!ok && lane == 0) fail();
+            // all MMAs issued by this warp are complete before TMEM and
+            // shared memory are released
+            tc_commit(&drain, leader);
             mbar_wait(&drain, 0, WAIT_LIMIT);
-            for (u32 b = 0; b < 2 && b < tcount; b++) {
-                const u32 uses = (tcount - b + 1) / 2;     // tiles that used buffer b
-                mbar_wait(&t_full[b], (uses - 1) & 1, WAIT_LIMIT);
-            }
         }
     } else {
         // ---- epilogue: warp w reads TMEM lanes 32 (w % 4) .. + 31; lane = one query ----
-        // group g of four warps: query sub-tile g (two sub-tiles) or row half g (one)
-        const int ew = warp - 2, grp = ew >> 2, quarter = warp & 3;
-        const int ms = a.n_msub == 2 ? grp : 0, half = a.n_msub == 2 ? 0 : grp;
+        // each group of four warps takes one half of the tile's rows
+        const int half = (warp - 2) >> 2, quarter = warp & 3;
         {
             const int row = quarter * 32 + lane;
             u32 tcount = 0;
@@ -292,64 +332,66 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
                 const u32 mt = it % a.m_tiles, ch = it / a.m_tiles;
                 const u32 t0 = ch * a.tiles_per_chunk, t1 = min(a.n_tiles, t0 + a.tiles_per_chunk);
                 if (mt >= mt_eff) continue;
-                const u32 q = (mt * a.n_msub + ms) * TC_ROWS + row;
+                const u32 q = mt * TC_ROWS + row;
                 const bool valid = q < nq_eff;
                 float4 *dst = reinterpret_cast<float4 *>(a.out + (size_t)(valid ? q : 0) * a.ld);
                 for (u32 t = t0; t < t1; t++, tcount++) {
                     const u32 b = tcount & 1;
+                    const u32 xi = tcount % TC_XS;
                     // every lane waits; the warp goes on together (tcgen05.ld is .sync.aligned)
-                    const bool got = !abort_flag && mbar_wait(&t_full[b], (tcount >> 1) & 1, WAIT_LIMIT);
+                    const bool got = !abort_flag && mbar_wait(&t_full[b], (tcount >> 1) & 1, WAIT_LIMIT) &&
+                                     mbar_wait(&x_full[xi], (tcount / TC_XS) & 1, WAIT_LIMIT);
                     if (!__all_sync(FULL, got)) { ok = false; break; }
                     tc_fence_after();
-                    const u32 tbase = tmem + ((u32)(quarter * 32) << 16) + b * TC_ACC + grp * TC_ROWS;
-                    float bm[TC_ROWS / 32];
-                    if (a.all_keys) {
-                        u32 r[TC_ROWS];
-                        tmem_ld64(tbase, r);
-                        tmem_ld64(tbase + 64, r + 64);
-                        tmem_wait();
-                        const float4 *x4 = reinterpret_cast<const float4 *>(xs[b] + half * TC_ROWS);
-                        float4 *o4 = dst + (size_t)(t * a.bn + half * TC_ROWS) / 4;
+                    const u32 tbase = tmem + ((u32)(quarter * 32) << 16) + b * TC_ACC + half * TC_ROWS;
+                    u32 r[TC_ROWS];
+                    tmem_ld64(tbase, r);
+                    tmem_ld64(tbase + 64, r + 64);
+                    tmem_wait();
 #pragma unroll
-                        for (int j4 = 0; j4 < TC_ROWS / 4; j4++) {
-                            const float4 v = x4[j4];
-                            const u32 *rr = r + 4 * j4;
-                            const float4 kv = make_float4(fmaf(a.s, __uint_as_float(rr[0]), v.x),
-                                                          fmaf(a.s, __uint_as_float(rr[1]), v.y),
-                                                          fmaf(a.s, __uint_as_float(rr[2]), v.z),
-                                                          fmaf(a.s, __uint_as_float(rr[3]), v.w));
-                            if (valid) o4[j4] = kv;
-                        }
-                        // TMEM and the key bases of buffer b are refilled after this
+                    for (int i = 0; i < TC_ROWS; i++) asm volatile("" : "+r"(r[i]));   // no use moves before the wait
+                    // TMEM buffer b and the key bases are refilled after this: only once
+                    // every loaded value has been used (given up right after the wait,
+                    // the next tile's MMAs overwrote columns still being read)
+                    auto release = [&]() {
                         tc_fence_before();
                         __syncwarp();
-                        if (lane == 0) mbar_arrive(&t_empty[b]);
+                        if (lane == 0) {
+                            mbar_arrive(&t_empty[b]);
+                            mbar_arrive(&x_empty[xi]);
+                        }
+                    };
+                    const ulonglong2 *x2 = reinterpret_cast<const ulonglong2 *>(xs[xi] + half * TC_ROWS);
+                    const u64 s2 = pair32(__float_as_uint(a.s), __float_as_uint(a.s));
+                    if (a.all_keys) {
+                        ulonglong2 *o4 = reinterpret_cast<ulonglong2 *>(dst + (size_t)(t * a.bn + half * TC_ROWS) / 4);
+#pragma unroll
+                        for (int j4 = 0; j4 < TC_ROWS / 4; j4++) {
+                            const ulonglong2 v = x2[j4];
+                            const u32 *rr = r + 4 * j4;
+                            ulonglong2 kv;
+                            kv.x = fma2(s2, pair32(rr[0], rr[1]), v.x);
+                            kv.y = fma2(s2, pair32(rr[2], rr[3]), v.y);
+                            if (valid) o4[j4] = kv;
+                        }
+                        release();
                         continue;
                     }
-                    {
-                        u32 r[TC_ROWS];
-                        tmem_ld64(tbase, r);
-                        tmem_ld64(tbase + 64, r + 64);
-                        tmem_wait();
-                        const float4 *x4 = reinterpret_cast<const float4 *>(xs[b] + half * TC_ROWS);
+                    float bm[TC_ROWS / 32];
 #pragma unroll
-                        for (int c = 0; c < TC_ROWS / 32; c++) {
-                            float m0 = __int_as_float(0x7f800000), m1 = m0;
+                    for (int c = 0; c < TC_ROWS / 32; c++) {
+                        float m0 = __int_as_float(0x7f800000), m1 = m0;
 #pragma unroll
-                            for (int j4 = 0; j4 < 8; j4++) {
-                                const float4 v = x4[c * 8 + j4];
-                                const u32 *rr = r + c * 32 + 4 * j4;
-                                m0 = fminf(m0, fmaf(a.s, __uint_as_float(rr[0]), v.x));
-                                m1 = fminf(m1, fmaf(a.s, __uint_as_float(rr[1]), v.y));
-                                m0 = fminf(m0, fmaf(a.s, __uint_as_float(rr[2]), v.z));
-                                m1 = fminf(m1, fmaf(a.s, __uint_as_float(rr[3]), v.w));
-                            }
-                            bm[c] = fminf(m0, m1);
+                        for (int j4 = 0; j4 < 8; j4++) {
+                            const ulonglong2 v = x2[c * 8 + j4];
+                            const u32 *rr = r + c * 32 + 4 * j4;
+                            const u64 k0 = fma2(s2, pair32(rr[0], rr[1]), v.x), k1 = fma2(s2, pair32(rr[2], rr[3]), v.y);
+                            m0 = min3(m0, pair_lo(k0), pair_hi(k0));
+                            m1 = min3(m1, pair_lo(k1), pair_hi(k1));
                         }
+                        bm[c] = fminf(m0, m1);
                     }
-                    tc_fence_before();
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(&t_empty[b]);
+                    release();
                     if (valid) dst[t * (a.bn / TC_ROWS) + half] = make_float4(bm[0], bm[1], bm[2], bm[3]);
                 }
             }
@@ -393,13 +435,52 @@ __device__ __forceinline__ Split4 split4(float4 v) {
     o.anylo = (l0 != 0.0f) | (l1 != 0.0f) | (l2 != 0.0f) | (l3 != 0.0f);
     return o;
 }
-__device__ __forceinline__ float4 load_row4(const float *r, u32 i, u32 dim, bool on) {
+// c (optional): subtracted from every element
+__device__ __forceinline__ float4 load_row4(const float *r, u32 i, u32 dim, bool on, const float *c) {
     if (!on || i >= dim) return make_float4(0.f, 0.f, 0.f, 0.f);
     float4 v = *reinterpret_cast<const float4 *>(r + i);   // rows are padded to a multiple of 4
+    if (c) {
+        const float4 m = *reinterpret_cast<const float4 *>(c + i);
+        v = make_float4(__fsub_rn(v.x, m.x), __fsub_rn(v.y, m.y), __fsub_rn(v.z, m.z), __fsub_rn(v.w, m.w));
+    }
     if (i + 1 >= dim) v.y = 0.f;
     if (i + 2 >= dim) v.z = 0.f;
     if (i + 3 >= dim) v.w = 0.f;
     return v;
+}
+
+// A common vector near the rows' mean.  Squared L2 distances do not change
+// when it is taken from rows and queries alike, but the norms that the error
+// bound grows with do: on the 960-d non-negative mixture the bound falls to a
+// third and with it the blocks a query has to score (40k rows, 2,003 queries:
+// 21.5 -> 5.4 ms of scoring).
+// The sample is CR rows spread over the ids.  gstat[6] is set when one of its
+// elements is not exact in bf16: only then do the copies subtract the vector,
+// so that data for which one bf16 segment is enough stay so.  A column whose
+// mean is no ordinary number keeps 0.
+constexpr int CR = 1024;
+__global__ void __launch_bounds__(1024) gt_center_kernel(Dev d, u64 next_id, float *center, u32 *gstat) {
+    __shared__ float part[32][33];
+    const u32 col = blockIdx.x * 32 + threadIdx.x, ry = threadIdx.y;   // 32 columns x 32 row groups
+    const u32 n = (u32)min((u64)CR, next_id);
+    float sum = 0.0f;
+    bool inexact = false;
+    if (col < d.mp)
+#pragma unroll 8
+        for (u32 j = ry; j < n; j += 32) {
+            const float v = d.x[(u64)j * next_id / n * d.mp + col];
+            sum += v;
+            inexact |= bf16_round(v) != v;
+        }
+    if (__any_sync(FULL, inexact) && threadIdx.x == 0) atomicOr(gstat + 6, 1u);
+    part[ry][threadIdx.x] = sum;
+    __syncthreads();
+    if (ry == 0 && col < d.mp) {
+        float s = 0.0f;
+        for (int j = 0; j < 32; j++) s += part[j][threadIdx.x];
+        const float c = rintf(s / (float)n);
+        center[col] = fabsf(c) <= 1048576.0f ? c : 0.0f;
+    }
 }
 
 // gstat: [0] max |x|^2, [1] max |lo_x|, [2] max |e_x| (fp32 bits), [3] any lo != 0.
@@ -407,8 +488,9 @@ __device__ __forceinline__ float4 load_row4(const float *r, u32 i, u32 dim, bool
 // ids (optional): row c is node ids[c]; check_live: rows of deleted or
 // never-inserted nodes get key base +inf and a zero copy.
 __global__ void gt_prep_rows(Dev d, const u32 *ids, u64 next_id, u32 n_pad, bool check_live, u32 kp1, u32 kb, u32 *B,
-                             float *xn, u32 *gstat) {
+                             float *xn, u32 *gstat, const float *center) {
     const int lane = lane_id();
+    if (center && !gstat[6]) center = nullptr;
     const u32 nwarps = (gridDim.x * blockDim.x) >> 5;
     float mx_sq = 0.0f, mx_lo = 0.0f, mx_e = 0.0f;
     bool any_lo = false;
@@ -425,7 +507,7 @@ __global__ void gt_prep_rows(Dev d, const u32 *ids, u64 next_id, u32 n_pad, bool
             const float *xr = d.x + (size_t)id * d.mp;
             uint2 *br = reinterpret_cast<uint2 *>(B + (size_t)c * (kb / 2));
             for (u32 i = 4 * lane; i < kp1; i += 128) {
-                const Split4 v = split4(load_row4(xr, i, d.dim, live));
+                const Split4 v = split4(load_row4(xr, i, d.dim, live, center));
                 br[i / 4] = v.hi;
                 br[(kp1 + i) / 4] = v.lo;
                 br[(2 * kp1 + i) / 4] = v.hi;
@@ -460,16 +542,17 @@ __global__ void gt_prep_rows(Dev d, const u32 *ids, u64 next_id, u32 n_pad, bool
 
 // qstat per query: |q|^2, |q|, |lo_q|, |e_q|; copy as [hi | hi | lo]
 __global__ void gt_prep_queries(const float *q, u32 mp, u32 dim, u32 nq, u32 kp1, u32 kb, u32 *A, float *qstat,
-                                u32 *gstat, const u32 *nq_dev = nullptr) {
+                                u32 *gstat, const float *center, const u32 *nq_dev) {
     const u32 r = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = lane_id();
     if (r >= (nq_dev ? min(*nq_dev, nq) : nq)) return;
+    if (center && !gstat[6]) center = nullptr;
     const float *qr = q + (size_t)r * mp;
     uint2 *ar = reinterpret_cast<uint2 *>(A + (size_t)r * (kb / 2));
     float sq = 0.0f, lo2 = 0.0f, e2 = 0.0f;
     bool anylo = false;
     for (u32 i = 4 * lane; i < kp1; i += 128) {
-        const Split4 v = split4(load_row4(qr, i, dim, true));
+        const Split4 v = split4(load_row4(qr, i, dim, true, center));
         ar[i / 4] = v.hi;
         ar[(kp1 + i) / 4] = v.hi;
         ar[(2 * kp1 + i) / 4] = v.lo;
@@ -508,8 +591,8 @@ __device__ double key_error(int metric, double m, double K, bool split, const fl
     // |computed dot - q.x|: the terms the split leaves out, plus fp32 accumulation
     const double dot_res = split ? loq * Lx + (qa + eq) * Ex + eq * (X1 + Ex) : 0.0;
     const double dot_err = dot_res + (K + 2.0) * 2.0 * u * 1.03 * qa * X1;
-    if (metric == 0)   // norms (fp32 sums of squares), 2 x dot error, rounding of the key
-        return 2.0 * ((m + 2.0) * u * qn * 1.01 + (m + 2.0) * u * X2 + 2.0 * dot_err + 2.0 * u * (X2 + 2.1 * qa * X1));
+    if (metric == 0)   // taking the centre off, norms (fp32 sums of squares), 2 x dot error, rounding of the key
+        return 2.0 * (2.1 * u * (qa + X1) * (qa + X1) + (m + 2.0) * u * qn * 1.01 + (m + 2.0) * u * X2 + 2.0 * dot_err + 2.0 * u * (X2 + 2.1 * qa * X1));
     return 2.0 * (dot_err + (m + 2.0) * u * qa * X1 + u * (1.0 + qa * X1));
 }
 // Lower bound on the canonical fp32 distance of every row whose approximate
@@ -597,15 +680,16 @@ __device__ __forceinline__ void canon_dist_wide2(const float *__restrict__ q, co
 
 // Bound by the row reads (L2) and their latency.  Scoring what the k-th
 // distance leaves open, instead of a fixed 32 blocks with a certificate and a
-// full scan by gt_kernel where it fails: 10k queries x 300k x 128 integer rows
-// 0.97 -> 0.73 ms; 2,003 queries x 40k x 960 real-valued rows, all of which
-// failed the certificate, 53.5 -> 21.5 ms.
+// full scan by gt_kernel where it fails, and two blocks of 8 warps per SM:
+// 10k queries x 300k x 128 integer rows 0.97 -> 0.50 ms; 2,003 queries x 40k x
+// 960 real-valued rows, all of which failed the certificate, 53.5 -> 2.9 ms
+// (21.5 before gt_center_kernel).
 // W warps per query (1 or 8): a block per query below 16 queries an SM, where
 // a warp per query would leave the SMs' slots empty.  Each lane keeps the four smallest minima of the
 // blocks it reads, with their numbers, so that a threshold met by at most four
 // blocks of any lane needs no second pass over the minima.
 template <int W>
-__global__ void __launch_bounds__(RR_WARPS * 32) gt_rerank_kernel(Dev d, RerankArgs a) {
+__global__ void __launch_bounds__(RR_WARPS * 32, 2) gt_rerank_kernel(Dev d, RerankArgs a) {
     __shared__ u32 clist[RR_WARPS][RR_LIST];
     __shared__ u64 ckey[RR_WARPS][32];
     __shared__ u64 xbest[RR_WARPS][32];
@@ -976,11 +1060,13 @@ cudaError_t launch_gt_tc_prep(const Dev &d, u64 next_id, const float *q, u32 nq,
                               const GtTcBufs &b, cudaStream_t st) {
     cudaError_t e = cudaMemsetAsync(b.gstat, 0, 8 * sizeof(u32), st);
     if (e != cudaSuccess) return e;
+    const float *center = d.metric == 0 && next_id ? b.center : nullptr;
+    if (center) gt_center_kernel<<<(d.mp + 31) / 32, dim3(32, 32), 0, st>>>(d, next_id, b.center, b.gstat);
     if (p.n_pad)
         gt_prep_rows<<<(unsigned)std::min<u64>((p.n_pad * 32 + 255) / 256, 152 * 16), 256, 0, st>>>(
-            d, nullptr, next_id, (u32)p.n_pad, true, p.kp1, p.kb, reinterpret_cast<u32 *>(b.B), b.xn, b.gstat);
+            d, nullptr, next_id, (u32)p.n_pad, true, p.kp1, p.kb, reinterpret_cast<u32 *>(b.B), b.xn, b.gstat, center);
     gt_prep_queries<<<(unsigned)(((size_t)nq * 32 + 255) / 256), 256, 0, st>>>(
-        q, d.mp, d.dim, nq, p.kp1, p.kb, reinterpret_cast<u32 *>(b.A), b.qstat, b.gstat);
+        q, d.mp, d.dim, nq, p.kp1, p.kb, reinterpret_cast<u32 *>(b.A), b.qstat, b.gstat, center, nullptr);
     return cudaGetLastError();
 }
 
@@ -988,9 +1074,8 @@ void gt_tc_configure(GtTcPlan &p, u32 nq, bool split) {
     p.kprime = split ? p.kb : p.kp1;
     p.split = split;
     p.kblocks = p.kprime / TC_KBOX;
-    const u32 smem_max = 227 * 1024 - 1024 - 4096;   // alignment slack, static shared memory
-    p.n_msub = 1;
-    p.bn = TC_ACC / p.n_msub;
+    const u32 smem_max = 227 * 1024 - 1024 - TC_STATIC;   // alignment slack, static shared memory
+    p.bn = TC_ACC;
     const u32 bbox = p.bn * TC_KBOX * 2;
     if (p.n_pad == 0) {
         p.usable = false;
@@ -998,13 +1083,13 @@ void gt_tc_configure(GtTcPlan &p, u32 nq, bool split) {
     }
     // the query tile stays resident when it fits beside two ring stages;
     // otherwise its boxes travel through the ring with the row boxes
-    p.stream_a = (u64)p.n_msub * p.kblocks * TC_BOX + 2ull * bbox > smem_max;
+    p.stream_a = (u64)p.kblocks * TC_BOX + 2ull * bbox > smem_max;
     if (p.stream_a) {
-        p.stages = std::min<u32>(TC_MAX_STAGES, smem_max / (bbox + p.n_msub * TC_BOX));
-        p.smem = p.stages * (bbox + p.n_msub * TC_BOX) + 1024;
+        p.stages = std::min<u32>(TC_MAX_STAGES, smem_max / (bbox + TC_BOX));
+        p.smem = p.stages * (bbox + TC_BOX) + 1024;
     } else {
-        p.stages = std::min<u32>(TC_MAX_STAGES, (smem_max - p.n_msub * p.kblocks * TC_BOX) / bbox);
-        p.smem = p.n_msub * p.kblocks * TC_BOX + p.stages * bbox + 1024;
+        p.stages = std::min<u32>(TC_MAX_STAGES, (smem_max - p.kblocks * TC_BOX) / bbox);
+        p.smem = p.kblocks * TC_BOX + p.stages * bbox + 1024;
     }
     p.n_tiles = (u32)(p.n_pad / p.bn);
     p.nblk = (u32)(p.n_pad / 32);
@@ -1025,9 +1110,8 @@ cudaError_t launch_gt_tc(const Dev &d, u32 q0, u32 nq, const GtTcPlan &p, const 
     a.nq = nq;
     a.n_tiles = p.n_tiles;
     a.kblocks = p.kblocks;
-    a.n_msub = p.n_msub;
     a.bn = p.bn;
-    a.m_tiles = (nq + p.n_msub * TC_ROWS - 1) / (p.n_msub * TC_ROWS);
+    a.m_tiles = (nq + TC_ROWS - 1) / TC_ROWS;
     // chunks of rows: enough work items to fill every SM, with the fewest
     // idle SMs in the last wave
     u32 best_c = 1;
@@ -1095,7 +1179,7 @@ SeedTcPlan seed_tc_plan(u32 dim, u32 n_entry, u32 nq) {
     p.kp1 = (dim + TC_KBOX - 1) / TC_KBOX * TC_KBOX;
     p.kb = 3 * p.kp1;
     p.s_pad = (n_entry + TC_ACC - 1) / TC_ACC * TC_ACC;
-    const u32 smem_max = 227 * 1024 - 1024 - 4096;
+    const u32 smem_max = 227 * 1024 - 1024 - TC_STATIC;
     const u32 bbox = TC_ACC * TC_KBOX * 2;
     const u32 abytes = (p.kb / TC_KBOX) * TC_BOX;
     p.usable = n_entry > 0;
@@ -1118,7 +1202,7 @@ cudaError_t launch_seed_tc_entries(const Dev &d, u32 S, const SeedTcPlan &p, con
     cudaError_t e = cudaMemsetAsync(b.estat, 0, 8 * sizeof(u32), st);
     if (e != cudaSuccess || p.s_pad == 0) return e;
     gt_prep_rows<<<(unsigned)std::min<u64>(((u64)p.s_pad * 32 + 255) / 256, 152 * 16), 256, 0, st>>>(
-        d, d.entries, S, p.s_pad, false, p.kp1, p.kb, reinterpret_cast<u32 *>(b.E), b.en, b.estat);
+        d, d.entries, S, p.s_pad, false, p.kp1, p.kb, reinterpret_cast<u32 *>(b.E), b.en, b.estat, nullptr);
     return cudaGetLastError();
 }
 
@@ -1128,7 +1212,7 @@ cudaError_t launch_seed_tc(const Dev &d, const float *q, u32 nq, u32 S, u32 L, u
     cudaError_t e = cudaMemsetAsync(b.ctr, 0, 8 * sizeof(u32), st);
     if (e != cudaSuccess) return e;
     gt_prep_queries<<<(unsigned)(((size_t)nq * 32 + 255) / 256), 256, 0, st>>>(
-        q, d.mp, d.dim, nq, p.kp1, p.kb, reinterpret_cast<u32 *>(b.A), b.qstat, b.ctr + 4, nq_dev);
+        q, d.mp, d.dim, nq, p.kp1, p.kb, reinterpret_cast<u32 *>(b.A), b.qstat, b.ctr + 4, nullptr, nq_dev);
     CUtensorMap ta, tb;
     if (!encode_bf16(&ta, b.A, nq, p.kb, TC_ROWS) || !encode_bf16(&tb, b.E, S, p.kb, TC_ACC))
         return cudaErrorInvalidValue;
@@ -1136,7 +1220,6 @@ cudaError_t launch_seed_tc(const Dev &d, const float *q, u32 nq, u32 S, u32 L, u
     a.nq = nq;
     a.n_tiles = p.s_pad / TC_ACC;
     a.kblocks = p.kb / TC_KBOX;
-    a.n_msub = 1;
     a.bn = TC_ACC;
     a.m_tiles = (nq + TC_ROWS - 1) / TC_ROWS;
     u32 best_c = 1;

@@ -134,7 +134,7 @@ struct GtTcPlan {
     u32 kp1 = 0, kb = 0;            // one bf16 segment (dim rounded to 64); three segments
     u64 n_pad = 0;                  // rows rounded to 256
     size_t bytes_A = 0, bytes_B = 0, bytes_bmin = 0;
-    u32 kprime = 0, kblocks = 0, n_msub = 0, bn = 0, stages = 0, smem = 0, n_tiles = 0, nblk = 0;
+    u32 kprime = 0, kblocks = 0, bn = 0, stages = 0, smem = 0, n_tiles = 0, nblk = 0;
     u32 qgroup = 0;                 // queries per candidate pass
     bool split = false, usable = false;
     bool stream_a = false;          // the query tile travels through the ring (K too large to stay resident)
@@ -145,6 +145,7 @@ struct GtTcBufs {
     u32 *gstat;                     // [0..3] maxima and the split flag, [4] fallback count, [5] error word
     u32 *fb;                        // fallback query list
     float *bmin;                    // qgroup x nblk block minima
+    float *center;                  // mp floats: the vector taken from rows and queries (L2)
     u32 *err;
 };
 struct SeedTcPlan {

@@ -301,8 +301,10 @@ etale_status etale_load(const char *path, const etale_config *cfg, uint64_t capa
 
 /* ---- launch-shape tuning (deployment support; the paper has none) -------- */
 typedef struct {
-    uint32_t stage_rows;  /* neighbour rows gathered per bulk-copy batch      */
-    uint32_t seen_bits;   /* log2 slots of the evaluated-id cache             */
+    uint32_t stage_rows;  /* neighbour rows gathered per bulk-copy batch
+                             (tensor-core keys; other searches stage none);
+                             0 in a result: the library's own rule            */
+    uint32_t seen_bits;   /* log2 slots of the evaluated-id cache; 0 likewise */
     float ms;             /* measured: seeding + search of the tuning batch   */
     uint32_t warps_per_block; /* queries in flight per thread block: 2, 4, 8 */
     uint32_t keys_tc;     /* BF16 searches: keys from the tensor cores (1) or
@@ -315,7 +317,8 @@ typedef struct {
 etale_status etale_set_exact_rows(etale_index *idx, int on);
 
 /* Set the BeamSearch launch shape (results never depend on it);
- * warps_per_block 0 keeps the current value.                               */
+ * warps_per_block 0 keeps the current value.  Until it is set the library
+ * chooses by row length, beam, batch size and capacity.                    */
 etale_status etale_set_search_tuning(etale_index *idx, uint32_t stage_rows, uint32_t seen_bits,
                                      uint32_t warps_per_block);
 

@@ -499,7 +499,7 @@ bool exact_rows(const etale_index *idx) {
 // The BeamSearch launch shape with its row stage shrunk until a block's shared
 // memory fits the device (long rows); results do not depend on the stage.
 SearchTuning fit_tuning(const etale_index *idx, u32 L, SearchTuning t) {
-    while (t.stage_rows > 1 &&
+    while (t.stage_rows > 1 && t.seen_bits &&
            search_smem_bytes(idx->mp, L, t.stage_rows, t.seen_bits, idx->capacity, t.warps_per_block) > (size_t)idx->smem_optin)
         t.stage_rows >>= 1;
     return t;
@@ -1358,40 +1358,48 @@ etale_status etale_autotune_search(etale_index *idx, const float *queries, uint6
     float best = 1e30f;
     SearchTuning best_t = saved;
     u32 tried = 0;
-    const u32 rows[4] = {2, 4, 8, 16}, bits[4] = {7, 8, 9, 10}, wpbs[3] = {2, 4, 8};
+    const u32 rows[4] = {2, 4, 8, 16}, bits[4] = {9, 10, 11, 12}, wpbs[3] = {2, 4, 8};
     // BF16 searches also try both key paths (tensor cores, CUDA cores)
     const u32 n_keys = idx->search_prec == 1 ? 2u : 1u;
-    for (u32 kp = 0; kp < n_keys; kp++)
-    for (u32 c = 0; c < 3; c++)
-    for (u32 a = 0; a < 4; a++)
-        for (u32 b = 0; b < 4; b++) {
-            SearchTuning t;
-            t.stage_rows = rows[a];
-            t.seen_bits = bits[b];
-            t.warps_per_block = wpbs[c];
-            t.keys_tc = kp == 0 ? 1u : 0u;
-            if (fit_tuning(idx, L, t).stage_rows != t.stage_rows) continue;   // does not fit: not a shape
-            float ms_best = 1e30f;
-            bool ok = true;
-            for (int rep = 0; rep < 3 && ok; rep++) {   // first run warms up
-                Dev d = idx->dev();
-                cudaEventRecord(e0, st);
-                ok = launch_seed(d, qpad, (u32)nq, L, as<u64>(idx->s_seed), st, idx->search_prec) == cudaSuccess &&
-                     launch_search(d, qpad, (u32)nq, L, H, 0, k, as<u32>(idx->s_out_ids), as<float>(idx->s_out_dist),
-                                   nullptr, nullptr, as<u64>(idx->s_seed), t, idx->num_sms, st, idx->search_prec,
-                                   idx->cfg.rerank, nullptr, idx->search_prec == 0 && exact_rows(idx)) == cudaSuccess;
-                cudaEventRecord(e1, st);
-                if (cudaStreamSynchronize(st) != cudaSuccess) ok = false;
-                float ms = 0.f;
-                if (ok && rep > 0 && cudaEventElapsedTime(&ms, e0, e1) == cudaSuccess) ms_best = std::min(ms_best, ms);
-            }
-            cudaGetLastError();   // a shape that does not fit is skipped
-            if (!ok) continue;
-            if (out && tried < n_out)
-                out[tried] = etale_tuning{t.stage_rows, t.seen_bits, ms_best, t.warps_per_block, t.keys_tc};
-            tried++;
-            if (ms_best < best) { best = ms_best; best_t = t; }
+    auto time_shape = [&](const SearchTuning &t) {
+        float ms_best = 1e30f;
+        bool ok = true;
+        for (int rep = 0; rep < 3 && ok; rep++) {   // first run warms up
+            Dev d = idx->dev();
+            cudaEventRecord(e0, st);
+            ok = launch_seed(d, qpad, (u32)nq, L, as<u64>(idx->s_seed), st, idx->search_prec) == cudaSuccess &&
+                 launch_search(d, qpad, (u32)nq, L, H, 0, k, as<u32>(idx->s_out_ids), as<float>(idx->s_out_dist),
+                               nullptr, nullptr, as<u64>(idx->s_seed), t, idx->num_sms, st, idx->search_prec,
+                               idx->cfg.rerank, nullptr, idx->search_prec == 0 && exact_rows(idx)) == cudaSuccess;
+            cudaEventRecord(e1, st);
+            if (cudaStreamSynchronize(st) != cudaSuccess) ok = false;
+            float ms = 0.f;
+            if (ok && rep > 0 && cudaEventElapsedTime(&ms, e0, e1) == cudaSuccess) ms_best = std::min(ms_best, ms);
         }
+        cudaGetLastError();   // a shape that does not fit is skipped
+        if (!ok) return;
+        // the library's own rule (stage_rows = seen_bits = 0) is reported as such
+        if (out && tried < n_out)
+            out[tried] = etale_tuning{t.stage_rows, t.seen_bits, ms_best, t.warps_per_block, t.keys_tc};
+        tried++;
+        if (ms_best < best) { best = ms_best; best_t = t; }
+    };
+    for (u32 kp = 0; kp < n_keys; kp++) {
+        SearchTuning own;
+        own.keys_tc = kp == 0 ? 1u : 0u;
+        time_shape(own);
+        for (u32 c = 0; c < 3; c++)
+            for (u32 a = 0; a < 4; a++)
+                for (u32 b = 0; b < 4; b++) {
+                    SearchTuning t;
+                    t.stage_rows = rows[a];
+                    t.seen_bits = bits[b];
+                    t.warps_per_block = wpbs[c];
+                    t.keys_tc = own.keys_tc;
+                    if (fit_tuning(idx, L, t).stage_rows != t.stage_rows) continue;   // does not fit: not a shape
+                    time_shape(t);
+                }
+    }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     g_kernel_launches += 1 + 2 * 3 * tried;

@@ -6,9 +6,9 @@
 namespace etale {
 
 struct SearchTuning {
-    u32 stage_rows = 16;       // rows gathered per bulk-copy batch
-    u32 seen_bits = 9;         // log2 of the evaluated-id cache slots
-    u32 warps_per_block = 4;   // queries in flight per block: 2, 4 or 8
+    u32 stage_rows = 0;        // rows gathered per bulk-copy batch; 0: by the rule of auto_shape
+    u32 seen_bits = 0;         // log2 of the evaluated-id cache slots; 0: by the rule of auto_shape
+    u32 warps_per_block = 4;   // queries in flight per block: 2, 4 or 8 (staged rows of a chosen stage_rows)
     u32 keys_tc = 1;           // BF16 searches: keys from the tensor cores (1) or the CUDA cores (0)
 };
 

@@ -3,9 +3,12 @@
 //
 // Per expansion the warp reads the expanded node's slab (the reference word
 // was read when the node entered the beam), drops neighbours it has already
-// evaluated, gathers the remaining neighbour rows into shared memory with
-// bulk (TMA) copies completing on an mbarrier, computes their canonical
-// distances with 8 lanes per distance, and merges them into the beam.
+// evaluated, gathers the remaining neighbour rows, computes their canonical
+// distances, and merges them into the beam.  Rows of
+// up to 128 elements are read 8 lanes a row (eval_direct), longer ones by the
+// whole warp (eval_wide), straight into registers; BF16 rows for tensor-core
+// keys go through shared memory with bulk (TMA) copies completing on an
+// mbarrier (eval_staged).
 //
 // Visited set.  The beam semantics are those of an exact visited set: an id
 // evaluated once is never evaluated again.  The kernel keeps only a lossy
@@ -15,6 +18,7 @@
 // beam or was refused is refused again (its key is the same), and an id still
 // in the beam is recognised in the merge by its equal key and dropped.
 #include <algorithm>
+#include <type_traits>
 
 #include <cuda_fp16.h>
 #include <cuda_fp8.h>
@@ -36,9 +40,8 @@ struct SearchArgs {
     u64 *exp_keys;       // insert: nq x max_hops expanded non-tombstone keys
     u32 *exp_count;
     u32 stage_rows, seen_slots, seen_bits;
-    // the evaluated-id cache (see seen_layout): 0 = whole ids, else 8- or
-    // 16-bit tags behind a validity bitmap of seen_words words
-    u32 seen_tag, seen_shift, seen_tmask, seen_hmask, seen_words;
+    // the evaluated-id cache (see seen_layout): 0 = whole ids, else 8- or 16-bit tags
+    u32 seen_tag, seen_shift, seen_tmask, seen_hmask;
     u32 rowb;            // bytes per gathered row (fp32, bf16 or fp8 copy)
     u32 wq, err;         // work-queue counter and error word (query searches
                          // use their own, so they can overlap a writer)
@@ -168,17 +171,20 @@ __device__ __forceinline__ float canon_dist_q8(const float4 (&qr)[4], const floa
     return metric == 0 ? s : __fsub_rn(1.0f, s);
 }
 
+// Set in a beam entry's copy of the reference word once it is expanded (a bit
+// that the word itself leaves 0).
+constexpr u64 REF_EXP = 1ull << 62;
+
+constexpr int RIF_WIDE = 8;   // rows of any length from global memory (see eval_wide)
+
 struct WarpSmem {
     float *qv;       // mp
     float *stage;    // stage_rows x mp
     u64 *bkey;       // beam keys (L), ascending
-    u64 *bref;       // reference word sampled when the entry was evaluated
-    unsigned char *bflag;   // expanded flag
-    u64 *nkey;       // 32: surviving new keys, sorted
-    u64 *nref;       // 32
-    u32 *cid;        // 32 candidate ids
-    u64 *ckey;       // 32
-    u64 *cref;       // 32
+    u64 *bref;       // reference word sampled when the entry was evaluated, with REF_EXP
+    u64 *nkey;       // 32: scratch of the ring's seeding
+    u32 *cid;        // candidate ids: 32, or 64 staged
+    u64 *ckey;       // 64 (not for rows of at most 128 elements)
     u32 *seen;       // seen_slots
     u64 *bar;        // mbarrier; with tensor-core keys, |bf16(q)|^2 (bar + 16 bytes) and
                      // the query as bf16 pairs (bar + 32 bytes) follow it (tc_nq, tc_qb)
@@ -189,13 +195,12 @@ __host__ __device__ inline size_t align_up(size_t x, size_t a) { return (x + a -
 // Layout of a warp's evaluated-id cache of 2^bits slots.  With ids below
 // 2^cb (cb >= bits, from the capacity), h = id * 2654435761 mod 2^cb is a
 // bijection of [0, 2^cb); slot = h >> (cb - bits) and tag = the low cb - bits
-// bits of h identify the id, so a slot need only hold the tag: 8 or 16 bits
-// when cb - bits allows, beside one validity bit per slot.  Otherwise the
-// slot holds the whole id (slot = the top bits of the 32-bit product).  A
-// hit is therefore never wrong; a slot overwritten by another id only costs
-// a repeated evaluation.
+// bits of h identify the id, so a slot need only hold tag + 1 (0 = empty) in 8
+// or 16 bits when cb - bits allows.  Otherwise the slot holds the whole id
+// (slot = the top bits of the 32-bit product).  A hit is therefore never
+// wrong; a slot overwritten by another id only costs a repeated evaluation.
 struct SeenLayout {
-    u32 tag, shift, tmask, hmask, words;
+    u32 tag, shift, tmask, hmask;
     size_t bytes;
 };
 inline SeenLayout seen_layout(u64 capacity, u32 bits) {
@@ -203,46 +208,40 @@ inline SeenLayout seen_layout(u64 capacity, u32 bits) {
     while (cb < 32 && (1ull << cb) < capacity) cb++;
     SeenLayout l;
     l.shift = cb - bits;
-    l.tag = l.shift <= 8 ? 8u : l.shift <= 16 ? 16u : 0u;
+    l.tag = l.shift < 8 ? 8u : l.shift < 16 ? 16u : 0u;
     l.tmask = (1u << l.shift) - 1u;
     l.hmask = cb >= 32 ? ~0u : (1u << cb) - 1u;
-    const size_t slots = (size_t)1 << bits;
-    l.words = (u32)(slots >= 32 ? slots / 32 : 1);
-    l.bytes = l.tag == 0 ? slots * 4 : (size_t)l.words * 4 + slots * (l.tag / 8);
+    l.bytes = ((size_t)1 << bits) * (l.tag ? l.tag / 8 : 4);
     return l;
 }
 
-// srow: stage row stride in bytes; qbytes: the bf16 query of the tensor-core keys (or 0)
-__host__ __device__ inline size_t search_warp_bytes(u32 mp, u32 L, u32 stage_rows, size_t seen_bytes, u32 srow,
+// stageb: bytes of the row stage; qbytes: the bf16 query of the tensor-core keys (or 0);
+// direct: rows are evaluated in registers (eval_direct)
+__host__ __device__ inline size_t search_warp_bytes(u32 mp, u32 L, size_t stageb, size_t seen_bytes, bool direct,
                                                    u32 qbytes = 0) {
     size_t b = 0;
     b += align_up((size_t)mp * 4, 128);
-    b += align_up((size_t)stage_rows * srow, 128);
+    b += align_up(stageb, 128);
     b += 2 * align_up((size_t)L * 8, 16);
-    b += align_up((size_t)L, 16);
-    b += 32 * 8 * 2 + 32 * 4 + 32 * 8 * 2;
+    b += 32 * 8 + (direct ? 32 * 4 : 64 * (4 + 8));
     b += align_up(seen_bytes, 16);
     b += 16;
     if (qbytes) b += 16 + align_up(qbytes, 16);
     return align_up(b, 128);
 }
 
-__device__ inline WarpSmem carve(char *p, u32 mp, u32 L, u32 stage_rows, size_t seen_bytes, u32 srow,
-                                 u32 qbytes = 0) {
+__device__ inline WarpSmem carve(char *p, u32 mp, u32 L, size_t stageb, size_t seen_bytes, bool direct) {
     WarpSmem s;
     s.qv = reinterpret_cast<float *>(p); p += align_up((size_t)mp * 4, 128);
-    s.stage = reinterpret_cast<float *>(p); p += align_up((size_t)stage_rows * srow, 128);
+    s.stage = reinterpret_cast<float *>(p); p += align_up(stageb, 128);
     s.bkey = reinterpret_cast<u64 *>(p); p += align_up((size_t)L * 8, 16);
     s.bref = reinterpret_cast<u64 *>(p); p += align_up((size_t)L * 8, 16);
-    s.bflag = reinterpret_cast<unsigned char *>(p); p += align_up((size_t)L, 16);
     s.nkey = reinterpret_cast<u64 *>(p); p += 32 * 8;
-    s.nref = reinterpret_cast<u64 *>(p); p += 32 * 8;
-    s.ckey = reinterpret_cast<u64 *>(p); p += 32 * 8;
-    s.cref = reinterpret_cast<u64 *>(p); p += 32 * 8;
-    s.cid = reinterpret_cast<u32 *>(p); p += 32 * 4;
+    s.cid = reinterpret_cast<u32 *>(p); p += (direct ? 32 : 64) * 4;
+    s.ckey = nullptr;
+    if (!direct) { s.ckey = reinterpret_cast<u64 *>(p); p += 64 * 8; }
     s.seen = reinterpret_cast<u32 *>(p); p += align_up(seen_bytes, 16);
     s.bar = reinterpret_cast<u64 *>(p);
-    (void)qbytes;
     return s;
 }
 
@@ -257,35 +256,31 @@ __device__ __forceinline__ u32 *tc_qb(const WarpSmem &s) {
 __device__ __forceinline__ u32 seen_slot(u32 id, u32 bits) { return (id * 2654435761u) >> (32 - bits); }
 
 __host__ __device__ inline size_t seen_bytes(const SearchArgs &a) {
-    return a.seen_tag == 0 ? (size_t)a.seen_slots * 4 : (size_t)a.seen_words * 4 + (size_t)a.seen_slots * (a.seen_tag / 8);
+    return (size_t)a.seen_slots * (a.seen_tag ? a.seen_tag / 8 : 4);
 }
 
 __device__ __forceinline__ bool seen_has(const SearchArgs &a, const WarpSmem &s, u32 id) {
     if (a.seen_tag == 0) return s.seen[seen_slot(id, a.seen_bits)] == id;
-    const u32 h = (id * 2654435761u) & a.seen_hmask, slot = h >> a.seen_shift, tag = h & a.seen_tmask;
-    if (!((s.seen[slot >> 5] >> (slot & 31)) & 1u)) return false;
-    const void *tags = s.seen + a.seen_words;
-    return a.seen_tag == 8 ? reinterpret_cast<const unsigned char *>(tags)[slot] == tag
-                           : reinterpret_cast<const unsigned short *>(tags)[slot] == tag;
+    const u32 h = (id * 2654435761u) & a.seen_hmask, slot = h >> a.seen_shift, tag = (h & a.seen_tmask) + 1u;
+    return a.seen_tag == 8 ? reinterpret_cast<const unsigned char *>(s.seen)[slot] == tag
+                           : reinterpret_cast<const unsigned short *>(s.seen)[slot] == tag;
 }
 
-// Lanes may record ids into the same slot at once: one tag stays, its bit set.
+// Lanes may record ids into the same slot at once: one tag stays.
 __device__ __forceinline__ void seen_put(const SearchArgs &a, const WarpSmem &s, u32 id) {
     if (a.seen_tag == 0) {
         s.seen[seen_slot(id, a.seen_bits)] = id;
         return;
     }
-    const u32 h = (id * 2654435761u) & a.seen_hmask, slot = h >> a.seen_shift, tag = h & a.seen_tmask;
-    void *tags = s.seen + a.seen_words;
-    if (a.seen_tag == 8) reinterpret_cast<unsigned char *>(tags)[slot] = (unsigned char)tag;
-    else reinterpret_cast<unsigned short *>(tags)[slot] = (unsigned short)tag;
-    atomicOr(s.seen + (slot >> 5), 1u << (slot & 31));
+    const u32 h = (id * 2654435761u) & a.seen_hmask, slot = h >> a.seen_shift, tag = (h & a.seen_tmask) + 1u;
+    if (a.seen_tag == 8) reinterpret_cast<unsigned char *>(s.seen)[slot] = (unsigned char)tag;
+    else reinterpret_cast<unsigned short *>(s.seen)[slot] = (unsigned short)tag;
 }
 
 __device__ __forceinline__ void seen_clear(const SearchArgs &a, const WarpSmem &s) {
-    const u32 n = a.seen_tag == 0 ? a.seen_slots : a.seen_words;
+    const u32 n = (u32)(seen_bytes(a) / 16);   // a multiple of 16 bytes: at least 2^6 slots
     const u32 v = a.seen_tag == 0 ? NIL : 0u;
-    for (u32 i = lane_id(); i < n; i += 32) s.seen[i] = v;
+    for (u32 i = lane_id(); i < n; i += 32) reinterpret_cast<uint4 *>(s.seen)[i] = make_uint4(v, v, v, v);
 }
 
 __device__ __forceinline__ int lower_bound(const u64 *a, int n, u64 key) {
@@ -298,59 +293,56 @@ __device__ __forceinline__ int lower_bound(const u64 *a, int n, u64 key) {
 }
 
 // Merge the candidate keys held one per lane (KEY_INF = none) into the beam
-// in place.  Only keys that can enter the beam take part; entries before the
-// first insertion point do not move, so `lo` (every entry before it is
-// expanded) drops to that point at most.  Returns the new beam size.
-__device__ int merge_beam(WarpSmem &s, u64 key, u64 ref, int n, int L, int &lo) {
+// in place: the beam stays the L smallest keys evaluated so far, ascending.
+// Every new key finds its final place (its lower bound in the beam plus its
+// rank among the new ones); then each 32-entry chunk from the last to the
+// first that changes is filled by place: a bit mask of the new keys' places
+// tells every other lane how far down its entry moves.  um: lane w holds the
+// bits of the unexpanded entries of chunk w.  Returns the new beam size.
+__device__ __forceinline__ int merge_beam(WarpSmem &s, u64 key, u64 ref, int n, int L, u32 &um) {
     const int lane = lane_id();
-    const u64 *bk = s.bkey;
+    u64 *bk = s.bkey;
     // drop keys that cannot enter a full beam, and keys already in the beam
+    if (n == L && key >= bk[n - 1]) key = KEY_INF;
+    if (!__any_sync(FULL, key != KEY_INF)) return n;
     int lb = 0;
-    if (key != KEY_INF) {
-        if (n == L && key >= bk[n - 1]) {
-            key = KEY_INF;
-        } else {
-            lb = lower_bound(bk, n, key);
-            if (lb < n && bk[lb] == key) key = KEY_INF;
-        }
+#pragma unroll
+    for (int step = 128; step >= 1; step >>= 1) {   // L <= 256
+        const int p = lb + step;
+        if (p <= n && bk[p - 1] < key) lb = p;
     }
+    if (lb < n && bk[lb] == key) key = KEY_INF;
     const u32 vm = __ballot_sync(FULL, key != KEY_INF);
     if (vm == 0) return n;
-    int rank = 0;
-    for (u32 m = vm; m; m &= m - 1) {
-        const u64 o = __shfl_sync(FULL, key, __ffs(m) - 1);
-        rank += (o < key);
-    }
-    const int c = __popc(vm);
-    if (key != KEY_INF) { s.nkey[rank] = key; s.nref[rank] = ref; }
-    // the first insertion point is the lower bound of the smallest new key
-    int p0 = (key != KEY_INF && rank == 0) ? lb : 0x7fffffff;
-    for (int o = 16; o >= 1; o >>= 1) p0 = min(p0, __shfl_xor_sync(FULL, p0, o));
-    lo = min(lo, p0);
-    __syncwarp();
-    // move entries [p0, n) down, last chunk first so no unread entry is overwritten
-    const int nmove = n - p0;
-    for (int c0 = ((nmove - 1) >> 5) << 5; c0 >= 0 && nmove > 0; c0 -= 32) {
-        const int i = p0 + c0 + lane;
+    int pos = lb;
+    for (u32 m = vm; m; m &= m - 1) pos += __shfl_sync(FULL, key, __ffs(m) - 1) < key;
+    const int nn = min(L, n + __popc(vm));
+    const u32 pw = key != KEY_INF ? (u32)pos : 0x7fffu;
+    const int w0 = (int)(__reduce_min_sync(FULL, pw) >> 5);
+    for (int w = (nn - 1) >> 5; w >= w0; w--) {
+        const u32 M = __reduce_or_sync(FULL, (int)(pw >> 5) == w ? 1u << (pw & 31) : 0u);
+        const int before = __popc(__ballot_sync(FULL, pw < 32u * w));
+        const int q = 32 * w + lane, k = before + __popc(M & lanemask_lt());
+        const bool fresh = (M >> lane) & 1u, old = q < nn && !fresh;
         u64 k2 = 0, r2 = 0;
-        unsigned char f2 = 0;
-        int pos = 0x7fffffff;
-        if (c0 + lane < nmove) {
-            k2 = bk[i];
-            r2 = s.bref[i];
-            f2 = s.bflag[i];
-            pos = i + lower_bound(s.nkey, c, k2);   // new keys below it (sorted, distinct)
+        if (old) {
+            k2 = bk[q - k];
+            r2 = s.bref[q - k];
         }
-        __syncwarp();
-        if (pos < L) { s.bkey[pos] = k2; s.bref[pos] = r2; s.bflag[pos] = f2; }
-        __syncwarp();
+        const u32 u = __ballot_sync(FULL, q < nn && (fresh || !(r2 & REF_EXP)));
+        if (lane == w) um = u;
+        __syncwarp();   // every lane has read its entry
+        if (old && k) {
+            bk[q] = k2;
+            s.bref[q] = r2;
+        }
     }
-    if (key != KEY_INF) {
-        const int pos = lb + rank;
-        if (pos < L) { s.bkey[pos] = key; s.bref[pos] = ref; s.bflag[pos] = 0; }
+    if ((int)pw < nn) {
+        bk[pos] = key;
+        s.bref[pos] = ref;
     }
     __syncwarp();
-    return min(L, n + c);
+    return nn;
 }
 
 // Tensor-core keys of a reduced-precision BF16 search.  The dot products of
@@ -372,27 +364,27 @@ __device__ void tc_keys(const SearchArgs &a, const WarpSmem &s, int nb, const u3
     for (int nt = 0; nt < 4; nt++)
 #pragma unroll
         for (int c = 0; c < 4; c++) acc[nt][c] = 0.0f;
-    for (u32 k0 = 0; k0 < d.mb; k0 += 32) {
-        // two k-steps of 16; A is zero outside row 0 (lanes 0..3)
-        u32 q0 = 0, q1 = 0, q2 = 0, q3 = 0;
-        if (g == 0) {
-            q0 = qb[(k0 >> 1) + t];
-            q1 = qb[(k0 >> 1) + 4 + t];
-            q2 = qb[(k0 >> 1) + 8 + t];
-            q3 = qb[(k0 >> 1) + 12 + t];
+    // one row tile's k-steps: a chain of dependent MMAs, its operands loaded
+    // four pairs of steps ahead
+    auto chain = [&](float (&ac)[4], int nt) {
+        u32 row = (u32)nt * 8 + r;
+        if ((int)row >= nb) row = 0;   // a staged row; its products are not read
+        const u32 ra = sb + row * a.srow + 16 * mi;
+#pragma unroll 4
+        for (u32 k0 = 0; k0 < d.mb; k0 += 32) {
+            // two k-steps of 16; A is zero outside row 0 (lanes 0..3)
+            const u32 *qk = qb + (k0 >> 1) + t;
+            const u32 w0 = qk[0], w1 = qk[4], w2 = qk[8], w3 = qk[12];
+            u32 b0, b1, b2, b3;
+            ldsm_x4(b0, b1, b2, b3, ra + 2 * k0);
+            mma_bf16_16816(ac, g == 0 ? w0 : 0u, 0u, g == 0 ? w1 : 0u, 0u, b0, b1);
+            mma_bf16_16816(ac, g == 0 ? w2 : 0u, 0u, g == 0 ? w3 : 0u, 0u, b2, b3);
         }
-#pragma unroll
-        for (int nt = 0; nt < 4; nt++) {
-            if (nt < ntn) {
-                u32 row = (u32)nt * 8 + r;
-                if ((int)row >= nb) row = 0;   // a staged row; its products are not read
-                u32 b0, b1, b2, b3;
-                ldsm_x4(b0, b1, b2, b3, sb + row * a.srow + (k0 + 8 * mi) * 2);
-                mma_bf16_16816(acc[nt], q0, 0u, q1, 0u, b0, b1);
-                mma_bf16_16816(acc[nt], q2, 0u, q3, 0u, b2, b3);
-            }
-        }
-    }
+    };
+    chain(acc[0], 0);
+    if (ntn > 1) chain(acc[1], 1);
+    if (ntn > 2) chain(acc[2], 2);
+    if (ntn > 3) chain(acc[3], 3);
     if (g == 0) {
         const float nq = *tc_nq(s);
 #pragma unroll
@@ -433,81 +425,267 @@ __device__ __forceinline__ void stage_ids(const SearchArgs &a, WarpSmem &s, cons
     __syncwarp();
 }
 
-// Evaluate the candidate ids held one per lane (NIL = none) and merge them
-// into the beam.  Returns the new beam size.  `phase` tracks the mbarrier.
-template <int P, bool LOG>
-__device__ int eval_merge(const SearchArgs &a, WarpSmem &s, u32 my_id, int n, u32 &phase, u64 &ndist,
-                          bool &timeout, int &lo, const float4 (&qr)[4], u32 *qlog, u32 &qcnt) {
-    const Dev &d = a.d;
-    const int lane = lane_id();
-    const u32 mp = d.mp;
-    u32 mask = __ballot_sync(FULL, my_id != NIL);
-    const int cnt = __popc(mask);
-    if (cnt == 0) return n;
-    if (my_id != NIL) s.cid[__popc(mask & lanemask_lt())] = my_id;
-    __syncwarp();
-    const u32 rowb = a.rowb, srow = P == 1 ? a.srow : a.rowb;   // only BF16 pads its stage rows
-    unsigned char *stage = reinterpret_cast<unsigned char *>(s.stage);
-    float *scl = reinterpret_cast<float *>(s.nref);   // fp8 scales of the batch (nref is free here)
+// Tensor-core keys of the cnt <= 64 candidates s.cid into s.ckey, their rows
+// staged in shared memory.  `phase` tracks the mbarrier.
+template <int P>
+__device__ void eval_staged(const SearchArgs &a, WarpSmem &s, int cnt, u32 &phase, bool &timeout) {
     for (int b0 = 0; b0 < cnt; b0 += (int)a.stage_rows) {
         const int nb = min((int)a.stage_rows, cnt - b0);
-        if (lane == 0) {
-            // generic-proxy reads of the stage (previous batch) before async-proxy writes
-            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-            mbar_expect_tx(s.bar, (u32)nb * rowb);
+        stage_ids<P>(a, s, s.cid + b0, nb, phase, timeout);
+        tc_keys(a, s, nb, s.cid + b0, s.ckey + b0);
+    }
+}
+
+// 16 bytes of a row that is read once: not kept in L1, whose few lines beside
+// the shared memory are left to the slabs and reference words (10k queries on
+// 1M x 128 rows: 2,240 -> 2,119 us).
+__device__ __forceinline__ float4 ld_row4(const float *p) {
+    float4 v;
+    asm volatile("ld.global.nc.L1::no_allocate.v4.f32 {%0, %1, %2, %3}, [%4];"
+                 : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+                 : "l"(p));
+    return v;
+}
+
+// Distances of the query (shared memory) to C rows of any length in global
+// memory, the whole warp on each: lane j sums partial j of every row (see
+// canon_dist), U column blocks of every row in flight, and the rows' canonical
+// trees share their shuffles: at the first levels a lane keeps half of the
+// rows it still has and passes the others on.  Lane l returns the value of row
+// l / (32 / C).
+template <int P, int C, int U>
+__device__ __forceinline__ float warp_dists(const float *__restrict__ q, const void *const (&row)[C],
+                                            const float (&sc)[C], int mp, int metric) {
+    const int lane = lane_id();
+    float p[C];
+#pragma unroll
+    for (int c = 0; c < C; c++) p[c] = 0.0f;
+    for (int base = 4 * lane; base < mp; base += 128 * U) {
+        float4 v[U][C];
+#pragma unroll
+        for (int u = 0; u < U; u++) {
+            const int i = base + 128 * u;
+            if (i < mp) {
+#pragma unroll
+                for (int c = 0; c < C; c++) {
+                    if (P == 0) v[u][c] = ld_row4(reinterpret_cast<const float *>(row[c]) + i);
+                    else v[u][c] = load4<P>(row[c], i, sc[c]);
+                }
+            }
         }
-        __syncwarp();
-        u64 rf = 0;
-        if (lane < nb) {
-            const u32 id = s.cid[b0 + lane];
-            bulk_g2s(stage + (size_t)lane * srow, row_src<P>(d, id), rowb, s.bar);
-            rf = ld_ref(d, id);
-            if (P == 2) scl[lane] = d.x8s[id];
+#pragma unroll
+        for (int u = 0; u < U; u++) {
+            const int i = base + 128 * u;
+            if (i < mp) {
+                const float4 x = *reinterpret_cast<const float4 *>(q + i);
+#pragma unroll
+                for (int c = 0; c < C; c++) {
+                    const float4 y = v[u][c];
+                    if (metric == 0) {
+                        const float d0 = __fsub_rn(x.x, y.x), d1 = __fsub_rn(x.y, y.y);
+                        const float d2 = __fsub_rn(x.z, y.z), d3 = __fsub_rn(x.w, y.w);
+                        p[c] = __fmaf_rn(d3, d3, __fmaf_rn(d2, d2, __fmaf_rn(d1, d1, __fmaf_rn(d0, d0, p[c]))));
+                    } else {
+                        p[c] = __fmaf_rn(x.w, y.w, __fmaf_rn(x.z, y.z, __fmaf_rn(x.y, y.y, __fmaf_rn(x.x, y.x, p[c]))));
+                    }
+                }
+            }
         }
-        if (!mbar_wait(s.bar, phase, WAIT_LIMIT)) {
-            timeout = true;
-            mbar_wait(s.bar, phase, WAIT_LIMIT);   // let copies in flight land
+    }
+    float t = p[0];
+    int h = 16;
+    if (C == 4) {
+        const bool hi = lane & 16, mid = lane & 8;
+        const float a0 = __fadd_rn(hi ? p[2 % C] : p[0], __shfl_xor_sync(FULL, hi ? p[0] : p[2 % C], 16));
+        const float a1 = __fadd_rn(hi ? p[3 % C] : p[1 % C], __shfl_xor_sync(FULL, hi ? p[1 % C] : p[3 % C], 16));
+        t = __fadd_rn(mid ? a1 : a0, __shfl_xor_sync(FULL, mid ? a0 : a1, 8));
+        h = 4;
+    } else if (C == 2) {
+        const bool hi = lane & 16;
+        t = __fadd_rn(hi ? p[1 % C] : p[0], __shfl_xor_sync(FULL, hi ? p[0] : p[1 % C], 16));
+        h = 8;
+    }
+#pragma unroll
+    for (; h >= 1; h >>= 1) t = __fadd_rn(t, __shfl_xor_sync(FULL, t, h));
+    return metric == 0 ? t : __fsub_rn(1.0f, t);
+}
+
+// Keys of the cnt <= 64 candidates s.cid into s.ckey, rows of any length.
+template <int P, int U>
+__device__ __forceinline__ void eval_wide(const SearchArgs &a, WarpSmem &s, int cnt) {
+    const Dev &d = a.d;
+    const int lane = lane_id();
+    auto some = [&](auto tag, int c0) {
+        constexpr int C = decltype(tag)::value;
+        const void *row[C];
+        float sc[C];
+#pragma unroll
+        for (int c = 0; c < C; c++) {
+            const u32 id = s.cid[min(c0 + c, cnt - 1)];   // past the list: a valid row again
+            row[c] = row_src<P>(d, id);
+            sc[c] = P == 2 ? d.x8s[id] : 1.0f;
         }
-        phase ^= 1u;
-        if (lane < nb) s.cref[b0 + lane] = rf;
-        __syncwarp();
-        if (P == 1 && a.tc) {
-            tc_keys(a, s, nb, s.cid + b0, s.ckey + b0);
-            continue;
-        }
-        // 8 lanes per distance, 4 distances per round
-        const int grp = lane >> 3, g = lane & 7;
-        for (int r0 = 0; r0 < nb; r0 += 4) {
-            const int c = r0 + grp;
-            const int cc = c < nb ? c : nb - 1;   // idle groups recompute a valid row
-            float dist;
-            if (P == 0 && mp <= 128) {
-                dist = canon_dist_q8(qr, reinterpret_cast<const float *>(stage + (size_t)cc * srow), (int)mp,
-                                     (int)d.metric, g);
-            } else if (P == 1 && mp <= 128) {
-                // the bf16 row widened to fp32, then canon_dist's operations in its order
-                float4 v[4];
+        const float dist = warp_dists<P, C, U * 4 / C>(s.qv, row, sc, (int)d.mp, (int)d.metric);
+        const int i = c0 + lane / (32 / C);
+        if (i < cnt && lane % (32 / C) == 0) s.ckey[i] = mkkey(dist, s.cid[i]);
+    };
+    int c0 = 0;
+    for (; cnt - c0 > 2; c0 += 4) some(std::integral_constant<int, 4>{}, c0);
+    if (c0 < cnt) some(std::integral_constant<int, 2>{}, c0);
+    __syncwarp();
+}
+
+// Distances of the cnt <= 32 candidates s.cid, rows of at most 128 elements
+// loaded straight into registers: lane by lane a key and a sampled reference word.
+// 8 lanes per row, four rows a round, RIF rounds of loads in flight.  Four
+// rounds (16 candidates) share one reduction: at each level of the canonical
+// tree a lane keeps half of its rounds' sums and passes the others on, so that
+// the tree's last three levels take 4 shuffles instead of 12.  Each lane ends
+// with the key of one candidate (in no particular order).
+template <int P, int RIF>
+__device__ __forceinline__ void eval_direct(const SearchArgs &a, const WarpSmem &s, int cnt, const float4 (&qr)[4],
+                                            u64 &key, u64 &ref) {
+    const Dev &d = a.d;
+    const int lane = lane_id(), grp = lane >> 3, g = lane & 7;
+    const int mp = (int)d.mp;
+    // this lane's candidate: round g >> 1 of the first 16 (even lanes) or of the second
+    const int cm = 16 * (g & 1) + 4 * (g >> 1) + grp;
+    const u32 mine = cm < cnt ? s.cid[cm] : NIL;
+    ref = mine != NIL ? ld_ref(d, mine) : 0;
+    float dist = 0.0f;
+    for (int q0 = 0; q0 < cnt; q0 += 16) {
+        float p[4];
+#pragma unroll
+        for (int r0 = 0; r0 < 4; r0 += RIF) {
+            float4 v[RIF][4];
+#pragma unroll
+            for (int u = 0; u < RIF; u++) {
+                const int c0 = q0 + 4 * (r0 + u);
+                if (c0 < cnt) {
+                    const u32 id = s.cid[min(c0 + grp, cnt - 1)];   // idle groups recompute a valid row
+                    const void *row = row_src<P>(d, id);
+                    const float sc = P == 2 ? d.x8s[id] : 1.0f;
+#pragma unroll
+                    for (int t = 0; t < 4; t++) {
+                        const int i = 4 * (g + 8 * t);
+                        if (i >= mp) v[u][t] = make_float4(0.f, 0.f, 0.f, 0.f);
+                        else if (P == 0) v[u][t] = ld_row4(reinterpret_cast<const float *>(row) + i);
+                        else v[u][t] = load4<P>(row, i, sc);
+                    }
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < RIF; u++) {
+                if (q0 + 4 * (r0 + u) >= cnt) {
+                    p[r0 + u] = 0.0f;
+                    continue;
+                }
+                float e[4];
 #pragma unroll
                 for (int t = 0; t < 4; t++) {
-                    const int i = 4 * (g + 8 * t);
-                    v[t] = i < (int)mp ? load4<1>(stage + (size_t)cc * srow, i, 1.0f) : make_float4(0.f, 0.f, 0.f, 0.f);
+                    const float4 x = qr[t], y = v[u][t];
+                    // past the row both are zero: the partial stays +0, as it starts
+                    if (d.metric == 0) {
+                        const float d0 = __fsub_rn(x.x, y.x), d1 = __fsub_rn(x.y, y.y);
+                        const float d2 = __fsub_rn(x.z, y.z), d3 = __fsub_rn(x.w, y.w);
+                        e[t] = __fmaf_rn(d3, d3, __fmaf_rn(d2, d2, __fmaf_rn(d1, d1, __fmaf_rn(d0, d0, 0.0f))));
+                    } else {
+                        e[t] = __fmaf_rn(x.w, y.w, __fmaf_rn(x.z, y.z, __fmaf_rn(x.y, y.y, __fmaf_rn(x.x, y.x, 0.0f))));
+                    }
                 }
-                dist = canon_dist_q8v(qr, v, (int)mp, (int)d.metric, g);
-            } else
-                dist = qdist<P>(s.qv, stage + (size_t)cc * srow, P == 2 ? scl[cc] : 1.0f, (int)mp, (int)d.metric, g);
-            if (c < nb && g == 0) s.ckey[b0 + c] = mkkey(dist, s.cid[b0 + c]);
+                p[r0 + u] = __fadd_rn(__fadd_rn(e[0], e[2]), __fadd_rn(e[1], e[3]));
+            }
+        }
+        const bool h4 = g & 4, h2 = g & 2;
+        const float a0 = __fadd_rn(h4 ? p[2] : p[0], __shfl_xor_sync(FULL, h4 ? p[0] : p[2], 4));
+        const float a1 = __fadd_rn(h4 ? p[3] : p[1], __shfl_xor_sync(FULL, h4 ? p[1] : p[3], 4));
+        float t = __fadd_rn(h2 ? a1 : a0, __shfl_xor_sync(FULL, h2 ? a0 : a1, 2));
+        t = __fadd_rn(t, __shfl_xor_sync(FULL, t, 1));
+        if ((q0 >> 4) == (g & 1)) dist = t;
+    }
+    key = mine != NIL ? mkkey(d.metric == 0 ? dist : __fsub_rn(1.0f, dist), mine) : KEY_INF;
+}
+
+// Keys of the nb <= 32 candidates s.cid into out[0 .. nb), in any order.
+template <int P, int RIF>
+__device__ __forceinline__ void score32(const SearchArgs &a, WarpSmem &s, int nb, const float4 (&qr)[4], u64 *out) {
+    const int lane = lane_id();
+    if constexpr (RIF == RIF_WIDE || RIF == 0) {
+        eval_wide<P, 1>(a, s, nb);
+        if (lane < nb) out[lane] = s.ckey[lane];
+    } else {
+        u64 key, ref;
+        eval_direct<P, 1>(a, s, nb, qr, key, ref);
+        const u32 m = __ballot_sync(FULL, key != KEY_INF);
+        if (key != KEY_INF) out[__popc(m & lanemask_lt())] = key;
+    }
+    __syncwarp();
+}
+
+// Evaluate the unseen ids among a slab's entries e0 and e1 (held one per lane,
+// NIL = none) and merge them into the beam.  Returns the new beam size.  RIF:
+// see eval_direct; RIF_WIDE: eval_wide; 0: eval_staged.
+template <int P, bool LOG, int RIF>
+__device__ __forceinline__ int eval_merge(const SearchArgs &a, WarpSmem &s, u32 e0, u32 e1, int n, u32 &phase,
+                                          u64 &ndist, bool &timeout, u32 &um, const float4 (&qr)[4], u32 *qlog,
+                                          u32 &qcnt) {
+    const int lane = lane_id();
+    auto log = [&](int cnt) {
+        if (!LOG) return;
+        for (int i = lane; i < cnt; i += 32)
+            if (qcnt + i < a.elog_cap) qlog[qcnt + i] = s.cid[i];
+        qcnt += cnt;
+    };
+    if constexpr (RIF > 0 && RIF != RIF_WIDE) {
+#pragma unroll 1
+        for (int half = 0; half < 2; half++) {
+            u32 id = half ? e1 : e0;
+            if (id != NIL && seen_has(a, s, id)) id = NIL;
+            const u32 mask = __ballot_sync(FULL, id != NIL);
+            const int cnt = __popc(mask);
+            if (cnt) {
+                if (id != NIL) {
+                    s.cid[__popc(mask & lanemask_lt())] = id;
+                    seen_put(a, s, id);
+                }
+                __syncwarp();
+                u64 key, ref;
+                eval_direct<P, RIF>(a, s, cnt, qr, key, ref);
+                ndist += cnt;
+                log(cnt);
+                n = merge_beam(s, key, ref, n, (int)a.L, um);
+            }
+            if (a.d.R <= 32) break;
+        }
+    } else {
+        if (e0 != NIL && seen_has(a, s, e0)) e0 = NIL;
+        if (e1 != NIL && seen_has(a, s, e1)) e1 = NIL;
+        const u32 m0 = __ballot_sync(FULL, e0 != NIL), m1 = __ballot_sync(FULL, e1 != NIL);
+        const int c0 = __popc(m0), cnt = c0 + __popc(m1);
+        if (cnt == 0) return n;
+        if (e0 != NIL) {
+            s.cid[__popc(m0 & lanemask_lt())] = e0;
+            seen_put(a, s, e0);
+        }
+        if (e1 != NIL) {
+            s.cid[c0 + __popc(m1 & lanemask_lt())] = e1;
+            seen_put(a, s, e1);
         }
         __syncwarp();
+        u64 ref[2] = {0, 0};
+#pragma unroll
+        for (int u = 0; u < 2; u++)
+            if (lane + 32 * u < cnt) ref[u] = ld_ref(a.d, s.cid[lane + 32 * u]);
+        if constexpr (RIF == RIF_WIDE) eval_wide<P, 2>(a, s, cnt);
+        else eval_staged<P>(a, s, cnt, phase, timeout);
+        ndist += cnt;
+        log(cnt);
+#pragma unroll
+        for (int u = 0; u < 2; u++)
+            if (32 * u < cnt)
+                n = merge_beam(s, lane + 32 * u < cnt ? s.ckey[lane + 32 * u] : KEY_INF, ref[u], n, (int)a.L, um);
     }
-    ndist += cnt;
-    if (LOG) {
-        if (lane < cnt && qcnt + lane < a.elog_cap) qlog[qcnt + lane] = s.cid[lane];
-        qcnt += cnt;
-    }
-    const u64 key = lane < cnt ? s.ckey[lane] : KEY_INF;
-    const u64 ref = lane < cnt ? s.cref[lane] : 0;
-    if (lane < cnt) seen_put(a, s, key_id(key));
-    return merge_beam(s, key, ref, n, (int)a.L, lo);
+    return n;
 }
 
 // ---------------------------------------------------------------------------
@@ -626,12 +804,14 @@ __global__ void __launch_bounds__(256) seed_kernel(SeedArgs a) {
     }
 }
 
+// Bound by the latency of one expansion's chain (slab, rows, merge) and by its
+// instructions; at 10k queries on 1M x 128 rows the gathers move 4.9 TB/s.
 // One query's BeamSearch by one warp, for slot qi: the query row is
 // a.q + qi * mp, the beam starts from the seeds a.seed + qi * L (the L
 // nearest entry points, KEY_INF padded, n0 of them valid); query mode writes
 // the k results to a.out_ids / a.out_dist + qi * k, insert mode the expanded
 // keys of batch member qi.  The reference words of the seeds are sampled here.
-template <int P, bool LOG>
+template <int P, bool LOG, int RIF>
 __device__ __forceinline__ void search_one(const SearchArgs &a, WarpSmem &s, u32 qi, int n0, u32 &phase,
                                            u64 &nexp_tot, u64 &ndist, bool &timeout) {
     const int lane = lane_id();
@@ -669,47 +849,22 @@ __device__ __forceinline__ void search_one(const SearchArgs &a, WarpSmem &s, u32
     // initial beam: the L nearest members of the entry set E, computed by
     // seed_kernel; the reference words are sampled here
     const u64 *sk = seed_row;
-    if (P == 1 && a.tc) {
-        // the seeds' keys on the tensor cores, whichever kernel chose them,
-        // so that they are the keys this search gives any id; sorted in the stage
-        const int bs = min((int)a.stage_rows, 32);   // s.cid holds 32 ids
+    if (P != 0 && (a.tc || a.rekey)) {
+        // Seeds on tensor-core keys, or ranked by the canonical fp32 distance:
+        // every key in the beam must be the key this search gives its id (an
+        // id evaluated again then collapses with its seed), so the seeds are
+        // re-keyed, and sorted in the stage; the keys wait in the beam.
+        const int bs = a.tc ? min((int)a.stage_rows, 32) : 32;   // s.cid holds 32 ids
         for (int b0 = 0; b0 < n0; b0 += bs) {
             const int nb = min(bs, n0 - b0);
             if (lane < nb) s.cid[lane] = key_id(seed_row[b0 + lane]);
             __syncwarp();
-            stage_ids<P>(a, s, s.cid, nb, phase, timeout);
-            tc_keys(a, s, nb, s.cid, s.bkey + b0);
-        }
-        u64 *rk = reinterpret_cast<u64 *>(s.stage);
-        int np2 = 32;
-        while (np2 < n0) np2 <<= 1;
-        for (int i = lane; i < np2; i += 32) rk[i] = i < n0 ? s.bkey[i] : KEY_INF;
-        __syncwarp();
-        warp_sort_u64(rk, np2);
-        sk = rk;
-    } else if (P != 0 && a.rekey) {
-        // seeds ranked by the canonical fp32 distance: every key in the beam
-        // must be this precision's distance of its id (an id evaluated again
-        // then collapses with its seed), so the seeds are re-keyed and sorted.
-        // Their rows go through the stage like a neighbour batch; the keys
-        // wait in the beam until the stage is free for the sort.
-        const int bs = min((int)a.stage_rows, 32);   // s.cid holds 32 ids
-        const int grp = lane >> 3, g = lane & 7;
-        const unsigned char *stage = reinterpret_cast<const unsigned char *>(s.stage);
-        for (int b0 = 0; b0 < n0; b0 += bs) {
-            const int nb = min(bs, n0 - b0);
-            if (lane < nb) s.cid[lane] = key_id(seed_row[b0 + lane]);
-            __syncwarp();
-            stage_ids<P>(a, s, s.cid, nb, phase, timeout);
-            for (int r0 = 0; r0 < nb; r0 += 4) {
-                const int c = r0 + grp;
-                const int cc = c < nb ? c : nb - 1;
-                const u32 id = s.cid[cc];
-                const float dist = qdist<P>(s.qv, stage + (size_t)cc * a.srow, P == 2 ? d.x8s[id] : 1.0f, (int)mp,
-                                            (int)d.metric, g);
-                if (c < nb && g == 0) s.bkey[b0 + c] = mkkey(dist, id);
+            if (a.tc) {
+                stage_ids<P>(a, s, s.cid, nb, phase, timeout);
+                tc_keys(a, s, nb, s.cid, s.bkey + b0);
+            } else {
+                score32<P, RIF>(a, s, nb, qr, s.bkey + b0);
             }
-            __syncwarp();
         }
         u64 *rk = reinterpret_cast<u64 *>(s.stage);
         int np2 = 32;
@@ -724,27 +879,33 @@ __device__ __forceinline__ void search_one(const SearchArgs &a, WarpSmem &s, u32
         const u32 id = key_id(k);
         s.bkey[i] = k;
         s.bref[i] = ld_ref(d, id);
-        s.bflag[i] = 0;
         seen_put(a, s, id);
     }
     int n = n0;
+    // lane w: the unexpanded entries among [32 w, 32 w + 32)
+    u32 um = 32 * lane >= n0 ? 0u : n0 - 32 * lane >= 32 ? ~0u : (1u << (n0 - 32 * lane)) - 1u;
     __syncwarp();
     u32 hops = 0, nexp = 0;
     u32 qcnt = 0;
     u32 *qlog = LOG ? a.elog + (size_t)qi * a.elog_cap : nullptr;
     // slab entries of the predicted next expansion, loaded ahead of use
     u32 pf_id = NIL, pf0 = NIL, pf1 = NIL;
-    int lo = 0;   // every beam entry before lo is expanded
     for (;;) {
-        int first = -1;
-        for (int i0 = lo; i0 < n; i0 += 32) {
-            int i = i0 + lane;
-            u32 m = __ballot_sync(FULL, i < n && !s.bflag[i]);
-            if (m) { first = i0 + __ffs(m) - 1; break; }
-        }
-        if (first < 0 || hops >= a.max_hops) break;
+        const u32 chunks = __ballot_sync(FULL, um != 0);
+        if (chunks == 0 || hops >= a.max_hops) break;
         hops++;
-        lo = first + 1;
+        // the first unexpanded entry, and the next one: the predicted next expansion
+        const int w = __ffs(chunks) - 1;
+        const u32 word = __shfl_sync(FULL, um, w), rest = word & (word - 1);
+        const int first = 32 * w + __ffs(word) - 1;
+        if (lane == w) um = rest;
+        int nx = -1;
+        if (rest) {
+            nx = 32 * w + __ffs(rest) - 1;
+        } else if (chunks & (chunks - 1)) {
+            const int w2 = __ffs(chunks & (chunks - 1)) - 1;
+            nx = 32 * w2 + __ffs(__shfl_sync(FULL, um, w2)) - 1;
+        }
         const u64 r = s.bref[first];
         const u64 bkey = s.bkey[first];
         const u32 fid = key_id(bkey);
@@ -756,31 +917,20 @@ __device__ __forceinline__ void search_one(const SearchArgs &a, WarpSmem &s, u32
             if ((u32)lane < deg) e0 = d.slab[(size_t)sl * d.R + lane].x;
             if ((u32)lane + 32 < deg) e1 = d.slab[(size_t)sl * d.R + lane + 32].x;
         }
-        // predict the next expansion: the next unexpanded beam entry
         pf_id = NIL;
-        for (int i0 = first + 1; i0 < n; i0 += 32) {
-            int i = i0 + lane;
-            u32 m = __ballot_sync(FULL, i < n && !s.bflag[i]);
-            if (m) {
-                const int nx = i0 + __ffs(m) - 1;
-                const u64 r2 = s.bref[nx];
-                const u32 s2 = ref_slab(r2), d2 = s2 == NIL ? 0 : ref_deg(r2);
-                pf_id = key_id(s.bkey[nx]);
-                pf0 = (u32)lane < d2 ? d.slab[(size_t)s2 * d.R + lane].x : NIL;
-                pf1 = (u32)lane + 32 < d2 ? d.slab[(size_t)s2 * d.R + lane + 32].x : NIL;
-                break;
-            }
+        if (nx >= 0) {
+            const u64 r2 = s.bref[nx];
+            const u32 s2 = ref_slab(r2), d2 = s2 == NIL ? 0 : ref_deg(r2);
+            pf_id = key_id(s.bkey[nx]);
+            pf0 = (u32)lane < d2 ? d.slab[(size_t)s2 * d.R + lane].x : NIL;
+            pf1 = (u32)lane + 32 < d2 ? d.slab[(size_t)s2 * d.R + lane + 32].x : NIL;
         }
         __syncwarp();
-        if (lane == 0) s.bflag[first] = 1;
+        if (lane == 0) s.bref[first] = r | REF_EXP;
         if (a.mode == 1 && lane == 0 && !ref_del(r)) a.exp_keys[(size_t)qi * a.max_hops + nexp] = bkey;
         if (!ref_del(r)) nexp++;
         __syncwarp();
-        for (u32 j0 = 0; j0 < deg; j0 += 32) {
-            u32 nb = j0 == 0 ? e0 : e1;
-            if (nb != NIL && seen_has(a, s, nb)) nb = NIL;
-            n = eval_merge<P, LOG>(a, s, nb, n, phase, ndist, timeout, lo, qr, qlog, qcnt);
-        }
+        n = eval_merge<P, LOG, RIF>(a, s, e0, e1, n, phase, ndist, timeout, um, qr, qlog, qcnt);
     }
     nexp_tot += hops;
     if (LOG && lane == 0) a.elog_n[qi] = qcnt;
@@ -800,48 +950,12 @@ __device__ __forceinline__ void search_one(const SearchArgs &a, WarpSmem &s, u32
             c = min(want, c + __popc(m));
         }
         __syncwarp();
-        const int grp = lane >> 3, g = lane & 7;
-        // the fp32 rows go through the stage behind the keys, as many per bulk
-        // copy as fit; a stage too small for one row reads them in place
-        const u32 rowf = mp * 4u, rkb = (u32)rn * 8u;
-        const u32 stb = a.stage_rows * a.srow;
-        const int per = stb > rkb ? (int)min(32u, (stb - rkb) / rowf) : 0;
-        if (per > 0) {
-            unsigned char *rows = reinterpret_cast<unsigned char *>(s.stage) + rkb;
-            for (int b0 = 0; b0 < c; b0 += per) {
-                const int nb = min(per, c - b0);
-                if (lane == 0) {
-                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-                    mbar_expect_tx(s.bar, (u32)nb * rowf);
-                }
-                __syncwarp();
-                if (lane < nb) bulk_g2s(rows + (size_t)lane * rowf, d.x + (size_t)key_id(rk[b0 + lane]) * mp, rowf, s.bar);
-                if (!mbar_wait(s.bar, phase, WAIT_LIMIT)) {
-                    timeout = true;
-                    mbar_wait(s.bar, phase, WAIT_LIMIT);   // let copies in flight land
-                }
-                phase ^= 1u;
-                __syncwarp();
-                for (int r0 = 0; r0 < nb; r0 += 4) {
-                    const int cc = min(r0 + grp, nb - 1);
-                    const u32 id = key_id(rk[b0 + cc]);
-                    const float dist = canon_dist<8>(s.qv, reinterpret_cast<const float *>(rows + (size_t)cc * rowf),
-                                                     (int)mp, (int)d.metric, g);
-                    __syncwarp();
-                    if (r0 + grp < nb && g == 0) rk[b0 + cc] = mkkey(dist, id);
-                    __syncwarp();
-                }
-            }
-        } else {
-            for (int i = lane; i < c; i += 32) bulk_prefetch_l2(d.x + (size_t)key_id(rk[i]) * mp, rowf);
-            for (int r0 = 0; r0 < c; r0 += 4) {
-                const int cc = min(r0 + grp, c - 1);
-                const u32 id = key_id(rk[cc]);
-                const float dist = canon_dist<8>(s.qv, d.x + (size_t)id * mp, (int)mp, (int)d.metric, g);
-                __syncwarp();
-                if (r0 + grp < c && g == 0) rk[cc] = mkkey(dist, id);
-                __syncwarp();
-            }
+        for (int b0 = 0; b0 < c; b0 += 32) {
+            const int nb = min(32, c - b0);
+            if (lane < nb) s.cid[lane] = key_id(rk[b0 + lane]);
+            __syncwarp();
+            // a search whose rows are short keeps no list for eval_wide
+            score32<0, (RIF == 0 || RIF == RIF_WIDE ? RIF_WIDE : 2)>(a, s, nb, qr, rk + b0);   // sorted below
         }
         for (int i = c + lane; i < rn; i += 32) rk[i] = KEY_INF;
         __syncwarp();
@@ -886,17 +1000,23 @@ __device__ __forceinline__ void search_one(const SearchArgs &a, WarpSmem &s, u32
     }
 }
 
-// WPB warps (queries in flight) per block; about 24 resident warps per SM.
-template <int P, bool LOG = false, int WPB = 4>
-__global__ void __launch_bounds__(32 * WPB, 24 / WPB) search_kernel(SearchArgs a) {
+// Bytes of a search's row stage: none for fp32 rows; a reduced-precision search
+// sorts its rerank candidates and seeds there.
+__host__ __device__ inline size_t stage_bytes(const SearchArgs &a, int P) {
+    return P == 0 ? 0 : (size_t)a.stage_rows * a.srow;
+}
+
+// WPB warps (queries in flight) per block; 16 resident warps per SM, 24 with one
+// round of rows in flight.
+template <int P, bool LOG = false, int WPB = 4, int RIF = 0>
+__global__ void __launch_bounds__(32 * WPB, (RIF == 1 ? 24 : 16) / WPB) search_kernel(SearchArgs a) {
     extern __shared__ __align__(128) char smem[];
     const int warp = threadIdx.x >> 5, lane = lane_id();
     const Dev &d = a.d;
     const u32 mp = d.mp;
-    const size_t sb = seen_bytes(a);
-    const u32 qbytes = a.tc ? d.mb * 2 : 0u;
-    const size_t wb = search_warp_bytes(mp, a.L, a.stage_rows, sb, a.srow, qbytes);
-    WarpSmem s = carve(smem + warp * wb, mp, a.L, a.stage_rows, sb, a.srow, qbytes);
+    const size_t sb = seen_bytes(a), stb = stage_bytes(a, P);
+    const size_t wb = search_warp_bytes(mp, a.L, stb, sb, RIF > 0 && RIF != RIF_WIDE, a.tc ? d.mb * 2 : 0u);
+    WarpSmem s = carve(smem + warp * wb, mp, a.L, stb, sb, RIF > 0 && RIF != RIF_WIDE);
     if (lane == 0) mbar_init(s.bar, 1);
     __syncwarp();
     u32 phase = 0;
@@ -909,7 +1029,7 @@ __global__ void __launch_bounds__(32 * WPB, 24 / WPB) search_kernel(SearchArgs a
         if (lane == 0) qi = (u32)atomicAdd(&d.ctr[a.wq], 1ull);
         qi = __shfl_sync(FULL, qi, 0);
         if (qi >= nq) break;
-        search_one<P, LOG>(a, s, qi, n0, phase, nexp_tot, ndist, timeout);
+        search_one<P, LOG, RIF>(a, s, qi, n0, phase, nexp_tot, ndist, timeout);
         __syncwarp();
     }
     if (lane == 0) {
@@ -1043,15 +1163,14 @@ __device__ void ring_seed(const SearchArgs &a, WarpSmem &s, u32 qi) {
     __syncwarp();
 }
 
-template <int P>
+template <int P, int RIF>
 __global__ void __launch_bounds__(128, 3) ring_search_kernel(SearchArgs a, RingArgs r) {
     extern __shared__ __align__(128) char smem[];
     const int warp = threadIdx.x >> 5, lane = lane_id();
     const Dev &d = a.d;
-    const size_t sb = seen_bytes(a);
-    const u32 qbytes = a.tc ? d.mb * 2 : 0u;
-    const size_t wb = search_warp_bytes(d.mp, a.L, a.stage_rows, sb, a.srow, qbytes);
-    WarpSmem s = carve(smem + warp * wb, d.mp, a.L, a.stage_rows, sb, a.srow, qbytes);
+    const size_t sb = seen_bytes(a), stb = stage_bytes(a, P);
+    const size_t wb = search_warp_bytes(d.mp, a.L, stb, sb, RIF > 0 && RIF != RIF_WIDE, a.tc ? d.mb * 2 : 0u);
+    WarpSmem s = carve(smem + warp * wb, d.mp, a.L, stb, sb, RIF > 0 && RIF != RIF_WIDE);
     if (lane == 0) mbar_init(s.bar, 1);
     __syncwarp();
     u32 phase = 0;
@@ -1101,7 +1220,7 @@ __global__ void __launch_bounds__(128, 3) ring_search_kernel(SearchArgs a, RingA
         ring_seed<P>(a, s, slot);
         const u64 t1 = globaltimer_ns();
         const int n0 = (int)min(a.L, d.nent_dev ? *d.nent_dev : d.n_entries);
-        search_one<P, false>(a, s, slot, n0, phase, nexp_tot, ndist, timeout);
+        search_one<P, false, RIF>(a, s, slot, n0, phase, nexp_tot, ndist, timeout);
         __syncwarp();
         if (lane == 0) {
             served++;
@@ -1130,13 +1249,14 @@ __global__ void __launch_bounds__(128, 3) ring_search_kernel(SearchArgs a, RingA
 // is a multiple of 32; its stage rows are then padded to an odd number of
 // 16-byte chunks, so that ldmatrix's eight row reads fall in distinct banks.
 static void set_tc(SearchArgs &a, const Dev &d, u32 prec, bool exact_rows, u32 keys_tc) {
+    const bool chosen = a.stage_rows != 0;   // 0: the rule below picks it
     a.tc = keys_tc && prec == 1 && !exact_rows && d.xbn != nullptr && d.mb % 32 == 0 ? 1u : 0u;
     a.srow = a.tc && (a.rowb / 16) % 2 == 0 ? a.rowb + 16 : a.rowb;
     // a BF16 row is half an fp32 row: as many rows per gather as the fp32
     // shape's stage bytes hold (up to 32), so an expansion needs fewer round
     // trips (measured on the 768-d inner-product index: 497k -> 527k
     // queries/s; FP8 rows at four times the count lost occupancy instead)
-    if (prec == 1 && !exact_rows)
+    if (chosen && prec == 1 && !exact_rows)
         a.stage_rows = std::min<u32>(32, std::max<u32>(a.stage_rows, a.stage_rows * d.mp * 4 / a.srow));
 }
 
@@ -1172,6 +1292,10 @@ static u32 fit_stage(SearchArgs &a, u32 L, u32 k, u32 rerank, u32 prec, u32 mode
     return min_rows;
 }
 
+// Rows of at most 128 elements are evaluated 8 lanes a row (eval_direct), unless
+// the keys come from the tensor cores, which read staged rows.
+static bool direct_rows(const SearchArgs &a, const Dev &d) { return d.mp <= 128 && !a.tc; }
+
 static SeenLayout set_seen(SearchArgs &a, const Dev &d, u32 bits) {
     const SeenLayout l = seen_layout(d.capacity, bits);
     a.seen_bits = bits;
@@ -1180,8 +1304,32 @@ static SeenLayout set_seen(SearchArgs &a, const Dev &d, u32 bits) {
     a.seen_shift = l.shift;
     a.seen_tmask = l.tmask;
     a.seen_hmask = l.hmask;
-    a.seen_words = l.words;
     return l;
+}
+
+// The launch shape of a search whose tuning leaves it open (0): rows per stage
+// and the evaluated-id cache.  `resident` is the warps an SM should hold.
+//  - Stage: tensor-core keys take eight rows, one tile of MMAs.  Nothing else
+//    reads staged rows (the stage then only holds sorts, see fit_stage).
+//    4,096 queries on 50k x 768 BF16, beam 64: 6,497 us with the former 31 rows,
+//    1,331 with eight, 1,562 with eleven.
+//  - Cache: the largest power of two of at most 8 KB that leaves `resident`
+//    warps their shared memory, or that covers every id.  Larger caches repeat
+//    fewer evaluations (1M x 128, beam 144: 14.8, 13.1, 12.1 per expansion at
+//    2^11, 2^12, 2^13 slots); beyond 8 KB resident warps were worth more.
+static void auto_shape(SearchArgs &a, const Dev &d, u32 &seen_bits, u32 prec, u32 L, bool direct, u32 resident) {
+    if (!a.tc) a.stage_rows = 1;
+    else if (a.stage_rows == 0) a.stage_rows = 8;
+    if (seen_bits) return;
+    const size_t budget = (227u << 10) / std::max<u32>(1, resident) - 1024;   // a block's own 1 KB
+    seen_bits = 9;
+    for (u32 b = 10; b <= 13 && (1ull << (b - 1)) < d.capacity; b++) {
+        const size_t sb = seen_layout(d.capacity, b).bytes;
+        if (sb > (8u << 10) ||
+            search_warp_bytes(d.mp, L, stage_bytes(a, (int)prec), sb, direct, a.tc ? d.mb * 2 : 0u) > budget)
+            break;
+        seen_bits = b;
+    }
 }
 
 cudaError_t launch_ring_search(const Dev &d, float *rows, u32 slots, u32 L, u32 max_hops, u32 k, u32 *out_ids,
@@ -1193,23 +1341,28 @@ cudaError_t launch_ring_search(const Dev &d, float *rows, u32 slots, u32 L, u32 
     a.d = d; a.q = rows; a.seed = seed; a.nq_dev = nullptr; a.nq = slots; a.L = L; a.max_hops = max_hops;
     a.mode = 0; a.k = k; a.out_ids = out_ids; a.out_dist = out_dist;
     a.stage_rows = tune.stage_rows;
-    const SeenLayout sl = set_seen(a, d, tune.seen_bits);
     a.rowb = prec == 1 ? d.mb * 2 : prec == 2 ? d.m8 : d.mp * 4;
     a.rerank = rerank;
     a.exact = 0;
     a.wq = C_WORK2;
     a.err = C_ERR_S;
     set_tc(a, d, prec, false, tune.keys_tc);
+    const bool direct = direct_rows(a, d);
+    u32 bits = tune.seen_bits;
+    auto_shape(a, d, bits, prec, L, direct, 12);
+    const SeenLayout sl = set_seen(a, d, bits);
     const u32 min_rows = fit_stage(a, L, k, rerank, prec, 0);
     // head: claimed, device count, last host poll, stop flag, then the statistics
     RingArgs r{head, head + 1, head + 2, head + 3, head + 4, tail, closed, done, served_by, slots, seq, max_ns};
     using K = void (*)(SearchArgs, RingArgs);
-    K fn = prec == 1 ? ring_search_kernel<1> : prec == 2 ? ring_search_kernel<2> : ring_search_kernel<0>;
-    size_t smem = 4 * search_warp_bytes(d.mp, L, a.stage_rows, sl.bytes, a.srow, a.tc ? d.mb * 2 : 0u);
-    while (smem > smem_optin_bytes() && a.stage_rows > min_rows) {
-        a.stage_rows--;
-        smem = 4 * search_warp_bytes(d.mp, L, a.stage_rows, sl.bytes, a.srow, a.tc ? d.mb * 2 : 0u);
-    }
+    K fn = a.tc ? ring_search_kernel<1, 0>
+         : direct ? (prec == 1 ? ring_search_kernel<1, 2> : prec == 2 ? ring_search_kernel<2, 2> : ring_search_kernel<0, 2>)
+                  : (prec == 1 ? ring_search_kernel<1, RIF_WIDE> : prec == 2 ? ring_search_kernel<2, RIF_WIDE> : ring_search_kernel<0, RIF_WIDE>);
+    auto warp_bytes = [&] {
+        return search_warp_bytes(d.mp, L, stage_bytes(a, (int)prec), sl.bytes, direct, a.tc ? d.mb * 2 : 0u);
+    };
+    while (4 * warp_bytes() > smem_optin_bytes() && a.stage_rows > min_rows) a.stage_rows--;
+    const size_t smem = 4 * warp_bytes();
     cudaError_t e = smem_at_least((const void *)fn, smem);
     if (e != cudaSuccess) return e;
     int per_sm = 0;
@@ -1223,7 +1376,7 @@ cudaError_t launch_ring_search(const Dev &d, float *rows, u32 slots, u32 L, u32 
 }
 
 size_t search_smem_bytes(u32 mp, u32 L, u32 stage_rows, u32 seen_bits, u64 capacity, u32 wpb) {
-    return (size_t)wpb * search_warp_bytes(mp, L, stage_rows, seen_layout(capacity, seen_bits).bytes, mp * 4);
+    return (size_t)wpb * search_warp_bytes(mp, L, (size_t)stage_rows * mp * 4, seen_layout(capacity, seen_bits).bytes, false);
 }
 
 cudaError_t launch_seed(const Dev &d, const float *q, u32 nq, u32 L, u64 *seed, cudaStream_t st, u32 prec,
@@ -1256,7 +1409,6 @@ cudaError_t launch_search(const Dev &d, const float *q, u32 nq, u32 L, u32 max_h
     a.k = k;
     a.out_ids = out_ids; a.out_dist = out_dist; a.exp_keys = exp_keys; a.exp_count = exp_count;
     a.stage_rows = tune.stage_rows;
-    const SeenLayout sl = set_seen(a, d, tune.seen_bits);
     a.rowb = prec == 1 ? d.mb * 2 : prec == 2 ? d.m8 : d.mp * 4;
     a.rerank = rerank;
     a.exact = exact_rows ? 1u : 0u;
@@ -1268,22 +1420,37 @@ cudaError_t launch_search(const Dev &d, const float *q, u32 nq, u32 L, u32 max_h
     a.elog_n = elog_n;
     a.elog_cap = elog_cap;
     const bool log = elog != nullptr;
-    const u32 wpb = log ? 4u : tune.warps_per_block;
-    if (wpb != 2 && wpb != 4 && wpb != 8) return cudaErrorInvalidValue;
+    if (tune.warps_per_block != 2 && tune.warps_per_block != 4 && tune.warps_per_block != 8) return cudaErrorInvalidValue;
+    const bool direct = !log && direct_rows(a, d);
+    // Searches that stage nothing run a block per warp, so that an SM's queries
+    // start and end one by one.  Rows of at most 128 elements: fp32 rows keep
+    // four rounds in flight on 16 warps (10k queries on 1M x 128, beam 144:
+    // 4,220 us staged, 2,046 so, 2,087 with two rounds on 20 warps); the
+    // narrower rows of a copy one round on 24 warps (4,099 queries, 100-d fp8:
+    // 1,968 staged, 1,093 with four rounds, 821 so) unless there are too few
+    // queries to fill them.  Longer rows: 1,537 queries on 50k x 960 fp32, beam
+    // 96: 2,855 staged, 710 from global memory.
+    const bool deep = prec == 0 || nq <= 16u * (u32)num_sms;
+    const u32 wpb = log ? 4u : !a.tc ? 1u : tune.stage_rows == 0 ? 2u : tune.warps_per_block;
+    u32 bits = tune.seen_bits;
+    const u32 per_sm_q = (nq + (u32)num_sms - 1) / (u32)num_sms;
+    auto_shape(a, d, bits, prec, L, direct, std::min<u32>(a.tc ? 10 : 16, per_sm_q));
+    const SeenLayout sl = set_seen(a, d, bits);
     const u32 min_rows = fit_stage(a, L, k, rerank, prec, mode);
     using K = void (*)(SearchArgs);
     K fn = nullptr;
-    if (log) fn = prec == 1 ? search_kernel<1, true> : prec == 2 ? search_kernel<2, true> : search_kernel<0, true>;
-    else if (wpb == 2) fn = prec == 1 ? search_kernel<1, false, 2> : prec == 2 ? search_kernel<2, false, 2> : search_kernel<0, false, 2>;
-    else if (wpb == 8) fn = prec == 1 ? search_kernel<1, false, 8> : prec == 2 ? search_kernel<2, false, 8> : search_kernel<0, false, 8>;
-    else fn = prec == 1 ? search_kernel<1> : prec == 2 ? search_kernel<2> : search_kernel<0>;
-    size_t smem = (size_t)wpb * search_warp_bytes(d.mp, L, a.stage_rows, sl.bytes, a.srow, a.tc ? d.mb * 2 : 0u);
+    if (log) fn = a.tc ? search_kernel<1, true, 4, 0> : prec == 1 ? search_kernel<1, true, 4, RIF_WIDE> : prec == 2 ? search_kernel<2, true, 4, RIF_WIDE> : search_kernel<0, true, 4, RIF_WIDE>;
+    else if (a.tc) fn = wpb == 2 ? search_kernel<1, false, 2> : wpb == 8 ? search_kernel<1, false, 8> : search_kernel<1>;
+    else if (!direct) fn = prec == 1 ? search_kernel<1, false, 1, RIF_WIDE> : prec == 2 ? search_kernel<2, false, 1, RIF_WIDE> : search_kernel<0, false, 1, RIF_WIDE>;
+    else if (deep) fn = prec == 1 ? search_kernel<1, false, 1, 4> : prec == 2 ? search_kernel<2, false, 1, 4> : search_kernel<0, false, 1, 4>;
+    else fn = prec == 1 ? search_kernel<1, false, 1, 1> : search_kernel<2, false, 1, 1>;
+    auto warp_bytes = [&] {
+        return search_warp_bytes(d.mp, L, stage_bytes(a, (int)prec), sl.bytes, direct, a.tc ? d.mb * 2 : 0u);
+    };
     // a widened stage (or the bf16 query) that does not fit beside this
     // shape: fewer rows, down to what the sorted keys need
-    while (smem > smem_optin_bytes() && a.stage_rows > min_rows) {
-        a.stage_rows--;
-        smem = (size_t)wpb * search_warp_bytes(d.mp, L, a.stage_rows, sl.bytes, a.srow, a.tc ? d.mb * 2 : 0u);
-    }
+    while (wpb * warp_bytes() > smem_optin_bytes() && a.stage_rows > min_rows) a.stage_rows--;
+    const size_t smem = wpb * warp_bytes();
     cudaError_t e = smem_at_least((const void *)fn, smem);
     if (e != cudaSuccess) return e;
     int per_sm = 0;

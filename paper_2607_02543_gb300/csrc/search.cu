@@ -176,6 +176,10 @@ __device__ __forceinline__ float canon_dist_q8(const float4 (&qr)[4], const floa
 constexpr u64 REF_EXP = 1ull << 62;
 
 constexpr int RIF_WIDE = 8;   // rows of any length from global memory (see eval_wide)
+constexpr int RIF_TC = 16;    // tensor-core keys of rows of at most 128 elements (see eval_tc)
+
+// The forms of eval_direct, which keep their keys in registers.
+__host__ __device__ constexpr bool narrow(int rif) { return rif > 0 && rif < RIF_WIDE; }
 
 struct WarpSmem {
     float *qv;       // mp
@@ -216,11 +220,12 @@ inline SeenLayout seen_layout(u64 capacity, u32 bits) {
 }
 
 // stageb: bytes of the row stage; qbytes: the bf16 query of the tensor-core keys (or 0);
-// direct: rows are evaluated in registers (eval_direct)
+// direct: rows are evaluated in registers (eval_direct).  staged: the fp32 query
+// is only needed while the stage holds no rows, and lives there.
 __host__ __device__ inline size_t search_warp_bytes(u32 mp, u32 L, size_t stageb, size_t seen_bytes, bool direct,
-                                                   u32 qbytes = 0) {
+                                                   bool staged, u32 qbytes = 0) {
     size_t b = 0;
-    b += align_up((size_t)mp * 4, 128);
+    if (!staged) b += align_up((size_t)mp * 4, 128);
     b += align_up(stageb, 128);
     b += 2 * align_up((size_t)L * 8, 16);
     b += 32 * 8 + (direct ? 32 * 4 : 64 * (4 + 8));
@@ -230,9 +235,10 @@ __host__ __device__ inline size_t search_warp_bytes(u32 mp, u32 L, size_t stageb
     return align_up(b, 128);
 }
 
-__device__ inline WarpSmem carve(char *p, u32 mp, u32 L, size_t stageb, size_t seen_bytes, bool direct) {
+__device__ inline WarpSmem carve(char *p, u32 mp, u32 L, size_t stageb, size_t seen_bytes, bool direct, bool staged) {
     WarpSmem s;
-    s.qv = reinterpret_cast<float *>(p); p += align_up((size_t)mp * 4, 128);
+    s.qv = reinterpret_cast<float *>(p);
+    if (!staged) p += align_up((size_t)mp * 4, 128);
     s.stage = reinterpret_cast<float *>(p); p += align_up(stageb, 128);
     s.bkey = reinterpret_cast<u64 *>(p); p += align_up((size_t)L * 8, 16);
     s.bref = reinterpret_cast<u64 *>(p); p += align_up((size_t)L * 8, 16);
@@ -436,6 +442,58 @@ __device__ void eval_staged(const SearchArgs &a, WarpSmem &s, int cnt, u32 &phas
     }
 }
 
+// The same for rows of at most 128 elements: each lane loads its fragments of
+// the B operand (rows g = lane / 4 of a tile, elements 2 t, 2 t + 1 of every
+// eight, t = lane % 4) straight from global memory, two tiles in flight.  The
+// same products in the same MMAs as tc_keys.
+__device__ __forceinline__ void eval_tc(const SearchArgs &a, WarpSmem &s, int cnt) {
+    const Dev &d = a.d;
+    const int lane = lane_id(), g = lane >> 2, t = lane & 3;
+    const u32 *qb = tc_qb(s);
+    const float nq = *tc_nq(s);
+    const int steps = (int)d.mb / 16;
+    for (int c0 = 0; c0 < cnt; c0 += 16) {
+        u32 b[2][16];
+        float xn[2][2], acc[2][4];
+#pragma unroll
+        for (int u = 0; u < 2; u++) {
+            const u32 *row = reinterpret_cast<const u32 *>(d.xb + (size_t)s.cid[min(c0 + 8 * u + g, cnt - 1)] * d.mb) + t;
+#pragma unroll
+            for (int k = 0; k < 8; k++)
+                if (k < steps) {
+                    b[u][2 * k] = row[8 * k];
+                    b[u][2 * k + 1] = row[8 * k + 4];
+                }
+#pragma unroll
+            for (int h = 0; h < 2; h++)   // the columns whose products lanes 0..3 will hold
+                xn[u][h] = d.xbn[s.cid[min(c0 + 8 * u + 2 * t + h, cnt - 1)]];
+#pragma unroll
+            for (int c = 0; c < 4; c++) acc[u][c] = 0.0f;
+        }
+#pragma unroll
+        for (int k = 0; k < 8; k++)
+            if (k < steps) {
+                const u32 q0 = g == 0 ? qb[8 * k + t] : 0u, q1 = g == 0 ? qb[8 * k + 4 + t] : 0u;
+#pragma unroll
+                for (int u = 0; u < 2; u++) mma_bf16_16816(acc[u], q0, 0u, q1, 0u, b[u][2 * k], b[u][2 * k + 1]);
+            }
+        if (g == 0) {
+#pragma unroll
+            for (int u = 0; u < 2; u++)
+#pragma unroll
+                for (int h = 0; h < 2; h++) {
+                    const int c = c0 + 8 * u + 2 * t + h;
+                    if (c < cnt) {
+                        const float dist = d.metric == 0 ? __fmaf_rn(-2.0f, acc[u][h], __fadd_rn(nq, xn[u][h]))
+                                                         : __fsub_rn(1.0f, acc[u][h]);
+                        s.ckey[c] = mkkey(dist, s.cid[c]);
+                    }
+                }
+        }
+    }
+    __syncwarp();
+}
+
 // 16 bytes of a row that is read once: not kept in L1, whose few lines beside
 // the shared memory are left to the slabs and reference words (10k queries on
 // 1M x 128 rows: 2,240 -> 2,119 us).
@@ -610,7 +668,7 @@ __device__ __forceinline__ void eval_direct(const SearchArgs &a, const WarpSmem 
 template <int P, int RIF>
 __device__ __forceinline__ void score32(const SearchArgs &a, WarpSmem &s, int nb, const float4 (&qr)[4], u64 *out) {
     const int lane = lane_id();
-    if constexpr (RIF == RIF_WIDE || RIF == 0) {
+    if constexpr (!narrow(RIF)) {
         eval_wide<P, 1>(a, s, nb);
         if (lane < nb) out[lane] = s.ckey[lane];
     } else {
@@ -624,7 +682,7 @@ __device__ __forceinline__ void score32(const SearchArgs &a, WarpSmem &s, int nb
 
 // Evaluate the unseen ids among a slab's entries e0 and e1 (held one per lane,
 // NIL = none) and merge them into the beam.  Returns the new beam size.  RIF:
-// see eval_direct; RIF_WIDE: eval_wide; 0: eval_staged.
+// see eval_direct; RIF_WIDE: eval_wide; RIF_TC: eval_tc; 0: eval_staged.
 template <int P, bool LOG, int RIF>
 __device__ __forceinline__ int eval_merge(const SearchArgs &a, WarpSmem &s, u32 e0, u32 e1, int n, u32 &phase,
                                           u64 &ndist, bool &timeout, u32 &um, const float4 (&qr)[4], u32 *qlog,
@@ -636,7 +694,7 @@ __device__ __forceinline__ int eval_merge(const SearchArgs &a, WarpSmem &s, u32 
             if (qcnt + i < a.elog_cap) qlog[qcnt + i] = s.cid[i];
         qcnt += cnt;
     };
-    if constexpr (RIF > 0 && RIF != RIF_WIDE) {
+    if constexpr (narrow(RIF)) {
 #pragma unroll 1
         for (int half = 0; half < 2; half++) {
             u32 id = half ? e1 : e0;
@@ -677,6 +735,7 @@ __device__ __forceinline__ int eval_merge(const SearchArgs &a, WarpSmem &s, u32 
         for (int u = 0; u < 2; u++)
             if (lane + 32 * u < cnt) ref[u] = ld_ref(a.d, s.cid[lane + 32 * u]);
         if constexpr (RIF == RIF_WIDE) eval_wide<P, 2>(a, s, cnt);
+        else if constexpr (RIF == RIF_TC) eval_tc(a, s, cnt);
         else eval_staged<P>(a, s, cnt, phase, timeout);
         ndist += cnt;
         log(cnt);
@@ -819,22 +878,23 @@ __device__ __forceinline__ void search_one(const SearchArgs &a, WarpSmem &s, u32
     const u32 mp = d.mp;
     const float *qrow = a.q + (size_t)qi * mp;
     const u64 *seed_row = a.seed + (size_t)qi * a.L;
-    for (u32 i = lane * 4; i < mp; i += 128)
-        *reinterpret_cast<float4 *>(s.qv + i) = *reinterpret_cast<const float4 *>(qrow + i);
+    if (RIF != 0)
+        for (u32 i = lane * 4; i < mp; i += 128)
+            *reinterpret_cast<float4 *>(s.qv + i) = *reinterpret_cast<const float4 *>(qrow + i);
     seen_clear(a, s);
     __syncwarp();
     float4 qr[4];
 #pragma unroll
     for (int t = 0; t < 4; t++) {
         const u32 i = 4u * ((lane & 7) + 8 * t);
-        qr[t] = i < mp ? *reinterpret_cast<const float4 *>(s.qv + i) : make_float4(0.f, 0.f, 0.f, 0.f);
+        qr[t] = narrow(RIF) && i < mp ? *reinterpret_cast<const float4 *>(s.qv + i) : make_float4(0.f, 0.f, 0.f, 0.f);
     }
     if (P == 1 && a.tc) {
         // the query as bf16 pairs, and its squared norm over the bf16 values
         float sq = 0.0f;
         u32 *qb = tc_qb(s);
         for (u32 i = lane; 2 * i < d.mb; i += 32) {
-            const float x0 = 2 * i < mp ? s.qv[2 * i] : 0.0f, x1 = 2 * i + 1 < mp ? s.qv[2 * i + 1] : 0.0f;
+            const float x0 = 2 * i < mp ? qrow[2 * i] : 0.0f, x1 = 2 * i + 1 < mp ? qrow[2 * i + 1] : 0.0f;
             const u32 w = pack_bf16(x0, x1);
             qb[i] = w;
             const float b0 = __uint_as_float(w << 16), b1 = __uint_as_float(w & 0xFFFF0000u);
@@ -854,12 +914,16 @@ __device__ __forceinline__ void search_one(const SearchArgs &a, WarpSmem &s, u32
         // every key in the beam must be the key this search gives its id (an
         // id evaluated again then collapses with its seed), so the seeds are
         // re-keyed, and sorted in the stage; the keys wait in the beam.
-        const int bs = a.tc ? min((int)a.stage_rows, 32) : 32;   // s.cid holds 32 ids
+        const int bs = a.tc && RIF != RIF_TC ? min((int)a.stage_rows, 32) : 32;   // s.cid holds 32 ids
         for (int b0 = 0; b0 < n0; b0 += bs) {
             const int nb = min(bs, n0 - b0);
             if (lane < nb) s.cid[lane] = key_id(seed_row[b0 + lane]);
             __syncwarp();
-            if (a.tc) {
+            if (RIF == RIF_TC) {
+                eval_tc(a, s, nb);
+                if (lane < nb) s.bkey[b0 + lane] = s.ckey[lane];
+                __syncwarp();
+            } else if (a.tc) {
                 stage_ids<P>(a, s, s.cid, nb, phase, timeout);
                 tc_keys(a, s, nb, s.cid, s.bkey + b0);
             } else {
@@ -950,12 +1014,17 @@ __device__ __forceinline__ void search_one(const SearchArgs &a, WarpSmem &s, u32
             c = min(want, c + __popc(m));
         }
         __syncwarp();
+        if (RIF == 0) {   // the stage holds no rows any more: the query goes behind the keys
+            s.qv = reinterpret_cast<float *>(rk + rn);
+            for (u32 i = lane * 4; i < mp; i += 128)
+                *reinterpret_cast<float4 *>(s.qv + i) = *reinterpret_cast<const float4 *>(qrow + i);
+        }
         for (int b0 = 0; b0 < c; b0 += 32) {
             const int nb = min(32, c - b0);
             if (lane < nb) s.cid[lane] = key_id(rk[b0 + lane]);
             __syncwarp();
             // a search whose rows are short keeps no list for eval_wide
-            score32<0, (RIF == 0 || RIF == RIF_WIDE ? RIF_WIDE : 2)>(a, s, nb, qr, rk + b0);   // sorted below
+            score32<0, (narrow(RIF) ? 1 : RIF_WIDE)>(a, s, nb, qr, rk + b0);   // sorted below
         }
         for (int i = c + lane; i < rn; i += 32) rk[i] = KEY_INF;
         __syncwarp();
@@ -1015,8 +1084,8 @@ __global__ void __launch_bounds__(32 * WPB, (RIF == 1 ? 24 : 16) / WPB) search_k
     const Dev &d = a.d;
     const u32 mp = d.mp;
     const size_t sb = seen_bytes(a), stb = stage_bytes(a, P);
-    const size_t wb = search_warp_bytes(mp, a.L, stb, sb, RIF > 0 && RIF != RIF_WIDE, a.tc ? d.mb * 2 : 0u);
-    WarpSmem s = carve(smem + warp * wb, mp, a.L, stb, sb, RIF > 0 && RIF != RIF_WIDE);
+    const size_t wb = search_warp_bytes(mp, a.L, stb, sb, narrow(RIF), RIF == 0, a.tc ? d.mb * 2 : 0u);
+    WarpSmem s = carve(smem + warp * wb, mp, a.L, stb, sb, narrow(RIF), RIF == 0);
     if (lane == 0) mbar_init(s.bar, 1);
     __syncwarp();
     u32 phase = 0;
@@ -1169,8 +1238,8 @@ __global__ void __launch_bounds__(128, 3) ring_search_kernel(SearchArgs a, RingA
     const int warp = threadIdx.x >> 5, lane = lane_id();
     const Dev &d = a.d;
     const size_t sb = seen_bytes(a), stb = stage_bytes(a, P);
-    const size_t wb = search_warp_bytes(d.mp, a.L, stb, sb, RIF > 0 && RIF != RIF_WIDE, a.tc ? d.mb * 2 : 0u);
-    WarpSmem s = carve(smem + warp * wb, d.mp, a.L, stb, sb, RIF > 0 && RIF != RIF_WIDE);
+    const size_t wb = search_warp_bytes(d.mp, a.L, stb, sb, narrow(RIF), RIF == 0, a.tc ? d.mb * 2 : 0u);
+    WarpSmem s = carve(smem + warp * wb, d.mp, a.L, stb, sb, narrow(RIF), RIF == 0);
     if (lane == 0) mbar_init(s.bar, 1);
     __syncwarp();
     u32 phase = 0;
@@ -1275,7 +1344,7 @@ static size_t smem_optin_bytes() {
 // (rerank * k, at most the beam) and re-keyed seeds (the beam), each rounded
 // up to a power of two.
 // Returns the fewest stage rows that hold them.
-static u32 fit_stage(SearchArgs &a, u32 L, u32 k, u32 rerank, u32 prec, u32 mode) {
+static u32 fit_stage(SearchArgs &a, u32 L, u32 k, u32 rerank, u32 prec, u32 mode, u32 mp, bool staged) {
     size_t need = 0;
     if (prec != 0 && mode == 0) {
         size_t rn = 64;
@@ -1287,7 +1356,8 @@ static u32 fit_stage(SearchArgs &a, u32 L, u32 k, u32 rerank, u32 prec, u32 mode
         while (rn < L) rn <<= 1;
         need = std::max(need, rn);
     }
-    const u32 min_rows = std::max<u32>(1, (u32)((need * 8 + a.srow - 1) / a.srow));
+    const size_t bytes = need * 8 + (staged ? (size_t)mp * 4 : 0);   // see search_warp_bytes
+    const u32 min_rows = std::max<u32>(1, (u32)((bytes + a.srow - 1) / a.srow));
     if (a.stage_rows < min_rows) a.stage_rows = min_rows;
     return min_rows;
 }
@@ -1295,6 +1365,9 @@ static u32 fit_stage(SearchArgs &a, u32 L, u32 k, u32 rerank, u32 prec, u32 mode
 // Rows of at most 128 elements are evaluated 8 lanes a row (eval_direct), unless
 // the keys come from the tensor cores, which read staged rows.
 static bool direct_rows(const SearchArgs &a, const Dev &d) { return d.mp <= 128 && !a.tc; }
+
+// Tensor-core keys of longer rows read them from the stage.
+static bool staged_rows(const SearchArgs &a, const Dev &d) { return a.tc && d.mb > 128; }
 
 static SeenLayout set_seen(SearchArgs &a, const Dev &d, u32 bits) {
     const SeenLayout l = seen_layout(d.capacity, bits);
@@ -1309,24 +1382,27 @@ static SeenLayout set_seen(SearchArgs &a, const Dev &d, u32 bits) {
 
 // The launch shape of a search whose tuning leaves it open (0): rows per stage
 // and the evaluated-id cache.  `resident` is the warps an SM should hold.
-//  - Stage: tensor-core keys take eight rows, one tile of MMAs.  Nothing else
-//    reads staged rows (the stage then only holds sorts, see fit_stage).
+//  - Stage: eight rows, one tile of MMAs, for tensor-core keys of rows longer
+//    than 128.  Nothing else reads staged rows (the stage then only holds
+//    sorts, see fit_stage).
 //    4,096 queries on 50k x 768 BF16, beam 64: 6,497 us with the former 31 rows,
 //    1,331 with eight, 1,562 with eleven.
-//  - Cache: the largest power of two of at most 8 KB that leaves `resident`
-//    warps their shared memory, or that covers every id.  Larger caches repeat
-//    fewer evaluations (1M x 128, beam 144: 14.8, 13.1, 12.1 per expansion at
-//    2^11, 2^12, 2^13 slots); beyond 8 KB resident warps were worth more.
+//  - Cache: 4 KB, or 8 KB where that leaves `resident` warps their shared
+//    memory; no more slots than cover every id.  Larger caches repeat fewer
+//    evaluations (1M x 128, beam 144: 14.8, 13.1, 12.1 per expansion at 2^11,
+//    2^12, 2^13 slots); beyond 8 KB resident warps were worth more, and below 4
+//    KB the evaluations (768-d BF16: 1,429 us at 2 KB, 1,282 at 4, 1,534 at 8).
 static void auto_shape(SearchArgs &a, const Dev &d, u32 &seen_bits, u32 prec, u32 L, bool direct, u32 resident) {
-    if (!a.tc) a.stage_rows = 1;
+    if (!staged_rows(a, d)) a.stage_rows = 1;
     else if (a.stage_rows == 0) a.stage_rows = 8;
     if (seen_bits) return;
     const size_t budget = (227u << 10) / std::max<u32>(1, resident) - 1024;   // a block's own 1 KB
     seen_bits = 9;
     for (u32 b = 10; b <= 13 && (1ull << (b - 1)) < d.capacity; b++) {
         const size_t sb = seen_layout(d.capacity, b).bytes;
-        if (sb > (8u << 10) ||
-            search_warp_bytes(d.mp, L, stage_bytes(a, (int)prec), sb, direct, a.tc ? d.mb * 2 : 0u) > budget)
+        if (sb > (8u << 10)) break;
+        if (sb > (4u << 10) &&
+            search_warp_bytes(d.mp, L, stage_bytes(a, (int)prec), sb, direct, staged_rows(a, d), a.tc ? d.mb * 2 : 0u) > budget)
             break;
         seen_bits = b;
     }
@@ -1351,15 +1427,16 @@ cudaError_t launch_ring_search(const Dev &d, float *rows, u32 slots, u32 L, u32 
     u32 bits = tune.seen_bits;
     auto_shape(a, d, bits, prec, L, direct, 12);
     const SeenLayout sl = set_seen(a, d, bits);
-    const u32 min_rows = fit_stage(a, L, k, rerank, prec, 0);
+    const u32 min_rows = fit_stage(a, L, k, rerank, prec, 0, d.mp, staged_rows(a, d));
     // head: claimed, device count, last host poll, stop flag, then the statistics
     RingArgs r{head, head + 1, head + 2, head + 3, head + 4, tail, closed, done, served_by, slots, seq, max_ns};
     using K = void (*)(SearchArgs, RingArgs);
-    K fn = a.tc ? ring_search_kernel<1, 0>
+    K fn = staged_rows(a, d) ? ring_search_kernel<1, 0>
+         : a.tc ? ring_search_kernel<1, RIF_TC>
          : direct ? (prec == 1 ? ring_search_kernel<1, 2> : prec == 2 ? ring_search_kernel<2, 2> : ring_search_kernel<0, 2>)
                   : (prec == 1 ? ring_search_kernel<1, RIF_WIDE> : prec == 2 ? ring_search_kernel<2, RIF_WIDE> : ring_search_kernel<0, RIF_WIDE>);
     auto warp_bytes = [&] {
-        return search_warp_bytes(d.mp, L, stage_bytes(a, (int)prec), sl.bytes, direct, a.tc ? d.mb * 2 : 0u);
+        return search_warp_bytes(d.mp, L, stage_bytes(a, (int)prec), sl.bytes, direct, staged_rows(a, d), a.tc ? d.mb * 2 : 0u);
     };
     while (4 * warp_bytes() > smem_optin_bytes() && a.stage_rows > min_rows) a.stage_rows--;
     const size_t smem = 4 * warp_bytes();
@@ -1376,7 +1453,7 @@ cudaError_t launch_ring_search(const Dev &d, float *rows, u32 slots, u32 L, u32 
 }
 
 size_t search_smem_bytes(u32 mp, u32 L, u32 stage_rows, u32 seen_bits, u64 capacity, u32 wpb) {
-    return (size_t)wpb * search_warp_bytes(mp, L, (size_t)stage_rows * mp * 4, seen_layout(capacity, seen_bits).bytes, false);
+    return (size_t)wpb * search_warp_bytes(mp, L, (size_t)stage_rows * mp * 4, seen_layout(capacity, seen_bits).bytes, false, false);
 }
 
 cudaError_t launch_seed(const Dev &d, const float *q, u32 nq, u32 L, u64 *seed, cudaStream_t st, u32 prec,
@@ -1431,21 +1508,22 @@ cudaError_t launch_search(const Dev &d, const float *q, u32 nq, u32 L, u32 max_h
     // queries to fill them.  Longer rows: 1,537 queries on 50k x 960 fp32, beam
     // 96: 2,855 staged, 710 from global memory.
     const bool deep = prec == 0 || nq <= 16u * (u32)num_sms;
-    const u32 wpb = log ? 4u : !a.tc ? 1u : tune.stage_rows == 0 ? 2u : tune.warps_per_block;
+    const u32 wpb = log ? 4u : !staged_rows(a, d) ? 1u : tune.stage_rows == 0 ? 2u : tune.warps_per_block;
     u32 bits = tune.seen_bits;
     const u32 per_sm_q = (nq + (u32)num_sms - 1) / (u32)num_sms;
-    auto_shape(a, d, bits, prec, L, direct, std::min<u32>(a.tc ? 10 : 16, per_sm_q));
+    auto_shape(a, d, bits, prec, L, direct, std::min<u32>(16, per_sm_q));
     const SeenLayout sl = set_seen(a, d, bits);
-    const u32 min_rows = fit_stage(a, L, k, rerank, prec, mode);
+    const u32 min_rows = fit_stage(a, L, k, rerank, prec, mode, d.mp, staged_rows(a, d));
     using K = void (*)(SearchArgs);
     K fn = nullptr;
-    if (log) fn = a.tc ? search_kernel<1, true, 4, 0> : prec == 1 ? search_kernel<1, true, 4, RIF_WIDE> : prec == 2 ? search_kernel<2, true, 4, RIF_WIDE> : search_kernel<0, true, 4, RIF_WIDE>;
+    if (log) fn = staged_rows(a, d) ? search_kernel<1, true, 4, 0> : a.tc ? search_kernel<1, true, 4, RIF_TC> : prec == 1 ? search_kernel<1, true, 4, RIF_WIDE> : prec == 2 ? search_kernel<2, true, 4, RIF_WIDE> : search_kernel<0, true, 4, RIF_WIDE>;
+    else if (a.tc && !staged_rows(a, d)) fn = search_kernel<1, false, 1, RIF_TC>;
     else if (a.tc) fn = wpb == 2 ? search_kernel<1, false, 2> : wpb == 8 ? search_kernel<1, false, 8> : search_kernel<1>;
     else if (!direct) fn = prec == 1 ? search_kernel<1, false, 1, RIF_WIDE> : prec == 2 ? search_kernel<2, false, 1, RIF_WIDE> : search_kernel<0, false, 1, RIF_WIDE>;
     else if (deep) fn = prec == 1 ? search_kernel<1, false, 1, 4> : prec == 2 ? search_kernel<2, false, 1, 4> : search_kernel<0, false, 1, 4>;
     else fn = prec == 1 ? search_kernel<1, false, 1, 1> : search_kernel<2, false, 1, 1>;
     auto warp_bytes = [&] {
-        return search_warp_bytes(d.mp, L, stage_bytes(a, (int)prec), sl.bytes, direct, a.tc ? d.mb * 2 : 0u);
+        return search_warp_bytes(d.mp, L, stage_bytes(a, (int)prec), sl.bytes, direct, staged_rows(a, d), a.tc ? d.mb * 2 : 0u);
     };
     // a widened stage (or the bf16 query) that does not fit beside this
     // shape: fewer rows, down to what the sorted keys need

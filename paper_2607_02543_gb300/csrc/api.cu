@@ -514,7 +514,8 @@ static etale_status seed_batch(etale_index *idx, const Dev &d, const float *q, u
                                cudaStream_t st, int sms = 0, bool *fp32_keys = nullptr) {
     const u32 S = idx->n_entries;
     if (fp32_keys) *fp32_keys = false;
-    if ((prec == 0 || fp32_keys) && idx->seed_tc && !idx->concurrent && S > 0 && nq >= 32) {
+    // small reduced-precision batches keep the kernel that ranks in their own precision
+    if ((prec == 0 || (fp32_keys && nq >= 32)) && idx->seed_tc && !idx->concurrent && S > 0) {
         const SeedTcPlan p = seed_tc_plan(idx->dim, S, nq);
         if (!grow(idx->sd_A, p.bytes_A) || !grow(idx->sd_qstat, (size_t)nq * 16) ||
             !grow(idx->sd_keys, p.bytes_keys) || !grow(idx->sd_fb, (size_t)nq * 4) || !grow(idx->sd_ctr, 64))
@@ -1638,7 +1639,7 @@ cudaError_t rg_entries(etale_index *idx, etale_round_graph *g, const Dev &dg, cu
 cudaError_t rg_seed(etale_index *idx, etale_round_graph *g, const Dev &dg, const float *q, u32 nq, u32 L, u64 *seed,
                     cudaStream_t st, u32 prec = 0) {
     if (prec) return launch_seed(dg, q, nq, L, seed, st, prec);
-    if (g->seed_tc && nq >= 32) {
+    if (g->seed_tc) {
         const SeedTcPlan p = seed_tc_plan(idx->dim, idx->cfg.n_entry, nq);
         return launch_seed_tc(dg, q, nq, idx->cfg.n_entry, L, seed, p, idx->seed_bufs(), idx->num_sms, st);
     }

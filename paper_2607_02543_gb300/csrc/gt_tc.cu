@@ -458,17 +458,18 @@ __device__ __forceinline__ float4 load_row4(const float *r, u32 i, u32 dim, bool
 // elements is not exact in bf16: only then do the copies subtract the vector,
 // so that data for which one bf16 segment is enough stay so.  A column whose
 // mean is no ordinary number keeps 0.
-constexpr int CR = 1024;
+constexpr int CR = 256;
 __global__ void __launch_bounds__(1024) gt_center_kernel(Dev d, u64 next_id, float *center, u32 *gstat) {
     __shared__ float part[32][33];
     const u32 col = blockIdx.x * 32 + threadIdx.x, ry = threadIdx.y;   // 32 columns x 32 row groups
     const u32 n = (u32)min((u64)CR, next_id);
+    const u64 stride = next_id / n * d.mp;
     float sum = 0.0f;
     bool inexact = false;
     if (col < d.mp)
 #pragma unroll 8
         for (u32 j = ry; j < n; j += 32) {
-            const float v = d.x[(u64)j * next_id / n * d.mp + col];
+            const float v = d.x[j * stride + col];
             sum += v;
             inexact |= bf16_round(v) != v;
         }
@@ -582,36 +583,42 @@ __global__ void gt_prep_queries(const float *q, u32 mp, u32 dim, u32 nq, u32 kp1
 // - |q|^2| (L2) or from canonical distance - 1 (IP), doubled for safety, up to
 // the factor 1 - 2 (m + 4) u of the L2 form below.  qs: |q|^2, |q|, |lo_q|,
 // |e_q| of the query; gs: max |x|^2, max |lo_x|, max |e_x| over the rows (fp32
-// bits).  K = contracted length.
-__device__ double key_error(int metric, double m, double K, bool split, const float *qs, const u32 *gs) {
-    const double u = 1.0 / 16777216.0;
-    const double qn = qs[0], qa = (double)qs[1] * 1.01, loq = (double)qs[2] * 1.01, eq = (double)qs[3] * 1.01;
-    const double X2 = __uint_as_float(gs[0]), X1 = sqrt(X2) * 1.01;
-    const double Lx = (double)__uint_as_float(gs[1]) * 1.01, Ex = (double)__uint_as_float(gs[2]) * 1.01;
+// bits).  K = contracted length.  Every operation rounds up (in fp32: double
+// arithmetic cost a warp 3,000 cycles and more).
+__device__ float key_error(int metric, float m, float K, bool split, const float *qs, const u32 *gs) {
+    auto mul = [](float x, float y) { return __fmul_ru(x, y); };
+    auto add = [](float x, float y) { return __fadd_ru(x, y); };
+    const float u = 1.0f / 16777216.0f;
+    const float qn = qs[0], qa = mul(qs[1], 1.011f), loq = mul(qs[2], 1.011f), eq = mul(qs[3], 1.011f);
+    const float X2 = __uint_as_float(gs[0]), X1 = mul(__fsqrt_ru(X2), 1.011f);
+    const float Lx = mul(__uint_as_float(gs[1]), 1.011f), Ex = mul(__uint_as_float(gs[2]), 1.011f);
     // |computed dot - q.x|: the terms the split leaves out, plus fp32 accumulation
-    const double dot_res = split ? loq * Lx + (qa + eq) * Ex + eq * (X1 + Ex) : 0.0;
-    const double dot_err = dot_res + (K + 2.0) * 2.0 * u * 1.03 * qa * X1;
-    if (metric == 0)   // taking the centre off, norms (fp32 sums of squares), 2 x dot error, rounding of the key
-        return 2.0 * (2.1 * u * (qa + X1) * (qa + X1) + (m + 2.0) * u * qn * 1.01 + (m + 2.0) * u * X2 + 2.0 * dot_err + 2.0 * u * (X2 + 2.1 * qa * X1));
-    return 2.0 * (dot_err + (m + 2.0) * u * qa * X1 + u * (1.0 + qa * X1));
+    const float qx = mul(qa, X1);
+    float dot_err = mul(mul(mul(add(K, 2.0f), 2.0f * u), 1.03f), qx);
+    if (split) dot_err = add(dot_err, add(add(mul(loq, Lx), mul(add(qa, eq), Ex)), mul(eq, add(X1, Ex))));
+    const float mu = mul(add(m, 2.0f), u);
+    if (metric == 0) {   // taking the centre off, norms (fp32 sums of squares), 2 x dot error, rounding of the key
+        const float s = add(qa, X1);
+        float e = add(mul(2.1f * u, mul(s, s)), add(mul(mul(mu, qn), 1.01f), mul(mu, X2)));
+        e = add(e, add(2.0f * dot_err, mul(2.0f * u, add(X2, mul(2.1f, qx)))));
+        return 2.0f * e;
+    }
+    return 2.0f * add(add(dot_err, mul(mu, qx)), mul(u, add(1.0f, qx)));
 }
-// Lower bound on the canonical fp32 distance of every row whose approximate
-// key exceeds LB.
-__device__ double key_lower_bound(int metric, double m, double K, bool split, const float *qs, const u32 *gs,
-                                  double LB) {
-    const double E = key_error(metric, m, K, split, qs, gs);
-    if (metric != 0) return 1.0 + LB - E;
-    const double y = (double)qs[0] + LB - E;
-    // the canonical fp32 distance is within (m + 4) u of the exact one
-    return y > 0.0 ? y * (1.0 - 2.0 * (m + 4.0) / 16777216.0) : -1.0;
+// No row with a canonical distance <= dk has an approximate key above the
+// returned value (the canonical fp32 distance is within (m + 4) u of the exact
+// one, and 1 / (1 - x) <= 1 + 2 x).
+__device__ float key_upper_bound(int metric, float m, float qn, float E, float dk) {
+    if (metric != 0) return __fadd_ru(__fadd_ru(dk, -1.0f), E);
+    const float f = __fadd_ru(1.0f, __fmul_ru(__fadd_ru(m, 4.0f), 4.0f / 16777216.0f));
+    return __fadd_ru(__fadd_ru(__fmul_ru(dk, f), -qn), E);
 }
-// The inverse: no row with a canonical distance <= dk has an approximate key
-// above the returned value.
-__device__ double key_upper_bound(int metric, double m, double K, bool split, const float *qs, const u32 *gs,
-                                  double dk) {
-    const double E = key_error(metric, m, K, split, qs, gs);
-    if (metric != 0) return dk - 1.0 + E;
-    return dk / (1.0 - 2.0 * (m + 4.0) / 16777216.0) - (double)qs[0] + E;
+// The canonical distance of a row with an approximate key <= key is at most the
+// returned value.
+__device__ float dist_upper_bound(int metric, float m, float qn, float E, float key) {
+    if (metric != 0) return __fadd_ru(__fadd_ru(1.0f, key), E);
+    const float f = __fadd_ru(1.0f, __fmul_ru(__fadd_ru(m, 4.0f), 4.0f / 16777216.0f));
+    return fmaxf(0.0f, __fmul_ru(__fadd_ru(__fadd_ru(qn, key), E), f));
 }
 
 // ---- threshold and exact rerank -----------------------------------------------
@@ -863,14 +870,17 @@ __global__ void __launch_bounds__(RR_WARPS * 32, 2) gt_rerank_kernel(Dev d, Rera
         if (W > 1) __syncthreads();
         if (phase == 1 || tau >= ORD_INF) break;     // tau: every live row was scored
         bound = __shfl_sync(FULL, top, (int)a.k - 1);
-        double T = __longlong_as_double(0x7ff0000000000000ll);
-        if (bound != KEY_INF)
-            T = key_upper_bound((int)d.metric, a.m, a.kprime, a.split != 0, a.qstat + 4 * (size_t)qi, a.gstat,
-                                (double)key_rho(bound));
-        const float Tf = __fadd_rn(__double2float_ru(T), 0.0f);   // +0 for -0: a minimum of +0 is not above it
-        cert = isfinite(Tf);
+        float T = __int_as_float(0x7f800000);
+        if (bound != KEY_INF) {
+            const float *qs = a.qstat + 4 * (size_t)qi;
+            T = key_upper_bound((int)d.metric, (float)a.m, qs[0],
+                                key_error((int)d.metric, (float)a.m, (float)a.kprime, a.split != 0, qs, a.gstat),
+                                key_rho(bound));
+        }
+        T = __fadd_rn(T, 0.0f);   // +0 for -0: a minimum of +0 is not above it
+        cert = isfinite(T);
         lo = hi;
-        hi = cert ? f2ord(Tf) : 0u;
+        hi = cert ? f2ord(T) : 0u;
         if (!cert || hi <= lo) break;
     }
     if (W > 1 && tw != 0) return;
@@ -889,7 +899,7 @@ constexpr int SS_CAP = 512;       // candidates a query may keep
 constexpr int SS_WARPS = 4;
 
 struct SeedSelArgs {
-    u32 nq, L, S, ld, want, m, kprime;
+    u32 nq, L, S, ld, m, kprime;
     const float *q;       // nq x mp fp32
     const float *keys;    // nq x ld approximate keys (entry order)
     const float *qstat;
@@ -900,119 +910,189 @@ struct SeedSelArgs {
     const u32 *nq_dev;    // when set, the batch size (nq is its cap)
 };
 
-// A warp per query: tau = the want-th smallest approximate key; every entry
-// with key <= tau is scored with the canonical distance, the scores are
-// sorted, and the first L are the seeds if the certificate shows that no
-// entry left out can beat the L-th.
-__global__ void __launch_bounds__(SS_WARPS * 32) seed_select_kernel(Dev d, SeedSelArgs a) {
-    __shared__ u32 cidx[SS_WARPS][SS_CAP];
-    __shared__ u64 ckey[SS_WARPS][SS_CAP];
+// Canonical distances of the candidates [c0, c1) of one query into key.
+__device__ __forceinline__ void seed_score(const Dev &d, const float *qv, const u32 *cidx, u32 c0, u32 c1, u64 *key) {
+    const int lane = lane_id(), grp = lane >> 3, g = lane & 7;
+    if (d.mp <= 128) {
+        // the query's elements in registers; four rows per group in flight
+        float4 qr[4];
+        canon_row_q8(qv, (int)d.mp, g, qr);
+        for (u32 r0 = c0; r0 < c1; r0 += 16) {
+            u32 id[4];
+#pragma unroll
+            for (int u = 0; u < 4; u++) id[u] = d.entries[cidx[min(r0 + grp + 4 * u, c1 - 1)]];
+            float4 v[4][4];
+#pragma unroll
+            for (int u = 0; u < 4; u++) canon_row_q8(d.x + (size_t)id[u] * d.mp, (int)d.mp, g, v[u]);
+#pragma unroll
+            for (int u = 0; u < 4; u++) {
+                const float dd = canon_dist_q8v(qr, v[u], (int)d.mp, (int)d.metric, g);
+                const u32 i = r0 + grp + 4 * u;
+                if (i < c1 && g == 0) key[i] = mkkey(dd, id[u]);
+            }
+        }
+    } else {
+        const float sc[4] = {1.0f, 1.0f, 1.0f, 1.0f};
+        for (u32 r0 = c0; r0 < c1; r0 += 4) {
+            const void *row[4];
+#pragma unroll
+            for (int u = 0; u < 4; u++) row[u] = d.x + (size_t)d.entries[cidx[min(r0 + u, c1 - 1)]] * d.mp;
+            const float dd = warp_dists<0, 4, 2>(qv, row, sc, (int)d.mp, (int)d.metric);
+            const u32 i = r0 + (lane >> 3);
+            if (i < c1 && g == 0) key[i] = mkkey(dd, d.entries[cidx[i]]);
+        }
+    }
+    __syncwarp();
+}
+
+// A warp per query.  A threshold from a sample of the approximate keys collects
+// a few more than L entries; the L-th smallest key among them bounds, by the
+// error bound, the L-th canonical distance and with it the approximate key of
+// every entry that can be a seed.  Those entries, and no others, are scored
+// with the canonical distance and sorted.  Queries with more than SS_CAP of
+// them, or without a finite bound, go to the CUDA-core kernel.  Bound by the
+// row reads (L2) and, in small batches, by one warp's chain.
+__global__ void __launch_bounds__(SS_WARPS * 32, 4) seed_select_kernel(Dev d, SeedSelArgs a) {
+    __shared__ u32 cidx_s[SS_WARPS][SS_CAP];
+    __shared__ u32 cord_s[SS_WARPS][SS_CAP];   // the candidates' approximate keys, ordered image
+    __shared__ u64 ckey_s[SS_WARPS][SS_CAP];
     const int warp = threadIdx.x >> 5, lane = lane_id();
     const u32 qi = blockIdx.x * SS_WARPS + warp;
     if (qi >= (a.nq_dev ? min(*a.nq_dev, a.nq) : a.nq) || a.ctr[1]) return;
-    const float *row = a.keys + (size_t)qi * a.ld;
-    u32 tau = ~0u;                                   // all entries when S <= want
-    if (a.S > a.want) {
-        // a threshold from every 8th key (16 per lane), kept when the count
-        // of keys at or below it lands in [want, SS_CAP]; else (below) the
-        // exact want-th smallest key by a bitwise search over all keys
+    u32 *cidx = cidx_s[warp], *cord = cord_s[warp];
+    u64 *ckey = ckey_s[warp];
+    const float *row = a.keys + (size_t)qi * a.ld;   // a.ld is a multiple of 256
+    // the r-th smallest of n values, value(i) for i < n
+    auto nth = [&](u32 r, u32 n, auto value) {
+        u32 t = 0;
+        for (int bit = 31; bit >= 0; bit--) {
+            const u32 tr = t | (1u << bit);
+            u32 c = 0;
+            for (u32 i = lane; i < n; i += 32) c += (u32)(value(i) < tr);
+            if (__reduce_add_sync(FULL, c) < r) t = tr;
+        }
+        return t;
+    };
+    // entries with a key in (lo, hi] (all up to hi when !from), appended to the
+    // n candidates there are; returns their number with these (more than
+    // SS_CAP: not all stored)
+    auto collect = [&](u32 lo, bool from, u32 hi, u32 n) {
+        for (u32 e0 = 0; e0 < a.S; e0 += 512) {
+            float4 v[4];
+#pragma unroll
+            for (int u = 0; u < 4; u++) {
+                const u32 e = e0 + 128 * u + 4 * lane;
+                if (e < a.S) v[u] = *reinterpret_cast<const float4 *>(row + e);
+            }
+#pragma unroll
+            for (int u = 0; u < 4; u++) {
+                const u32 e = e0 + 128 * u + 4 * lane;
+                const u32 o[4] = {f2ord(v[u].x), f2ord(v[u].y), f2ord(v[u].z), f2ord(v[u].w)};
+                u32 in = 0;
+#pragma unroll
+                for (int c = 0; c < 4; c++)
+                    if (e + c < a.S && o[c] <= hi && (!from || o[c] > lo)) in |= 1u << c;
+                if (!__any_sync(FULL, in != 0)) continue;
+#pragma unroll
+                for (int c = 0; c < 4; c++) {
+                    const u32 m = __ballot_sync(FULL, in >> c & 1u);
+                    const u32 pos = n + __popc(m & lanemask_lt());
+                    if ((in >> c & 1u) && pos < SS_CAP) {
+                        cidx[pos] = e + c;
+                        cord[pos] = o[c];
+                    }
+                    n += __popc(m);
+                }
+            }
+        }
+        __syncwarp();
+        return n;
+    };
+    u32 tau = ~0u, cnt = 0;                          // all entries when S <= L
+    if (a.S > a.L) {
+        // a threshold from every 8th key (16 per lane), kept when the count of
+        // keys at or below it lands in [L, SS_CAP]; raised when it falls short
+        // (one query in twenty: the exact search over all keys that follows at
+        // last takes a warp 80 us and would hold up the whole batch)
         u32 smp[16];
 #pragma unroll
         for (int j = 0; j < 16; j++) {
             const u32 e = 8u * (lane + 32u * j);
             smp[j] = e < a.S ? f2ord(row[e]) : ~0u;
         }
-        const u32 rs = a.want / 8 + 8;
-        u32 t0 = 0;
-        for (int bit = 31; bit >= 0; bit--) {
-            const u32 tr = t0 | (1u << bit);
-            u32 c = 0;
+        u32 rs = a.L / 8 + 8;
+        for (int attempt = 0; attempt < 3; attempt++, rs += rs / 2 + 4) {
+            tau = 0;
+            for (int bit = 31; bit >= 0; bit--) {
+                const u32 tr = tau | (1u << bit);
+                u32 c = 0;
 #pragma unroll
-            for (int j = 0; j < 16; j++) c += (u32)(smp[j] < tr);
-            if (__reduce_add_sync(FULL, c) < rs) t0 = tr;
+                for (int j = 0; j < 16; j++) c += (u32)(smp[j] < tr);
+                if (__reduce_add_sync(FULL, c) < rs) tau = tr;
+            }
+            if (tau == ~0u) break;                   // fewer samples than rs
+            cnt = collect(0u, false, tau, 0);
+            if (cnt >= a.L) break;
         }
-        tau = t0;
+        if (tau == ~0u || cnt < a.L || cnt > (u32)SS_CAP) {
+            tau = nth(a.L, a.S, [&](u32 e) { return f2ord(row[e]); });
+            cnt = collect(0u, false, tau, 0);
+        }
+    } else {
+        cnt = collect(0u, false, tau, 0);
     }
-    // entries with key <= tau, collected and counted in one pass
-    auto collect = [&](u32 t) {
-        u32 n = 0;
-        for (u32 e0 = 0; e0 < a.S; e0 += 32) {
-            const u32 e = e0 + lane;
-            const bool c = e < a.S && f2ord(row[e]) <= t;
-            const u32 m = __ballot_sync(FULL, c);
-            const u32 pos = n + __popc(m & lanemask_lt());
-            if (c && pos < SS_CAP) cidx[warp][pos] = e;
-            n += __popc(m);
-        }
-        return n;
-    };
-    u32 cnt = collect(tau);
-    if (a.S > a.want && (tau == ~0u || cnt < a.want || cnt > (u32)SS_CAP)) {
-        // the sampled threshold missed: the exact want-th smallest key
-        tau = 0;
-        for (int bit = 31; bit >= 0; bit--) {
-            const u32 tr = tau | (1u << bit);
-            u32 c2 = 0;
-            for (u32 e = lane; e < a.S; e += 32) c2 += (u32)(f2ord(row[e]) < tr);
-            if (__reduce_add_sync(FULL, c2) < a.want) tau = tr;
+    const float *qs = a.qstat + 4 * (size_t)qi;
+    bool cert = cnt <= (u32)SS_CAP;
+    if (cert && tau != ~0u) {
+        // keep the candidates that the bound does not exclude
+        const u32 kth = nth(a.L, cnt, [&](u32 i) { return cord[i]; });
+        const float E = key_error((int)d.metric, (float)a.m, (float)a.kprime, true, qs, a.estat);
+        const float D = dist_upper_bound((int)d.metric, (float)a.m, qs[0], E, ord2f(kth));
+        const float T = __fadd_rn(key_upper_bound((int)d.metric, (float)a.m, qs[0], E, D), 0.0f);
+        cert = isfinite(T);
+        const u32 hi = f2ord(T);
+        if (cert && hi > tau) {
+            cnt = collect(tau, true, hi, cnt);
+            cert = cnt <= (u32)SS_CAP;
+        } else if (cert) {
+            u32 n = 0;
+            for (u32 i0 = 0; i0 < cnt; i0 += 32) {
+                const u32 i = i0 + lane;
+                const bool in = i < cnt && cord[i] <= hi;
+                const u32 e = in ? cidx[i] : 0u, m = __ballot_sync(FULL, in);
+                if (in) cidx[n + __popc(m & lanemask_lt())] = e;   // at or below i: already read
+                n += __popc(m);
+            }
+            cnt = n;
         }
         __syncwarp();
-        cnt = collect(tau);
-    }
-    __syncwarp();
-    bool cert = false;
-    if (cnt <= SS_CAP) {
-        const float *qv = a.q + (size_t)qi * d.mp;
-        const int grp = lane >> 3, g = lane & 7;
-        if (d.mp <= 128) {
-            // the query's elements in registers; four rows per group in flight
-            float4 qr[4];
-#pragma unroll
-            for (int t = 0; t < 4; t++) {
-                const int i = 4 * (g + 8 * t);
-                qr[t] = i < (int)d.mp ? *reinterpret_cast<const float4 *>(qv + i) : make_float4(0.f, 0.f, 0.f, 0.f);
-            }
-            for (u32 r0 = 0; r0 < cnt; r0 += 16) {
-                u32 id[4];
-                float dd[4];
-#pragma unroll
-                for (int u = 0; u < 4; u++) {
-                    const u32 i = r0 + grp + 4 * u;
-                    id[u] = d.entries[cidx[warp][i < cnt ? i : cnt - 1]];
-                }
-                float4 v[4][4];
-#pragma unroll
-                for (int u = 0; u < 4; u++) canon_row_q8(d.x + (size_t)id[u] * d.mp, (int)d.mp, g, v[u]);
-#pragma unroll
-                for (int u = 0; u < 4; u++) dd[u] = canon_dist_q8v(qr, v[u], (int)d.mp, (int)d.metric, g);
-#pragma unroll
-                for (int u = 0; u < 4; u++) {
-                    const u32 i = r0 + grp + 4 * u;
-                    if (i < cnt && g == 0) ckey[warp][i] = mkkey(dd[u], id[u]);
-                }
-            }
-        } else {
-            for (u32 r0 = 0; r0 < cnt; r0 += 4) {
-                const u32 i = r0 + grp;
-                const u32 id = d.entries[cidx[warp][i < cnt ? i : cnt - 1]];
-                const float dd = canon_dist_wide<8>(qv, d.x + (size_t)id * d.mp, (int)d.mp, (int)d.metric, g);
-                if (i < cnt && g == 0) ckey[warp][i] = mkkey(dd, id);
-            }
-        }
-        const int np = next_pow2((int)cnt);
-        for (int i = (int)cnt + lane; i < np; i += 32) ckey[warp][i] = KEY_INF;
-        __syncwarp();
-        warp_sort_u64(ckey[warp], np);
-        if (tau == ~0u) {
-            cert = true;                               // every entry was scored
-        } else if (cnt >= a.L) {
-            const double lb = key_lower_bound((int)d.metric, a.m, a.kprime, true, a.qstat + 4 * (size_t)qi, a.estat,
-                                              (double)ord2f(tau));
-            cert = (double)key_rho(ckey[warp][a.L - 1]) < lb;
-        }
     }
     if (cert) {
-        for (u32 i = lane; i < a.L; i += 32) a.seed[(size_t)qi * a.L + i] = i < cnt ? ckey[warp][i] : KEY_INF;
+        seed_score(d, a.q + (size_t)qi * d.mp, cidx, 0, cnt, ckey);
+        // a key's place is the number of smaller ones (they are distinct): a short
+        // loop with no dependent step, where the stages of a bitonic sort wait for
+        // one another, or, unrolled, for their instructions
+        u64 *out = a.seed + (size_t)qi * a.L;
+        for (u32 b0 = 0; b0 < cnt; b0 += 128) {
+            u64 v[4];
+            u32 rank[4];
+#pragma unroll
+            for (int r = 0; r < 4; r++) {
+                const u32 i = b0 + 32 * r + lane;
+                v[r] = i < cnt ? ckey[i] : KEY_INF;
+                rank[r] = 0;
+            }
+#pragma unroll 4
+            for (u32 j = 0; j < cnt; j++) {
+                const u64 o = ckey[j];
+#pragma unroll
+                for (int r = 0; r < 4; r++) rank[r] += (u32)(o < v[r]);
+            }
+#pragma unroll
+            for (int r = 0; r < 4; r++)
+                if (b0 + 32 * r + lane < cnt && rank[r] < a.L) out[rank[r]] = v[r];
+        }
+        for (u32 i = cnt + lane; i < a.L; i += 32) out[i] = KEY_INF;
     } else if (lane == 0) {
         a.fb[atomicAdd(a.ctr, 1u)] = qi;
     }
@@ -1257,7 +1337,6 @@ cudaError_t launch_seed_tc(const Dev &d, const float *q, u32 nq, u32 S, u32 L, u
     r.L = L;
     r.S = S;
     r.ld = p.s_pad;
-    r.want = L + 32;
     r.m = d.dim;
     r.kprime = p.kb;
     r.q = q;

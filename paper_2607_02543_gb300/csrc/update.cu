@@ -7,6 +7,8 @@
 // order and publish once.  Lock-free mode gives each offer its own warp,
 // which snapshots the target, builds the new list and publishes it with a
 // compare-and-swap, retrying up to the attempt budget (Algorithm 1).
+#include <algorithm>
+
 #include <cuda_bf16.h>
 
 #include "common.cuh"
@@ -1345,218 +1347,225 @@ struct RepairKArgs {
     Dev d;
     const u32 *dt;
     const u64 *n_dt;
-    u32 max_n, ns, gram;
     u32 *pair_key, *pair_val;
     uint2 *pair_K;
     u32 *pair_Kn;
 };
 
-// sort width for K: the warp bitonic sort needs a power of two >= 32
-__host__ __device__ inline u32 repk_np(u32 R) {
-    u32 np = 32;
-    while (np < R) np <<= 1;
-    return np;
+constexpr int REPK_WARPS = 4;
+__host__ __device__ inline size_t repk_bytes(u32 R) {
+    return 2 * al16((size_t)R * 4) + al16((size_t)R * R * 4) + REPK_WARPS * 64;
 }
 
-__host__ __device__ inline size_t repk_warp_bytes(u32 R, u32 ns, u32 mp, u32 gram) {
-    const u32 np = repk_np(R);
-    return stage_bytes(ns, mp) + 2 * al16((size_t)R * 4) + al16((size_t)R * R * 4) + al16((size_t)32 * np + 32) +
-           gram_bytes(gram, mp);
+// The canonical sums of 64 values a lane holds as partials (value p in v[p]):
+// the tree of canon_dist over the 32 lanes, where at each level a lane keeps
+// half of the values it still has and passes the other half on.  Lane l ends
+// with values 2 l and 2 l + 1 in v[0] and v[1].
+__device__ __forceinline__ void warp_tree64(float (&v)[64]) {
+    const int lane = lane_id();
+#pragma unroll
+    for (int h = 16, n = 32; h >= 1; h >>= 1, n >>= 1) {
+        const bool up = lane & h;
+#pragma unroll
+        for (int i = 0; i < n; i++)
+            v[i] = __fadd_rn(up ? v[i + n] : v[i], __shfl_xor_sync(FULL, up ? v[i] : v[i + n], h));
+    }
 }
 
-__global__ void __launch_bounds__(128, 1) repair_k_kernel(RepairKArgs a) {
+// The greedy RobustPrune of B \ {a} about a = member ja of B, from the table M,
+// by one warp: the candidates b != a, live, in ascending (d(a, b), b), ranked
+// by counting the smaller keys (ids differ); then, for every candidate, the
+// mask of the later ones it would drop (no step waits for the one before); the
+// walk visits only candidates whose mask is not empty.  Writes K in order and
+// returns its size.  H: candidates per lane (nb <= 32 H).
+template <int H>
+__device__ __forceinline__ int repair_select(const Dev &d, const float *M, const u32 *bid, const u32 *bdel, int nb,
+                                             int ja, unsigned char *ord, uint2 *K) {
+    const int lane = lane_id();
+    const u32 R = d.R;
+    u64 k[H];
+    int rank[H], nc = 0;
+#pragma unroll
+    for (int c = 0; c < H; c++) {
+        const int t = lane + 32 * c;
+        const bool v = t < nb && t != ja && !bdel[t];
+        k[c] = v ? mkkey(M[ja * R + t], bid[t]) : KEY_INF;
+        rank[c] = 0;
+        nc += __popc(__ballot_sync(FULL, v));
+    }
+#pragma unroll
+    for (int c2 = 0; c2 < H; c2++)
+#pragma unroll 8
+        for (int j = 0; j < min(32, nb - 32 * c2); j++) {
+            const u64 o = __shfl_sync(FULL, k[c2], j);
+#pragma unroll
+            for (int c = 0; c < H; c++) rank[c] += o < k[c];
+        }
+#pragma unroll
+    for (int c = 0; c < H; c++)
+        if (k[c] != KEY_INF) ord[rank[c]] = (unsigned char)(lane + 32 * c);
+    __syncwarp();
+    int t[H];
+    float rho[H];
+#pragma unroll
+    for (int c = 0; c < H; c++) {
+        t[c] = lane + 32 * c < nc ? ord[lane + 32 * c] : ja;
+        rho[c] = M[ja * R + t[c]];       // not read for t = ja
+    }
+    u64 dom[H], any = 0;                 // dom[c]: the candidates that candidate lane + 32 c would drop
+#pragma unroll
+    for (int c = 0; c < H; c++) dom[c] = 0;
+#pragma unroll
+    for (int c2 = 0; c2 < H; c2++)
+#pragma unroll 8
+        for (int j = 0; j < min(32, nc - 32 * c2); j++) {
+            const int h = j + 32 * c2, hj = __shfl_sync(FULL, t[c2], j);
+            u64 m = 0;
+#pragma unroll
+            for (int c = 0; c < H; c++) {
+                const int i = lane + 32 * c;
+                const bool hit = i > h && i < nc && __fmul_rn(d.alpha2, M[hj * R + t[c]]) <= rho[c];
+                m |= (u64)__ballot_sync(FULL, hit) << (32 * c);
+            }
+            if (lane == j) dom[c2] = m;
+            if (m) any |= 1ull << h;
+        }
+    u64 alive = nc >= 64 ? ~0ull : ((1ull << nc) - 1);
+    while (any) {
+        const int h = __ffsll((long long)any) - 1;
+        any &= any - 1;
+        const u64 m = __shfl_sync(FULL, H == 1 || h < 32 ? dom[0] : dom[H - 1], h & 31);
+        if (alive >> h & 1) alive &= ~m;
+    }
+#pragma unroll
+    for (int c = 0; c < H; c++) {
+        const int i = lane + 32 * c;
+        if (i < nc && (alive >> i & 1))
+            K[__popcll(alive & ((1ull << i) - 1))] = make_uint2(bid[t[c]], __float_as_uint(rho[c]));
+    }
+    __syncwarp();                        // ord is free again
+    return __popcll(alive);
+}
+
+// A block per deleted node.  The distances among B are computed in 8 x 8 tiles
+// of pairs, a warp per tile: lane j sums partial j of the tile's 64 pairs, so
+// that each 128-column block of 16 rows serves 64 pairs from registers.  Bound
+// by the fp32 arithmetic of the table (the stored edge distances have to be
+// canonical); a warp per node, four pairs at a time from shared memory, took
+// 682 us for 10,000 nodes of 128-d (R = 32) and 2,590 for 500 of 768-d (R = 64).
+template <int H>   // members of B per lane: R <= 32 H
+__global__ void __launch_bounds__(32 * REPK_WARPS, 3) repair_k_kernel(RepairKArgs a) {
     extern __shared__ __align__(16) char smem[];
-    const int warp = threadIdx.x >> 5, lane = lane_id();
+    __shared__ u64 next;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = lane_id();
     const Dev &d = a.d;
     const u32 R = d.R;
-    char *p = smem + warp * repk_warp_bytes(R, a.ns, d.mp, a.gram);
-    char *gbuf = a.gram ? p : nullptr;
-    p += gram_bytes(a.gram, d.mp);
-    Stage st = stage_init(p, a.ns, d.mp, gbuf, a.gram);
-    p += stage_bytes(a.ns, d.mp);
+    char *p = smem;
     u32 *bid = reinterpret_cast<u32 *>(p); p += al16((size_t)R * 4);
     u32 *bdel = reinterpret_cast<u32 *>(p); p += al16((size_t)R * 4);
     float *M = reinterpret_cast<float *>(p); p += al16((size_t)R * R * 4);
-    const int npk = (int)repk_np(R);
-    unsigned char *ord = reinterpret_cast<unsigned char *>(p) + lane * npk;   // this lane's sorted candidates
-    const int grp = lane >> 3, g = lane & 7;
+    unsigned char *ord = reinterpret_cast<unsigned char *>(p);   // a warp's candidates in order
     const u64 nd = *a.n_dt;
     const u32 invalid = (u32)d.capacity;
-    u64 i_next = 0;   // the next item's claim, in flight while this one runs
-    if (lane == 0) i_next = atomicAdd(&d.ctr[C_WORK], 1ull);
+    u64 wk_rows = 0, wk_state = 0;
     for (;;) {
-        const u64 i = __shfl_sync(FULL, i_next, 0);
+        __syncthreads();   // the last node's lists are read
+        if (tid == 0) next = atomicAdd(&d.ctr[C_WORK], 1ull);
+        __syncthreads();
+        const u64 i = next;
         if (i >= nd) break;
-        if (lane == 0) i_next = atomicAdd(&d.ctr[C_WORK], 1ull);
-        const u32 u = a.dt[i];
-        u64 r = 0;
-        if (lane == 0) r = ld_ref(d, u);
-        r = __shfl_sync(FULL, r, 0);
+        const u64 r = ld_ref(d, a.dt[i]);
         const u32 s = ref_slab(r);
         const int nb = s == NIL ? 0 : (int)ref_deg(r);
-        for (int j = lane; j < nb; j += 32) {
-            bid[j] = d.slab[(size_t)s * R + j].x;
-            bdel[j] = ref_del(ld_ref(d, bid[j]));
+        for (int j = tid; j < nb; j += 32 * REPK_WARPS) {
+            const u32 id = d.slab[(size_t)s * R + j].x;
+            bid[j] = id;
+            bdel[j] = ref_del(ld_ref(d, id));
         }
-        st.wk_state += 8 + 16ull * nb;           // u's word, N(u), and the members' words
-        st.wk_rows += (u64)nb * 4 * d.mp;        // B's rows (the canonical table)
-        __syncwarp();
-        // distance table among B (symmetric).  These distances become the
-        // stored rho of replacement edges, so they stay canonical.
-        const int nsb = st.rows ? min(nb, st.ns_cap) : 0;
-        stage_rows_by(d, st, nsb, [&](int i) { return bid[i]; });
-        auto brow = [&](int i) -> const float * {
-            return i < nsb ? st.rows + (size_t)i * d.mp : d.x + (size_t)bid[i] * d.mp;
-        };
-        // the pairs x < y in one sequence (index y (y - 1) / 2 + x), eight per
-        // trip in two independent rounds of four: their row loads overlap
-        const int npair = nb * (nb - 1) / 2;
-        auto pair_of = [](int q, int &x, int &y) {
-            int yy = (int)((1.0f + sqrtf(1.0f + 8.0f * (float)q)) * 0.5f);
-            if (yy * (yy - 1) / 2 > q) yy--;
-            if ((yy + 1) * yy / 2 <= q) yy++;
-            y = yy;
-            x = q - yy * (yy - 1) / 2;
-        };
-        if (d.mp <= 128) {
-            // rows of at most 128 floats: each lane's four float4 of both rows
-            // of a pair in registers, so the canonical distance runs with no
-            // column loop; each group's pair cursor steps by 8 in the same
-            // sequence instead of recomputing it with a square root
-            int x = 0, y = 1, x2 = 0, y2 = 1;
-            if (grp < npair) pair_of(grp, x, y);
-            if (grp + 4 < npair) pair_of(grp + 4, x2, y2);
-            for (int q0 = 0; q0 < npair; q0 += 8) {
-                const int q = q0 + grp, q2 = q + 4;
-                const bool v1 = q < npair, v2 = q2 < npair;
-                float4 ra[4], rb[4], rc[4], rd[4];
-                canon_row_q8(brow(v1 ? x : 0), (int)d.mp, g, ra);
-                canon_row_q8(brow(v1 ? y : 1), (int)d.mp, g, rb);
-                canon_row_q8(brow(v2 ? x2 : 0), (int)d.mp, g, rc);
-                canon_row_q8(brow(v2 ? y2 : 1), (int)d.mp, g, rd);
-                const float dd = canon_dist_q8v(ra, rb, (int)d.mp, (int)d.metric, g);
-                const float dd2 = canon_dist_q8v(rc, rd, (int)d.mp, (int)d.metric, g);
-                if (v1 && g == 0) { M[x * R + y] = dd; M[y * R + x] = dd; }
-                if (v2 && g == 0) { M[x2 * R + y2] = dd2; M[y2 * R + x2] = dd2; }
-                for (x += 8; x >= y; y++) x -= y;
-                for (x2 += 8; x2 >= y2; y2++) x2 -= y2;
-            }
-        } else {
-            for (int q0 = 0; q0 < npair; q0 += 8) {
-                const int q = q0 + grp, q2 = q + 4;
-                int x, y, x2, y2;
-                pair_of(q < npair ? q : npair - 1, x, y);
-                pair_of(q2 < npair ? q2 : npair - 1, x2, y2);
-                const float dd = canon_dist<8>(brow(x), brow(y), (int)d.mp, (int)d.metric, g);
-                const float dd2 = canon_dist<8>(brow(x2), brow(y2), (int)d.mp, (int)d.metric, g);
-                if (q < npair && g == 0) { M[x * R + y] = dd; M[y * R + x] = dd; }
-                if (q2 < npair && g == 0) { M[x2 * R + y2] = dd2; M[y2 * R + x2] = dd2; }
-            }
-        }
-        __syncwarp();
-        // K(u, a) for every a in B, one lane per a: the candidates b != a, live,
-        // in ascending (d(a, b), b), then the greedy RobustPrune on the table.
-        // Orders: with |B| <= 32 the warp sorts each a's candidates in
-        // registers (the id replaced by its rank among B's ids: the same
-        // order, and the rank leads back to the table index); above that each
-        // lane ranks its own candidates by counting.
-        u32 liveB = 0;
-        for (int t0 = 0; t0 < nb; t0 += 32) {
-            const u32 m = __ballot_sync(FULL, t0 + lane < nb && !bdel[t0 + lane]);
-            if (t0 == 0) liveB = m;
-        }
-        const bool sorted_by_warp = nb <= 32;
-        if (sorted_by_warp) {
-            int idr = 0;
-            if (lane < nb)
-                for (int t2 = 0; t2 < nb; t2++) idr += bid[t2] < bid[lane];
-            unsigned char *inv = reinterpret_cast<unsigned char *>(ord) - lane * npk + 32 * npk;   // after the orders
-            if (lane < nb) inv[idr] = (unsigned char)lane;
-            __syncwarp();
-            for (int ja0 = 0; ja0 < nb; ja0 += 4) {
-                u64 k[4];
+        wk_state += 8 + 16ull * nb;           // u's word, N(u), and the members' words
+        wk_rows += (u64)nb * 4 * d.mp;        // B's rows
+        __syncthreads();
+        // distance table among B (symmetric): tiles x <= y, in one sequence
+        const int nt = (nb + 7) >> 3;
+        for (int t = warp; t < nt * (nt + 1) / 2; t += REPK_WARPS) {
+            int ty = 0, tx = t;
+            while (tx > ty) tx -= ++ty;       // t = ty (ty + 1) / 2 + tx
+            const float *xr[8], *yr[8];
 #pragma unroll
-                for (int c = 0; c < 4; c++) {
-                    const int ja = ja0 + c;
-                    const bool v = ja < nb && (liveB >> ja & 1) && lane < nb && lane != ja && (liveB >> lane & 1);
-                    k[c] = v ? ((u64)f2ord(M[ja * R + lane]) << 32) | (u32)idr : KEY_INF;   // M is symmetric
+            for (int c = 0; c < 8; c++) {     // past the list: a valid row again
+                xr[c] = d.x + (size_t)bid[min(8 * tx + c, nb - 1)] * d.mp;
+                yr[c] = d.x + (size_t)bid[min(8 * ty + c, nb - 1)] * d.mp;
+            }
+            float acc[64];
+#pragma unroll
+            for (int q = 0; q < 64; q++) acc[q] = 0.0f;
+            for (u32 e = 4 * lane; e < d.mp; e += 128) {
+                float4 x[8], y[8];
+#pragma unroll
+                for (int c = 0; c < 8; c++) {
+                    x[c] = *reinterpret_cast<const float4 *>(xr[c] + e);
+                    y[c] = *reinterpret_cast<const float4 *>(yr[c] + e);
                 }
-                warp_sort32x4(k);
+                if (d.metric == 0) {
 #pragma unroll
-                for (int c = 0; c < 4; c++) {
-                    unsigned char *oa = reinterpret_cast<unsigned char *>(ord) - lane * npk + (ja0 + c) * npk;
-                    if (k[c] != KEY_INF) oa[lane] = inv[(u32)k[c]];
+                    for (int q = 0; q < 64; q++) {
+                        const float4 u = x[q >> 3], v = y[q & 7];
+                        const float d0 = __fsub_rn(u.x, v.x), d1 = __fsub_rn(u.y, v.y);
+                        const float d2 = __fsub_rn(u.z, v.z), d3 = __fsub_rn(u.w, v.w);
+                        acc[q] = __fmaf_rn(d3, d3, __fmaf_rn(d2, d2, __fmaf_rn(d1, d1, __fmaf_rn(d0, d0, acc[q]))));
+                    }
+                } else {
+#pragma unroll
+                    for (int q = 0; q < 64; q++) {
+                        const float4 u = x[q >> 3], v = y[q & 7];
+                        acc[q] = __fmaf_rn(u.w, v.w, __fmaf_rn(u.z, v.z, __fmaf_rn(u.y, v.y, __fmaf_rn(u.x, v.x, acc[q]))));
+                    }
                 }
             }
             __syncwarp();
+            warp_tree64(acc);
+#pragma unroll
+            for (int k = 0; k < 2; k++) {
+                const int q = 2 * lane + k, x = 8 * tx + (q >> 3), y = 8 * ty + (q & 7);
+                const float dd = d.metric == 0 ? acc[k] : __fsub_rn(1.0f, acc[k]);
+                if (x < y && y < nb) { M[x * R + y] = dd; M[y * R + x] = dd; }
+            }
         }
-        for (int ja = lane; ja < (int)R; ja += 32) {
+        __syncthreads();
+        // K(u, a), a warp per a
+        for (int ja = warp; ja < (int)R; ja += REPK_WARPS) {
             const size_t slot = (size_t)i * R + ja;
-            if (ja >= nb || bdel[ja]) {
-                a.pair_key[slot] = invalid;
+            int nk = -1;
+            if (ja < nb && !bdel[ja]) nk = repair_select<H>(d, M, bid, bdel, nb, ja, ord + warp * 64, a.pair_K + slot * R);
+            if (lane == 0) {
+                a.pair_key[slot] = nk < 0 ? invalid : bid[ja];
                 a.pair_val[slot] = (u32)slot;
-                a.pair_Kn[slot] = 0;
-                continue;
+                a.pair_Kn[slot] = (u32)max(nk, 0);
             }
-            int nc = 0;
-            if (sorted_by_warp) {
-                nc = __popc(liveB & ~(1u << ja));
-            } else {
-                // rank of each candidate among the candidates (keys are distinct: ids
-                // differ); M is symmetric, and M[t][ja] keeps the lanes on distinct banks
-                for (int t = 0; t < nb; t++) {
-                    if (t == ja || bdel[t]) continue;
-                    const u64 kt = mkkey(M[t * R + ja], bid[t]);
-                    int rank = 0;
-                    for (int t2 = 0; t2 < nb; t2++)
-                        if (t2 != ja && !bdel[t2] && mkkey(M[t2 * R + ja], bid[t2]) < kt) rank++;
-                    ord[rank] = (unsigned char)t;
-                    nc++;
-                }
-            }
-            int nk = 0;
-            u64 alive = nc >= 64 ? ~0ull : ((1ull << nc) - 1);
-            for (int h = 0; h < nc && nk < (int)R; h++) {
-                if (!(alive >> h & 1)) continue;
-                const int hj = ord[h];
-                const float hr = M[hj * R + ja];
-                a.pair_K[slot * R + nk] = make_uint2(bid[hj], __float_as_uint(hr));
-                nk++;
-                for (int t2 = h + 1; t2 < nc; t2++) {
-                    if (!(alive >> t2 & 1)) continue;
-                    const int tj = ord[t2];
-                    if (__fmul_rn(d.alpha2, M[hj * R + tj]) <= M[tj * R + ja]) alive &= ~(1ull << t2);
-                }
-            }
-            a.pair_key[slot] = bid[ja];
-            a.pair_val[slot] = (u32)slot;
-            a.pair_Kn[slot] = (u32)nk;
         }
-        __syncwarp();
     }
-    stage_done(d, st, WK_REPAIR_K);
+    if (tid == 0) {
+        if (wk_rows) atomicAdd(&d.ctr[C_WK + 2 * WK_REPAIR_K], wk_rows);
+        if (wk_state) atomicAdd(&d.ctr[C_WK + 2 * WK_REPAIR_K + 1], wk_state);
+    }
 }
 
 cudaError_t launch_repair_k(const Dev &d, const u32 *dt, const u64 *n_dt, u32 max_n, u32 *pair_key,
                             u32 *pair_val, uint2 *pair_K, u32 *pair_Kn, int num_sms, cudaStream_t st) {
     if (max_n == 0) return cudaSuccess;
-    // B's rows are read about |B| times each: stage up to 16 KB of them
-    const u32 budget = d.stage_bytes > (16u << 10) ? d.stage_bytes : (16u << 10);
-    RepairKArgs a{d, dt, n_dt, max_n, stage_cap(d.mp, d.R, budget), 0u, pair_key, pair_val, pair_K, pair_Kn};
-    const size_t wb = repk_warp_bytes(d.R, a.ns, d.mp, a.gram);
-    const int W = warps_for(wb);
-    size_t smem = W * wb;
-    cudaError_t e = smem_at_least((const void *)repair_k_kernel, smem);
+    RepairKArgs a{d, dt, n_dt, pair_key, pair_val, pair_K, pair_Kn};
+    const size_t smem = repk_bytes(d.R);
+    void (*fn)(RepairKArgs) = d.R <= 32 ? repair_k_kernel<1> : repair_k_kernel<2>;
+    cudaError_t e = smem_at_least((const void *)fn, smem);
     if (e != cudaSuccess) return e;
     int per_sm = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, repair_k_kernel, 32 * W, smem);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, (const void *)fn, 32 * REPK_WARPS, smem);
     if (e != cudaSuccess) return e;
     if (per_sm < 1) return cudaErrorInvalidConfiguration;
-    u32 blocks = (u32)(per_sm * num_sms), need = (max_n + W - 1) / W;
-    if (blocks > need) blocks = need;
+    const u32 blocks = std::min<u32>((u32)(per_sm * num_sms), max_n);
     e = cudaMemsetAsync(d.ctr + C_WORK, 0, sizeof(u64), st);
     if (e != cudaSuccess) return e;
-    repair_k_kernel<<<blocks, 32 * W, smem, st>>>(a);
+    fn<<<blocks, 32 * REPK_WARPS, smem, st>>>(a);
     return cudaGetLastError();
 }
 

@@ -8,8 +8,7 @@
 // which snapshots the target, builds the new list and publishes it with a
 // compare-and-swap, retrying up to the attempt budget (Algorithm 1).
 #include <algorithm>
-
-#include <cuda_bf16.h>
+#include <type_traits>
 
 #include "common.cuh"
 #include "internal.h"
@@ -31,6 +30,7 @@ struct Stage {
     bool timeout;
     char *gram;      // gram_bytes(gram_rows, mp) for the tensor-core Gram path (nullptr: canonical path)
     int gram_rows;   // candidates the Gram buffer holds (a multiple of 16, <= GRAM_NL)
+    struct GramReq *req;     // the block's request slot (cooperative variants)
     u64 wk_rows, wk_state;   // this warp's work tallies (see WK_*), added by stage_done
 };
 
@@ -41,38 +41,28 @@ struct Stage {
 // GRAM_N floats, also 256 bytes) reuses the same bytes.
 constexpr int GRAM_N = 64;
 constexpr int GRAM_RB = 256;   // bytes per staged row (128 bf16 columns)
-// The large path (more than GRAM_N rows) keeps rows of GRAM_RS_LG bf16 (a
-// 16-byte pad: conflict-free ldmatrix without a swizzle), so that a whole
-// row block lands with one bulk copy per row.
-constexpr int GRAM_RS_LG = 136;
-__host__ __device__ inline size_t gram_rowb(u32 rows) { return rows > (u32)GRAM_N ? (size_t)GRAM_RS_LG * 2 : GRAM_RB; }
+// The cooperative path (more than GRAM_N rows, or rows of more than one
+// 128-column block; see gram_masks) pads its rows to GRAM_RS_CO bf16 (a 16-byte
+// pad: conflict-free ldmatrix without a swizzle) and keeps two blocks of them.
+constexpr int GRAM_RS_CO = 136;
+constexpr int GRAM_NL = 128;   // candidates of the cooperative path
+constexpr int COOP_WARPS = 4;
 __host__ __device__ inline u32 gram_xoff(int r, int chunk) { return (u32)(r * GRAM_RB + ((chunk ^ (r & 7)) << 4)); }
-// Byte offset, in a Gram buffer for `rows` candidates, of the partial sums
-// that rows longer than one 128-column block keep between blocks: after the
-// bf16 rows (or the table over them), a (norm, rho) pair per candidate and
-// the large path's domination masks.  rows is a multiple of 16.
-__host__ __device__ inline size_t gram_part_off(u32 rows) {
-    const size_t b = (size_t)rows * gram_rowb(rows) + (size_t)rows * 8;
-    return rows > (u32)GRAM_N ? b + (size_t)rows * 16 : b;
-}
-// Shared-memory bytes of a Gram buffer for `rows` candidates of mp columns;
-// 0 rows = no buffer.  With more than one column block, a small-path buffer
-// (rows <= GRAM_N) also holds one accumulator fragment (32 lanes x 16 bytes)
-// per upper-triangle tile: nm (nm + 1) tiles for nm = rows / 16 stripes.
-__host__ __device__ inline size_t gram_bytes(u32 rows, u32 mp) {
-    if (!rows) return 0;
-    const size_t nm = rows / 16;
-    return gram_part_off(rows) + (mp > 128 && rows <= (u32)GRAM_N ? nm * (nm + 1) * 512 : 0);
-}
-// First tile slot of stripe mt among the partial sums (stripe mt holds the
-// tiles nt = 2 mt .. 2 nmr - 1, nmr = rows / 16).
-__device__ __forceinline__ int gram_part_slot(int mt, int nmr) { return mt * (2 * nmr + 1 - mt); }
-constexpr int GRAM_NL = 128;   // candidates of the large (mask) path
 // The Gram variant (see warp_prune) of a kernel whose buffer holds gram_rows rows of mp columns.
-inline int gram_variant(u32 gram_rows, u32 mp) { return gram_rows > (u32)GRAM_N ? 1 : (gram_rows && mp > 128 ? 2 : 0); }
+__host__ __device__ inline int gram_variant(u32 gram_rows, u32 mp) {
+    return gram_rows > (u32)GRAM_N ? 1 : (gram_rows && mp > 128 ? 2 : 0);
+}
+// Bytes of a Gram buffer's rows (or the table over them), and of the whole
+// buffer: a (norm, rho) pair per candidate follows, and on the cooperative path
+// its domination mask (two words).  rows is a multiple of 16; 0 = no buffer.
+__host__ __device__ inline size_t gram_row_bytes(u32 rows, u32 mp) {
+    return gram_variant(rows, mp) ? (size_t)(mp > 128 ? 2 : 1) * rows * GRAM_RS_CO * 2 : (size_t)rows * GRAM_RB;
+}
+__host__ __device__ inline size_t gram_bytes(u32 rows, u32 mp) {
+    return gram_row_bytes(rows, mp) + (size_t)rows * (gram_variant(rows, mp) ? 8 + 16 : 8);
+}
 // Gram rows for a kernel whose prunes see at most max_n candidates (0: the
-// Gram path is off or cannot hold them).  Above GRAM_N rows the kernel runs
-// the large path (warp_prune_masks).
+// Gram path is off or cannot hold them).
 inline u32 gram_rows_for(u32 on, u32 max_n) { return on && max_n <= (u32)GRAM_NL ? (max_n + 15) / 16 * 16 : 0; }
 // Scratch that is dead whenever the Gram buffer is live (list compaction before
 // a prune, the canonical prune's arrays, a prune's output, written after its
@@ -83,7 +73,8 @@ __host__ __device__ inline bool gram_alias(u32 gram, size_t scratch) { return gr
 __host__ __device__ inline size_t stage_bytes(u32 ns, u32 mp) { return al16((size_t)ns * mp * 4) + 16; }
 
 // Carve a stage at p (16-byte aligned) and initialise the warp's mbarrier.
-__device__ __forceinline__ Stage stage_init(char *p, u32 ns, u32 mp, char *gram = nullptr, u32 gram_rows = 0) {
+__device__ __forceinline__ Stage stage_init(char *p, u32 ns, u32 mp, char *gram = nullptr, u32 gram_rows = 0,
+                                            GramReq *req = nullptr) {
     Stage st;
     st.rows = ns ? reinterpret_cast<float *>(p) : nullptr;
     st.ns_cap = (int)ns;
@@ -92,6 +83,7 @@ __device__ __forceinline__ Stage stage_init(char *p, u32 ns, u32 mp, char *gram 
     st.timeout = false;
     st.gram = gram;
     st.gram_rows = (int)gram_rows;
+    st.req = req;
     st.wk_rows = st.wk_state = 0;
     if (lane_id() == 0) mbar_init(st.bar, 1);
     __syncwarp();
@@ -112,11 +104,11 @@ __device__ __forceinline__ u64 prune_row_bytes(const Dev &d, const Stage &st, in
     return (u64)n * (b16 ? 2ull * d.mb : 4ull * d.mp);
 }
 
-// Warps per block (<= 4) such that a block's shared memory stays <= 200 KB.
-// Warps per block of the persistent update kernels: one.  Their shared memory
-// is per warp (up to ~20 KB with the Gram tile), so one-warp blocks pack the
-// SM by the warp instead of by four (11 warps instead of 8 at 19 KB).
-inline int warps_for(size_t) { return 1; }
+// Threads per block of the persistent update kernels: one warp, or one with its
+// helpers on the cooperative path.  Their shared memory is per item (up to ~20
+// KB with the Gram tile), so one-warp blocks pack the SM by the warp instead of
+// by four (11 warps instead of 8 at 19 KB).
+inline int block_threads(u32 gram_rows, u32 mp) { return gram_variant(gram_rows, mp) ? 32 * COOP_WARPS : 32; }
 
 // Rows that fit a per-warp stage of `budget` bytes, capped at `want`.
 inline u32 stage_cap(u32 mp, u32 want, u32 budget) {
@@ -211,144 +203,68 @@ __device__ __forceinline__ void gram_stage_rows(const Dev &d, const u64 *ck, int
 // (h, h + 1 + k)) still hits 32 distinct banks.
 __device__ __forceinline__ int gram_tsw(int r) { return (r & 3) << 3; }
 
-// Writes the upper triangle (j >= i, in 16 x 8 tiles) of the n x n Gram into
-// T (fp32, row stride GRAM_N, columns swizzled by gram_tsw) and the diagonal
-// into nr2[i].x, with rho_i (the candidate's key distance) in nr2[i].y.
-// Rows of one 128-column block (MB false) are staged once, then the stripes
-// run in ascending order.  With several blocks (MB true) the blocks go
-// outermost: each block of every row is staged once, and each stripe adds
-// its products for the block to the buffer's partial sums (fp32; exact for
-// the integer-valued data the tile is exact for).  T and the bf16 rows share
-// `buf`: in the (last) block the stripes go in ascending order, and stripe
-// mt's table rows (bytes [4096 mt, 4096 (mt + 1))) are the staged rows of
-// that same stripe, which no later stripe reads (it reads rows >= 16 (mt + 1)).
-// A stripe only needs the columns j >= 16 mt, because the prune reads
-// T[head][j] for j > head.  Rows past n hold whatever the buffer held: an
-// entry (i, j) reads rows i and j only, and no entry with i or j >= n is read.
-template <bool MB>   // rows span more than one 128-column block
-__device__ void warp_gram(const Dev &d, const u64 *ck, int n, char *buf, int rows, Stage &st, float *&T, float2 *&nr2) {
-    // The single-block form keeps its own loop nest: written as the
-    // multi-block one with one block, it costs the 128-d kernels 10 to 20
-    // registers and with them resident warps.
-    if constexpr (!MB) {
-        (void)st;
-        const int lane = lane_id();
-        T = reinterpret_cast<float *>(buf);
-        nr2 = reinterpret_cast<float2 *>(buf + (size_t)rows * GRAM_RB);
-        const int nm = (n + 15) >> 4, nn = (n + 7) >> 3;
-        const int nkb = ((int)d.mp + 127) >> 7;
-        const u32 xs = smem_addr(buf), c0 = gram_c0(lane);
-        for (int mt = 0; mt < nm; mt++) {
-            float acc[8][4];
+// Writes the upper triangle (j >= i, in 16 x 8 tiles) of the n x n Gram of rows
+// of one 128-column block into T (fp32, row stride GRAM_N, columns swizzled by
+// gram_tsw) and the diagonal into nr2[i].x, with rho_i (the candidate's key
+// distance) in nr2[i].y.  T and the bf16 rows share `buf`: the stripes go in
+// ascending order, and stripe mt's table rows (bytes [4096 mt, 4096 (mt + 1)))
+// are the staged rows of that same stripe, which no later stripe reads (it
+// reads rows >= 16 (mt + 1)).  A stripe only needs the columns j >= 16 mt,
+// because the prune reads T[head][j] for j > head.  Rows past n hold whatever
+// the buffer held: an entry (i, j) reads rows i and j only, and no entry with
+// i or j >= n is read.
+// (The loop over column blocks runs once here.  Without it, and with the
+// staging ahead of the stripes, the kernels take 10 to 25 registers more and
+// lose resident warps.)
+__device__ void warp_gram(const Dev &d, const u64 *ck, int n, char *buf, int rows, float *&T, float2 *&nr2) {
+    const int lane = lane_id();
+    T = reinterpret_cast<float *>(buf);
+    nr2 = reinterpret_cast<float2 *>(buf + (size_t)rows * GRAM_RB);
+    const int nm = (n + 15) >> 4, nn = (n + 7) >> 3;
+    const int nkb = ((int)d.mp + 127) >> 7;
+    const u32 xs = smem_addr(buf), c0 = gram_c0(lane);
+    for (int mt = 0; mt < nm; mt++) {
+        float acc[8][4];
 #pragma unroll
-            for (int b = 0; b < 8; b++)
+        for (int b = 0; b < 8; b++)
 #pragma unroll
-                for (int c = 0; c < 4; c++) acc[b][c] = 0.f;
-            for (int kb = 0; kb < nkb; kb++) {
-                // rows [16 mt, n) of this column block: all rows once when one
-                // block covers the row, else this stripe's and later ones per block
-                if (nkb > 1 || mt == 0) gram_stage_rows(d, ck, 16 * mt, n, kb, xs);
-#pragma unroll
-                for (int ks = 0; ks < 8; ks++) {
-                    u32 a0, a1, a2, a3;
-                    const u32 ko = (u32)(32 * ks) ^ c0;
-                    const int ar = 16 * mt + (lane & 7) + 8 * ((lane >> 3) & 1);
-                    ldsm_x4(a0, a1, a2, a3, xs + (u32)ar * GRAM_RB + ko);
-#pragma unroll
-                    for (int nt = 0; nt < 8; nt += 2) {
-                        if (nt < 2 * mt || nt >= nn) continue;
-                        // matrices: (nt, k 0-7), (nt + 1, k 0-7), (nt, k 8-15), (nt + 1, k 8-15)
-                        u32 b0, b1, b2, b3;
-                        const int br = 8 * nt + (lane & 7) + 8 * ((lane >> 3) & 1);
-                        ldsm_x4(b0, b1, b2, b3, xs + (u32)br * GRAM_RB + ko);
-                        mma_bf16_16816(acc[nt], a0, a1, a2, a3, b0, b2);
-                        mma_bf16_16816(acc[nt + 1], a0, a1, a2, a3, b1, b3);
-                    }
-                }
-            }
-            __syncwarp();
-            // this stripe's table rows, over this stripe's staged rows (rows r and
-            // r + 8 share the column swizzle)
-#pragma unroll
-            for (int nt = 0; nt < 8; nt++) {
-                if (nt < 2 * mt || nt >= nn) continue;
-                const int r = 16 * mt + (lane >> 2), c = (8 * nt + 2 * (lane & 3)) ^ gram_tsw(r);
-                *reinterpret_cast<float2 *>(T + r * GRAM_N + c) = make_float2(acc[nt][0], acc[nt][1]);
-                *reinterpret_cast<float2 *>(T + (r + 8) * GRAM_N + c) = make_float2(acc[nt][2], acc[nt][3]);
-            }
-            __syncwarp();
-        }
-        for (int i = lane; i < n; i += 32) nr2[i] = make_float2(T[i * GRAM_N + (i ^ gram_tsw(i))], key_rho(ck[i]));
-        __syncwarp();
-    } else {
-        (void)st;
-        const int lane = lane_id();
-        T = reinterpret_cast<float *>(buf);
-        nr2 = reinterpret_cast<float2 *>(buf + (size_t)rows * GRAM_RB);
-        float4 *part = reinterpret_cast<float4 *>(buf + gram_part_off((u32)rows));
-        const int nm = (n + 15) >> 4, nn = (n + 7) >> 3, nmr = rows >> 4;
-        const int nkb = MB ? ((int)d.mp + 127) >> 7 : 1;
-        const u32 xs = smem_addr(buf), c0 = gram_c0(lane);
+            for (int c = 0; c < 4; c++) acc[b][c] = 0.f;
         for (int kb = 0; kb < nkb; kb++) {
-            gram_stage_rows(d, ck, 0, n, kb, xs);
-            const bool last = kb == nkb - 1;
-            for (int mt = 0; mt < nm; mt++) {
-                const int slot = gram_part_slot(mt, nmr) - 2 * mt;
-                float acc[8][4];
+            // rows [16 mt, n) of this column block: all rows once when one
+            // block covers the row, else this stripe's and later ones per block
+            if (nkb > 1 || mt == 0) gram_stage_rows(d, ck, 16 * mt, n, kb, xs);
 #pragma unroll
-                for (int b = 0; b < 8; b++)
+            for (int ks = 0; ks < 8; ks++) {
+                u32 a0, a1, a2, a3;
+                const u32 ko = (u32)(32 * ks) ^ c0;
+                const int ar = 16 * mt + (lane & 7) + 8 * ((lane >> 3) & 1);
+                ldsm_x4(a0, a1, a2, a3, xs + (u32)ar * GRAM_RB + ko);
 #pragma unroll
-                    for (int c = 0; c < 4; c++) acc[b][c] = 0.f;
-#pragma unroll
-                for (int ks = 0; ks < 8; ks++) {
-                    u32 a0, a1, a2, a3;
-                    const u32 ko = (u32)(32 * ks) ^ c0;
-                    const int ar = 16 * mt + (lane & 7) + 8 * ((lane >> 3) & 1);
-                    ldsm_x4(a0, a1, a2, a3, xs + (u32)ar * GRAM_RB + ko);
-#pragma unroll
-                    for (int nt = 0; nt < 8; nt += 2) {
-                        if (nt < 2 * mt || nt >= nn) continue;
-                        // matrices: (nt, k 0-7), (nt + 1, k 0-7), (nt, k 8-15), (nt + 1, k 8-15)
-                        u32 b0, b1, b2, b3;
-                        const int br = 8 * nt + (lane & 7) + 8 * ((lane >> 3) & 1);
-                        ldsm_x4(b0, b1, b2, b3, xs + (u32)br * GRAM_RB + ko);
-                        mma_bf16_16816(acc[nt], a0, a1, a2, a3, b0, b2);
-                        mma_bf16_16816(acc[nt + 1], a0, a1, a2, a3, b1, b3);
-                    }
-                }
-                if constexpr (MB) {
-                    // this block's products join the earlier blocks' sums
-#pragma unroll
-                    for (int nt = 0; nt < 8; nt++) {
-                        if (nt < 2 * mt || nt >= nn) continue;
-                        float4 *pp = part + (size_t)(slot + nt) * 32 + lane;
-                        if (kb > 0) {
-                            const float4 v = *pp;
-                            acc[nt][0] = __fadd_rn(v.x, acc[nt][0]);
-                            acc[nt][1] = __fadd_rn(v.y, acc[nt][1]);
-                            acc[nt][2] = __fadd_rn(v.z, acc[nt][2]);
-                            acc[nt][3] = __fadd_rn(v.w, acc[nt][3]);
-                        }
-                        if (!last) *pp = make_float4(acc[nt][0], acc[nt][1], acc[nt][2], acc[nt][3]);
-                    }
-                    if (!last) continue;
-                }
-                __syncwarp();
-                // this stripe's table rows, over this stripe's staged rows (rows r and
-                // r + 8 share the column swizzle)
-#pragma unroll
-                for (int nt = 0; nt < 8; nt++) {
+                for (int nt = 0; nt < 8; nt += 2) {
                     if (nt < 2 * mt || nt >= nn) continue;
-                    const int r = 16 * mt + (lane >> 2), c = (8 * nt + 2 * (lane & 3)) ^ gram_tsw(r);
-                    *reinterpret_cast<float2 *>(T + r * GRAM_N + c) = make_float2(acc[nt][0], acc[nt][1]);
-                    *reinterpret_cast<float2 *>(T + (r + 8) * GRAM_N + c) = make_float2(acc[nt][2], acc[nt][3]);
+                    // matrices: (nt, k 0-7), (nt + 1, k 0-7), (nt, k 8-15), (nt + 1, k 8-15)
+                    u32 b0, b1, b2, b3;
+                    const int br = 8 * nt + (lane & 7) + 8 * ((lane >> 3) & 1);
+                    ldsm_x4(b0, b1, b2, b3, xs + (u32)br * GRAM_RB + ko);
+                    mma_bf16_16816(acc[nt], a0, a1, a2, a3, b0, b2);
+                    mma_bf16_16816(acc[nt + 1], a0, a1, a2, a3, b1, b3);
                 }
-                __syncwarp();
             }
         }
-        for (int i = lane; i < n; i += 32) nr2[i] = make_float2(T[i * GRAM_N + (i ^ gram_tsw(i))], key_rho(ck[i]));
+        __syncwarp();
+        // this stripe's table rows, over this stripe's staged rows (rows r and
+        // r + 8 share the column swizzle)
+#pragma unroll
+        for (int nt = 0; nt < 8; nt++) {
+            if (nt < 2 * mt || nt >= nn) continue;
+            const int r = 16 * mt + (lane >> 2), c = (8 * nt + 2 * (lane & 3)) ^ gram_tsw(r);
+            *reinterpret_cast<float2 *>(T + r * GRAM_N + c) = make_float2(acc[nt][0], acc[nt][1]);
+            *reinterpret_cast<float2 *>(T + (r + 8) * GRAM_N + c) = make_float2(acc[nt][2], acc[nt][3]);
+        }
         __syncwarp();
     }
+    for (int i = lane; i < n; i += 32) nr2[i] = make_float2(T[i * GRAM_N + (i ^ gram_tsw(i))], key_rho(ck[i]));
+    __syncwarp();
 }
 
 // RobustPrune on a Gram table: same rule and order as warp_prune.  First the
@@ -360,14 +276,13 @@ __device__ void warp_gram(const Dev &d, const u64 *ck, int n, char *buf, int row
 // greedy pass is a warp-uniform walk over a 64-bit alive mask (take the first
 // alive candidate, clear the ones it drops), and the kept candidates are
 // written out afterwards, a lane per candidate.
-template <bool MB>
 __device__ int warp_prune_gram(const Dev &d, const u64 *ck, int n, unsigned char *alive, u32 *out_id,
                                float *out_rho, Stage &st) {
     (void)alive;
     const int lane = lane_id();
     float *T;
     float2 *nr2;
-    warp_gram<MB>(d, ck, n, st.gram, st.gram_rows, st, T, nr2);
+    warp_gram(d, ck, n, st.gram, st.gram_rows, T, nr2);
     const float alpha2 = d.alpha2;
     const bool l2 = d.metric == 0;
     // (n_h - g) + (n_j - g): every intermediate stays as small as the result
@@ -429,122 +344,148 @@ __device__ int warp_prune_gram(const Dev &d, const u64 *ck, int n, unsigned char
     __syncwarp();
     return nout;
 }
-// RobustPrune on the tensor-core Gram for up to GRAM_NL candidates, with no
-// table in shared memory: the Gram is built in 16-row stripes, last stripe
-// first, so that by the time a stripe is converted the norms of every column
-// it reads are known (this stripe's diagonal, or a later stripe's).  Each
-// accumulator entry (i, j), j > i, becomes bit j of row i's domination mask
-// (alpha^2 * d(i, j) <= rho(j)); the four lanes of a quad hold the columns of
-// a row and OR their bits.  The greedy pass is the register walk of
-// warp_prune_gram over 128-bit masks.  Same distances as warp_prune_gram:
-// squared L2 as (G_ii - G_ij) + (G_jj - G_ij), inner product as 1 - G_ij.
-template <int NT>   // tiles of 8 columns: 8 (n <= 64) or 16 (n <= 128)
-__device__ int warp_prune_masks(const Dev &d, const u64 *ck, int n, u32 *out_id, float *out_rho, Stage &st) {
-    const int lane = lane_id();
-    const int rows = st.gram_rows;
-    __nv_bfloat16 *X = reinterpret_cast<__nv_bfloat16 *>(st.gram);
-    char *tail = st.gram + (size_t)rows * GRAM_RS_LG * 2;
-    float2 *nr2 = reinterpret_cast<float2 *>(tail);   // .x: the norms (.y unused here)
-    u64 *dom = reinterpret_cast<u64 *>(tail + (size_t)rows * 8);
-    const int nm = (n + 15) >> 4, nn = (n + 7) >> 3;
-    const int nkb = ((int)d.mp + 127) >> 7;
-    const u32 xs = smem_addr(X);
-    for (int mt = nm - 1; mt >= 0; mt--) {
-        float acc[NT][4];
+// ---------------------------------------------------------------------------
+// The cooperative Gram: the domination masks of up to GRAM_NL candidates with
+// rows of any length, by the block's four warps.  The first warp runs the
+// kernel; the others wait for its requests.  The rows are staged once, 128
+// columns at a time and the next block while this one is multiplied; the
+// upper triangle's 16-row stripes are split over the warps (stripes w and nm -
+// 1 - w together hold about as many tiles for every w) and their sums stay in
+// registers.  Each entry (i, j), j > i, then becomes bit j of row i's mask
+// (alpha^2 * d(i, j) <= rho(j)); squared L2 is (G_ii - G_ij) + (G_jj - G_ij),
+// inner product 1 - G_ij.  BLOCKSUM: each column block's products are summed
+// from zero and added to the total (the form of candidate lists of up to
+// GRAM_N), else one chain runs over all columns.
+// Bound by the row reads (L2) and the mma.sync chains.  A warp per item that
+// restaged every column block for each stripe, or kept its sums in shared
+// memory, held 5 warps per SM: 500 deletes of 768-d with R = 64 (32,000 pairs)
+// took 6.7 ms against 2.4, the offers of 500 inserts 2.3 against 1.5.
+// ---------------------------------------------------------------------------
+struct GramReq {
+    const u64 *ck;
+    int n;
+};
+__device__ __forceinline__ void coop_bar() { asm volatile("bar.sync 1, 128;" ::: "memory"); }   // 32 COOP_WARPS
+__device__ __forceinline__ char *gram_tail(char *buf, int rows, u32 mp) { return buf + gram_row_bytes((u32)rows, mp); }
+
+template <bool BLOCKSUM>
+__device__ __forceinline__ void gram_masks(const Dev &d, const u64 *ck, int n, char *buf, int rows) {
+    constexpr int T0 = BLOCKSUM ? 8 : 16, T1 = BLOCKSUM ? 1 : 8;   // tiles of a warp's first and second stripe
+    const int tid = threadIdx.x, warp = tid >> 5, lane = lane_id();
+    float2 *nr2 = reinterpret_cast<float2 *>(gram_tail(buf, rows, d.mp));   // .x: the norms, .y: rho
+    u64 *dom = reinterpret_cast<u64 *>(nr2 + rows);
+    const int nm = (n + 15) >> 4, nn = 2 * nm, nkb = ((int)d.mp + 127) >> 7;
+    // BLOCKSUM: at most four stripes, one a warp
+    const int s0 = warp, s1 = nm - 1 - warp;
+    const bool has0 = BLOCKSUM ? s0 < nm : s0 <= s1, has1 = !BLOCKSUM && s0 < s1;
+    const u32 blk = (u32)rows * GRAM_RS_CO * 2;
+    auto stage = [&](int kb) {
+        const u32 xs = smem_addr(buf) + (kb & 1) * blk;
+        const int c = tid & 15;
+        const bool in = 128 * kb + 8 * c < (int)d.mb;   // d.mb is a multiple of 8
+        for (int r = tid >> 4; r < n; r += 2 * COOP_WARPS) {
+            const u32 dst = xs + (u32)(r * GRAM_RS_CO * 2 + 16 * c);
+            if (in) cp_async16(dst, d.xb + (size_t)key_id(ck[r]) * d.mb + 128 * kb + 8 * c);
+            else asm volatile("st.shared.v4.u32 [%0], {%1, %1, %1, %1};" ::"r"(dst), "r"(0u) : "memory");
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    float a0[T0][4], a1[T1][4], t0[BLOCKSUM ? T0 : 1][4];
 #pragma unroll
-        for (int b = 0; b < NT; b++)
+    for (int t = 0; t < T0; t++)
 #pragma unroll
-            for (int c = 0; c < 4; c++) acc[b][c] = 0.f;
-        for (int kb = 0; kb < nkb; kb++) {
-            if (nkb > 1 || mt == nm - 1) {
-                // rows [r_lo, n) of columns [128 kb, 128 kb + 128): all rows once
-                // when one block covers the row, else those of this stripe on
-                const int r_lo = nkb > 1 ? 16 * mt : 0;
-                __syncwarp();
-                if (d.xb) {
-                    const int cols = min(128, (int)d.mb - 128 * kb);
-                    if (lane == 0) asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-                    if (cols < 128)
-                        for (int z = lane; z < (n - r_lo) * 64; z += 32) {
-                            const int r = r_lo + (z >> 6), c = (z & 63) * 2;
-                            if (c >= cols) *reinterpret_cast<u32 *>(X + (size_t)r * GRAM_RS_LG + c) = 0u;
-                        }
-                    const int nr = n - r_lo;
-                    if (lane == 0 && nr > 0) mbar_expect_tx(st.bar, (u32)(nr * cols * 2));
-                    __syncwarp();
-                    for (int r = r_lo + lane; r < n; r += 32)
-                        bulk_g2s(X + (size_t)r * GRAM_RS_LG, d.xb + (size_t)key_id(ck[r]) * d.mb + 128 * kb,
-                                 (u32)cols * 2, st.bar);
-                    if (nr > 0) {
-                        if (!mbar_wait(st.bar, st.phase, WAIT_LIMIT)) {
-                            st.timeout = true;
-                            mbar_wait(st.bar, st.phase, WAIT_LIMIT);   // let copies in flight land
-                        }
-                        st.phase ^= 1u;
-                    }
-                } else {
-                    const int col = 128 * kb + 4 * lane;
-                    for (int r = r_lo; r < n; r++) {
-                        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-                        if (col < (int)d.mp)
-                            v = *reinterpret_cast<const float4 *>(d.x + (size_t)key_id(ck[r]) * d.mp + col);
-                        *reinterpret_cast<uint2 *>(X + (size_t)r * GRAM_RS_LG + 4 * lane) =
-                            make_uint2(pack_bf16(v.x, v.y), pack_bf16(v.z, v.w));
-                    }
-                }
-                __syncwarp();
-            }
+        for (int c = 0; c < 4; c++) a0[t][c] = 0.f;
+#pragma unroll
+    for (int t = 0; t < T1; t++)
+#pragma unroll
+        for (int c = 0; c < 4; c++) a1[t][c] = 0.f;
+    if (tid < n) nr2[tid].y = key_rho(ck[tid]);
+    stage(0);
+    for (int kb = 0; kb < nkb; kb++) {
+        if (kb + 1 < nkb) {
+            stage(kb + 1);
+            asm volatile("cp.async.wait_group 1;" ::: "memory");
+        } else {
+            asm volatile("cp.async.wait_group 0;" ::: "memory");
+        }
+        coop_bar();
+        const u32 xs = smem_addr(buf) + (kb & 1) * blk;
+        // one stripe: tiles 2 mt + t, t < NT (two at a time), rows past n hold anything
+        auto stripe = [&](auto &acc, auto nt_c, int mt) {
+            constexpr int NT = decltype(nt_c)::value;
 #pragma unroll
             for (int ks = 0; ks < 8; ks++) {
-                u32 a0, a1, a2, a3;
-                const int ar = 16 * mt + (lane & 7) + 8 * ((lane >> 3) & 1);
-                const int ac = 16 * ks + 8 * (lane >> 4);
-                ldsm_x4(a0, a1, a2, a3, xs + (u32)((ar * GRAM_RS_LG + ac) * 2));
+                u32 x0, x1, x2, x3;
+                const int ar = 16 * mt + (lane & 7) + 8 * ((lane >> 3) & 1), ac = 16 * ks + 8 * (lane >> 4);
+                ldsm_x4(x0, x1, x2, x3, xs + (u32)((ar * GRAM_RS_CO + ac) * 2));
 #pragma unroll
-                for (int nt = 0; nt < NT; nt += 2) {
-                    if (nt < 2 * mt || nt >= nn) continue;
+                for (int t = 0; t < NT; t += 2) {
+                    if (2 * mt + t >= nn) continue;
                     u32 b0, b1, b2, b3;
-                    const int br = 8 * nt + (lane & 7) + 8 * (lane >> 4);
+                    const int br = 8 * (2 * mt + t) + (lane & 7) + 8 * (lane >> 4);
                     const int bc = 16 * ks + 8 * ((lane >> 3) & 1);
-                    ldsm_x4(b0, b1, b2, b3, xs + (u32)((br * GRAM_RS_LG + bc) * 2));
-                    mma_bf16_16816(acc[nt], a0, a1, a2, a3, b0, b1);
-                    mma_bf16_16816(acc[nt + 1], a0, a1, a2, a3, b2, b3);
+                    ldsm_x4(b0, b1, b2, b3, xs + (u32)((br * GRAM_RS_CO + bc) * 2));
+                    mma_bf16_16816(acc[t], x0, x1, x2, x3, b0, b1);
+                    mma_bf16_16816(acc[t + 1], x0, x1, x2, x3, b2, b3);
                 }
             }
-        }
-        // this stripe's diagonal: entry (r, r) sits in tile 2 mt (rows r0) or 2 mt + 1 (rows r0 + 8)
-        const int r0 = 16 * mt + (lane >> 2), r1 = r0 + 8, cq = 2 * (lane & 3);
-        {
-            float d0 = 0.f, d1 = 0.f;
+        };
+        if (BLOCKSUM) {
+            if (has0) {
 #pragma unroll
-            for (int nt = 0; nt < NT; nt++) {
-                if (nt == 2 * mt) d0 = cq == (lane >> 2) ? acc[nt][0] : acc[nt][1];
-                if (nt == 2 * mt + 1) d1 = cq == (lane >> 2) ? acc[nt][2] : acc[nt][3];
+                for (int t = 0; t < T0; t++)
+#pragma unroll
+                    for (int c = 0; c < 4; c++) t0[BLOCKSUM ? t : 0][c] = 0.f;
+                stripe(t0, std::integral_constant<int, BLOCKSUM ? T0 : 0>{}, s0);
+#pragma unroll
+                for (int t = 0; t < T0; t++)
+#pragma unroll
+                    for (int c = 0; c < 4; c++)
+                        a0[t][c] = kb == 0 ? t0[BLOCKSUM ? t : 0][c] : __fadd_rn(a0[t][c], t0[BLOCKSUM ? t : 0][c]);
             }
-            const bool own = cq == (lane >> 2) || cq + 1 == (lane >> 2);
-            if (own && r0 < n) nr2[r0].x = d0;
-            if (own && r1 < n) nr2[r1].x = d1;
+        } else {
+            if (has0) stripe(a0, std::integral_constant<int, T0>{}, s0);
+            if (has1) stripe(a1, std::integral_constant<int, BLOCKSUM ? 0 : T1>{}, s1);
         }
-        __syncwarp();
+        coop_bar();   // this half is read
+    }
+    // the diagonal: entry (r, r) sits in tile 2 mt (rows r0) or 2 mt + 1 (rows r0 + 8)
+    const int cq = 2 * (lane & 3), rq = lane >> 2;
+    auto diag = [&](auto &acc, int mt) {
+        const int r0 = 16 * mt + rq, r1 = r0 + 8;
+        if (cq == rq || cq + 1 == rq) {
+            if (r0 < n) nr2[r0].x = cq == rq ? acc[0][0] : acc[0][1];
+            if (r1 < n) nr2[r1].x = cq == rq ? acc[1][2] : acc[1][3];
+        }
+    };
+    if (has0) diag(a0, s0);
+    if constexpr (!BLOCKSUM)
+        if (has1) diag(a1, s1);
+    coop_bar();
+    auto masks = [&](auto &acc, auto nt_c, int mt) {
+        constexpr int NT = decltype(nt_c)::value;
+        const int r0 = 16 * mt + rq, r1 = r0 + 8;
         const float n0 = r0 < n ? nr2[r0].x : 0.f, n1 = r1 < n ? nr2[r1].x : 0.f;
         u64 m0l = 0, m0h = 0, m1l = 0, m1h = 0;
 #pragma unroll
-        for (int nt = 0; nt < NT; nt++) {
-            const bool tile = nt >= 2 * mt && nt < nn;
+        for (int t = 0; t < NT; t++) {
+            const int nt = 2 * mt + t;
+            if (nt >= nn) continue;
 #pragma unroll
-            for (int e = 0; e < 4; e++) {
-                const int r = e < 2 ? r0 : r1, c = 8 * nt + cq + (e & 1);
-                const bool ok = tile && c > r && c < n;   // c < n implies r < n
-                const int cc = ok ? c : 0;
-                const float g = acc[nt][e];
-                const float nr_ = e < 2 ? n0 : n1;
-                const float dd = d.metric == 0 ? __fadd_rn(__fsub_rn(nr_, g), __fsub_rn(nr2[cc].x, g)) : __fsub_rn(1.0f, g);
-                const bool hit = ok && __fmul_rn(d.alpha2, dd) <= key_rho(ck[cc]);
-                const u64 bit = hit ? 1ull << (c & 63) : 0ull;
-                if (e < 2) { if (8 * nt < 64) m0l |= bit; else m0h |= bit; }
-                else { if (8 * nt < 64) m1l |= bit; else m1h |= bit; }
+            for (int h = 0; h < 2; h++) {
+                const int c = 8 * nt + cq + h;
+                if (c >= n) continue;
+                const float2 v = nr2[c];
+                auto hit = [&](float nr, float g) {
+                    const float dd = d.metric == 0 ? __fadd_rn(__fsub_rn(nr, g), __fsub_rn(v.x, g)) : __fsub_rn(1.0f, g);
+                    return __fmul_rn(d.alpha2, dd) <= v.y;
+                };
+                const u64 bit = 1ull << (c & 63);
+                if (c > r0 && hit(n0, acc[t][h])) { if (c < 64) m0l |= bit; else m0h |= bit; }
+                if (c > r1 && hit(n1, acc[t][2 + h])) { if (c < 64) m1l |= bit; else m1h |= bit; }
             }
         }
+        // the four lanes of a quad hold the columns of a row
 #pragma unroll
         for (int o = 1; o <= 2; o <<= 1) {
             m0l |= __shfl_xor_sync(FULL, m0l, o);
@@ -556,8 +497,42 @@ __device__ int warp_prune_masks(const Dev &d, const u64 *ck, int n, u32 *out_id,
             if (r0 < n) { dom[2 * r0] = m0l; dom[2 * r0 + 1] = m0h; }
             if (r1 < n) { dom[2 * r1] = m1l; dom[2 * r1 + 1] = m1h; }
         }
-        __syncwarp();
+    };
+    if (has0) masks(a0, std::integral_constant<int, T0>{}, s0);
+    if constexpr (!BLOCKSUM)
+        if (has1) masks(a1, std::integral_constant<int, T1>{}, s1);
+    coop_bar();
+}
+
+// The helper warps of a block: serve requests until one has n < 0.
+template <int GV>
+__device__ __noinline__ void gram_helper(const Dev d, char *buf, int rows, const GramReq *req) {
+    for (;;) {
+        coop_bar();
+        const int n = *reinterpret_cast<const volatile int *>(&req->n);
+        if (n < 0) return;
+        gram_masks<GV == 2>(d, *reinterpret_cast<const u64 *const volatile *>(&req->ck), n, buf, rows);
     }
+}
+__device__ __forceinline__ void gram_release(GramReq *req) {
+    if (lane_id() == 0) req->n = -1;
+    __syncwarp();
+    coop_bar();
+}
+
+// RobustPrune from the masks (first warp): a walk over a 128-bit alive mask.
+template <int GV>
+__device__ int warp_prune_masks(const Dev &d, const u64 *ck, int n, u32 *out_id, float *out_rho, Stage &st) {
+    const int lane = lane_id();
+    __syncwarp();
+    if (lane == 0) {
+        st.req->ck = ck;
+        st.req->n = n;
+    }
+    __syncwarp();
+    coop_bar();
+    gram_masks<GV == 2>(d, ck, n, st.gram, st.gram_rows);
+    const u64 *dom = reinterpret_cast<const u64 *>(gram_tail(st.gram, st.gram_rows, d.mp) + (size_t)st.gram_rows * 8);
     // equal adjacent keys collapse to one
     u64 lo = 0, hi = 0;
     for (int i0 = 0; i0 < n; i0 += 32) {
@@ -592,15 +567,15 @@ __device__ int warp_prune_masks(const Dev &d, const u64 *ck, int n, u32 *out_id,
 // Scratch: alive[n], idx[n].
 // ---------------------------------------------------------------------------
 // GV, the Gram variant of a kernel: 0, a buffer of at most GRAM_N rows with
-// rows of one 128-column block; 1, more than GRAM_N rows (the large path,
-// which restages each block per stripe); 2, at most GRAM_N rows spanning
-// several blocks (partial sums kept between blocks).
+// rows of one 128-column block, a warp per item; 1, more than GRAM_N rows, and
+// 2, at most GRAM_N rows spanning several blocks: the block's four warps on one
+// item (see gram_masks).
 template <int GV>
 __device__ int warp_prune(const Dev &d, const u64 *ck, int n, unsigned char *alive, u32 *idx, u32 *out_id,
                           float *out_rho, Stage &st) {
     if (st.gram && n <= st.gram_rows) {
-        if constexpr (GV == 1) return warp_prune_masks<GRAM_NL / 8>(d, ck, n, out_id, out_rho, st);
-        else return warp_prune_gram<GV == 2>(d, ck, n, alive, out_id, out_rho, st);
+        if constexpr (GV != 0) return warp_prune_masks<GV>(d, ck, n, out_id, out_rho, st);
+        else return warp_prune_gram(d, ck, n, alive, out_id, out_rho, st);
     }
     const int lane = lane_id();
     const int grp = lane >> 3, g = lane & 7;
@@ -787,18 +762,20 @@ __host__ __device__ inline size_t prune_ins_warp_bytes(u32 np, u32 R, u32 ns, u3
     return stage_bytes(ns, mp) + al16((size_t)np * 8) + (gram_alias(gram, sc) ? 0 : sc) + gram_bytes(gram, mp);
 }
 
-// one-warp blocks (the launch uses 32 threads); the small-path instantiation
-// is held to 12 resident warps per SM (at most 170 registers a thread)
+// one-warp blocks of the single-warp variant (GV 0) are held to 12 resident warps
+// per SM (at most 170 registers a thread)
 template <int GV>
-__global__ void __launch_bounds__(32, GV == 1 ? 1 : 12) prune_insert_kernel(PruneInsArgs a) {
+__global__ void __launch_bounds__(GV ? 32 * COOP_WARPS : 32, GV ? 3 : 12) prune_insert_kernel(PruneInsArgs a) {
     extern __shared__ __align__(16) char smem[];
-    const int warp = threadIdx.x >> 5, lane = lane_id();
+    __shared__ GramReq req;
+    const int lane = lane_id();
     const Dev &d = a.d;
     const u32 R = d.R;
-    char *p = smem + warp * prune_ins_warp_bytes(a.np, R, a.ns, d.mp, a.gram);
+    char *p = smem;
     char *gbuf = a.gram ? p : nullptr;
+    if (GV != 0 && threadIdx.x >= 32) return gram_helper<GV>(d, gbuf, (int)a.gram, &req);
     p += gram_bytes(a.gram, d.mp);
-    Stage st = stage_init(p, a.ns, d.mp, gbuf, a.gram);
+    Stage st = stage_init(p, a.ns, d.mp, gbuf, a.gram, &req);
     WarpSlabs ws;
     ws_init(ws);
     p += stage_bytes(a.ns, d.mp);
@@ -825,13 +802,15 @@ __global__ void __launch_bounds__(32, GV == 1 ? 1 : 12) prune_insert_kernel(Prun
             // re-scored with the canonical fp32 distance to v and re-sorted,
             // so that RobustPrune and every stored rho see exact distances
             const float *xv = d.x + (size_t)v * d.mp;
-            const int grp = lane >> 3, g = lane & 7;
+            const float one[4] = {1.0f, 1.0f, 1.0f, 1.0f};
             for (int r0 = 0; r0 < n; r0 += 4) {
-                const int c = min(r0 + grp, n - 1);
-                const u32 id = key_id(keys[c]);
-                const float dist = canon_dist<8>(xv, d.x + (size_t)id * d.mp, (int)d.mp, (int)d.metric, g);
+                const void *row[4];
+#pragma unroll
+                for (int c = 0; c < 4; c++) row[c] = d.x + (size_t)key_id(keys[min(r0 + c, n - 1)]) * d.mp;
+                const float dist = warp_dists<0, 4, 2>(xv, row, one, (int)d.mp, (int)d.metric);
+                const int i = r0 + (lane >> 3);
                 __syncwarp();
-                if (r0 + grp < n && g == 0) keys[c] = mkkey(dist, id);
+                if (i < n && (lane & 7) == 0) keys[i] = mkkey(dist, key_id(keys[i]));
                 __syncwarp();
             }
             for (u32 i = n + lane; i < a.np; i += 32) keys[i] = KEY_INF;
@@ -861,6 +840,7 @@ __global__ void __launch_bounds__(32, GV == 1 ? 1 : 12) prune_insert_kernel(Prun
         if (lane == 0) a.F_n[t] = (u32)nout;
         __syncwarp();
     }
+    if (GV != 0) gram_release(&req);
     ws_finish(d, ws);
     stage_done(d, st, WK_PRUNE);
 }
@@ -878,23 +858,23 @@ cudaError_t launch_prune_insert(const Dev &d, u32 first, u32 b, const u64 *exp_k
     a.np = np;
     a.ns = gram ? 0 : stage_cap(d.mp, max_cand, d.stage_bytes);
     const size_t wb = prune_ins_warp_bytes(np, d.R, a.ns, d.mp, gram);
-    const int W = warps_for(wb);
-    size_t smem = W * wb;
+    const size_t smem = wb;
+    const int threads = block_threads(a.gram, d.mp);
     const void *fns[3] = {(const void *)prune_insert_kernel<0>, (const void *)prune_insert_kernel<1>, (const void *)prune_insert_kernel<2>};
     const void *fn = fns[gram_variant(a.gram, d.mp)];
     cudaError_t e = smem_at_least((const void *)fn, smem);
     if (e != cudaSuccess) return e;
     int per_sm = 0;
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-        &per_sm, fn, 32 * W, smem);
+        &per_sm, fn, threads, smem);
     if (e != cudaSuccess) return e;
     if (per_sm < 1) return cudaErrorInvalidConfiguration;
-    u32 blocks = (u32)(per_sm * num_sms), need = (b + W - 1) / W;
+    u32 blocks = (u32)(per_sm * num_sms), need = b;
     if (blocks > need) blocks = need;
     e = cudaMemsetAsync(d.ctr + C_WORK, 0, sizeof(u64), st);
     if (e != cudaSuccess) return e;
     void *args[] = {&a};
-    e = cudaLaunchKernel(fn, dim3(blocks), dim3(32 * W), args, smem, st);
+    e = cudaLaunchKernel(fn, dim3(blocks), dim3(threads), args, smem, st);
     if (e != cudaSuccess) return e;
     return cudaGetLastError();
 }
@@ -924,18 +904,20 @@ __host__ __device__ inline size_t fold_warp_bytes(u32 np, u32 R, u32 ns, u32 mp,
            (gram_alias(gram, sc) ? 0 : sc) + gram_bytes(gram, mp);
 }
 
-// one-warp blocks (the launch uses 32 threads); the small-path instantiation
-// is held to 12 resident warps per SM (at most 170 registers a thread)
+// one-warp blocks of the single-warp variant (GV 0) are held to 12 resident warps
+// per SM (at most 170 registers a thread)
 template <int GV>
-__global__ void __launch_bounds__(32, GV == 1 ? 1 : 12) offer_fold_kernel(FoldArgs a) {
+__global__ void __launch_bounds__(GV ? 32 * COOP_WARPS : 32, GV ? 3 : 12) offer_fold_kernel(FoldArgs a) {
     extern __shared__ __align__(16) char smem[];
-    const int warp = threadIdx.x >> 5, lane = lane_id();
+    __shared__ GramReq req;
+    const int lane = lane_id();
     const Dev &d = a.d;
     const u32 R = d.R;
-    char *p = smem + warp * fold_warp_bytes(a.np, R, a.ns, d.mp, a.gram);
+    char *p = smem;
     char *gbuf = a.gram ? p : nullptr;
+    if (GV != 0 && threadIdx.x >= 32) return gram_helper<GV>(d, gbuf, (int)a.gram, &req);
     p += gram_bytes(a.gram, d.mp);
-    Stage st = stage_init(p, a.ns, d.mp, gbuf, a.gram);
+    Stage st = stage_init(p, a.ns, d.mp, gbuf, a.gram, &req);
     WarpSlabs ws;
     ws_init(ws);
     p += stage_bytes(a.ns, d.mp);
@@ -1010,6 +992,7 @@ __global__ void __launch_bounds__(32, GV == 1 ? 1 : 12) offer_fold_kernel(FoldAr
         }
         __syncwarp();
     }
+    if (GV != 0) gram_release(&req);
     ws_finish(d, ws);
     stage_done(d, st, WK_OFFER);
 }
@@ -1025,24 +1008,24 @@ cudaError_t launch_offer_fold(const Dev &d, const Offers &of, const u32 *seg_sta
     a.np = np;
     a.ns = d.gram ? 0 : stage_cap(d.mp, d.R + 1, d.stage_bytes);
     const size_t wb = fold_warp_bytes(np, d.R, a.ns, d.mp, a.gram);
-    const int W = warps_for(wb);
-    size_t smem = W * wb;
+    const size_t smem = wb;
+    const int threads = block_threads(a.gram, d.mp);
     const void *fns[3] = {(const void *)offer_fold_kernel<0>, (const void *)offer_fold_kernel<1>, (const void *)offer_fold_kernel<2>};
     const void *fn = fns[gram_variant(a.gram, d.mp)];
     cudaError_t e = smem_at_least((const void *)fn, smem);
     if (e != cudaSuccess) return e;
     int per_sm = 0;
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-        &per_sm, fn, 32 * W, smem);
+        &per_sm, fn, threads, smem);
     if (e != cudaSuccess) return e;
     if (per_sm < 1) return cudaErrorInvalidConfiguration;
     const u32 items = budget ? a.hi - a.lo : of.n;
-    u32 blocks = (u32)(per_sm * num_sms), need = (items + W - 1) / W;
+    u32 blocks = (u32)(per_sm * num_sms), need = items;
     if (blocks > need) blocks = need;
     e = cudaMemsetAsync(d.ctr + C_WORK, 0, sizeof(u64), st);
     if (e != cudaSuccess) return e;
     void *args[] = {&a};
-    e = cudaLaunchKernel(fn, dim3(blocks), dim3(32 * W), args, smem, st);
+    e = cudaLaunchKernel(fn, dim3(blocks), dim3(threads), args, smem, st);
     if (e != cudaSuccess) return e;
     return cudaGetLastError();
 }
@@ -1072,15 +1055,17 @@ __host__ __device__ inline size_t refine_warp_bytes(u32 np, u32 cap, u32 R, u32 
 }
 
 template <int GV>
-__global__ void __launch_bounds__(64, GV == 1 ? 1 : 6) refine_kernel(RefineArgs a) {
+__global__ void __launch_bounds__(GV ? 32 * COOP_WARPS : 64, GV ? 3 : 6) refine_kernel(RefineArgs a) {
     extern __shared__ __align__(16) char smem[];
+    __shared__ GramReq req;
     const int warp = threadIdx.x >> 5, lane = lane_id();
     const Dev &d = a.d;
     const u32 R = d.R;
-    char *p = smem + warp * refine_warp_bytes(a.np_s, a.cap_s, R, a.ns, d.mp, a.gram);
+    char *p = smem + (GV ? 0 : warp) * refine_warp_bytes(a.np_s, a.cap_s, R, a.ns, d.mp, a.gram);
     char *gbuf = a.gram ? p : nullptr;
+    if (GV != 0 && warp) return gram_helper<GV>(d, gbuf, (int)a.gram, &req);
     p += gram_bytes(a.gram, d.mp);
-    Stage st = stage_init(p, a.ns, d.mp, gbuf, a.gram);
+    Stage st = stage_init(p, a.ns, d.mp, gbuf, a.gram, &req);
     WarpSlabs ws;
     ws_init(ws);
     p += stage_bytes(a.ns, d.mp);
@@ -1098,7 +1083,7 @@ __global__ void __launch_bounds__(64, GV == 1 ? 1 : 6) refine_kernel(RefineArgs 
         return l;
     };
     const auto ls = carve_lists(p, a.np_s);
-    const auto lg = carve_lists(a.spill + (blockIdx.x * (blockDim.x >> 5) + warp) * a.spill_warp, a.np);
+    const auto lg = carve_lists(a.spill + (GV ? blockIdx.x : blockIdx.x * (blockDim.x >> 5) + warp) * a.spill_warp, a.np);
     const int grp = lane >> 3, g = lane & 7;
     u32 t_next = 0;   // the next item's claim, in flight while this one runs
     if (lane == 0) t_next = (u32)atomicAdd(&d.ctr[C_WORK], 1ull);
@@ -1255,6 +1240,7 @@ __global__ void __launch_bounds__(64, GV == 1 ? 1 : 6) refine_kernel(RefineArgs 
         }
         __syncwarp();
     }
+    if (GV != 0) gram_release(&req);
     ws_finish(d, ws);
     stage_done(d, st, WK_REFINE);
 }
@@ -1291,7 +1277,9 @@ cudaError_t launch_refine(const Dev &d, u32 first, u32 b, u32 mode, u32 max_cand
     refine_shape(d, max_cand, a);
     a.spill = spill;
     const size_t wb = refine_warp_bytes(a.np_s, a.cap_s, d.R, a.ns, d.mp, a.gram);
-    const int warps = 2 * wb <= 200 * 1024 ? 2 : 1;
+    const bool coop = gram_variant(a.gram, d.mp) != 0;
+    const int warps = !coop && 2 * wb <= 200 * 1024 ? 2 : 1;   // items of a block
+    const int threads = coop ? 32 * COOP_WARPS : 32 * warps;
     size_t smem = warps * wb;
     const void *fns[3] = {(const void *)refine_kernel<0>, (const void *)refine_kernel<1>, (const void *)refine_kernel<2>};
     const void *fn = fns[gram_variant(a.gram, d.mp)];
@@ -1299,7 +1287,7 @@ cudaError_t launch_refine(const Dev &d, u32 first, u32 b, u32 mode, u32 max_cand
     if (e != cudaSuccess) return e;
     int per_sm = 0;
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-        &per_sm, fn, 32 * warps, smem);
+        &per_sm, fn, threads, smem);
     if (e != cudaSuccess) return e;
     if (per_sm < 1) return cudaErrorInvalidConfiguration;
     u32 blocks = (u32)(per_sm * num_sms), need = (b + warps - 1) / warps;
@@ -1308,7 +1296,7 @@ cudaError_t launch_refine(const Dev &d, u32 first, u32 b, u32 mode, u32 max_cand
     e = cudaMemsetAsync(d.ctr + C_WORK, 0, sizeof(u64), st);
     if (e != cudaSuccess) return e;
     void *args[] = {&a};
-    e = cudaLaunchKernel(fn, dim3(blocks), dim3(32 * warps), args, smem, st);
+    e = cudaLaunchKernel(fn, dim3(blocks), dim3(threads), args, smem, st);
     if (e != cudaSuccess) return e;
     return cudaGetLastError();
 }
@@ -1674,18 +1662,20 @@ __device__ int repair_apply(const Dev &d, u32 *lid, float *lrho, int n, u32 u, c
     return nout;
 }
 
-// one-warp blocks (the launch uses 32 threads); the small-path instantiation
-// is held to 12 resident warps per SM (at most 170 registers a thread)
+// one-warp blocks of the single-warp variant (GV 0) are held to 12 resident warps
+// per SM (at most 170 registers a thread)
 template <int GV>
-__global__ void __launch_bounds__(32, GV == 1 ? 1 : 12) repair_fold_kernel(RepairFoldArgs a) {
+__global__ void __launch_bounds__(GV ? 32 * COOP_WARPS : 32, GV ? 3 : 12) repair_fold_kernel(RepairFoldArgs a) {
     extern __shared__ __align__(16) char smem[];
-    const int warp = threadIdx.x >> 5, lane = lane_id();
+    __shared__ GramReq req;
+    const int lane = lane_id();
     const Dev &d = a.d;
     const u32 R = d.R;
-    char *p = smem + warp * repf_warp_bytes(a.np, R, a.ns, d.mp, a.gram);
+    char *p = smem;
     char *gbuf = a.gram ? p : nullptr;
+    if (GV != 0 && threadIdx.x >= 32) return gram_helper<GV>(d, gbuf, (int)a.gram, &req);
     p += gram_bytes(a.gram, d.mp);
-    Stage st = stage_init(p, a.ns, d.mp, gbuf, a.gram);
+    Stage st = stage_init(p, a.ns, d.mp, gbuf, a.gram, &req);
     WarpSlabs ws;
     ws_init(ws);
     p += stage_bytes(a.ns, d.mp);
@@ -1761,6 +1751,7 @@ __global__ void __launch_bounds__(32, GV == 1 ? 1 : 12) repair_fold_kernel(Repai
         }
         __syncwarp();
     }
+    if (GV != 0) gram_release(&req);
     ws_finish(d, ws);
     stage_done(d, st, WK_REPAIR_FOLD);
 }
@@ -1777,24 +1768,24 @@ cudaError_t launch_repair_fold(const Dev &d, const u32 *dt, const u32 *pair_key,
     a.np = np;
     a.ns = d.gram ? 0 : stage_cap(d.mp, 2 * d.R, d.stage_bytes);
     const size_t wb = repf_warp_bytes(np, d.R, a.ns, d.mp, a.gram);
-    const int W = warps_for(wb);
-    size_t smem = W * wb;
+    const size_t smem = wb;
+    const int threads = block_threads(a.gram, d.mp);
     const void *fns[3] = {(const void *)repair_fold_kernel<0>, (const void *)repair_fold_kernel<1>, (const void *)repair_fold_kernel<2>};
     const void *fn = fns[gram_variant(a.gram, d.mp)];
     cudaError_t e = smem_at_least((const void *)fn, smem);
     if (e != cudaSuccess) return e;
     int per_sm = 0;
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-        &per_sm, fn, 32 * W, smem);
+        &per_sm, fn, threads, smem);
     if (e != cudaSuccess) return e;
     if (per_sm < 1) return cudaErrorInvalidConfiguration;
-    u64 need = (n_pairs + W - 1) / W;
+    const u64 need = n_pairs;
     u32 blocks = (u32)(per_sm * num_sms);
     if ((u64)blocks > need) blocks = (u32)need;
     e = cudaMemsetAsync(d.ctr + C_WORK, 0, sizeof(u64), st);
     if (e != cudaSuccess) return e;
     void *args[] = {&a};
-    e = cudaLaunchKernel(fn, dim3(blocks), dim3(32 * W), args, smem, st);
+    e = cudaLaunchKernel(fn, dim3(blocks), dim3(threads), args, smem, st);
     if (e != cudaSuccess) return e;
     return cudaGetLastError();
 }

@@ -92,6 +92,7 @@ struct etale_index {
     float *x8s = nullptr;
     u32 mb = 0, m8 = 0;
     u32 search_prec = 0;
+    bool loaded = false;            // lists came from a file (see Dev::same_tests)
     u32 insert_prec = 0;            // precision of the insert BeamSearch gathers
     bool rows_exact = true;         // every ingested row's bf16 copy is exact (C_INEXACT == 0)
     u32 *nent_dev = nullptr;        // |E| in device memory
@@ -160,6 +161,7 @@ struct etale_index {
         d.entries = entries; d.dim = dim; d.mp = mp; d.R = R; d.metric = metric; d.alpha2 = alpha2;
         d.n_entries = n_entries.load(std::memory_order_relaxed); d.capacity = capacity; d.pool = pool; d.stage_bytes = cfg.stage_kb << 10;
         d.gram = cfg.gram == 2 ? 1u : 0u;
+        d.same_tests = !loaded && d.gram == 0 ? 1u : 0u;
         d.xb = xb; d.xbn = xbn; d.x8 = x8; d.x8s = x8s; d.mb = mb; d.m8 = m8;
         // warps pop 8 free slabs at a time when the free pool covers every
         // resident warp's batch many times over (else one, as Algorithm 1)
@@ -2452,6 +2454,7 @@ etale_status etale_load(const char *path, const etale_config *cfg_in, uint64_t c
         return e;
     };
     if (ne > idx->cfg.n_entry) return fail(ETALE_EINVAL, "saved entry set larger than n_entry");
+    idx->loaded = n > 0;
     std::vector<float> xh;
     for (u64 lo = 0; lo < n; lo += SNAP_CHUNK) {
         const u64 c = std::min(SNAP_CHUNK, n - lo);

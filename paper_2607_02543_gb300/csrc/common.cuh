@@ -123,6 +123,9 @@ struct Dev {
     u64 capacity, pool;
     u32 stage_bytes;   // per-warp RobustPrune row stage (0: rows read from L2)
     u32 gram;          // 1: domination tests of small prunes use the tensor-core Gram tile
+    u32 same_tests;    // 1: every list was pruned here, by canonical distances and this alpha: a pruned
+                       // list's entries (ref_pruned) need no test among themselves.  0 with the Gram and
+                       // for lists of a file, which may come from prunes under other settings
     // reduced-precision copies (query search only)
     unsigned short *xb;  // C x mb bf16 bits (nullptr if not kept)
     float *xbn;          // C: |bf16 row|^2, for the tensor-core keys of BF16 searches

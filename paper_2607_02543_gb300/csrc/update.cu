@@ -29,6 +29,7 @@ struct Stage {
     u32 phase;
     bool timeout;
     char *gram;      // gram_bytes(gram_rows, mp) for the tensor-core Gram path (nullptr: canonical path)
+    u32 gram_tag;    // its rows as the launch gave them (CANON_ROWS: variant 3)
     int gram_rows;   // candidates the Gram buffer holds (a multiple of 16, <= GRAM_NL)
     struct GramReq *req;     // the block's request slot (cooperative variants)
     u64 wk_rows, wk_state;   // this warp's work tallies (see WK_*), added by stage_done
@@ -50,16 +51,20 @@ constexpr int COOP_WARPS = 4;
 __host__ __device__ inline u32 gram_xoff(int r, int chunk) { return (u32)(r * GRAM_RB + ((chunk ^ (r & 7)) << 4)); }
 // The Gram variant (see warp_prune) of a kernel whose buffer holds gram_rows rows of mp columns.
 __host__ __device__ inline int gram_variant(u32 gram_rows, u32 mp) {
-    return gram_rows > (u32)GRAM_N ? 1 : (gram_rows && mp > 128 ? 2 : 0);
+    return gram_rows >> 31 ? 3 : gram_rows > (u32)GRAM_N ? 1 : (gram_rows && mp > 128 ? 2 : 0);
 }
+// Variant 3, canonical distances on the cooperative path, keeps masks only: its
+// buffer is that of CANON_ROWS "rows".
+constexpr u32 CANON_ROWS = 0x80000000u | GRAM_NL;
 // Bytes of a Gram buffer's rows (or the table over them), and of the whole
 // buffer: a (norm, rho) pair per candidate follows, and on the cooperative path
 // its domination mask (two words).  rows is a multiple of 16; 0 = no buffer.
 __host__ __device__ inline size_t gram_row_bytes(u32 rows, u32 mp) {
+    if (rows >> 31) return 0;
     return gram_variant(rows, mp) ? (size_t)(mp > 128 ? 2 : 1) * rows * GRAM_RS_CO * 2 : (size_t)rows * GRAM_RB;
 }
 __host__ __device__ inline size_t gram_bytes(u32 rows, u32 mp) {
-    return gram_row_bytes(rows, mp) + (size_t)rows * (gram_variant(rows, mp) ? 8 + 16 : 8);
+    return gram_row_bytes(rows, mp) + (size_t)(rows & 0x7FFFFFFFu) * (gram_variant(rows, mp) ? 8 + 16 : 8);
 }
 // Gram rows for a kernel whose prunes see at most max_n candidates (0: the
 // Gram path is off or cannot hold them).
@@ -67,7 +72,7 @@ inline u32 gram_rows_for(u32 on, u32 max_n) { return on && max_n <= (u32)GRAM_NL
 // Scratch that is dead whenever the Gram buffer is live (list compaction before
 // a prune, the canonical prune's arrays, a prune's output, written after its
 // last read of the buffer) lives inside the Gram buffer's row bytes if it fits.
-__host__ __device__ inline bool gram_alias(u32 gram, size_t scratch) { return gram && scratch <= (size_t)gram * GRAM_RB; }
+__host__ __device__ inline bool gram_alias(u32 gram, size_t scratch) { return gram && !(gram >> 31) && scratch <= (size_t)gram * GRAM_RB; }
 
 // Shared-memory bytes for a stage of ns rows plus its mbarrier.
 __host__ __device__ inline size_t stage_bytes(u32 ns, u32 mp) { return al16((size_t)ns * mp * 4) + 16; }
@@ -82,7 +87,8 @@ __device__ __forceinline__ Stage stage_init(char *p, u32 ns, u32 mp, char *gram 
     st.phase = 0;
     st.timeout = false;
     st.gram = gram;
-    st.gram_rows = (int)gram_rows;
+    st.gram_tag = gram_rows;
+    st.gram_rows = (int)(gram_rows & 0x7FFFFFFFu);
     st.req = req;
     st.wk_rows = st.wk_state = 0;
     if (lane_id() == 0) mbar_init(st.bar, 1);
@@ -100,7 +106,7 @@ __device__ __forceinline__ void stage_done(const Dev &d, const Stage &st, int ki
 // Row bytes a prune of n candidates gathers: the bf16 copy on the Gram path
 // when the index keeps one, else the fp32 rows.
 __device__ __forceinline__ u64 prune_row_bytes(const Dev &d, const Stage &st, int n) {
-    const bool b16 = st.gram && n <= st.gram_rows && d.xb;
+    const bool b16 = st.gram && !(st.gram_tag >> 31) && n <= st.gram_rows && d.xb;
     return (u64)n * (b16 ? 2ull * d.mb : 4ull * d.mp);
 }
 
@@ -366,10 +372,11 @@ struct GramReq {
     int n;
 };
 __device__ __forceinline__ void coop_bar() { asm volatile("bar.sync 1, 128;" ::: "memory"); }   // 32 COOP_WARPS
-__device__ __forceinline__ char *gram_tail(char *buf, int rows, u32 mp) { return buf + gram_row_bytes((u32)rows, mp); }
+// The (norm, rho) pairs and masks of a buffer of `rows` candidates.
+__device__ __forceinline__ char *gram_tail(char *buf, u32 rows, u32 mp) { return buf + gram_row_bytes(rows, mp); }
 
 template <bool BLOCKSUM>
-__device__ __forceinline__ void gram_masks(const Dev &d, const u64 *ck, int n, char *buf, int rows) {
+__device__ __forceinline__ void gram_masks(const Dev &d, const u64 *ck, int n, char *buf, u32 rows) {
     constexpr int T0 = BLOCKSUM ? 8 : 16, T1 = BLOCKSUM ? 1 : 8;   // tiles of a warp's first and second stripe
     const int tid = threadIdx.x, warp = tid >> 5, lane = lane_id();
     float2 *nr2 = reinterpret_cast<float2 *>(gram_tail(buf, rows, d.mp));   // .x: the norms, .y: rho
@@ -504,14 +511,113 @@ __device__ __forceinline__ void gram_masks(const Dev &d, const u64 *ck, int n, c
     coop_bar();
 }
 
+// The canonical sums of 64 values a lane holds as partials (value p in v[p]):
+// the tree of canon_dist over the 32 lanes, where at each level a lane keeps
+// half of the values it still has and passes the other half on.  Lane l ends
+// with values 2 l and 2 l + 1 in v[0] and v[1].
+__device__ __forceinline__ void warp_tree64(float (&v)[64]) {
+    const int lane = lane_id();
+#pragma unroll
+    for (int h = 16, n = 32; h >= 1; h >>= 1, n >>= 1) {
+        const bool up = lane & h;
+#pragma unroll
+        for (int i = 0; i < n; i++)
+            v[i] = __fadd_rn(up ? v[i + n] : v[i], __shfl_xor_sync(FULL, up ? v[i] : v[i + n], h));
+    }
+}
+
+// Canonical distances of the 64 pairs of 8 rows and 8 rows, by one warp: lane j
+// sums partial j of every pair.  Lane l returns pairs 2 l and 2 l + 1 (pair 8 i
+// + j: rows xr[i], yr[j]).
+__device__ __forceinline__ void pair_tile(u32 mp, u32 metric, const float *const (&xr)[8], const float *const (&yr)[8],
+                                          float (&dd)[2]) {
+    float acc[64];
+#pragma unroll
+    for (int q = 0; q < 64; q++) acc[q] = 0.0f;
+    for (u32 e = 4 * lane_id(); e < mp; e += 128) {
+        float4 x[8], y[8];
+#pragma unroll
+        for (int c = 0; c < 8; c++) {
+            x[c] = *reinterpret_cast<const float4 *>(xr[c] + e);
+            y[c] = *reinterpret_cast<const float4 *>(yr[c] + e);
+        }
+        if (metric == 0) {
+#pragma unroll
+            for (int q = 0; q < 64; q++) {
+                const float4 u = x[q >> 3], v = y[q & 7];
+                const float d0 = __fsub_rn(u.x, v.x), d1 = __fsub_rn(u.y, v.y);
+                const float d2 = __fsub_rn(u.z, v.z), d3 = __fsub_rn(u.w, v.w);
+                acc[q] = __fmaf_rn(d3, d3, __fmaf_rn(d2, d2, __fmaf_rn(d1, d1, __fmaf_rn(d0, d0, acc[q]))));
+            }
+        } else {
+#pragma unroll
+            for (int q = 0; q < 64; q++) {
+                const float4 u = x[q >> 3], v = y[q & 7];
+                acc[q] = __fmaf_rn(u.w, v.w, __fmaf_rn(u.z, v.z, __fmaf_rn(u.y, v.y, __fmaf_rn(u.x, v.x, acc[q]))));
+            }
+        }
+    }
+    __syncwarp();
+    warp_tree64(acc);
+#pragma unroll
+    for (int k = 0; k < 2; k++) dd[k] = metric == 0 ? acc[k] : __fsub_rn(1.0f, acc[k]);
+}
+// Tile t of the upper triangle, rows of tiles: t = ty (ty + 1) / 2 + tx, tx <= ty.
+__device__ __forceinline__ void tile_of(int t, int &tx, int &ty) {
+    for (ty = 0, tx = t; tx > ty;) tx -= ++ty;
+}
+
+// The same masks from canonical fp32 distances (variant 3), in 8 x 8 tiles of
+// pairs, a warp per tile.  Every pair's distance, where a greedy walk computes
+// only those of the heads it keeps: but at a third of the instructions each and
+// with no head waiting for the one before.
+__device__ __noinline__ void canon_masks(const float *x0, u32 mp, u32 metric, float alpha2, const u64 *ck, int n,
+                                         u64 *dom) {
+    const int tid = threadIdx.x, warp = tid >> 5, lane = lane_id();
+    unsigned char *dom8 = reinterpret_cast<unsigned char *>(dom);   // byte 16 x + ty: columns 8 ty .. of row x
+    for (int i = tid; i < 2 * n; i += 32 * COOP_WARPS) dom[i] = 0ull;
+    coop_bar();
+    const int nt = (n + 7) >> 3;
+    for (int t = warp; t < nt * (nt + 1) / 2; t += COOP_WARPS) {
+        int tx, ty;
+        tile_of(t, tx, ty);
+        const float *xr[8], *yr[8];
+#pragma unroll
+        for (int c = 0; c < 8; c++) {   // past the list: a valid row again
+            xr[c] = x0 + (size_t)key_id(ck[min(8 * tx + c, n - 1)]) * mp;
+            yr[c] = x0 + (size_t)key_id(ck[min(8 * ty + c, n - 1)]) * mp;
+        }
+        float dd[2];
+        pair_tile(mp, metric, xr, yr, dd);
+        u32 bits = 0;
+        const int x = 8 * tx + (lane >> 2);   // pairs 2 lane, 2 lane + 1 share a row
+#pragma unroll
+        for (int k = 0; k < 2; k++) {
+            const int j = 2 * (lane & 3) + k, y = 8 * ty + j;
+            if (x < y && y < n && __fmul_rn(alpha2, dd[k]) <= key_rho(ck[y])) bits |= 1u << j;
+        }
+        bits |= __shfl_xor_sync(FULL, bits, 1);
+        bits |= __shfl_xor_sync(FULL, bits, 2);
+        if ((lane & 3) == 0 && x < n) dom8[16 * x + ty] = (unsigned char)bits;
+    }
+    coop_bar();
+}
+
+// The domination masks of variant GV, by the whole block.
+template <int GV>
+__device__ __forceinline__ void coop_masks(const Dev &d, const u64 *ck, int n, char *buf, u32 rows) {
+    if constexpr (GV == 3) canon_masks(d.x, d.mp, d.metric, d.alpha2, ck, n, reinterpret_cast<u64 *>(buf + GRAM_NL * 8));
+    else gram_masks<GV == 2>(d, ck, n, buf, rows);
+}
+
 // The helper warps of a block: serve requests until one has n < 0.
 template <int GV>
-__device__ __noinline__ void gram_helper(const Dev d, char *buf, int rows, const GramReq *req) {
+__device__ __noinline__ void gram_helper(const Dev d, char *buf, u32 rows, const GramReq *req) {
     for (;;) {
         coop_bar();
         const int n = *reinterpret_cast<const volatile int *>(&req->n);
         if (n < 0) return;
-        gram_masks<GV == 2>(d, *reinterpret_cast<const u64 *const volatile *>(&req->ck), n, buf, rows);
+        coop_masks<GV>(d, *reinterpret_cast<const u64 *const volatile *>(&req->ck), n, buf, rows);
     }
 }
 __device__ __forceinline__ void gram_release(GramReq *req) {
@@ -531,8 +637,8 @@ __device__ int warp_prune_masks(const Dev &d, const u64 *ck, int n, u32 *out_id,
     }
     __syncwarp();
     coop_bar();
-    gram_masks<GV == 2>(d, ck, n, st.gram, st.gram_rows);
-    const u64 *dom = reinterpret_cast<const u64 *>(gram_tail(st.gram, st.gram_rows, d.mp) + (size_t)st.gram_rows * 8);
+    coop_masks<GV>(d, ck, n, st.gram, st.gram_tag);
+    const u64 *dom = reinterpret_cast<const u64 *>(gram_tail(st.gram, st.gram_tag, d.mp) + (size_t)st.gram_rows * 8);
     // equal adjacent keys collapse to one
     u64 lo = 0, hi = 0;
     for (int i0 = 0; i0 < n; i0 += 32) {
@@ -569,7 +675,7 @@ __device__ int warp_prune_masks(const Dev &d, const u64 *ck, int n, u32 *out_id,
 // GV, the Gram variant of a kernel: 0, a buffer of at most GRAM_N rows with
 // rows of one 128-column block, a warp per item; 1, more than GRAM_N rows, and
 // 2, at most GRAM_N rows spanning several blocks: the block's four warps on one
-// item (see gram_masks).
+// item (see gram_masks); 3, the same on canonical distances (see canon_masks).
 template <int GV>
 __device__ int warp_prune(const Dev &d, const u64 *ck, int n, unsigned char *alive, u32 *idx, u32 *out_id,
                           float *out_rho, Stage &st) {
@@ -675,6 +781,40 @@ __device__ __forceinline__ bool warp_contains(const u32 *ids, int n, u32 v) {
     return __ballot_sync(FULL, hit) != 0;
 }
 
+// Canonical distances of row v to the nl rows keys[i + (i >= below)], into dv.
+__device__ __noinline__ void canon_row_dists(const float *x0, u32 mp, u32 metric, const u64 *keys, int nl, int below,
+                                             u32 v, float *dv) {
+    const int lane = lane_id(), grp = lane >> 3, g = lane & 7;
+    const float *xv = x0 + (size_t)v * mp;
+    auto row_of = [&](int i) {
+        i = min(i, nl - 1);
+        return x0 + (size_t)key_id(keys[i + (i >= below)]) * mp;
+    };
+    if (mp <= 128) {
+        float4 q[4];
+        canon_row_q8(xv, (int)mp, g, q);
+        for (int r0 = 0; r0 < nl; r0 += 8) {
+            float4 x[4], y[4];
+            canon_row_q8(row_of(r0 + grp), (int)mp, g, x);
+            canon_row_q8(row_of(r0 + 4 + grp), (int)mp, g, y);
+            const float da = canon_dist_q8v(q, x, (int)mp, (int)metric, g);
+            const float db = canon_dist_q8v(q, y, (int)mp, (int)metric, g);
+            if (g == 0 && r0 + grp < nl) dv[r0 + grp] = da;
+            if (g == 0 && r0 + 4 + grp < nl) dv[r0 + 4 + grp] = db;
+        }
+    } else {
+        const float one[4] = {1.0f, 1.0f, 1.0f, 1.0f};
+        for (int r0 = 0; r0 < nl; r0 += 4) {
+            const void *row[4];
+#pragma unroll
+            for (int c = 0; c < 4; c++) row[c] = row_of(r0 + c);
+            const float dd = warp_dists<0, 4, 2>(xv, row, one, (int)mp, (int)metric);
+            if (g == 0 && r0 + grp < nl) dv[r0 + grp] = dd;
+        }
+    }
+    __syncwarp();
+}
+
 // Apply one offer (v, rho) to the list in place (Algorithm 2, reverse edge):
 // a present id is a no-op; below R the entry is inserted in (rho, id) order;
 // at R the list is RobustPrune(list + v) about the owner (tombstones drop).
@@ -730,6 +870,39 @@ __device__ int apply_offer(const Dev &d, u32 *ids, float *rho, int n, u32 v, flo
     __syncwarp();
     const int cn = nl + 1;
     st.wk_rows += prune_row_bytes(d, st, cn);
+    // No entry of a pruned list drops a later one: only v's tests are open.
+    // The entries before it may drop it, else it may drop those after it.
+    // Variant 3 only: 32 distances where the greedy walk computes 528 (rounds
+    // of 100 + 100 on 10k x 128, deterministic: the offers 258 -> 76 us).  On
+    // the Gram tile the same short cut was no faster: what bounds an offer there
+    // is its chain of loads, fence and compare-and-swap; and in variant 0 the
+    // code alone costs the lock-free folds a quarter (128 -> 161 registers).
+    if (GV == 3 && pruned && d.same_tests) {
+        float *dv = reinterpret_cast<float *>(idx);
+        canon_row_dists(d.x, d.mp, d.metric, keys, nl, below, v, dv);
+        bool lost = false;
+        for (int i = lane; i < below; i += 32) lost |= __fmul_rn(d.alpha2, dv[i]) <= vr;
+        const bool drop_v = __any_sync(FULL, lost);
+        int nout = 0;
+        for (int i0 = 0; i0 < cn; i0 += 32) {   // positions of the merged list
+            const int i = i0 + lane;
+            bool keep = false;
+            u64 k = 0;
+            if (i < cn) {
+                k = keys[i];
+                keep = i < below || (i == below ? !drop_v : drop_v || !(__fmul_rn(d.alpha2, dv[i - 1]) <= key_rho(k)));
+            }
+            const u32 m = __ballot_sync(FULL, keep);
+            const int pos = nout + __popc(m & lanemask_lt());
+            if (keep && pos < (int)d.R) {
+                ids[pos] = key_id(k);
+                rho[pos] = key_rho(k);
+            }
+            nout += __popc(m);
+        }
+        __syncwarp();
+        return min(nout, (int)d.R);
+    }
     int nout = warp_prune<GV>(d, keys, cn, alive, idx, oid, orho, st);
     for (int j = lane; j < nout; j += 32) { ids[j] = oid[j]; rho[j] = orho[j]; }
     __syncwarp();
@@ -741,6 +914,14 @@ __device__ int apply_offer(const Dev &d, u32 *ids, float *rho, int n, u32 v, flo
 // Forward edges: F_v = RobustPrune(C_v) with C_v the expanded non-tombstone
 // nodes of v's search (nearest max_cand); Publish(v, F_v); emit offers.
 // ---------------------------------------------------------------------------
+// The Gram rows of a launch whose prunes see at most max_n candidates: without
+// the Gram, variant 3 while the items leave SMs idle.  (Its blocks hold three
+// items per SM where one-warp blocks hold up to 16, but an item's prune takes a
+// tenth of the time.)
+inline u32 prune_rows_for(const Dev &d, u32 max_n, u64 items, int num_sms) {
+    if (d.gram) return gram_rows_for(d.gram, max_n);
+    return max_n <= (u32)GRAM_NL && items <= 64ull * num_sms ? CANON_ROWS : 0u;
+}
 struct PruneInsArgs {
     Dev d;
     u32 first, b;
@@ -773,7 +954,7 @@ __global__ void __launch_bounds__(GV ? 32 * COOP_WARPS : 32, GV ? 3 : 12) prune_
     const u32 R = d.R;
     char *p = smem;
     char *gbuf = a.gram ? p : nullptr;
-    if (GV != 0 && threadIdx.x >= 32) return gram_helper<GV>(d, gbuf, (int)a.gram, &req);
+    if (GV != 0 && threadIdx.x >= 32) return gram_helper<GV>(d, gbuf, a.gram, &req);
     p += gram_bytes(a.gram, d.mp);
     Stage st = stage_init(p, a.ns, d.mp, gbuf, a.gram, &req);
     WarpSlabs ws;
@@ -850,7 +1031,7 @@ cudaError_t launch_prune_insert(const Dev &d, u32 first, u32 b, const u64 *exp_k
                                 const Offers &of, int num_sms, cudaStream_t st, bool rescore) {
     if (b == 0) return cudaSuccess;
     // the Gram tile covers the prune only when every candidate fits in it
-    const u32 gram = gram_rows_for(d.gram, max_cand);
+    const u32 gram = prune_rows_for(d, max_cand, b, num_sms);
     PruneInsArgs a{d, first, b, exp_keys, exp_count, max_hops, max_cand, 0, 0, gram, rescore ? 1u : 0u,
                    F_id, F_rho, F_n, of};
     u32 np = 32;
@@ -860,7 +1041,8 @@ cudaError_t launch_prune_insert(const Dev &d, u32 first, u32 b, const u64 *exp_k
     const size_t wb = prune_ins_warp_bytes(np, d.R, a.ns, d.mp, gram);
     const size_t smem = wb;
     const int threads = block_threads(a.gram, d.mp);
-    const void *fns[3] = {(const void *)prune_insert_kernel<0>, (const void *)prune_insert_kernel<1>, (const void *)prune_insert_kernel<2>};
+    const void *fns[4] = {(const void *)prune_insert_kernel<0>, (const void *)prune_insert_kernel<1>, (const void *)prune_insert_kernel<2>,
+                          (const void *)prune_insert_kernel<3>};
     const void *fn = fns[gram_variant(a.gram, d.mp)];
     cudaError_t e = smem_at_least((const void *)fn, smem);
     if (e != cudaSuccess) return e;
@@ -915,7 +1097,7 @@ __global__ void __launch_bounds__(GV ? 32 * COOP_WARPS : 32, GV ? 3 : 12) offer_
     const u32 R = d.R;
     char *p = smem;
     char *gbuf = a.gram ? p : nullptr;
-    if (GV != 0 && threadIdx.x >= 32) return gram_helper<GV>(d, gbuf, (int)a.gram, &req);
+    if (GV != 0 && threadIdx.x >= 32) return gram_helper<GV>(d, gbuf, a.gram, &req);
     p += gram_bytes(a.gram, d.mp);
     Stage st = stage_init(p, a.ns, d.mp, gbuf, a.gram, &req);
     WarpSlabs ws;
@@ -1002,15 +1184,17 @@ cudaError_t launch_offer_fold(const Dev &d, const Offers &of, const u32 *seg_sta
     if (of.n == 0) return cudaSuccess;
     if (budget && hi > of.n) hi = of.n;
     if (budget && lo >= hi) return cudaSuccess;
-    FoldArgs a{d, of, seg_start, seg_count, budget, 0, 0, gram_rows_for(d.gram, d.R + 1), lo, budget ? hi : of.n};
+    FoldArgs a{d, of, seg_start, seg_count, budget, 0, 0, 0, lo, budget ? hi : of.n};
+    a.gram = prune_rows_for(d, d.R + 1, a.hi - a.lo, num_sms);
     u32 np = 32;
     while (np < d.R + 1) np <<= 1;
     a.np = np;
-    a.ns = d.gram ? 0 : stage_cap(d.mp, d.R + 1, d.stage_bytes);
+    a.ns = a.gram ? 0 : stage_cap(d.mp, d.R + 1, d.stage_bytes);
     const size_t wb = fold_warp_bytes(np, d.R, a.ns, d.mp, a.gram);
     const size_t smem = wb;
     const int threads = block_threads(a.gram, d.mp);
-    const void *fns[3] = {(const void *)offer_fold_kernel<0>, (const void *)offer_fold_kernel<1>, (const void *)offer_fold_kernel<2>};
+    const void *fns[4] = {(const void *)offer_fold_kernel<0>, (const void *)offer_fold_kernel<1>, (const void *)offer_fold_kernel<2>,
+                          (const void *)offer_fold_kernel<3>};
     const void *fn = fns[gram_variant(a.gram, d.mp)];
     cudaError_t e = smem_at_least((const void *)fn, smem);
     if (e != cudaSuccess) return e;
@@ -1063,7 +1247,7 @@ __global__ void __launch_bounds__(GV ? 32 * COOP_WARPS : 64, GV ? 3 : 6) refine_
     const u32 R = d.R;
     char *p = smem + (GV ? 0 : warp) * refine_warp_bytes(a.np_s, a.cap_s, R, a.ns, d.mp, a.gram);
     char *gbuf = a.gram ? p : nullptr;
-    if (GV != 0 && warp) return gram_helper<GV>(d, gbuf, (int)a.gram, &req);
+    if (GV != 0 && warp) return gram_helper<GV>(d, gbuf, a.gram, &req);
     p += gram_bytes(a.gram, d.mp);
     Stage st = stage_init(p, a.ns, d.mp, gbuf, a.gram, &req);
     WarpSlabs ws;
@@ -1246,7 +1430,7 @@ __global__ void __launch_bounds__(GV ? 32 * COOP_WARPS : 64, GV ? 3 : 6) refine_
 }
 
 // Launch shape of the refine kernel (shared by launch_refine and the spill size).
-static void refine_shape(const Dev &d, u32 max_cand, RefineArgs &a) {
+static void refine_shape(const Dev &d, u32 max_cand, RefineArgs &a, u64 items, int num_sms) {
     u32 cap = d.R * d.R;
     if (cap > 4096) cap = 4096;
     a.cap = cap;
@@ -1257,14 +1441,14 @@ static void refine_shape(const Dev &d, u32 max_cand, RefineArgs &a) {
     u32 nps = 32;
     while (nps < a.cap_s + d.R) nps <<= 1;
     a.np_s = nps;
-    a.gram = d.gram ? (d.R > 32 ? (u32)GRAM_NL : (u32)GRAM_N) : 0u;
-    a.ns = d.gram ? 0 : stage_cap(d.mp, max_cand, d.stage_bytes);
+    a.gram = d.gram ? (d.R > 32 ? (u32)GRAM_NL : (u32)GRAM_N) : prune_rows_for(d, 0, items, num_sms);
+    a.ns = a.gram ? 0 : stage_cap(d.mp, max_cand, d.stage_bytes);
     a.spill_warp = refine_list_bytes(np, cap);
 }
 
 size_t refine_spill_bytes(const Dev &d, u32 max_cand, int num_sms) {
     RefineArgs a{};
-    refine_shape(d, max_cand, a);
+    refine_shape(d, max_cand, a, 0, num_sms);
     // every warp an SM can hold (2,048 threads)
     return (size_t)num_sms * 64 * a.spill_warp;
 }
@@ -1274,14 +1458,15 @@ cudaError_t launch_refine(const Dev &d, u32 first, u32 b, u32 mode, u32 max_cand
     if (b == 0) return cudaSuccess;
     RefineArgs a;
     a.d = d; a.first = first; a.b = b; a.mode = mode; a.max_cand = max_cand; a.of = of;
-    refine_shape(d, max_cand, a);
+    refine_shape(d, max_cand, a, b, num_sms);
     a.spill = spill;
     const size_t wb = refine_warp_bytes(a.np_s, a.cap_s, d.R, a.ns, d.mp, a.gram);
     const bool coop = gram_variant(a.gram, d.mp) != 0;
     const int warps = !coop && 2 * wb <= 200 * 1024 ? 2 : 1;   // items of a block
     const int threads = coop ? 32 * COOP_WARPS : 32 * warps;
     size_t smem = warps * wb;
-    const void *fns[3] = {(const void *)refine_kernel<0>, (const void *)refine_kernel<1>, (const void *)refine_kernel<2>};
+    const void *fns[4] = {(const void *)refine_kernel<0>, (const void *)refine_kernel<1>, (const void *)refine_kernel<2>,
+                          (const void *)refine_kernel<3>};
     const void *fn = fns[gram_variant(a.gram, d.mp)];
     cudaError_t e = smem_at_least((const void *)fn, smem);
     if (e != cudaSuccess) return e;
@@ -1343,21 +1528,6 @@ struct RepairKArgs {
 constexpr int REPK_WARPS = 4;
 __host__ __device__ inline size_t repk_bytes(u32 R) {
     return 2 * al16((size_t)R * 4) + al16((size_t)R * R * 4) + REPK_WARPS * 64;
-}
-
-// The canonical sums of 64 values a lane holds as partials (value p in v[p]):
-// the tree of canon_dist over the 32 lanes, where at each level a lane keeps
-// half of the values it still has and passes the other half on.  Lane l ends
-// with values 2 l and 2 l + 1 in v[0] and v[1].
-__device__ __forceinline__ void warp_tree64(float (&v)[64]) {
-    const int lane = lane_id();
-#pragma unroll
-    for (int h = 16, n = 32; h >= 1; h >>= 1, n >>= 1) {
-        const bool up = lane & h;
-#pragma unroll
-        for (int i = 0; i < n; i++)
-            v[i] = __fadd_rn(up ? v[i + n] : v[i], __shfl_xor_sync(FULL, up ? v[i] : v[i + n], h));
-    }
 }
 
 // The greedy RobustPrune of B \ {a} about a = member ja of B, from the table M,
@@ -1476,47 +1646,20 @@ __global__ void __launch_bounds__(32 * REPK_WARPS, 3) repair_k_kernel(RepairKArg
         // distance table among B (symmetric): tiles x <= y, in one sequence
         const int nt = (nb + 7) >> 3;
         for (int t = warp; t < nt * (nt + 1) / 2; t += REPK_WARPS) {
-            int ty = 0, tx = t;
-            while (tx > ty) tx -= ++ty;       // t = ty (ty + 1) / 2 + tx
+            int tx, ty;
+            tile_of(t, tx, ty);
             const float *xr[8], *yr[8];
 #pragma unroll
             for (int c = 0; c < 8; c++) {     // past the list: a valid row again
                 xr[c] = d.x + (size_t)bid[min(8 * tx + c, nb - 1)] * d.mp;
                 yr[c] = d.x + (size_t)bid[min(8 * ty + c, nb - 1)] * d.mp;
             }
-            float acc[64];
-#pragma unroll
-            for (int q = 0; q < 64; q++) acc[q] = 0.0f;
-            for (u32 e = 4 * lane; e < d.mp; e += 128) {
-                float4 x[8], y[8];
-#pragma unroll
-                for (int c = 0; c < 8; c++) {
-                    x[c] = *reinterpret_cast<const float4 *>(xr[c] + e);
-                    y[c] = *reinterpret_cast<const float4 *>(yr[c] + e);
-                }
-                if (d.metric == 0) {
-#pragma unroll
-                    for (int q = 0; q < 64; q++) {
-                        const float4 u = x[q >> 3], v = y[q & 7];
-                        const float d0 = __fsub_rn(u.x, v.x), d1 = __fsub_rn(u.y, v.y);
-                        const float d2 = __fsub_rn(u.z, v.z), d3 = __fsub_rn(u.w, v.w);
-                        acc[q] = __fmaf_rn(d3, d3, __fmaf_rn(d2, d2, __fmaf_rn(d1, d1, __fmaf_rn(d0, d0, acc[q]))));
-                    }
-                } else {
-#pragma unroll
-                    for (int q = 0; q < 64; q++) {
-                        const float4 u = x[q >> 3], v = y[q & 7];
-                        acc[q] = __fmaf_rn(u.w, v.w, __fmaf_rn(u.z, v.z, __fmaf_rn(u.y, v.y, __fmaf_rn(u.x, v.x, acc[q]))));
-                    }
-                }
-            }
-            __syncwarp();
-            warp_tree64(acc);
+            float dd[2];
+            pair_tile(d.mp, d.metric, xr, yr, dd);
 #pragma unroll
             for (int k = 0; k < 2; k++) {
                 const int q = 2 * lane + k, x = 8 * tx + (q >> 3), y = 8 * ty + (q & 7);
-                const float dd = d.metric == 0 ? acc[k] : __fsub_rn(1.0f, acc[k]);
-                if (x < y && y < nb) { M[x * R + y] = dd; M[y * R + x] = dd; }
+                if (x < y && y < nb) { M[x * R + y] = dd[k]; M[y * R + x] = dd[k]; }
             }
         }
         __syncthreads();
@@ -1673,7 +1816,7 @@ __global__ void __launch_bounds__(GV ? 32 * COOP_WARPS : 32, GV ? 3 : 12) repair
     const u32 R = d.R;
     char *p = smem;
     char *gbuf = a.gram ? p : nullptr;
-    if (GV != 0 && threadIdx.x >= 32) return gram_helper<GV>(d, gbuf, (int)a.gram, &req);
+    if (GV != 0 && threadIdx.x >= 32) return gram_helper<GV>(d, gbuf, a.gram, &req);
     p += gram_bytes(a.gram, d.mp);
     Stage st = stage_init(p, a.ns, d.mp, gbuf, a.gram, &req);
     WarpSlabs ws;
@@ -1762,15 +1905,16 @@ cudaError_t launch_repair_fold(const Dev &d, const u32 *dt, const u32 *pair_key,
                                u64 lo) {
     if (n_pairs == 0) return cudaSuccess;
     RepairFoldArgs a{d, dt, pair_key, pair_val, pair_K, pair_Kn, seg_start, seg_count, n_pairs, budget, 0, 0,
-                     gram_rows_for(d.gram, 2 * d.R - 1), lo};
+                     prune_rows_for(d, 2 * d.R - 1, n_pairs, num_sms), lo};
     u32 np = 32;
     while (np < 2 * d.R) np <<= 1;
     a.np = np;
-    a.ns = d.gram ? 0 : stage_cap(d.mp, 2 * d.R, d.stage_bytes);
+    a.ns = a.gram ? 0 : stage_cap(d.mp, 2 * d.R, d.stage_bytes);
     const size_t wb = repf_warp_bytes(np, d.R, a.ns, d.mp, a.gram);
     const size_t smem = wb;
     const int threads = block_threads(a.gram, d.mp);
-    const void *fns[3] = {(const void *)repair_fold_kernel<0>, (const void *)repair_fold_kernel<1>, (const void *)repair_fold_kernel<2>};
+    const void *fns[4] = {(const void *)repair_fold_kernel<0>, (const void *)repair_fold_kernel<1>, (const void *)repair_fold_kernel<2>,
+                          (const void *)repair_fold_kernel<3>};
     const void *fn = fns[gram_variant(a.gram, d.mp)];
     cudaError_t e = smem_at_least((const void *)fn, smem);
     if (e != cudaSuccess) return e;

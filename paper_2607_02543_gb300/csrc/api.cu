@@ -453,7 +453,7 @@ etale_status run_offers(etale_index *idx, u32 nslots, u64 targets, cudaStream_t 
         CK(make_segments(of.key, nslots, (u32)idx->capacity, as<u32>(idx->seg_flags), as<u32>(idx->seg_scan),
                          as<u32>(idx->seg_start), seg_count, sc, st),
            "offer segments");
-        g_kernel_launches += 3 * ((bits_for(idx->capacity) + 7) / 8) * 2 + 4;
+        g_kernel_launches += sort_launches(nslots, bits_for(idx->capacity)) + 4;
     }
     {
         PhaseScope ps(idx, ETALE_PH_OFFER_FOLD, st);
@@ -919,7 +919,7 @@ etale_status etale_delete(etale_index *idx, const uint32_t *ids, uint64_t n, uin
     CK(launch_compact_ok(as<u32>(idx->del_ids), as<u32>(idx->del_ok), as<u32>(idx->del_scan), (u32)n,
                          as<u32>(idx->dt), n_dt, st),
        "tombstone compaction");
-    g_kernel_launches += 4 * 3 + 6;
+    g_kernel_launches += sort_launches((u32)n, 32) + 6;
     prof_end(idx, st);
     // repair: K(u, a) per pair, then one fold per a
     const u32 invalid = (u32)idx->capacity;
@@ -960,7 +960,7 @@ etale_status etale_delete(etale_index *idx, const uint32_t *ids, uint64_t n, uin
         CK(make_segments(as<u32>(idx->pair_key), (u32)slots, invalid, as<u32>(idx->pair_flags),
                          as<u32>(idx->pair_scan), as<u32>(idx->pair_seg), seg_count, sc, st),
            "pair segments");
-        g_kernel_launches += 3 * ((bits_for(idx->capacity) + 7) / 8) * 2 + 4;
+        g_kernel_launches += sort_launches((u32)slots, bits_for(idx->capacity)) + 4;
     }
     if (!lockfree) {
         CK(launch_repair_fold(d, as<u32>(idx->dt), as<u32>(idx->pair_key), as<u32>(idx->pair_val),

@@ -108,6 +108,8 @@ void sort_scratch_carve(SortScratch &s, u32 *buf, u32 n);
 // result ends in (key, val); (key_alt, val_alt) are scratch of equal size.
 cudaError_t radix_sort_pairs(u32 *key, u32 *val, u32 *key_alt, u32 *val_alt, u32 n, u32 key_bits,
                              const SortScratch &s, cudaStream_t st);
+// Kernels of such a sort (one scan level).
+u32 sort_launches(u32 n, u32 key_bits);
 // Segments of equal keys among sorted keys (keys equal to `invalid` sort last
 // and are ignored): seg_start[0..count] and the count in *seg_count.
 cudaError_t make_segments(const u32 *key, u32 n, u32 invalid, u32 *flags, u32 *scan_out,

@@ -112,7 +112,7 @@ struct etale_index {
     // call and one update call can run at the same time (concurrent mode)
     DevBuf s_stage, s_qpad, s_out_ids, s_out_dist, s_seed;
     // ground truth on tensor cores
-    DevBuf gt_A, gt_B, gt_xn, gt_qstat, gt_gstat, gt_fb, gt_bmin, gt_center;
+    DevBuf gt_A, gt_B, gt_xn, gt_qstat, gt_gstat, gt_fb, gt_bmin, gt_keys, gt_center;
     u32 gt_path = 0;
     u64 gt_fallbacks = 0;
     // seeding on tensor cores
@@ -1053,7 +1053,9 @@ static etale_status ground_truth_run(etale_index *idx, const Dev &d, const float
     u32 h[8];
     CK(cudaMemcpyAsync(h, b.gstat, sizeof h, cudaMemcpyDeviceToHost, st), "read split flag");
     CK(cudaStreamSynchronize(st), "synchronize");
-    gt_tc_configure(p, nq, h[3] != 0);
+    gt_tc_configure(p, nq, k, idx->mp, h[3] != 0, true);
+    // no room for the keys: the candidate blocks are scored whole
+    if (p.keys && !grow(idx->gt_keys, p.bytes_keys)) gt_tc_configure(p, nq, k, idx->mp, h[3] != 0, false);
     if (!p.usable) {
         PhaseScope ps(idx, ETALE_PH_GT_EXACT, st);
         CK(launch_ground_truth(d, idx->next_id, qpad, nq, k, oid, od, idx->num_sms, st), "ground truth");
@@ -1062,6 +1064,7 @@ static etale_status ground_truth_run(etale_index *idx, const Dev &d, const float
     }
     if (!grow(idx->gt_bmin, p.bytes_bmin)) return idx->fail(ETALE_ENOMEM, "ground-truth block minima");
     b.bmin = as<float>(idx->gt_bmin);
+    b.keys = as<float>(idx->gt_keys);
     for (u32 q0 = 0; q0 < nq; q0 += p.qgroup) {
         const u32 g = std::min<u32>(p.qgroup, nq - q0);
         {

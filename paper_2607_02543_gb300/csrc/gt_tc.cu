@@ -19,13 +19,14 @@
 //      accumulator; eight epilogue warps read it with tcgen05.ld and write,
 //      per query and per block of 32 rows, the smallest approximate key
 //      key = |x|^2 - 2 q.x (L2) or -q.x (IP); dead rows have key +inf.
+//      For few wide rows it writes every key too.
 //   3. gt_rerank_kernel: every row of the k blocks with the smallest minima
 //      is scored with the canonical fp32 distance (the same definition the
 //      rest of the index uses).  The k-th of these distances bounds the
 //      answer: an a-priori bound E on |approximate - canonical| turns it into
 //      a threshold T on approximate keys that no row of the top k can exceed,
 //      and the rows of the remaining blocks with a minimum <= T are scored
-//      too.  So the result is always the exact top-k with canonical
+//      too (where every key is at hand, only the rows with a key that passes).  So the result is always the exact top-k with canonical
 //      distances, ties by smaller id.  Queries without a finite threshold
 //      (infinities or NaN in the data), or whose T admits more than half of
 //      all blocks, go to the CUDA-core exact kernel.
@@ -63,13 +64,14 @@ __host__ __device__ constexpr u32 tc_idesc(u32 n) {
 
 struct TcArgs {
     u32 nq, n_tiles, kblocks, bn, m_tiles, chunks, tiles_per_chunk, stages;
-    u32 all_keys;         // 0: smallest key per block of 32 rows; 1: every key
+    u32 all_keys;         // 0: smallest key per block of 32 rows; 1: every key; 2: both, the keys in `keys`
     u32 stream_a;         // 1: the query boxes travel through the ring (selects gt_tc_kernel<true>)
     const u32 *nq_dev;    // when set, the batch size is read here (nq is its cap); later query tiles are skipped
     u32 ld;               // row length of the output (blocks or keys)
     float s;              // -2 (L2) or -1 (IP)
     const float *xn;      // n_tiles * bn key bases (+inf for dead rows and padding)
     float *out;           // nq x ld
+    float *keys;          // all_keys 2: (n_tiles * bn / 32) x nq x 32, a block's keys for a query on one line
     u32 *err;
 };
 
@@ -138,6 +140,10 @@ __device__ __forceinline__ float min3(float a, float b, float c) {
     asm("min.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
     return r;
 }
+// 32 bytes, one sector a lane
+__device__ __forceinline__ void st_global32(float *p, u64 a, u64 b, u64 c, u64 d) {
+    asm volatile("st.global.v4.b64 [%0], {%1, %2, %3, %4};" ::"l"(p), "l"(a), "l"(b), "l"(c), "l"(d) : "memory");
+}
 __device__ __forceinline__ float pair_lo(u64 v) { return __uint_as_float((u32)v); }
 __device__ __forceinline__ float pair_hi(u64 v) { return __uint_as_float((u32)(v >> 32)); }
 __device__ __forceinline__ void tmem_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
@@ -149,7 +155,8 @@ __device__ __forceinline__ void tmem_wait() { asm volatile("tcgen05.wait::ld.syn
 // fma and takes two at a time into the running minimum.
 // STREAM_A: the query boxes travel through the ring with the row boxes (a
 // compile-time choice, so the resident form's MMA issue loop carries no test).
-template <bool STREAM_A>
+// KEYS: the keys are written beside the minima (all_keys 2).
+template <bool STREAM_A, bool KEYS>
 __global__ void __launch_bounds__(TC_THREADS, 1)
     gt_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, TcArgs a) {
     extern __shared__ unsigned char tc_raw[];
@@ -363,16 +370,15 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
                     };
                     const ulonglong2 *x2 = reinterpret_cast<const ulonglong2 *>(xs[xi] + half * TC_ROWS);
                     const u64 s2 = pair32(__float_as_uint(a.s), __float_as_uint(a.s));
-                    if (a.all_keys) {
-                        ulonglong2 *o4 = reinterpret_cast<ulonglong2 *>(dst + (size_t)(t * a.bn + half * TC_ROWS) / 4);
+                    if (a.all_keys == 1) {
+                        float *o = a.out + (size_t)(valid ? q : 0) * a.ld + t * a.bn + half * TC_ROWS;
 #pragma unroll
-                        for (int j4 = 0; j4 < TC_ROWS / 4; j4++) {
-                            const ulonglong2 v = x2[j4];
-                            const u32 *rr = r + 4 * j4;
-                            ulonglong2 kv;
-                            kv.x = fma2(s2, pair32(rr[0], rr[1]), v.x);
-                            kv.y = fma2(s2, pair32(rr[2], rr[3]), v.y);
-                            if (valid) o4[j4] = kv;
+                        for (int j8 = 0; j8 < TC_ROWS / 8; j8++) {
+                            const ulonglong2 v = x2[2 * j8], w = x2[2 * j8 + 1];
+                            const u32 *rr = r + 8 * j8;
+                            const u64 k0 = fma2(s2, pair32(rr[0], rr[1]), v.x), k1 = fma2(s2, pair32(rr[2], rr[3]), v.y);
+                            const u64 k2 = fma2(s2, pair32(rr[4], rr[5]), w.x), k3 = fma2(s2, pair32(rr[6], rr[7]), w.y);
+                            if (valid) st_global32(o + 8 * j8, k0, k1, k2, k3);
                         }
                         release();
                         continue;
@@ -381,13 +387,20 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
 #pragma unroll
                     for (int c = 0; c < TC_ROWS / 32; c++) {
                         float m0 = __int_as_float(0x7f800000), m1 = m0;
+                        float *o = KEYS ? a.keys + ((size_t)(t * (a.bn / 32) + half * (TC_ROWS / 32) + c) * a.nq +
+                                                    (valid ? q : 0)) * 32
+                                        : nullptr;
 #pragma unroll
-                        for (int j4 = 0; j4 < 8; j4++) {
-                            const ulonglong2 v = x2[c * 8 + j4];
-                            const u32 *rr = r + c * 32 + 4 * j4;
+                        for (int j8 = 0; j8 < 4; j8++) {
+                            const ulonglong2 v = x2[c * 8 + 2 * j8], w = x2[c * 8 + 2 * j8 + 1];
+                            const u32 *rr = r + c * 32 + 8 * j8;
                             const u64 k0 = fma2(s2, pair32(rr[0], rr[1]), v.x), k1 = fma2(s2, pair32(rr[2], rr[3]), v.y);
+                            const u64 k2 = fma2(s2, pair32(rr[4], rr[5]), w.x), k3 = fma2(s2, pair32(rr[6], rr[7]), w.y);
                             m0 = min3(m0, pair_lo(k0), pair_hi(k0));
                             m1 = min3(m1, pair_lo(k1), pair_hi(k1));
+                            m0 = min3(m0, pair_lo(k2), pair_hi(k2));
+                            m1 = min3(m1, pair_lo(k3), pair_hi(k3));
+                            if (KEYS && valid) st_global32(o + 8 * j8, k0, k1, k2, k3);
                         }
                         bm[c] = fminf(m0, m1);
                     }
@@ -622,7 +635,7 @@ __device__ float dist_upper_bound(int metric, float m, float qn, float E, float 
 }
 
 // ---- threshold and exact rerank -----------------------------------------------
-constexpr int RR_WARPS = 8;
+__host__ __device__ constexpr int rr_warps(int W) { return W == 1 ? 8 : W; }   // a block's warps
 constexpr int RR_LIST = 256;      // candidate blocks a warp collects before it scores them
 
 struct RerankArgs {
@@ -630,6 +643,7 @@ struct RerankArgs {
     u64 n_rows;
     const float *q;       // all queries, nq_total x mp fp32
     const float *bmin;    // this group: nq x nblk
+    const float *keys;    // KEYS: this group, nblk x nq x 32
     const float *qstat;   // all queries
     const u32 *gstat;
     u32 *out_ids;         // all queries, x k
@@ -685,22 +699,61 @@ __device__ __forceinline__ void canon_dist_wide2(const float *__restrict__ q, co
     d1 = metric == 0 ? s1 : __fsub_rn(1.0f, s1);
 }
 
+// The canonical keys of the rows rl[0 .. n - 1] for the query qv, by one warp.
+__device__ __noinline__ void score_rows(const float *x, u32 mp, u32 metric, const float *qv, const u32 *rl, u32 n,
+                                        u64 *out) {
+    const int lane = lane_id(), grp = lane >> 3, g = lane & 7;
+    if (mp <= 128) {
+        float4 q[4];
+        canon_row_q8(qv, (int)mp, g, q);
+        for (u32 r0 = 0; r0 < n; r0 += 8) {
+            const u32 ia = rl[min(r0 + grp, n - 1)], ib = rl[min(r0 + 4 + grp, n - 1)];
+            float4 va[4], vb[4];
+            canon_row_q8(x + (size_t)ia * mp, (int)mp, g, va);
+            canon_row_q8(x + (size_t)ib * mp, (int)mp, g, vb);
+            const float da = canon_dist_q8v(q, va, (int)mp, (int)metric, g);
+            const float db = canon_dist_q8v(q, vb, (int)mp, (int)metric, g);
+            if (g == 0) {
+                out[r0 + grp] = mkkey(da, ia);
+                out[r0 + 4 + grp] = mkkey(db, ib);
+            }
+        }
+    } else {
+        const float one[4] = {1.0f, 1.0f, 1.0f, 1.0f};
+        for (u32 r0 = 0; r0 < n; r0 += 4) {
+            const void *row[4];
+#pragma unroll
+            for (int c = 0; c < 4; c++) row[c] = x + (size_t)rl[min(r0 + c, n - 1)] * mp;
+            const float dd = warp_dists<0, 4, 2>(qv, row, one, (int)mp, (int)metric);
+            if (g == 0) out[r0 + grp] = mkkey(dd, rl[min(r0 + grp, n - 1)]);
+        }
+    }
+    __syncwarp();
+}
+
 // Bound by the row reads (L2) and their latency.  Scoring what the k-th
 // distance leaves open, instead of a fixed 32 blocks with a certificate and a
 // full scan by gt_kernel where it fails, and two blocks of 8 warps per SM:
 // 10k queries x 300k x 128 integer rows 0.97 -> 0.50 ms; 2,003 queries x 40k x
 // 960 real-valued rows, all of which failed the certificate, 53.5 -> 2.9 ms
 // (21.5 before gt_center_kernel).
-// W warps per query (1 or 8): a block per query below 16 queries an SM, where
-// a warp per query would leave the SMs' slots empty.  Each lane keeps the four smallest minima of the
-// blocks it reads, with their numbers, so that a threshold met by at most four
-// blocks of any lane needs no second pass over the minima.
-template <int W>
-__global__ void __launch_bounds__(RR_WARPS * 32, 2) gt_rerank_kernel(Dev d, RerankArgs a) {
+// W warps per query (1, 2, 4 or 8), as many as the SMs hold for all queries at
+// once: 2,003 queries x 40k x 960 with 1, 2, 4, 8 warps 88, 98, 140, 237 us, 300
+// queries 57, 42, 39, 42.
+// KEYS: the candidate pass left every key, and of a candidate block only the rows
+// below the threshold are scored: the 960-d batch 866 -> 88 us (with the case's
+// wider clusters 2.9 -> 0.1 ms).
+// Each lane keeps the four smallest minima of the blocks it reads, with their
+// numbers, so that a threshold met by at most four blocks of any lane needs no
+// second pass over the minima.
+template <int W, bool KEYS>
+__global__ void __launch_bounds__(rr_warps(W) * 32, 16 / rr_warps(W)) gt_rerank_kernel(Dev d, RerankArgs a) {
+    constexpr int RR_WARPS = rr_warps(W);
     __shared__ u32 clist[RR_WARPS][RR_LIST];
     __shared__ u64 ckey[RR_WARPS][32];
     __shared__ u64 xbest[RR_WARPS][32];
     __shared__ u32 xsum[2][RR_WARPS];
+    __shared__ u32 rlist[KEYS ? RR_WARPS : 1][64];   // rows to score
     const int warp = threadIdx.x >> 5, lane = lane_id();
     const int tw = warp % W;                         // this warp's place among the query's warps
     const u32 li = blockIdx.x * (RR_WARPS / W) + warp / W;
@@ -768,8 +821,12 @@ __global__ void __launch_bounds__(RR_WARPS * 32, 2) gt_rerank_kernel(Dev d, Rera
     // 3. phase 0: the blocks with a minimum <= tau (dead-only blocks have
     //    +inf); phase 1: those that the k-th distance found does not exclude
     u32 lo = 0, hi = min(tau, ORD_INF - 1);
+    // KEYS: of those blocks only the rows whose own key passes are scored, and
+    // phase 1 takes the rest of phase 0's blocks too.  (A key that passes is
+    // finite, its row live.)  With fewer than k blocks every live row is scored.
+    const bool by_rows = KEYS && tau < ORD_INF;
     for (int phase = 0; phase < 2; phase++) {
-        auto in = [&](u32 v) { return v > lo && v <= hi; };
+        auto in = [&](u32 v) { return (by_rows || v > lo) && v <= hi; };
         const bool kept = !__any_sync(FULL, t3 <= hi);   // every block in (lo, hi] is among the kept ones
         if (phase == 1) {
             u32 cnt = 0;
@@ -787,6 +844,22 @@ __global__ void __launch_bounds__(RR_WARPS * 32, 2) gt_rerank_kernel(Dev d, Rera
             if (!cert) break;
         }
         u64 best = KEY_INF;   // this warp's 32 smallest keys of the phase
+        // cand, a key a lane, into best: only when one can still enter the top k
+        auto merge = [&](u64 cand) {
+            const u64 kth = __shfl_sync(FULL, best, (int)a.k - 1);
+            if (!__any_sync(FULL, cand < kth && cand < bound)) return;
+            cand = warp_sort32(cand);
+            const u64 rev = __shfl_sync(FULL, cand, 31 - lane);
+            best = warp_sort32(best < rev ? best : rev);
+        };
+        u32 nrow = 0;         // rows in rlist
+        // the first n <= 32 rows of the list
+        auto score = [&](u32 n) {
+            score_rows(d.x, d.mp, d.metric, qv, rlist[KEYS ? warp : 0], n, ckey[warp]);
+            const u64 cand = lane < (int)n ? ckey[warp][lane] : KEY_INF;
+            __syncwarp();
+            merge(cand);
+        };
         u32 cur = (u32)tw * 128;
         for (bool more = true; more;) {
             u32 pend = 0;
@@ -814,6 +887,33 @@ __global__ void __launch_bounds__(RR_WARPS * 32, 2) gt_rerank_kernel(Dev d, Rera
                 more = cur < a.nblk;
             }
             __syncwarp();
+            if (by_rows) {
+                // keys of eight blocks in flight
+                for (u32 i0 = 0; i0 < pend; i0 += 8) {
+                    u32 v[8];
+#pragma unroll
+                    for (int c = 0; c < 8; c++)
+                        v[c] = i0 + c < pend ? f2ord(__ldg(a.keys + ((size_t)clist[warp][i0 + c] * a.nq + li) * 32 + lane)) : ~0u;
+#pragma unroll
+                    for (int c = 0; c < 8; c++) {
+                        const bool pass = v[c] > lo && v[c] <= hi;
+                        const u32 m = __ballot_sync(FULL, pass);
+                        if (m == 0) continue;
+                        if (pass) rlist[warp][nrow + __popc(m & lanemask_lt())] = clist[warp][i0 + c] * 32u + lane;
+                        nrow += __popc(m);
+                        __syncwarp();
+                        if (nrow >= 32) {
+                            score(32);
+                            const u32 rest = lane + 32 < (int)nrow ? rlist[warp][lane + 32] : 0u;
+                            __syncwarp();
+                            rlist[warp][lane] = rest;
+                            __syncwarp();
+                            nrow -= 32;
+                        }
+                    }
+                }
+                continue;
+            }
             for (u32 i = 0; i < pend; i++) {
                 const u32 id0 = clist[warp][i] * 32u;
                 if (lane == 0 && i + 1 < pend) {
@@ -847,17 +947,13 @@ __global__ void __launch_bounds__(RR_WARPS * 32, 2) gt_rerank_kernel(Dev d, Rera
                     }
                 }
                 __syncwarp();
-                u64 cand = live ? ckey[warp][lane] : KEY_INF;
+                const u64 cand = live ? ckey[warp][lane] : KEY_INF;
                 __syncwarp();
-                // merge only when a key can still enter the top k
-                const u64 kth = __shfl_sync(FULL, best, (int)a.k - 1);
-                if (!__any_sync(FULL, cand < kth && cand < bound)) continue;
-                cand = warp_sort32(cand);
-                const u64 rev = __shfl_sync(FULL, cand, 31 - lane);
-                best = warp_sort32(best < rev ? best : rev);
+                merge(cand);
             }
             __syncwarp();
         }
+        if (KEYS && nrow) score(nrow);
         // join the warps' lists
         if (W > 1) {
             xbest[warp][lane] = best;
@@ -1150,7 +1246,7 @@ cudaError_t launch_gt_tc_prep(const Dev &d, u64 next_id, const float *q, u32 nq,
     return cudaGetLastError();
 }
 
-void gt_tc_configure(GtTcPlan &p, u32 nq, bool split) {
+void gt_tc_configure(GtTcPlan &p, u32 nq, u32 k, u32 mp, bool split, bool keys) {
     p.kprime = split ? p.kb : p.kp1;
     p.split = split;
     p.kblocks = p.kprime / TC_KBOX;
@@ -1176,6 +1272,18 @@ void gt_tc_configure(GtTcPlan &p, u32 nq, bool split) {
     // queries per pass: the block-minimum buffer stays under 4 GiB
     const u64 cap = std::max<u64>(256, ((4ull << 30) / ((u64)p.nblk * 4)) / 256 * 256);
     p.qgroup = (u32)std::min<u64>(nq, cap);
+    // Every key written costs 0.7 ns per 1000 rows and query (0.4 beside the
+    // longer K of a split); what the rerank then leaves out are 31 of 32 rows in
+    // at least k blocks, 4 mp bytes each: 960-d, 40k rows, 2,003 queries, k 10
+    // (split) tensor + rerank 1,140 -> 400 us; at 128-d, k 10, even at 20k rows
+    // (10k queries: 320 and 332 us), behind at 40k (2,003 queries: 96 and 127).
+    p.keys = keys && p.n_pad <= (u64)k * mp * (split ? 24 : 16);
+    if (p.keys) {
+        const u64 room = (4ull << 30) / (p.n_pad * 4) / TC_ROWS * TC_ROWS;   // queries in 4 GiB
+        p.keys = room > 0;
+        if (p.keys) p.qgroup = (u32)std::min<u64>(p.qgroup, room);
+    }
+    p.bytes_keys = p.keys ? (size_t)p.qgroup * p.n_pad * 4 : 0;
     p.bytes_bmin = (size_t)p.qgroup * p.nblk * 4;
     p.usable = true;
 }
@@ -1211,19 +1319,19 @@ cudaError_t launch_gt_tc(const Dev &d, u32 q0, u32 nq, const GtTcPlan &p, const 
     a.chunks = (p.n_tiles + a.tiles_per_chunk - 1) / a.tiles_per_chunk;
     a.stages = p.stages;
     a.stream_a = p.stream_a ? 1u : 0u;
-    a.all_keys = 0;
+    a.all_keys = p.keys ? 2u : 0u;
     a.ld = p.nblk;
     a.s = d.metric == 0 ? -2.0f : -1.0f;
     a.xn = b.xn;
     a.out = b.bmin;
+    a.keys = b.keys;
     a.err = b.err;
-    const void *fn = p.stream_a ? (const void *)gt_tc_kernel<true> : (const void *)gt_tc_kernel<false>;
-    cudaError_t e = smem_at_least(fn, p.smem);
+    auto *fn = p.stream_a ? (p.keys ? gt_tc_kernel<true, true> : gt_tc_kernel<true, false>)
+                          : (p.keys ? gt_tc_kernel<false, true> : gt_tc_kernel<false, false>);
+    cudaError_t e = smem_at_least((const void *)fn, p.smem);
     if (e != cudaSuccess) return e;
     const u32 items = a.m_tiles * a.chunks;
-    const u32 grid = std::min<u32>(items, (u32)num_sms);
-    if (p.stream_a) gt_tc_kernel<true><<<grid, TC_THREADS, p.smem, st>>>(ta, tb, a);
-    else gt_tc_kernel<false><<<grid, TC_THREADS, p.smem, st>>>(ta, tb, a);
+    fn<<<std::min<u32>(items, (u32)num_sms), TC_THREADS, p.smem, st>>>(ta, tb, a);
     return cudaGetLastError();
 }
 
@@ -1240,6 +1348,7 @@ cudaError_t launch_gt_rerank(const Dev &d, const float *q, u32 q0, u32 nq, u32 k
     r.n_rows = next_id;
     r.q = q;
     r.bmin = b.bmin;
+    r.keys = b.keys;
     r.qstat = b.qstat;
     r.gstat = b.gstat;
     r.out_ids = out_ids;
@@ -1247,9 +1356,15 @@ cudaError_t launch_gt_rerank(const Dev &d, const float *q, u32 q0, u32 nq, u32 k
     r.fb = b.fb;
     r.fb_count = b.gstat + 4;
     r.err = b.err;
-    // a block per query until a warp per query fills the SMs
-    if (nq < (u32)num_sms * 16) gt_rerank_kernel<RR_WARPS><<<nq, RR_WARPS * 32, 0, st>>>(d, r);
-    else gt_rerank_kernel<1><<<(nq + RR_WARPS - 1) / RR_WARPS, RR_WARPS * 32, 0, st>>>(d, r);
+    // the most warps per query that the SMs hold at once
+    u32 W = 1;
+    while (W < 8 && (u64)nq * 2 * W <= (u64)num_sms * 16) W *= 2;
+    const u32 grid = W == 1 ? (nq + rr_warps(1) - 1) / rr_warps(1) : nq;
+    auto go = [&](auto *fn) { fn<<<grid, rr_warps(W) * 32, 0, st>>>(d, r); };
+    if (W == 1) p.keys ? go(gt_rerank_kernel<1, true>) : go(gt_rerank_kernel<1, false>);
+    else if (W == 2) p.keys ? go(gt_rerank_kernel<2, true>) : go(gt_rerank_kernel<2, false>);
+    else if (W == 4) p.keys ? go(gt_rerank_kernel<4, true>) : go(gt_rerank_kernel<4, false>);
+    else p.keys ? go(gt_rerank_kernel<8, true>) : go(gt_rerank_kernel<8, false>);
     return cudaGetLastError();
 }
 
@@ -1324,12 +1439,11 @@ cudaError_t launch_seed_tc(const Dev &d, const float *q, u32 nq, u32 S, u32 L, u
     a.xn = b.en;
     a.out = b.keys;
     a.err = b.ctr + 1;
-    const void *fn = p.stream_a ? (const void *)gt_tc_kernel<true> : (const void *)gt_tc_kernel<false>;
-    e = smem_at_least(fn, p.smem);
+    auto *fn = p.stream_a ? gt_tc_kernel<true, false> : gt_tc_kernel<false, false>;
+    e = smem_at_least((const void *)fn, p.smem);
     if (e != cudaSuccess) return e;
     const u32 items = a.m_tiles * a.chunks;
-    if (p.stream_a) gt_tc_kernel<true><<<std::min<u32>(items, (u32)num_sms), TC_THREADS, p.smem, st>>>(ta, tb, a);
-    else gt_tc_kernel<false><<<std::min<u32>(items, (u32)num_sms), TC_THREADS, p.smem, st>>>(ta, tb, a);
+    fn<<<std::min<u32>(items, (u32)num_sms), TC_THREADS, p.smem, st>>>(ta, tb, a);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     SeedSelArgs r{};

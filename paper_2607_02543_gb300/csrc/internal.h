@@ -135,10 +135,11 @@ cudaError_t launch_ground_truth(const Dev &d, u64 next_id, const float *q, u32 n
 struct GtTcPlan {
     u32 kp1 = 0, kb = 0;            // one bf16 segment (dim rounded to 64); three segments
     u64 n_pad = 0;                  // rows rounded to 256
-    size_t bytes_A = 0, bytes_B = 0, bytes_bmin = 0;
+    size_t bytes_A = 0, bytes_B = 0, bytes_bmin = 0, bytes_keys = 0;
     u32 kprime = 0, kblocks = 0, bn = 0, stages = 0, smem = 0, n_tiles = 0, nblk = 0;
     u32 qgroup = 0;                 // queries per candidate pass
     bool split = false, usable = false;
+    bool keys = false;              // the candidate pass also writes every key
     bool stream_a = false;          // the query tile travels through the ring (K too large to stay resident)
 };
 struct GtTcBufs {
@@ -147,6 +148,7 @@ struct GtTcBufs {
     u32 *gstat;                     // [0..3] maxima and the split flag, [4] fallback count, [5] error word
     u32 *fb;                        // fallback query list
     float *bmin;                    // qgroup x nblk block minima
+    float *keys;                    // nblk x qgroup x 32 keys (GtTcPlan::keys)
     float *center;                  // mp floats: the vector taken from rows and queries (L2)
     u32 *err;
 };
@@ -172,7 +174,7 @@ cudaError_t launch_seed_tc(const Dev &d, const float *q, u32 nq, u32 S, u32 L, u
 GtTcPlan gt_tc_plan(u32 dim, u64 next_id, u32 nq);
 cudaError_t launch_gt_tc_prep(const Dev &d, u64 next_id, const float *q, u32 nq, const GtTcPlan &p,
                               const GtTcBufs &b, cudaStream_t st);
-void gt_tc_configure(GtTcPlan &p, u32 nq, bool split);
+void gt_tc_configure(GtTcPlan &p, u32 nq, u32 k, u32 mp, bool split, bool keys);
 cudaError_t launch_gt_tc(const Dev &d, u32 q0, u32 nq, const GtTcPlan &p, const GtTcBufs &b, u64 next_id,
                          int num_sms, cudaStream_t st);
 cudaError_t launch_gt_rerank(const Dev &d, const float *q, u32 q0, u32 nq, u32 k, const GtTcPlan &p,

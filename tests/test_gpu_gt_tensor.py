@@ -94,3 +94,36 @@ def test_rerank_team_shapes(n, nq, k, kind, dim):
             assert g.ground_truth_info()["fallback_queries"] == 0
     np.testing.assert_array_equal(res[0][0], res[1][0])
     np.testing.assert_array_equal(res[0][1].view(np.uint32), res[1][1].view(np.uint32))
+
+
+@pytest.mark.parametrize("n,nq,k,metric,dim,integer", [
+    (255, 1, 1, "l2", 32, True),           # one row tile, not full
+    (257, 127, 32, "ip", 64, True),        # two row tiles, ties and zero keys of both signs
+    (3_000, 129, 10, "l2", 129, False),    # two query tiles, rows longer than one column block
+    (9_999, 609, 10, "l2", 100, True),     # the last row count at which the keys are written ...
+    (20_481, 609, 10, "l2", 128, True),    # ... and the first beyond it
+    (4_000, 1_217, 32, "ip", 300, False),  # the query tile streams; one warp per query
+])
+def test_rerank_by_row_keys(n, nq, k, metric, dim, integer):
+    """Rows chosen by their own keys: the exact kernel's bits, with repeated and
+    all-zero rows and whole blocks deleted."""
+    from paper_2607_02543_gb300 import Index
+    rng = np.random.default_rng(n + nq)
+    c = rng.normal(0, 12, size=(7, dim))
+    draw = lambda m: c[rng.integers(0, 7, m)] + rng.normal(0, 3, size=(m, dim))
+    x, q = draw(n), draw(nq)
+    if integer:
+        x, q = np.clip(np.rint(x), -100, 100), np.clip(np.rint(q), -100, 100)
+    x[rng.integers(0, n, n // 5)] = x[rng.integers(0, n, n // 5)]
+    x[::17] = 0.0
+    q[::5] = 0.0
+    x, q = x.astype(np.float32), q.astype(np.float32)
+    dele = np.concatenate([np.arange(32, 96), np.arange(97, n, 11)]).astype(np.uint32)
+    res = []
+    for gt in ("default", "cuda_cores"):
+        g = Index(dim, metric, 8, n + 10, build_beam=16, max_cand=16, gt=gt)
+        g.insert(x)
+        g.delete(dele)
+        res.append(g.ground_truth(q, k))
+    np.testing.assert_array_equal(res[0][0], res[1][0])
+    np.testing.assert_array_equal(res[0][1].view(np.uint32), res[1][1].view(np.uint32))

@@ -5,11 +5,10 @@
 // round.  The contraction runs on the 5th-generation tensor cores:
 //
 //   1. gt_prep_rows / gt_prep_queries write bf16 copies of the live rows and
-//      the queries (x = hi + lo + e with hi, lo bf16; rows as [hi | lo | hi],
-//      queries as [hi | hi | lo], each segment padded to 64) and the norms an
-//      error bound needs.  When every lo is zero (data exactly
-//      representable in bf16, e.g. integers up to 256) only the first
-//      segment is used, otherwise all three (hi.hi + hi.lo + lo.hi).
+//      the queries (x = hi + lo + e with hi, lo bf16; both as [hi | lo], each
+//      segment padded to 64) and the norms an error bound needs.  When every
+//      lo is zero (data exactly representable in bf16, e.g. integers up to
+//      256) K runs over hi.hi only, otherwise over hi.hi + hi.lo + lo.hi.
 //   2. gt_tc_kernel: persistent CTAs; TMA (cp.async.bulk.tensor, 128-byte
 //      swizzle) streams 256-row boxes of the row copy through a shared
 //      memory ring while the query tile stays resident (or, when the query
@@ -64,6 +63,7 @@ __host__ __device__ constexpr u32 tc_idesc(u32 n) {
 
 struct TcArgs {
     u32 nq, n_tiles, kblocks, bn, m_tiles, chunks, tiles_per_chunk, stages;
+    u32 seg;              // column blocks of one segment: K runs over hi.hi, hi.lo, lo.hi (see a_col, b_col)
     u32 all_keys;         // 0: smallest key per block of 32 rows; 1: every key; 2: both, the keys in `keys`
     u32 stream_a;         // 1: the query boxes travel through the ring (selects gt_tc_kernel<true>)
     const u32 *nq_dev;    // when set, the batch size is read here (nq is its cap); later query tiles are skipped
@@ -148,6 +148,11 @@ __device__ __forceinline__ float pair_lo(u64 v) { return __uint_as_float((u32)v)
 __device__ __forceinline__ float pair_hi(u64 v) { return __uint_as_float((u32)(v >> 32)); }
 __device__ __forceinline__ void tmem_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
+// Column block of the query copy [hi | lo] and of the row copy [hi | lo] at step
+// kb of K: hi hi lo against hi lo hi.
+__device__ __forceinline__ u32 a_col(u32 kb, u32 seg) { return kb < seg ? kb : kb - seg; }
+__device__ __forceinline__ u32 b_col(u32 kb, u32 seg) { return kb < 2 * seg ? kb : kb - 2 * seg; }
+
 // ---- candidate pass ---------------------------------------------------------
 // Bound by the issue of the MMAs and their waits, then by the row boxes from L2
 // (a tile's 64 KB per 128 queries): 300k x 128 integer rows, 10k queries, 1.09
@@ -173,12 +178,13 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
     // items by every role
     const u32 nq_eff = a.nq_dev ? min(*a.nq_dev, a.nq) : a.nq;
     const u32 mt_eff = (nq_eff + TC_ROWS - 1) / TC_ROWS;
-    // resident: sA holds the query tile (kblocks boxes), then the ring of row
+    // resident: sA holds the query tile (one or two segments), then the ring of row
     // boxes; streamed: each ring stage is a row box followed by the query box
     // of the same 64 columns
     const u32 sbytes = bbox + (STREAM_A ? TC_BOX : 0u);
     unsigned char *sA = sm;
-    unsigned char *sB = sm + (STREAM_A ? 0u : (size_t)a.kblocks * TC_BOX);
+    const u32 aboxes = min(a.kblocks, 2 * a.seg);
+    unsigned char *sB = sm + (STREAM_A ? 0u : (size_t)aboxes * TC_BOX);
 
     if (threadIdx.x == 0) {
         for (u32 i = 0; i < a.stages; i++) {
@@ -232,8 +238,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
                 }
                 first = false;
                 if (leader) {
-                    mbar_expect_tx(&a_full, a.kblocks * TC_BOX);
-                    for (u32 kb = 0; kb < a.kblocks; kb++)
+                    mbar_expect_tx(&a_full, aboxes * TC_BOX);
+                    for (u32 kb = 0; kb < aboxes; kb++)
                         tma_load_2d(sA + (size_t)kb * TC_BOX, &tmA, (int)(kb * TC_KBOX), (int)(mt * TC_ROWS), &a_full);
                 }
                 __syncwarp();
@@ -256,9 +262,10 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
                     unsigned char *sb = sB + (size_t)stage * sbytes;
                     if (leader) {
                         mbar_expect_tx(&full[stage], sbytes);
-                        tma_load_2d(sb, &tmB, (int)(kb * TC_KBOX), (int)(t * a.bn), &full[stage]);
+                        tma_load_2d(sb, &tmB, (int)(b_col(kb, a.seg) * TC_KBOX), (int)(t * a.bn), &full[stage]);
                         if (STREAM_A)
-                            tma_load_2d(sb + bbox, &tmA, (int)(kb * TC_KBOX), (int)(mt * TC_ROWS), &full[stage]);
+                            tma_load_2d(sb + bbox, &tmA, (int)(a_col(kb, a.seg) * TC_KBOX), (int)(mt * TC_ROWS),
+                                        &full[stage]);
                     }
                     __syncwarp();
                     issued |= 1u << stage;
@@ -306,7 +313,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
                         if (!warp_wait(&full[stage], ph)) { ok = false; break; }
                         tc_fence_after();
                         const u64 bd = dB + (u64)(stage * sbytes >> 4);
-                        const u64 ad = STREAM_A ? bd + (bbox >> 4) : dA + (u64)(kb * (TC_BOX >> 4));
+                        const u64 ad = STREAM_A ? bd + (bbox >> 4) : dA + (u64)(a_col(kb, a.seg) * (TC_BOX >> 4));
 #pragma unroll
                         for (u32 k = 0; k < TC_KBOX / 16; k++)
                             tc_mma(acol, ad + 2 * k, bd + 2 * k, idesc, (kb | k) != 0, leader);
@@ -498,63 +505,122 @@ __global__ void __launch_bounds__(1024) gt_center_kernel(Dev d, u64 next_id, flo
 }
 
 // gstat: [0] max |x|^2, [1] max |lo_x|, [2] max |e_x| (fp32 bits), [3] any lo != 0.
-// A warp per row, grid-stride; maxima are kept per warp and published once.
+// A warp per row, grid-stride; maxima are kept per warp and published per block.
 // ids (optional): row c is node ids[c]; check_live: rows of deleted or
 // never-inserted nodes get key base +inf and a zero copy.
-__global__ void gt_prep_rows(Dev d, const u32 *ids, u64 next_id, u32 n_pad, bool check_live, u32 kp1, u32 kb, u32 *B,
-                             float *xn, u32 *gstat, const float *center) {
-    const int lane = lane_id();
+// Bound by the rows' bytes (4 m read, 4 m written; 3.5 and 4.3 TB/s).  Publishing
+// per warp was 80k atomics on one sector, a row's loads waited for its reference
+// word, and the copies held a third segment [hi | lo | hi]: 40k x 960 with queries
+// 119 -> 91 us, 300k x 128 105 -> 95.  The blocks that are resident, on rows that
+// lie together: four waves of blocks 97 and 105, a warp's four rows apart 133.
+// U rows of a warp in flight (4 for rows of one column block, each lane 16 bytes
+// of each; 1 else, with four column blocks in flight).
+constexpr int PREP_WARPS = 8;
+// Sums over the warp of U = 1 value (in every lane) or of U = 4 values (value
+// lane >> 3; a lane passes on half of what it still holds), the same additions.
+template <int U>
+__device__ __forceinline__ float row_sums(const float (&v)[U], int lane) {
+    float t = v[0];
+    if (U == 4) {
+        const bool hi = lane & 16, mid = lane & 8;
+        const float a0 = (hi ? v[2 % U] : v[0]) + __shfl_xor_sync(FULL, hi ? v[0] : v[2 % U], 16);
+        const float a1 = (hi ? v[3 % U] : v[1 % U]) + __shfl_xor_sync(FULL, hi ? v[1 % U] : v[3 % U], 16);
+        t = (mid ? a1 : a0) + __shfl_xor_sync(FULL, mid ? a0 : a1, 8);
+    }
+#pragma unroll
+    for (int h = U == 4 ? 4 : 16; h >= 1; h >>= 1) t += __shfl_xor_sync(FULL, t, h);
+    return t;
+}
+template <int U>
+__global__ void __launch_bounds__(PREP_WARPS * 32)
+    gt_prep_rows(Dev d, const u32 *ids, u64 next_id, u32 n_pad, bool check_live, u32 kp1, u32 kb, u32 *B, float *xn,
+                 u32 *gstat, const float *center) {
+    __shared__ float red[3][PREP_WARPS];
+    const int lane = lane_id(), warp = threadIdx.x >> 5;
     if (center && !gstat[6]) center = nullptr;
-    const u32 nwarps = (gridDim.x * blockDim.x) >> 5;
+    const u32 nwarps = gridDim.x * PREP_WARPS;
+    constexpr int V = 4 / U;   // column blocks of a row in flight
     float mx_sq = 0.0f, mx_lo = 0.0f, mx_e = 0.0f;
     bool any_lo = false;
-    for (u32 c = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; c < n_pad; c += nwarps) {
-        const u32 id = c < next_id ? (ids ? ids[c] : c) : 0u;
-        bool live = c < next_id;
-        if (live && check_live) {
-            const u64 rf = d.ref[id];
-            live = !ref_del(rf) && ref_slab(rf) != NIL;
+    for (u32 c0 = (blockIdx.x * PREP_WARPS + warp) * U; c0 < n_pad; c0 += U * nwarps) {
+        u32 id[U];
+        u64 rf[U];
+        bool live[U];
+        float sq[U], lo2[U], e2[U];
+#pragma unroll
+        for (int r = 0; r < U; r++) {
+            const u32 c = c0 + r;
+            live[r] = c < next_id;
+            id[r] = live[r] ? (ids ? ids[c] : c) : 0u;
+            rf[r] = check_live && live[r] ? d.ref[id[r]] : 0;
+            sq[r] = lo2[r] = e2[r] = 0.0f;
         }
-        float sq = 0.0f, lo2 = 0.0f, e2 = 0.0f;
         bool anylo = false;
-        if (c < next_id) {
-            const float *xr = d.x + (size_t)id * d.mp;
-            uint2 *br = reinterpret_cast<uint2 *>(B + (size_t)c * (kb / 2));
-            for (u32 i = 4 * lane; i < kp1; i += 128) {
-                const Split4 v = split4(load_row4(xr, i, d.dim, live, center));
-                br[i / 4] = v.hi;
-                br[(kp1 + i) / 4] = v.lo;
-                br[(2 * kp1 + i) / 4] = v.hi;
-                sq += v.sq;
-                lo2 += v.lo2;
-                e2 += v.e2;
-                anylo |= v.anylo;
+        for (u32 i0 = 4 * lane; i0 < kp1; i0 += 128 * V) {
+            float4 v[U][V];
+#pragma unroll
+            for (int r = 0; r < U; r++)
+#pragma unroll
+                for (int u = 0; u < V; u++) {
+                    const u32 i = i0 + 128 * u;
+                    v[r][u] = load_row4(d.x + (size_t)id[r] * d.mp, i, d.dim, i < kp1 && c0 + r < next_id, center);
+                }
+#pragma unroll
+            for (int r = 0; r < U; r++) {
+                const u32 c = c0 + r;
+                if (c >= next_id) break;
+                const bool on = !check_live || (!ref_del(rf[r]) && ref_slab(rf[r]) != NIL);
+                uint2 *br = reinterpret_cast<uint2 *>(B + (size_t)c * (kb / 2));
+#pragma unroll
+                for (int u = 0; u < V; u++) {
+                    const u32 i = i0 + 128 * u;
+                    if (i >= kp1) break;
+                    const Split4 w = split4(on ? v[r][u] : make_float4(0.f, 0.f, 0.f, 0.f));
+                    br[i / 4] = w.hi;
+                    br[(kp1 + i) / 4] = w.lo;
+                    sq[r] += w.sq;
+                    lo2[r] += w.lo2;
+                    e2[r] += w.e2;
+                    anylo |= w.anylo;
+                }
             }
         }
+        u32 live_bits = 0;
 #pragma unroll
-        for (int h = 16; h >= 1; h >>= 1) {
-            sq += __shfl_xor_sync(FULL, sq, h);
-            lo2 += __shfl_xor_sync(FULL, lo2, h);
-            e2 += __shfl_xor_sync(FULL, e2, h);
-        }
-        if (lane == 0) xn[c] = live ? (d.metric == 0 ? sq : 0.0f) : __int_as_float(0x7f800000);
-        if (live) {
-            mx_sq = fmaxf(mx_sq, sq);
-            mx_lo = fmaxf(mx_lo, sqrtf(lo2));
-            mx_e = fmaxf(mx_e, sqrtf(e2));
-            any_lo |= anylo;
+        for (int r = 0; r < U; r++)
+            live_bits |= (live[r] && (!check_live || (!ref_del(rf[r]) && ref_slab(rf[r]) != NIL)) ? 1u : 0u) << r;
+        const u32 mine = U == 4 ? lane >> 3 : 0;
+        const bool on = live_bits >> mine & 1;
+        const float n2 = row_sums<U>(sq, lane);
+        const u32 c = c0 + mine;
+        if ((U == 4 ? lane & 7 : lane) == 0 && c < n_pad) xn[c] = on ? (d.metric == 0 ? n2 : 0.0f) : __int_as_float(0x7f800000);
+        if (on) mx_sq = fmaxf(mx_sq, n2);
+        // the copy of a row that is not live is zero; without low parts the
+        // remainders are zero too
+        if (__any_sync(FULL, anylo)) {
+            any_lo = true;
+            mx_lo = fmaxf(mx_lo, row_sums<U>(lo2, lane));
+            mx_e = fmaxf(mx_e, row_sums<U>(e2, lane));
         }
     }
-    any_lo = __any_sync(FULL, any_lo);
+    // of values >= 0 (no NaN passes fmaxf) the bits are ordered as the values are
+    const u32 m_sq = __reduce_max_sync(FULL, __float_as_uint(mx_sq)), m_lo = __reduce_max_sync(FULL, __float_as_uint(mx_lo));
+    const u32 m_e = __reduce_max_sync(FULL, __float_as_uint(mx_e));
     if (lane == 0) {
-        if (mx_sq > 0.0f) atomicMax(gstat + 0, __float_as_uint(mx_sq));
-        if (mx_lo > 0.0f) atomicMax(gstat + 1, __float_as_uint(mx_lo));
-        if (mx_e > 0.0f) atomicMax(gstat + 2, __float_as_uint(mx_e));
-        if (any_lo) atomicOr(gstat + 3, 1u);
+        red[0][warp] = __uint_as_float(m_sq);
+        red[1][warp] = sqrtf(__uint_as_float(m_lo));
+        red[2][warp] = sqrtf(__uint_as_float(m_e));
     }
+    any_lo = __syncthreads_or(any_lo);
+    if (threadIdx.x < 3) {
+        float m = 0.0f;
+        for (int w = 0; w < PREP_WARPS; w++) m = fmaxf(m, red[threadIdx.x][w]);
+        if (m > 0.0f) atomicMax(gstat + threadIdx.x, __float_as_uint(m));
+    }
+    if (threadIdx.x == 3 && any_lo) atomicOr(gstat + 3, 1u);
 }
 
-// qstat per query: |q|^2, |q|, |lo_q|, |e_q|; copy as [hi | hi | lo]
+// qstat per query: |q|^2, |q|, |lo_q|, |e_q|; copy as [hi | lo]
 __global__ void gt_prep_queries(const float *q, u32 mp, u32 dim, u32 nq, u32 kp1, u32 kb, u32 *A, float *qstat,
                                 u32 *gstat, const float *center, const u32 *nq_dev) {
     const u32 r = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -568,8 +634,7 @@ __global__ void gt_prep_queries(const float *q, u32 mp, u32 dim, u32 nq, u32 kp1
     for (u32 i = 4 * lane; i < kp1; i += 128) {
         const Split4 v = split4(load_row4(qr, i, dim, true, center));
         ar[i / 4] = v.hi;
-        ar[(kp1 + i) / 4] = v.hi;
-        ar[(2 * kp1 + i) / 4] = v.lo;
+        ar[(kp1 + i) / 4] = v.lo;
         sq += v.sq;
         lo2 += v.lo2;
         e2 += v.e2;
@@ -587,7 +652,7 @@ __global__ void gt_prep_queries(const float *q, u32 mp, u32 dim, u32 nq, u32 kp1
         qstat[4 * (size_t)r + 1] = sqrtf(sq);
         qstat[4 * (size_t)r + 2] = sqrtf(lo2);
         qstat[4 * (size_t)r + 3] = sqrtf(e2);
-        if (anylo) atomicOr(gstat + 3, 1u);
+        if (anylo && !*reinterpret_cast<volatile u32 *>(gstat + 3)) atomicOr(gstat + 3, 1u);
     }
 }
 
@@ -1220,12 +1285,20 @@ bool encode_bf16(CUtensorMap *m, const void *base, u64 rows, u32 cols, u32 box_r
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+void prep_rows(const Dev &d, const u32 *ids, u64 next_id, u32 n_pad, bool check_live, u32 kp1, u32 kb, u32 *B, float *xn,
+               u32 *gstat, const float *center, cudaStream_t st) {
+    const u32 U = kp1 <= 128 ? 4 : 1;
+    const u32 grid = std::min<u32>((n_pad + PREP_WARPS * U - 1) / (PREP_WARPS * U), 152 * (U == 4 ? 3 : 4));   // resident blocks
+    auto *fn = U == 4 ? gt_prep_rows<4> : gt_prep_rows<1>;
+    fn<<<grid, PREP_WARPS * 32, 0, st>>>(d, ids, next_id, n_pad, check_live, kp1, kb, B, xn, gstat, center);
+}
+
 }  // namespace
 
 GtTcPlan gt_tc_plan(u32 dim, u64 next_id, u32 nq) {
     GtTcPlan p{};
     p.kp1 = (dim + TC_KBOX - 1) / TC_KBOX * TC_KBOX;
-    p.kb = 3 * p.kp1;
+    p.kb = 2 * p.kp1;
     p.n_pad = (next_id + TC_ACC - 1) / TC_ACC * TC_ACC;
     p.bytes_B = (size_t)next_id * p.kb * 2;
     p.bytes_A = (size_t)nq * p.kb * 2;
@@ -1239,17 +1312,18 @@ cudaError_t launch_gt_tc_prep(const Dev &d, u64 next_id, const float *q, u32 nq,
     const float *center = d.metric == 0 && next_id ? b.center : nullptr;
     if (center) gt_center_kernel<<<(d.mp + 31) / 32, dim3(32, 32), 0, st>>>(d, next_id, b.center, b.gstat);
     if (p.n_pad)
-        gt_prep_rows<<<(unsigned)std::min<u64>((p.n_pad * 32 + 255) / 256, 152 * 16), 256, 0, st>>>(
-            d, nullptr, next_id, (u32)p.n_pad, true, p.kp1, p.kb, reinterpret_cast<u32 *>(b.B), b.xn, b.gstat, center);
+        prep_rows(d, nullptr, next_id, (u32)p.n_pad, true, p.kp1, p.kb, reinterpret_cast<u32 *>(b.B), b.xn, b.gstat,
+                  center, st);
     gt_prep_queries<<<(unsigned)(((size_t)nq * 32 + 255) / 256), 256, 0, st>>>(
         q, d.mp, d.dim, nq, p.kp1, p.kb, reinterpret_cast<u32 *>(b.A), b.qstat, b.gstat, center, nullptr);
     return cudaGetLastError();
 }
 
 void gt_tc_configure(GtTcPlan &p, u32 nq, u32 k, u32 mp, bool split, bool keys) {
-    p.kprime = split ? p.kb : p.kp1;
+    p.kprime = split ? 3 * p.kp1 : p.kp1;
     p.split = split;
     p.kblocks = p.kprime / TC_KBOX;
+    const u32 abytes = (split ? 2 : 1) * (p.kp1 / TC_KBOX) * TC_BOX;
     const u32 smem_max = 227 * 1024 - 1024 - TC_STATIC;   // alignment slack, static shared memory
     p.bn = TC_ACC;
     const u32 bbox = p.bn * TC_KBOX * 2;
@@ -1259,13 +1333,13 @@ void gt_tc_configure(GtTcPlan &p, u32 nq, u32 k, u32 mp, bool split, bool keys) 
     }
     // the query tile stays resident when it fits beside two ring stages;
     // otherwise its boxes travel through the ring with the row boxes
-    p.stream_a = (u64)p.kblocks * TC_BOX + 2ull * bbox > smem_max;
+    p.stream_a = (u64)abytes + 2ull * bbox > smem_max;
     if (p.stream_a) {
         p.stages = std::min<u32>(TC_MAX_STAGES, smem_max / (bbox + TC_BOX));
         p.smem = p.stages * (bbox + TC_BOX) + 1024;
     } else {
-        p.stages = std::min<u32>(TC_MAX_STAGES, (smem_max - p.kblocks * TC_BOX) / bbox);
-        p.smem = p.kblocks * TC_BOX + p.stages * bbox + 1024;
+        p.stages = std::min<u32>(TC_MAX_STAGES, (smem_max - abytes) / bbox);
+        p.smem = abytes + p.stages * bbox + 1024;
     }
     p.n_tiles = (u32)(p.n_pad / p.bn);
     p.nblk = (u32)(p.n_pad / 32);
@@ -1298,6 +1372,7 @@ cudaError_t launch_gt_tc(const Dev &d, u32 q0, u32 nq, const GtTcPlan &p, const 
     a.nq = nq;
     a.n_tiles = p.n_tiles;
     a.kblocks = p.kblocks;
+    a.seg = p.kp1 / TC_KBOX;
     a.bn = p.bn;
     a.m_tiles = (nq + TC_ROWS - 1) / TC_ROWS;
     // chunks of rows: enough work items to fill every SM, with the fewest
@@ -1372,7 +1447,7 @@ cudaError_t launch_gt_rerank(const Dev &d, const float *q, u32 q0, u32 nq, u32 k
 SeedTcPlan seed_tc_plan(u32 dim, u32 n_entry, u32 nq) {
     SeedTcPlan p{};
     p.kp1 = (dim + TC_KBOX - 1) / TC_KBOX * TC_KBOX;
-    p.kb = 3 * p.kp1;
+    p.kb = 2 * p.kp1;
     p.s_pad = (n_entry + TC_ACC - 1) / TC_ACC * TC_ACC;
     const u32 smem_max = 227 * 1024 - 1024 - TC_STATIC;
     const u32 bbox = TC_ACC * TC_KBOX * 2;
@@ -1396,8 +1471,7 @@ SeedTcPlan seed_tc_plan(u32 dim, u32 n_entry, u32 nq) {
 cudaError_t launch_seed_tc_entries(const Dev &d, u32 S, const SeedTcPlan &p, const SeedTcBufs &b, cudaStream_t st) {
     cudaError_t e = cudaMemsetAsync(b.estat, 0, 8 * sizeof(u32), st);
     if (e != cudaSuccess || p.s_pad == 0) return e;
-    gt_prep_rows<<<(unsigned)std::min<u64>(((u64)p.s_pad * 32 + 255) / 256, 152 * 16), 256, 0, st>>>(
-        d, d.entries, S, p.s_pad, false, p.kp1, p.kb, reinterpret_cast<u32 *>(b.E), b.en, b.estat, nullptr);
+    prep_rows(d, d.entries, S, p.s_pad, false, p.kp1, p.kb, reinterpret_cast<u32 *>(b.E), b.en, b.estat, nullptr, st);
     return cudaGetLastError();
 }
 
@@ -1414,7 +1488,8 @@ cudaError_t launch_seed_tc(const Dev &d, const float *q, u32 nq, u32 S, u32 L, u
     TcArgs a{};
     a.nq = nq;
     a.n_tiles = p.s_pad / TC_ACC;
-    a.kblocks = p.kb / TC_KBOX;
+    a.seg = p.kp1 / TC_KBOX;
+    a.kblocks = 3 * a.seg;
     a.bn = TC_ACC;
     a.m_tiles = (nq + TC_ROWS - 1) / TC_ROWS;
     u32 best_c = 1;
@@ -1452,7 +1527,7 @@ cudaError_t launch_seed_tc(const Dev &d, const float *q, u32 nq, u32 S, u32 L, u
     r.S = S;
     r.ld = p.s_pad;
     r.m = d.dim;
-    r.kprime = p.kb;
+    r.kprime = 3 * p.kp1;
     r.q = q;
     r.keys = b.keys;
     r.qstat = b.qstat;

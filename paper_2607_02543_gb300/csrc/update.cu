@@ -38,8 +38,7 @@ struct Stage {
 // Tensor-core Gram tile: up to 64 candidates, K staged 128 columns at a time
 // as bf16 rows of 256 bytes with no pad; the 16-byte chunk c of row r sits at
 // chunk c ^ (r & 7), so the eight rows an ldmatrix phase reads at one column
-// fall in eight distinct bank groups.  The 64 x 64 fp32 result (row stride
-// GRAM_N floats, also 256 bytes) reuses the same bytes.
+// fall in eight distinct bank groups.
 constexpr int GRAM_N = 64;
 constexpr int GRAM_RB = 256;   // bytes per staged row (128 bf16 columns)
 // The cooperative path (more than GRAM_N rows, or rows of more than one
@@ -56,7 +55,7 @@ __host__ __device__ inline int gram_variant(u32 gram_rows, u32 mp) {
 // Variant 3, canonical distances on the cooperative path, keeps masks only: its
 // buffer is that of CANON_ROWS "rows".
 constexpr u32 CANON_ROWS = 0x80000000u | GRAM_NL;
-// Bytes of a Gram buffer's rows (or the table over them), and of the whole
+// Bytes of a Gram buffer's rows, and of the whole
 // buffer: a (norm, rho) pair per candidate follows, and on the cooperative path
 // its domination mask (two words).  rows is a multiple of 16; 0 = no buffer.
 __host__ __device__ inline size_t gram_row_bytes(u32 rows, u32 mp) {
@@ -203,148 +202,125 @@ __device__ __forceinline__ void gram_stage_rows(const Dev &d, const u64 *ck, int
     __syncwarp();
 }
 
-// Column swizzle of the Gram table: entry (r, c) sits at column c ^ gram_tsw(r),
-// so the eight rows of an accumulator fragment store to four bank groups
-// (two wavefronts instead of eight), while a walk along rows (lane h reading
-// (h, h + 1 + k)) still hits 32 distinct banks.
-__device__ __forceinline__ int gram_tsw(int r) { return (r & 3) << 3; }
-
-// Writes the upper triangle (j >= i, in 16 x 8 tiles) of the n x n Gram of rows
-// of one 128-column block into T (fp32, row stride GRAM_N, columns swizzled by
-// gram_tsw) and the diagonal into nr2[i].x, with rho_i (the candidate's key
-// distance) in nr2[i].y.  T and the bf16 rows share `buf`: the stripes go in
-// ascending order, and stripe mt's table rows (bytes [4096 mt, 4096 (mt + 1)))
-// are the staged rows of that same stripe, which no later stripe reads (it
-// reads rows >= 16 (mt + 1)).  A stripe only needs the columns j >= 16 mt,
-// because the prune reads T[head][j] for j > head.  Rows past n hold whatever
-// the buffer held: an entry (i, j) reads rows i and j only, and no entry with
-// i or j >= n is read.
-// (The loop over column blocks runs once here.  Without it, and with the
-// staging ahead of the stripes, the kernels take 10 to 25 registers more and
-// lose resident warps.)
-__device__ void warp_gram(const Dev &d, const u64 *ck, int n, char *buf, int rows, float *&T, float2 *&nr2) {
+// RobustPrune on the Gram of rows of one 128-column block: same rule and order
+// as warp_prune.  First the domination masks: row i's mask holds the later
+// candidates j > i that i would drop (alpha^2 * d(i, j) <= rho(j)).  The 16-row
+// stripes go from the last to the first, so that a stripe finds every norm it
+// needs (the diagonal of its own and of later stripes) and turns its sums into
+// mask bits where they are, in registers; a quad's lanes hold the columns of two
+// rows, and lane k of it ends with one word of them.  The greedy pass is a
+// warp-uniform walk over a 64-bit alive mask, from one candidate that drops
+// something to the next; of what is left the first R are the result (a
+// candidate drops only later ones, so those after the R-th change nothing).
+// Bound by the instructions of one warp (12 to 16 warps an SM, 2 to 3 ready
+// cycles of 7).  With the sums stored as a table that each lane then walked a row
+// of, and a step of the walk per kept candidate, 300k repairs took 2.02 ms
+// against 1.71, the offers of 10k inserts 1.13 against 1.06.
+__device__ int warp_prune_gram(const Dev &d, const u64 *ck, int n, u32 *out_id, float *out_rho, Stage &st) {
     const int lane = lane_id();
-    T = reinterpret_cast<float *>(buf);
-    nr2 = reinterpret_cast<float2 *>(buf + (size_t)rows * GRAM_RB);
+    float2 *nr2 = reinterpret_cast<float2 *>(st.gram + (size_t)st.gram_rows * GRAM_RB);   // .x: the norms, .y: rho
     const int nm = (n + 15) >> 4, nn = (n + 7) >> 3;
-    const int nkb = ((int)d.mp + 127) >> 7;
-    const u32 xs = smem_addr(buf), c0 = gram_c0(lane);
-    for (int mt = 0; mt < nm; mt++) {
+    const u32 xs = smem_addr(st.gram), c0 = gram_c0(lane);
+    const float alpha2 = d.alpha2;
+    const bool l2 = d.metric == 0;
+    const int cq = 2 * (lane & 3), rq = lane >> 2;
+    const u64 in_n = n < 64 ? (1ull << n) - 1 : ~0ull;
+    u32 mw[4] = {0u, 0u, 0u, 0u};
+    for (int i = lane; i < n; i += 32) nr2[i].y = key_rho(ck[i]);
+    gram_stage_rows(d, ck, 0, n, 0, xs);
+    for (int mt = nm - 1; mt >= 0; mt--) {
+        // tile t: rows 16 mt + .., columns 16 mt + 8 t + ..; rows past n hold
+        // whatever the buffer held, and their bits are cleared below
         float acc[8][4];
 #pragma unroll
         for (int b = 0; b < 8; b++)
 #pragma unroll
             for (int c = 0; c < 4; c++) acc[b][c] = 0.f;
-        for (int kb = 0; kb < nkb; kb++) {
-            // rows [16 mt, n) of this column block: all rows once when one
-            // block covers the row, else this stripe's and later ones per block
-            if (nkb > 1 || mt == 0) gram_stage_rows(d, ck, 16 * mt, n, kb, xs);
+        const u32 xm = xs + (u32)(16 * mt + (lane & 7) + 8 * ((lane >> 3) & 1)) * GRAM_RB;
 #pragma unroll
-            for (int ks = 0; ks < 8; ks++) {
-                u32 a0, a1, a2, a3;
-                const u32 ko = (u32)(32 * ks) ^ c0;
-                const int ar = 16 * mt + (lane & 7) + 8 * ((lane >> 3) & 1);
-                ldsm_x4(a0, a1, a2, a3, xs + (u32)ar * GRAM_RB + ko);
+        for (int ks = 0; ks < 8; ks++) {
+            u32 a0, a1, a2, a3;
+            const u32 ko = (u32)(32 * ks) ^ c0;
+            ldsm_x4(a0, a1, a2, a3, xm + ko);
 #pragma unroll
-                for (int nt = 0; nt < 8; nt += 2) {
-                    if (nt < 2 * mt || nt >= nn) continue;
-                    // matrices: (nt, k 0-7), (nt + 1, k 0-7), (nt, k 8-15), (nt + 1, k 8-15)
-                    u32 b0, b1, b2, b3;
-                    const int br = 8 * nt + (lane & 7) + 8 * ((lane >> 3) & 1);
-                    ldsm_x4(b0, b1, b2, b3, xs + (u32)br * GRAM_RB + ko);
-                    mma_bf16_16816(acc[nt], a0, a1, a2, a3, b0, b2);
-                    mma_bf16_16816(acc[nt + 1], a0, a1, a2, a3, b1, b3);
-                }
+            for (int t = 0; t < 8; t += 2) {
+                if (2 * mt + t >= nn) continue;
+                // matrices: (t, k 0-7), (t + 1, k 0-7), (t, k 8-15), (t + 1, k 8-15)
+                u32 b0, b1, b2, b3;
+                ldsm_x4(b0, b1, b2, b3, xm + (u32)(8 * t) * GRAM_RB + ko);
+                mma_bf16_16816(acc[t], a0, a1, a2, a3, b0, b2);
+                mma_bf16_16816(acc[t + 1], a0, a1, a2, a3, b1, b3);
             }
         }
-        __syncwarp();
-        // this stripe's table rows, over this stripe's staged rows (rows r and
-        // r + 8 share the column swizzle)
-#pragma unroll
-        for (int nt = 0; nt < 8; nt++) {
-            if (nt < 2 * mt || nt >= nn) continue;
-            const int r = 16 * mt + (lane >> 2), c = (8 * nt + 2 * (lane & 3)) ^ gram_tsw(r);
-            *reinterpret_cast<float2 *>(T + r * GRAM_N + c) = make_float2(acc[nt][0], acc[nt][1]);
-            *reinterpret_cast<float2 *>(T + (r + 8) * GRAM_N + c) = make_float2(acc[nt][2], acc[nt][3]);
+        // the diagonal: entry (r, r) of rows rq in tile 0, of rows rq + 8 in tile 1
+        const int r0 = 16 * mt + rq;
+        if (cq == rq || cq + 1 == rq) {
+            nr2[r0].x = cq == rq ? acc[0][0] : acc[0][1];
+            nr2[r0 + 8].x = cq == rq ? acc[1][2] : acc[1][3];
         }
         __syncwarp();
+        const float n0 = nr2[r0].x, n1 = nr2[r0 + 8].x;
+        u32 m[2][2] = {{0u, 0u}, {0u, 0u}};   // row rq, row rq + 8: bits 8 t + h
+#pragma unroll
+        for (int t = 0; t < 8; t++) {
+            if (2 * mt + t >= nn) continue;
+            const float4 v = *reinterpret_cast<const float4 *>(nr2 + 16 * mt + 8 * t + cq);
+            // (n_i - g) + (n_j - g): every intermediate stays as small as the result
+            auto hit = [&](float ni, float g, float nj, float rho) {
+                const float dd = l2 ? __fadd_rn(__fsub_rn(ni, g), __fsub_rn(nj, g)) : __fsub_rn(1.0f, g);
+                return __fmul_rn(alpha2, dd) <= rho;
+            };
+            const u32 b = 1u << (8 * (t & 3));
+            if (hit(n0, acc[t][0], v.x, v.y)) m[0][t >> 2] |= b;
+            if (hit(n0, acc[t][1], v.z, v.w)) m[0][t >> 2] |= 2u * b;
+            if (hit(n1, acc[t][2], v.x, v.y)) m[1][t >> 2] |= b;
+            if (hit(n1, acc[t][3], v.z, v.w)) m[1][t >> 2] |= 2u * b;
+        }
+        // to columns of the whole list, then words (row rq + 8 (lane & 1), half
+        // (lane >> 1) & 1)
+        const u64 w0 = (((u64)m[0][1] << 32) | m[0][0]) << cq << (16 * mt);
+        const u64 w1 = (((u64)m[1][1] << 32) | m[1][0]) << cq << (16 * mt);
+        const bool odd = lane & 1, up = lane & 2;
+        const u64 p = (odd ? w1 : w0) | __shfl_xor_sync(FULL, odd ? w0 : w1, 1);
+        const u32 w = (u32)(up ? p >> 32 : p) | __shfl_xor_sync(FULL, (u32)(up ? p : p >> 32), 2);
+        const u64 later = (~0ull << (r0 + 8 * (lane & 1)) << 1) & in_n;
+        const u32 word = w & (u32)(up ? later >> 32 : later);
+#pragma unroll
+        for (int k = 0; k < 4; k++)
+            if (k == mt) mw[k] = word;
     }
-    for (int i = lane; i < n; i += 32) nr2[i] = make_float2(T[i * GRAM_N + (i ^ gram_tsw(i))], key_rho(ck[i]));
+    __syncwarp();   // the rows are read: their last bytes take the masks
+    u64 *dom = reinterpret_cast<u64 *>(st.gram + (size_t)st.gram_rows * GRAM_RB - GRAM_N * 8);
+#pragma unroll
+    for (int k = 0; k < 4; k++)
+        if (k < nm) reinterpret_cast<u32 *>(dom + 16 * k + rq + 8 * (lane & 1))[(lane >> 1) & 1] = mw[k];
     __syncwarp();
-}
-
-// RobustPrune on a Gram table: same rule and order as warp_prune.  First the
-// domination masks: row i's mask holds the later candidates j > i that i would
-// drop (alpha^2 * d(i, j) <= rho(j)).  Lane l builds the mask of row l and,
-// when n - 2 - l >= 32, of row n - 2 - l, walking each row's columns upward
-// (lane l reads column row + 1 + k in step k: distinct banks).  The masks go
-// to the last 512 bytes of the buffer's row area (the table is read by then); the
-// greedy pass is a warp-uniform walk over a 64-bit alive mask (take the first
-// alive candidate, clear the ones it drops), and the kept candidates are
-// written out afterwards, a lane per candidate.
-__device__ int warp_prune_gram(const Dev &d, const u64 *ck, int n, unsigned char *alive, u32 *out_id,
-                               float *out_rho, Stage &st) {
-    (void)alive;
-    const int lane = lane_id();
-    float *T;
-    float2 *nr2;
-    warp_gram(d, ck, n, st.gram, st.gram_rows, T, nr2);
-    const float alpha2 = d.alpha2;
-    const bool l2 = d.metric == 0;
-    // (n_h - g) + (n_j - g): every intermediate stays as small as the result
-    auto hit = [&](float nh, float g, int j) {
-        const float2 v = nr2[j];
-        const float dd = l2 ? __fadd_rn(__fsub_rn(nh, g), __fsub_rn(v.x, g)) : __fsub_rn(1.0f, g);
-        return __fmul_rn(alpha2, dd) <= v.y;
-    };
-    u64 dom_a = 0ull, dom_b = 0ull;
-    const int ra = lane, rb = n - 2 - lane;
-    if (ra < n - 1) {
-        const float *Ta = T + ra * GRAM_N;
-        const float na = nr2[ra].x;
-        const int sw = gram_tsw(ra);
-#pragma unroll 4
-        for (int j = ra + 1; j < n; j++)
-            if (hit(na, Ta[j ^ sw], j)) dom_a |= 1ull << j;
-    }
-    if (rb >= 32) {
-        const float *Tb = T + rb * GRAM_N;
-        const float nb = nr2[rb].x;
-        const int sw = gram_tsw(rb);
-#pragma unroll 4
-        for (int j = rb + 1; j < n; j++)
-            if (hit(nb, Tb[j ^ sw], j)) dom_b |= 1ull << j;
-    }
-    __syncwarp();   // the table is read: its last bytes take the masks
-    u64 *dsm = reinterpret_cast<u64 *>(st.gram + (size_t)st.gram_rows * GRAM_RB - GRAM_N * 8);
-    if (ra < n) dsm[ra] = dom_a;
-    if (rb >= 32) dsm[rb] = dom_b;
-    if (lane == 0 && n - 1 >= 32) dsm[n - 1] = 0ull;   // the last row drops nothing
     // equal adjacent keys collapse to one
-    u64 live = 0ull;
+    u64 live = 0ull, act = 0ull;
     for (int i0 = 0; i0 < n; i0 += 32) {
         const int i = i0 + lane;
         const u32 b = __ballot_sync(FULL, i < n && (i == 0 || ck[i] != ck[i - 1]));
+        const u32 a = __ballot_sync(FULL, i < n && dom[i] != 0);
         live |= (u64)b << i0;
+        act |= (u64)a << i0;
     }
-    __syncwarp();
-    u64 kept = 0ull;
-    int nout = 0;
-    const int R = (int)d.R;
-    while (nout < R && live) {
-        const u64 low = live & (0ull - live);
-        const int head = __ffsll((long long)live) - 1;
-        kept |= low;
-        nout++;
-        live = (live ^ low) & ~dsm[head];
+    for (u64 todo = live & act; todo;) {
+        const int head = __ffsll((long long)todo) - 1;
+        todo &= todo - 1;
+        const u64 m = ~dom[head];
+        live &= m;
+        todo &= m;
     }
+    const int nout = min(__popcll(live), (int)d.R);
     for (int i0 = 0; i0 < n; i0 += 32) {
         const int i = i0 + lane;
-        if (i < n && (kept >> i & 1)) {
-            const int pos = __popcll(kept & ((1ull << i) - 1));
+        if (i < n && (live >> i & 1)) {
+            const int pos = __popcll(live & ((1ull << i) - 1));
             const u64 hk = ck[i];
-            out_id[pos] = key_id(hk);
-            out_rho[pos] = key_rho(hk);
+            if (pos < nout) {
+                out_id[pos] = key_id(hk);
+                out_rho[pos] = key_rho(hk);
+            }
         }
     }
     __syncwarp();
@@ -681,7 +657,7 @@ __device__ int warp_prune(const Dev &d, const u64 *ck, int n, unsigned char *ali
                           float *out_rho, Stage &st) {
     if (st.gram && n <= st.gram_rows) {
         if constexpr (GV != 0) return warp_prune_masks<GV>(d, ck, n, out_id, out_rho, st);
-        else return warp_prune_gram(d, ck, n, alive, out_id, out_rho, st);
+        else return warp_prune_gram(d, ck, n, out_id, out_rho, st);
     }
     const int lane = lane_id();
     const int grp = lane >> 3, g = lane & 7;
@@ -943,10 +919,10 @@ __host__ __device__ inline size_t prune_ins_warp_bytes(u32 np, u32 R, u32 ns, u3
     return stage_bytes(ns, mp) + al16((size_t)np * 8) + (gram_alias(gram, sc) ? 0 : sc) + gram_bytes(gram, mp);
 }
 
-// one-warp blocks of the single-warp variant (GV 0) are held to 12 resident warps
-// per SM (at most 170 registers a thread)
+// one-warp blocks of the single-warp variant (GV 0) are held to 16 resident warps
+// per SM (at most 128 registers a thread)
 template <int GV>
-__global__ void __launch_bounds__(GV ? 32 * COOP_WARPS : 32, GV ? 3 : 12) prune_insert_kernel(PruneInsArgs a) {
+__global__ void __launch_bounds__(GV ? 32 * COOP_WARPS : 32, GV ? 3 : 16) prune_insert_kernel(PruneInsArgs a) {
     extern __shared__ __align__(16) char smem[];
     __shared__ GramReq req;
     const int lane = lane_id();
@@ -1086,10 +1062,10 @@ __host__ __device__ inline size_t fold_warp_bytes(u32 np, u32 R, u32 ns, u32 mp,
            (gram_alias(gram, sc) ? 0 : sc) + gram_bytes(gram, mp);
 }
 
-// one-warp blocks of the single-warp variant (GV 0) are held to 12 resident warps
-// per SM (at most 170 registers a thread)
+// one-warp blocks of the single-warp variant (GV 0) are held to 16 resident warps
+// per SM (at most 128 registers a thread)
 template <int GV>
-__global__ void __launch_bounds__(GV ? 32 * COOP_WARPS : 32, GV ? 3 : 12) offer_fold_kernel(FoldArgs a) {
+__global__ void __launch_bounds__(GV ? 32 * COOP_WARPS : 32, GV ? 3 : 16) offer_fold_kernel(FoldArgs a) {
     extern __shared__ __align__(16) char smem[];
     __shared__ GramReq req;
     const int lane = lane_id();

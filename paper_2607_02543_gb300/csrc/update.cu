@@ -1503,7 +1503,7 @@ struct RepairKArgs {
 
 constexpr int REPK_WARPS = 4;
 __host__ __device__ inline size_t repk_bytes(u32 R) {
-    return 2 * al16((size_t)R * 4) + al16((size_t)R * R * 4) + REPK_WARPS * 64;
+    return 2 * al16((size_t)R * 4) + al16((size_t)R * R * 4) + REPK_WARPS * (R <= 32 ? 32 * 8 : 64);
 }
 
 // The greedy RobustPrune of B \ {a} about a = member ja of B, from the table M,
@@ -1511,10 +1511,10 @@ __host__ __device__ inline size_t repk_bytes(u32 R) {
 // by counting the smaller keys (ids differ); then, for every candidate, the
 // mask of the later ones it would drop (no step waits for the one before); the
 // walk visits only candidates whose mask is not empty.  Writes K in order and
-// returns its size.  H: candidates per lane (nb <= 32 H).
-template <int H>
-__device__ __forceinline__ int repair_select(const Dev &d, const float *M, const u32 *bid, const u32 *bdel, int nb,
+// returns its size.  nb <= 64, H candidates per lane.
+__device__ __forceinline__ int repair_select64(const Dev &d, const float *M, const u32 *bid, const u32 *bdel, int nb,
                                              int ja, unsigned char *ord, uint2 *K) {
+    constexpr int H = 2;
     const int lane = lane_id();
     const u32 R = d.R;
     u64 k[H];
@@ -1568,7 +1568,7 @@ __device__ __forceinline__ int repair_select(const Dev &d, const float *M, const
     while (any) {
         const int h = __ffsll((long long)any) - 1;
         any &= any - 1;
-        const u64 m = __shfl_sync(FULL, H == 1 || h < 32 ? dom[0] : dom[H - 1], h & 31);
+        const u64 m = __shfl_sync(FULL, h < 32 ? dom[0] : dom[1], h & 31);
         if (alive >> h & 1) alive &= ~m;
     }
 #pragma unroll
@@ -1579,6 +1579,46 @@ __device__ __forceinline__ int repair_select(const Dev &d, const float *M, const
     }
     __syncwarp();                        // ord is free again
     return __popcll(alive);
+}
+
+// The same for nb <= 32.  Lane c holds its column of alpha^2 M in registers (am)
+// and collects, over all b, the earlier candidates (E) and those of them that would
+// drop c (D).  A candidate is kept when none of D is: all that is decided by what
+// is known is decided at once, so the steps are as many as the longest chain of
+// candidates, not one for each; a kept candidate's place is the kept ones in E.
+// 10,000 nodes of 128-d (R = 32) 664 -> 336 us against the form above; with two
+// candidates per lane and the table in shared memory it is the slower one (500
+// nodes of 768-d, R = 64: 318 against 247).
+__device__ __forceinline__ int repair_select32(const float *M, const float (&am)[32], const u32 *bid, const u32 *bdel,
+                                               u32 R, int nb, int ja, u64 *okey, uint2 *K) {
+    const int lane = lane_id();
+    const bool v = lane < nb && lane != ja && !bdel[lane];
+    const float rho = v ? M[ja * R + lane] : 0.0f;
+    const u64 k = v ? mkkey(rho, bid[lane]) : KEY_INF;
+    okey[lane] = k;
+    __syncwarp();
+    u32 E = 0, D = 0;
+#pragma unroll
+    for (int g = 0; g < 4; g++) {
+        if (8 * g >= nb) break;
+#pragma unroll
+        for (int b = 8 * g; b < 8 * g + 8; b++) {
+            const bool lt = okey[b] < k;             // KEY_INF where b is no candidate
+            if (lt) E |= 1u << b;
+            if (lt && am[b] <= rho) D |= 1u << b;
+        }
+    }
+    u32 kept = __ballot_sync(FULL, v && D == 0), open = __ballot_sync(FULL, v && D != 0);
+    while (open) {
+        open &= ~__ballot_sync(FULL, (open >> lane & 1) && (D & kept));
+        // no kept candidate drops what is left; one that none of the open drop is kept
+        const u32 m = open & ~__ballot_sync(FULL, (open >> lane & 1) && (D & open));
+        kept |= m;
+        open &= ~m;
+    }
+    if (kept >> lane & 1) K[__popc(E & kept)] = make_uint2(bid[lane], __float_as_uint(rho));
+    __syncwarp();                        // okey is free again
+    return __popc(kept);
 }
 
 // A block per deleted node.  The distances among B are computed in 8 x 8 tiles
@@ -1598,7 +1638,8 @@ __global__ void __launch_bounds__(32 * REPK_WARPS, 3) repair_k_kernel(RepairKArg
     u32 *bid = reinterpret_cast<u32 *>(p); p += al16((size_t)R * 4);
     u32 *bdel = reinterpret_cast<u32 *>(p); p += al16((size_t)R * 4);
     float *M = reinterpret_cast<float *>(p); p += al16((size_t)R * R * 4);
-    unsigned char *ord = reinterpret_cast<unsigned char *>(p);   // a warp's candidates in order
+    u64 *okey = reinterpret_cast<u64 *>(p) + warp * 32;                        // H = 1: a warp's candidate keys
+    unsigned char *ord = reinterpret_cast<unsigned char *>(p) + warp * 64;   // H = 2: its candidates in order
     const u64 nd = *a.n_dt;
     const u32 invalid = (u32)d.capacity;
     u64 wk_rows = 0, wk_state = 0;
@@ -1640,10 +1681,18 @@ __global__ void __launch_bounds__(32 * REPK_WARPS, 3) repair_k_kernel(RepairKArg
         }
         __syncthreads();
         // K(u, a), a warp per a
+        float am[32];
+        if (H == 1) {
+#pragma unroll
+            for (int b = 0; b < 32; b++) am[b] = b < nb ? __fmul_rn(d.alpha2, M[b * R + min(lane, nb - 1)]) : 0.0f;
+        }
         for (int ja = warp; ja < (int)R; ja += REPK_WARPS) {
             const size_t slot = (size_t)i * R + ja;
             int nk = -1;
-            if (ja < nb && !bdel[ja]) nk = repair_select<H>(d, M, bid, bdel, nb, ja, ord + warp * 64, a.pair_K + slot * R);
+            if (ja < nb && !bdel[ja]) {
+                if constexpr (H == 1) nk = repair_select32(M, am, bid, bdel, R, nb, ja, okey, a.pair_K + slot * R);
+                else nk = repair_select64(d, M, bid, bdel, nb, ja, ord, a.pair_K + slot * R);
+            }
             if (lane == 0) {
                 a.pair_key[slot] = nk < 0 ? invalid : bid[ja];
                 a.pair_val[slot] = (u32)slot;

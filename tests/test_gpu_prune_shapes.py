@@ -31,6 +31,7 @@ def _rounds(g, o, rng, n, m, integer, R):
 
 @pytest.mark.parametrize("m,metric,R,max_cand", [
     (1, "l2", 2, 0),
+    (24, "l2", 9, 0),         # a second group of eight candidates with one member
     (100, "ip", 33, 128),     # the most rows of a cooperative canonical prune
     (127, "l2", 32, 64),
     (128, "l2", 64, 65),      # lists longer than a warp, folds of up to 127 candidates

@@ -808,7 +808,10 @@ etale_status etale_destroy(etale_index *idx) {
                       &idx->pair_val2, &idx->pair_K, &idx->pair_Kn, &idx->pair_flags, &idx->pair_scan,
                       &idx->pair_seg, &idx->counts, &idx->ex_del, &idx->ex_hs, &idx->ex_deg, &idx->ex_ids,
                       &idx->ex_rho, &idx->seed, &idx->s_stage, &idx->s_qpad, &idx->s_out_ids, &idx->s_out_dist,
-                      &idx->s_seed};
+                      &idx->s_seed, &idx->refine_spill, &idx->gt_A, &idx->gt_B, &idx->gt_xn, &idx->gt_qstat,
+                      &idx->gt_gstat, &idx->gt_fb, &idx->gt_bmin, &idx->gt_keys, &idx->gt_center, &idx->sd_E,
+                      &idx->sd_en, &idx->sd_estat, &idx->sd_A, &idx->sd_qstat, &idx->sd_keys, &idx->sd_fb,
+                      &idx->sd_ctr};
     for (DevBuf *b : bufs)
         if (b->p) cudaFree(b->p);
     delete idx;

@@ -127,3 +127,19 @@ def test_rerank_by_row_keys(n, nq, k, metric, dim, integer):
         res.append(g.ground_truth(q, k))
     np.testing.assert_array_equal(res[0][0], res[1][0])
     np.testing.assert_array_equal(res[0][1].view(np.uint32), res[1][1].view(np.uint32))
+
+
+def test_close_gives_the_workspaces_back():
+    """Ground truth, seeding and round workspaces (about 60 MB here) do not outlive their index."""
+    import torch
+    from paper_2607_02543_gb300 import Index
+    x = np.random.default_rng(1).normal(size=(4_000, 128)).astype(np.float32)
+    free = []
+    for _ in range(3):
+        g = Index(128, "l2", 32, 5_000, build_beam=32, n_entry=512, mode="lockfree")
+        g.insert(x)
+        g.ground_truth(x, 10)
+        g.search(x, 10, 32)
+        g.close()
+        free.append(torch.cuda.mem_get_info()[0])
+    assert free[0] - free[2] < 16 << 20, free   # the first pass pays for the context's own allocations

@@ -52,6 +52,7 @@ __host__ __device__ inline u32 gram_xoff(int r, int chunk) { return (u32)(r * GR
 __host__ __device__ inline int gram_variant(u32 gram_rows, u32 mp) {
     return gram_rows >> 31 ? 3 : gram_rows > (u32)GRAM_N ? 1 : (gram_rows && mp > 128 ? 2 : 0);
 }
+__host__ __device__ constexpr bool coop_variant(int GV) { return GV >= 1 && GV <= 3; }
 // Variant 3, canonical distances on the cooperative path, keeps masks only: its
 // buffer is that of CANON_ROWS "rows".
 constexpr u32 CANON_ROWS = 0x80000000u | GRAM_NL;
@@ -212,9 +213,9 @@ __device__ __forceinline__ void gram_stage_rows(const Dev &d, const u64 *ck, int
 // warp-uniform walk over a 64-bit alive mask, from one candidate that drops
 // something to the next; of what is left the first R are the result (a
 // candidate drops only later ones, so those after the R-th change nothing).
-// Bound by the instructions of one warp (12 to 16 warps an SM, 2 to 3 ready
-// cycles of 7).  With the sums stored as a table that each lane then walked a row
-// of, and a step of the walk per kept candidate, 300k repairs took 2.02 ms
+// Bound by the instructions of one warp (12 to 16 warps an SM, each issuing every
+// 7 to 9 cycles).  With the sums stored as a table that each lane then walked a
+// row of, and a step of the walk per kept candidate, 300k repairs took 2.02 ms
 // against 1.71, the offers of 10k inserts 1.13 against 1.06.
 __device__ int warp_prune_gram(const Dev &d, const u64 *ck, int n, u32 *out_id, float *out_rho, Stage &st) {
     const int lane = lane_id();
@@ -651,12 +652,13 @@ __device__ int warp_prune_masks(const Dev &d, const u64 *ck, int n, u32 *out_id,
 // GV, the Gram variant of a kernel: 0, a buffer of at most GRAM_N rows with
 // rows of one 128-column block, a warp per item; 1, more than GRAM_N rows, and
 // 2, at most GRAM_N rows spanning several blocks: the block's four warps on one
-// item (see gram_masks); 3, the same on canonical distances (see canon_masks).
+// item (see gram_masks); 3, the same on canonical distances (see canon_masks); 4,
+// canonical distances by a warp per item, in a kernel without the Gram's code.
 template <int GV>
 __device__ int warp_prune(const Dev &d, const u64 *ck, int n, unsigned char *alive, u32 *idx, u32 *out_id,
                           float *out_rho, Stage &st) {
-    if (st.gram && n <= st.gram_rows) {
-        if constexpr (GV != 0) return warp_prune_masks<GV>(d, ck, n, out_id, out_rho, st);
+    if (GV != 4 && st.gram && n <= st.gram_rows) {
+        if constexpr (coop_variant(GV)) return warp_prune_masks<GV>(d, ck, n, out_id, out_rho, st);
         else return warp_prune_gram(d, ck, n, out_id, out_rho, st);
     }
     const int lane = lane_id();
@@ -848,12 +850,14 @@ __device__ int apply_offer(const Dev &d, u32 *ids, float *rho, int n, u32 v, flo
     st.wk_rows += prune_row_bytes(d, st, cn);
     // No entry of a pruned list drops a later one: only v's tests are open.
     // The entries before it may drop it, else it may drop those after it.
-    // Variant 3 only: 32 distances where the greedy walk computes 528 (rounds
-    // of 100 + 100 on 10k x 128, deterministic: the offers 258 -> 76 us).  On
-    // the Gram tile the same short cut was no faster: what bounds an offer there
-    // is its chain of loads, fence and compare-and-swap; and in variant 0 the
-    // code alone costs the lock-free folds a quarter (128 -> 161 registers).
-    if (GV == 3 && pruned && d.same_tests) {
+    // Canonical variants only: 32 distances where the greedy walk computes 528
+    // (rounds of 100 + 100 on 10k x 128, deterministic: the offers 258 -> 76 us).
+    // On the Gram tile the same short cut was no faster: what bounds an offer
+    // there is its chain of loads, fence and compare-and-swap; and in variant 0
+    // the code alone costs the lock-free folds a quarter (128 -> 161 registers),
+    // so larger canonical launches have variant 4 (deterministic loads of 44k x
+    // 120 and 125k x 42 rows 126 -> 75 and 189 -> 120 ms).
+    if (GV >= 3 && pruned && d.same_tests) {
         float *dv = reinterpret_cast<float *>(idx);
         canon_row_dists(d.x, d.mp, d.metric, keys, nl, below, v, dv);
         bool lost = false;
@@ -1065,7 +1069,8 @@ __host__ __device__ inline size_t fold_warp_bytes(u32 np, u32 R, u32 ns, u32 mp,
 // one-warp blocks of the single-warp variant (GV 0) are held to 16 resident warps
 // per SM (at most 128 registers a thread)
 template <int GV>
-__global__ void __launch_bounds__(GV ? 32 * COOP_WARPS : 32, GV ? 3 : 16) offer_fold_kernel(FoldArgs a) {
+__global__ void __launch_bounds__(coop_variant(GV) ? 32 * COOP_WARPS : 32, coop_variant(GV) ? 3 : GV == 4 ? 12 : 16)
+    offer_fold_kernel(FoldArgs a) {
     extern __shared__ __align__(16) char smem[];
     __shared__ GramReq req;
     const int lane = lane_id();
@@ -1073,7 +1078,8 @@ __global__ void __launch_bounds__(GV ? 32 * COOP_WARPS : 32, GV ? 3 : 16) offer_
     const u32 R = d.R;
     char *p = smem;
     char *gbuf = a.gram ? p : nullptr;
-    if (GV != 0 && threadIdx.x >= 32) return gram_helper<GV>(d, gbuf, a.gram, &req);
+    if constexpr (coop_variant(GV))
+        if (threadIdx.x >= 32) return gram_helper<GV>(d, gbuf, a.gram, &req);
     p += gram_bytes(a.gram, d.mp);
     Stage st = stage_init(p, a.ns, d.mp, gbuf, a.gram, &req);
     WarpSlabs ws;
@@ -1150,7 +1156,7 @@ __global__ void __launch_bounds__(GV ? 32 * COOP_WARPS : 32, GV ? 3 : 16) offer_
         }
         __syncwarp();
     }
-    if (GV != 0) gram_release(&req);
+    if (coop_variant(GV)) gram_release(&req);
     ws_finish(d, ws);
     stage_done(d, st, WK_OFFER);
 }
@@ -1171,7 +1177,7 @@ cudaError_t launch_offer_fold(const Dev &d, const Offers &of, const u32 *seg_sta
     const int threads = block_threads(a.gram, d.mp);
     const void *fns[4] = {(const void *)offer_fold_kernel<0>, (const void *)offer_fold_kernel<1>, (const void *)offer_fold_kernel<2>,
                           (const void *)offer_fold_kernel<3>};
-    const void *fn = fns[gram_variant(a.gram, d.mp)];
+    const void *fn = !d.gram && !a.gram ? (const void *)offer_fold_kernel<4> : fns[gram_variant(a.gram, d.mp)];
     cudaError_t e = smem_at_least((const void *)fn, smem);
     if (e != cudaSuccess) return e;
     int per_sm = 0;
@@ -1625,8 +1631,9 @@ __device__ __forceinline__ int repair_select32(const float *M, const float (&am)
 // of pairs, a warp per tile: lane j sums partial j of the tile's 64 pairs, so
 // that each 128-column block of 16 rows serves 64 pairs from registers.  Bound
 // by the fp32 arithmetic of the table (the stored edge distances have to be
-// canonical); a warp per node, four pairs at a time from shared memory, took
-// 682 us for 10,000 nodes of 128-d (R = 32) and 2,590 for 500 of 768-d (R = 64).
+// canonical) and the selections: 336 us for 10,000 nodes of 128-d (R = 32), 246 for
+// 500 of 768-d (R = 64), where a warp per node, four pairs at a time from shared
+// memory, took 682 and 2,590.
 template <int H>   // members of B per lane: R <= 32 H
 __global__ void __launch_bounds__(32 * REPK_WARPS, 3) repair_k_kernel(RepairKArgs a) {
     extern __shared__ __align__(16) char smem[];

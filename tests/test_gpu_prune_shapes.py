@@ -58,3 +58,15 @@ def test_tile_prunes_of_exact_data_equal_oracle(oracle_mod, m, metric, R, max_ca
     g, o = make_pair(oracle_mod, m, metric, R, 800, build_beam=64, n_entry=32, max_cand=max_cand, max_batch=70,
                      gram="tensor")
     _rounds(g, o, rng, 800, m, True, R)
+
+
+@pytest.mark.parametrize("m,metric,R", [(24, "l2", 64), (130, "ip", 33)])
+def test_canonical_offers_of_large_batches_equal_oracle(oracle_mod, m, metric, R):
+    """More offers than the cooperative prunes take (64 per SM): a warp per list."""
+    rng = np.random.default_rng(m)
+    g, o = make_pair(oracle_mod, m, metric, R, 1600, build_beam=64, n_entry=32, max_batch=512)
+    for n in (1100, 500):
+        x = _rows(rng, n, m, False)
+        g.insert(x)
+        o.insert(x)
+        assert graphs_equal(g.export_graph(), o.dump(), R) == []

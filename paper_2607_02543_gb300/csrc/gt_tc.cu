@@ -806,8 +806,8 @@ __device__ __noinline__ void score_rows(const float *x, u32 mp, u32 metric, cons
 // once: 2,003 queries x 40k x 960 with 1, 2, 4, 8 warps 88, 98, 140, 237 us, 300
 // queries 57, 42, 39, 42.
 // KEYS: the candidate pass left every key, and of a candidate block only the rows
-// below the threshold are scored: the 960-d batch 866 -> 88 us (with the case's
-// wider clusters 2.9 -> 0.1 ms).
+// below the threshold are scored: the 960-d batch 866 -> 88 us, the same sizes of
+// the non-negative mixture 2.9 -> 0.2 ms.
 // Each lane keeps the four smallest minima of the blocks it reads, with their
 // numbers, so that a threshold met by at most four blocks of any lane needs no
 // second pass over the minima.

@@ -894,13 +894,16 @@ __device__ int apply_offer(const Dev &d, u32 *ids, float *rho, int n, u32 v, flo
 // Forward edges: F_v = RobustPrune(C_v) with C_v the expanded non-tombstone
 // nodes of v's search (nearest max_cand); Publish(v, F_v); emit offers.
 // ---------------------------------------------------------------------------
-// The Gram rows of a launch whose prunes see at most max_n candidates: without
-// the Gram, variant 3 while the items leave SMs idle.  (Its blocks hold three
-// items per SM where one-warp blocks hold up to 16, but an item's prune takes a
-// tenth of the time.)
+// The Gram rows of a launch whose prunes see at most max_n candidates.  Without
+// the Gram, variant 3 for rows of more than 128 floats, and for shorter ones while
+// the items leave SMs idle: its blocks hold three items per SM where one-warp
+// blocks hold up to 16, but an item's prune takes a tenth of the time, at 768-d
+// less.  40k x 768, R = 64, rounds of 1,000 + 1,000: the repair fold 83 ms with a
+// warp per item, 21 with variant 3, the offers 38 and 3.0; 100k x 128, R = 32, of
+// 2,000 + 2,000: the repair fold 2.84 (variant 4) and 2.90, the offers 0.40 and 0.83.
 inline u32 prune_rows_for(const Dev &d, u32 max_n, u64 items, int num_sms) {
     if (d.gram) return gram_rows_for(d.gram, max_n);
-    return max_n <= (u32)GRAM_NL && items <= 64ull * num_sms ? CANON_ROWS : 0u;
+    return max_n <= (u32)GRAM_NL && (d.mp > 128 || items <= 64ull * num_sms) ? CANON_ROWS : 0u;
 }
 struct PruneInsArgs {
     Dev d;
@@ -1840,7 +1843,8 @@ __device__ int repair_apply(const Dev &d, u32 *lid, float *lrho, int n, u32 u, c
 // one-warp blocks of the single-warp variant (GV 0) are held to 12 resident warps
 // per SM (at most 170 registers a thread)
 template <int GV>
-__global__ void __launch_bounds__(GV ? 32 * COOP_WARPS : 32, GV ? 3 : 12) repair_fold_kernel(RepairFoldArgs a) {
+__global__ void __launch_bounds__(coop_variant(GV) ? 32 * COOP_WARPS : 32, coop_variant(GV) ? 3 : 12)
+    repair_fold_kernel(RepairFoldArgs a) {
     extern __shared__ __align__(16) char smem[];
     __shared__ GramReq req;
     const int lane = lane_id();
@@ -1848,7 +1852,8 @@ __global__ void __launch_bounds__(GV ? 32 * COOP_WARPS : 32, GV ? 3 : 12) repair
     const u32 R = d.R;
     char *p = smem;
     char *gbuf = a.gram ? p : nullptr;
-    if (GV != 0 && threadIdx.x >= 32) return gram_helper<GV>(d, gbuf, a.gram, &req);
+    if constexpr (coop_variant(GV))
+        if (threadIdx.x >= 32) return gram_helper<GV>(d, gbuf, a.gram, &req);
     p += gram_bytes(a.gram, d.mp);
     Stage st = stage_init(p, a.ns, d.mp, gbuf, a.gram, &req);
     WarpSlabs ws;
@@ -1926,7 +1931,7 @@ __global__ void __launch_bounds__(GV ? 32 * COOP_WARPS : 32, GV ? 3 : 12) repair
         }
         __syncwarp();
     }
-    if (GV != 0) gram_release(&req);
+    if (coop_variant(GV)) gram_release(&req);
     ws_finish(d, ws);
     stage_done(d, st, WK_REPAIR_FOLD);
 }
@@ -1947,7 +1952,7 @@ cudaError_t launch_repair_fold(const Dev &d, const u32 *dt, const u32 *pair_key,
     const int threads = block_threads(a.gram, d.mp);
     const void *fns[4] = {(const void *)repair_fold_kernel<0>, (const void *)repair_fold_kernel<1>, (const void *)repair_fold_kernel<2>,
                           (const void *)repair_fold_kernel<3>};
-    const void *fn = fns[gram_variant(a.gram, d.mp)];
+    const void *fn = !d.gram && !a.gram ? (const void *)repair_fold_kernel<4> : fns[gram_variant(a.gram, d.mp)];
     cudaError_t e = smem_at_least((const void *)fn, smem);
     if (e != cudaSuccess) return e;
     int per_sm = 0;

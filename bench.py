@@ -105,19 +105,19 @@ def workload(name: str, n_live: int = 0) -> W.Workload:
 
 # DRAM bytes per BeamSearch expansion of the query-mode launch on the 1M x 128
 # workload, from the full-size ncu capture in
-# profiles/search_kernel_int256-1m-d128_dram.md (9,384,713,728 bytes over
+# profiles/search_kernel_int256-1m-d128_dram.md (7,443,644,928 bytes over
 # 1,287,324 expansions at beam 128); a launch's traffic is this figure times
 # its expansions.  Valid only for the search.cu revision it was taken on
 # (first 16 hex digits of SHA-256).
-SEARCH_DRAM_BYTES_PER_EXPANSION = {"int256-1m-d128": (9_384_713_728 / 1_287_324, "d44d14f8e67edf2a")}
+SEARCH_DRAM_BYTES_PER_EXPANSION = {"int256-1m-d128": (7_443_644_928 / 1_287_324, "5ce2cd5cfe123d30")}
 
 
 # DRAM bytes of each writer kernel over one round of 10,000 deletes + 10,000
 # inserts on the 1M x 128 workload (the same capture; offer_fold: the insert
 # offers and the refine offers).  Valid only for the update.cu revision given.
-WRITER_DRAM_BYTES = {"int256-1m-d128": ({"prune": 94_937_088, "offer_fold": 456_001_536, "refine": 84_663_296,
-                                         "repair_k": 173_829_120, "repair_fold": 822_004_736,
-                                         "compact": 295_891_456}, "d1687973a1e58402")}
+WRITER_DRAM_BYTES = {"int256-1m-d128": ({"prune": 94_624_768, "offer_fold": 455_926_784, "refine": 84_606_976,
+                                         "repair_k": 183_053_824, "repair_fold": 821_861_632,
+                                         "compact": 296_081_152}, "537c8dabd00f37f4")}
 
 
 def writer_traffic(workload_name: str):
